@@ -810,7 +810,7 @@ int apf_solve_S_grad_batch(apf_ctx *const *ctx, int nb, int objective, const dou
         cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), s);
     }
     cudaEventRecord(c0->ev[0], s);
-    for (int b = 0; b < nb; ++b) launch_boundary(ctx[b], s);
+    launch_boundary_n(ctx, nb, s);
     cudaEventRecord(c0->ev[1], s);
     int rc = mixed_eliminate_n(ctx, nb, s);
     if (rc != APF_OK) { cudaStreamSynchronize(s); return rc; }

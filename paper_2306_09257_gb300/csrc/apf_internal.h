@@ -38,6 +38,8 @@ __host__ __device__ __forceinline__ float2 fmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+constexpr int APF_MAX_BATCH = 16;  // designs per apf_solve_S_grad_batch call
+
 // ---------------------------------------------------------------------------
 // Grid description passed by value to kernels.
 // ---------------------------------------------------------------------------
@@ -162,6 +164,7 @@ GridDev make_grid(const apf_ctx *c);
 
 // boundary.cu
 void launch_boundary(apf_ctx *c, cudaStream_t s);
+void launch_boundary_n(apf_ctx *const *cs, int nb, cudaStream_t s);  // contexts of one grid
 void launch_build_rhs(apf_ctx *c, double2 *E, cudaStream_t s);
 void launch_adjoint_rhs(apf_ctx *c, const double2 *Gamma, double2 *E, cudaStream_t s);
 void launch_source_row(apf_ctx *c, double2 *q, cudaStream_t s);
@@ -200,7 +203,6 @@ int mixed_eliminate(apf_ctx *c, cudaStream_t s);
 int mixed_fields_begin(apf_ctx *c, cudaStream_t s);
 int mixed_refine(apf_ctx *c, cudaStream_t s);
 // the same steps for a batch of designs (shared launches), see apf_solve_S_grad_batch
-constexpr int APF_MAX_BATCH = 16;
 int mixed_eliminate_n(apf_ctx *const *cs, int nb, cudaStream_t s);
 int mixed_fields_begin_n(apf_ctx *const *cs, int nb, cudaStream_t s);
 int mixed_refine_n(apf_ctx *const *cs, int nb, cudaStream_t s, int *rcs);
