@@ -144,11 +144,12 @@ static int ensure_workspace(apf_ctx *c) {
     AL(c->d_modes, 4 * nx); AL(c->d_stretch, 2 * (c->ny + 1)); AL(c->d_coef, ncol); AL(c->d_circ, 2 * nx); AL(c->d_tw, nx / 2);
     if (c->precision == APF_FP64) {
         AL(c->d_G, h * nx * nx);
-        AL(c->d_scr1, nx * nx / 2); AL(c->d_scr2, nx * nx / 2);
+        AL(c->d_scr1, nx * nx); AL(c->d_scr2, nx * nx);
+        AL(c->d_T, 2 * std::max<long long>(ncol, nin) * nx);
     }
     // fields: the single-elimination solve's n_in + n_out columns, or the
     // conventional adjoint method's n_in forward and n_in adjoint columns
-    AL(c->d_E, h * std::max<long long>(ncol, 2LL * nin) * nx); AL(c->d_T, ncol * nx); AL(c->d_fft, ncol * nx);
+    AL(c->d_E, h * std::max<long long>(ncol, 2LL * nin) * nx); AL(c->d_fft, ncol * nx);
     if (c->precision != APF_FP64) { AL(c->d_R, h * ncol * nx); }
     AL(c->d_S, (long long)nout * nin); AL(c->d_Gam, (long long)nout * nin);
     AL(c->d_Q, h * nout * nx); AL(c->d_grad, h * nx);
@@ -445,24 +446,6 @@ int apf_get_stats(const apf_ctx *c, apf_stats *st) {
 // ---------------------------------------------------------------------------
 // Solve pipeline
 // ---------------------------------------------------------------------------
-void fields64(apf_ctx *c, cudaStream_t s) {
-    int nf = c->cf, ncol = c->cf + c->ca;
-    long long nx = c->nx, L = (long long)ncol * nx, nn = nx * nx;
-    double2 *E = c->d_Ew;
-    const double2 one = cmk(1, 0), zero = cmk(0, 0);
-    // forward chain Y_j = G_{j-1} Y_{j-1} (forward columns; Y_0 = R_0)
-    for (int j = 1; j < c->h; ++j)
-        zgemm(c, false, false, nf, c->nx, c->nx, one, E + (j - 1) * L, nx, 0, c->d_G + (j - 1) * nn, nx, 0,
-              zero, E + j * L, nx, 0, 1, s);
-    // back substitution E_{h-1} = G_{h-1} Y_{h-1}; E_j = G_j (Y_j + E_{j+1})
-    for (int j = c->h - 1; j >= 0; --j) {
-        if (j == c->h - 1) launch_copy(c, c->d_T, E + j * L, L, s);
-        else launch_add(c, c->d_T, E + j * L, E + (j + 1) * L, L, s);
-        zgemm(c, false, false, ncol, c->nx, c->nx, one, c->d_T, nx, 0, c->d_G + j * nn, nx, 0, zero,
-              E + j * L, nx, 0, 1, s);
-    }
-}
-
 // Everything up to the first host synchronization: boundary elimination, slab
 // elimination and the first field sweep of the current column layout (0 or 1).
 // Captured once per layout into a CUDA graph.
@@ -474,12 +457,7 @@ static int main_body(apf_ctx *c, cudaStream_t s) {
     record_event(c, c->ev[1], s);
     int rc = APF_OK;
     if (c->precision == APF_FP64) {
-        long long nx = c->nx, nn = nx * nx;
-        for (int j = 0; j < c->h; ++j) {
-            double2 *X = c->d_G + j * nn;
-            launch_assemble64(c, j, X, j > 0 ? c->d_G + (j - 1) * nn : nullptr, s);
-            invert_sym64(c, X, c->nx, nx, c->d_scr1, c->d_scr2, s);
-        }
+        eliminate64(c, s);
     } else {
         rc = mixed_eliminate(c, s);
         if (rc != APF_OK) return rc;

@@ -99,9 +99,9 @@ struct apf_ctx {
     double2 *d_circ = nullptr;   // 2*nx: circulant generators of Sigma_bot, Sigma_top
     double2 *d_tw = nullptr;     // nx/2 twiddles exp(-2 pi i k / nx)
     double2 *d_G = nullptr;      // h*nx*nx   (float64 mode)
-    double2 *d_scr1 = nullptr, *d_scr2 = nullptr;  // recursion scratch, nx*nx/2 each
+    double2 *d_scr1 = nullptr, *d_scr2 = nullptr;  // recursion scratch, nx*nx each (two blocks at a time)
     double2 *d_E = nullptr;      // h*ncol*nx fields, [row][column][x]
-    double2 *d_T = nullptr;      // ncol*nx temp
+    double2 *d_T = nullptr;      // 2*ncol*nx temp (float64 mode)
     double2 *d_R = nullptr;      // h*ncol*nx residual (mixed)
     double2 *d_S = nullptr, *d_Gam = nullptr;  // n_out*n_in
     double2 *d_qsrc = nullptr;   // nx: source-row coefficient q[m] of the substrate side
@@ -177,14 +177,13 @@ void launch_fft(apf_ctx *c, const double2 *in, double2 *out, int n, int batch, l
 int fft_smem_bytes(int n);
 
 // slab64.cu
-void launch_assemble64(apf_ctx *c, int row, double2 *X, const double2 *Gprev, cudaStream_t s);
-void zgemm(apf_ctx *c, bool ta, bool tb, int M, int N, int K, double2 alpha,
+void zgemm(apf_ctx *c, bool ta, bool sym, int M, int N, int K, double2 alpha,
            const double2 *A, long long lda, long long sA,
            const double2 *B, long long ldb, long long sB, double2 beta,
-           double2 *C, long long ldc, long long sC, int batch, cudaStream_t s);
-void invert_sym64(apf_ctx *c, double2 *X, int n, long long ld, double2 *scr1, double2 *scr2, cudaStream_t s);
-void launch_add(apf_ctx *c, double2 *T, const double2 *a, const double2 *b, long long n, cudaStream_t s);
-void launch_copy(apf_ctx *c, double2 *dst, const double2 *src, long long n, cudaStream_t s);
+           double2 *C, long long ldc, long long sC, int batch, cudaStream_t s, int M2 = 0);
+void eliminate64(apf_ctx *c, cudaStream_t s);
+void launch_add(apf_ctx *c, double2 *T, const double2 *a, long long da, const double2 *b, long long db, long long n,
+                int nz, cudaStream_t s);
 void launch_zero(apf_ctx *c, void *dst, long long bytes, cudaStream_t s);
 
 void fields64(apf_ctx *c, cudaStream_t s);

@@ -137,10 +137,10 @@ extern "C" int apf_solve_S_noalloc(int nx, int ny, int npml_bot, int npml_top, d
     c.d_circ = (double2 *)carve(sizeof(double2) * 2 * n);
     c.d_tw = (double2 *)carve(sizeof(double2) * n / 2);
     c.d_G = (double2 *)carve(sizeof(double2) * h * n * n);
-    c.d_scr1 = (double2 *)carve(sizeof(double2) * n * n / 2);
-    c.d_scr2 = (double2 *)carve(sizeof(double2) * n * n / 2);
+    c.d_scr1 = (double2 *)carve(sizeof(double2) * n * n);
+    c.d_scr2 = (double2 *)carve(sizeof(double2) * n * n);
     c.d_E = (double2 *)carve(sizeof(double2) * h * ncol * n);
-    c.d_T = (double2 *)carve(sizeof(double2) * ncol * n);
+    c.d_T = (double2 *)carve(sizeof(double2) * 2 * ncol * n);
     c.d_fft = (double2 *)carve(sizeof(double2) * ncol * n);
     c.d_S = (double2 *)carve(sizeof(double2) * n_in * n_out);
     c.d_flags = (int *)carve(sizeof(int) * 4);
@@ -158,11 +158,7 @@ extern "C" int apf_solve_S_noalloc(int nx, int ny, int npml_bot, int npml_top, d
     }
     launch_twiddles(&c, s);
     launch_boundary(&c, s);
-    for (int j = 0; j < h; ++j) {
-        double2 *X = c.d_G + (long long)j * n * n;
-        launch_assemble64(&c, j, X, j > 0 ? c.d_G + (long long)(j - 1) * n * n : nullptr, s);
-        invert_sym64(&c, X, nx, n, c.d_scr1, c.d_scr2, s);
-    }
+    eliminate64(&c, s);
     launch_zero(&c, c.d_E, sizeof(double2) * h * ncol * n, s);  // the fields must start at zero
     launch_build_rhs(&c, c.d_E, s);
     fields64(&c, s);
