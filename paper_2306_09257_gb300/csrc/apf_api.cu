@@ -150,7 +150,7 @@ static int ensure_workspace(apf_ctx *c) {
     // fields: the single-elimination solve's n_in + n_out columns, or the
     // conventional adjoint method's n_in forward and n_in adjoint columns
     AL(c->d_E, h * std::max<long long>(ncol, 2LL * nin) * nx); AL(c->d_fft, ncol * nx);
-    if (c->precision != APF_FP64) { AL(c->d_R, h * ncol * nx); }
+    if (c->precision != APF_FP64) { AL(c->d_R, 2 * std::max<long long>(ncol, nin) * nx); }
     AL(c->d_S, (long long)nout * nin); AL(c->d_Gam, (long long)nout * nin);
     AL(c->d_Q, h * nout * nx); AL(c->d_grad, h * nx);
     AL(c->d_f, 8); AL(c->d_colnorm, 2 * ncol); AL(c->d_flags, 4);
@@ -446,6 +446,14 @@ int apf_get_stats(const apf_ctx *c, apf_stats *st) {
 // ---------------------------------------------------------------------------
 // Solve pipeline
 // ---------------------------------------------------------------------------
+// Mixed mode: only the first and the last slab row of the right-hand side are
+// not zero; d_R holds these two.
+static void build_rhs_rows(apf_ctx *c, cudaStream_t s) {
+    const int rows = std::min(c->h, 2);
+    launch_zero(c, c->d_R, sizeof(double2) * rows * (long long)(c->cf + c->ca) * c->nx, s);
+    launch_build_rhs(c, c->d_R, rows, s);
+}
+
 // Everything up to the first host synchronization: boundary elimination, slab
 // elimination and the first field sweep of the current column layout (0 or 1).
 // Captured once per layout into a CUDA graph.
@@ -463,11 +471,14 @@ static int main_body(apf_ctx *c, cudaStream_t s) {
         if (rc != APF_OK) return rc;
     }
     record_event(c, c->ev[2], s);
-    launch_zero(c, c->d_Ew, sizeof(double2) * c->h * L, s);
-    launch_build_rhs(c, c->d_Ew, s);
-    if (c->precision == APF_FP64) fields64(c, s);
-    else rc = mixed_fields_begin(c, s);
-    return rc;
+    if (c->precision == APF_FP64) {
+        launch_zero(c, c->d_Ew, sizeof(double2) * c->h * L, s);
+        launch_build_rhs(c, c->d_Ew, c->h, s);
+        fields64(c, s);
+        return APF_OK;
+    }
+    build_rhs_rows(c, s);
+    return mixed_fields_begin(c, s);
 }
 
 // Second pass of the conventional adjoint method (layout 2): the adjoint
@@ -475,9 +486,12 @@ static int main_body(apf_ctx *c, cudaStream_t s) {
 // sweep through the stored elimination.
 static int adjoint_body(apf_ctx *c, cudaStream_t s) {
     long long L = (long long)(c->cf + c->ca) * c->nx;
-    launch_zero(c, c->d_Ew, sizeof(double2) * c->h * L, s);
-    launch_adjoint_rhs(c, c->d_Gam, c->d_Ew + (long long)(c->h - 1) * L, s);
-    if (c->precision == APF_FP64) {
+    const bool f64 = c->precision == APF_FP64;
+    const int rows = f64 ? c->h : std::min(c->h, 2);  // mixed: the first and last row only, in d_R
+    double2 *R = f64 ? c->d_Ew : c->d_R;
+    launch_zero(c, R, sizeof(double2) * rows * L, s);
+    launch_adjoint_rhs(c, c->d_Gam, R + (long long)(rows - 1) * L, s);
+    if (f64) {
         fields64(c, s);
         return APF_OK;
     }
@@ -793,11 +807,7 @@ int apf_solve_S_grad_batch(apf_ctx *const *ctx, int nb, int objective, const dou
     int rc = mixed_eliminate_n(ctx, nb, s);
     if (rc != APF_OK) { cudaStreamSynchronize(s); return rc; }
     cudaEventRecord(c0->ev[2], s);
-    for (int b = 0; b < nb; ++b) {
-        apf_ctx *c = ctx[b];
-        launch_zero(c, c->d_Ew, sizeof(double2) * c->h * (long long)(c->cf + c->ca) * c->nx, s);
-        launch_build_rhs(c, c->d_Ew, s);
-    }
+    for (int b = 0; b < nb; ++b) build_rhs_rows(ctx[b], s);
     rc = mixed_fields_begin_n(ctx, nb, s);
     if (rc != APF_OK) { cudaStreamSynchronize(s); return rc; }
     int rcs[APF_MAX_BATCH] = {};

@@ -102,7 +102,7 @@ struct apf_ctx {
     double2 *d_scr1 = nullptr, *d_scr2 = nullptr;  // recursion scratch, nx*nx each (two blocks at a time)
     double2 *d_E = nullptr;      // h*ncol*nx fields, [row][column][x]
     double2 *d_T = nullptr;      // 2*ncol*nx temp (float64 mode)
-    double2 *d_R = nullptr;      // h*ncol*nx residual (mixed)
+    double2 *d_R = nullptr;      // 2*ncol*nx right-hand side, first and last slab row (mixed)
     double2 *d_S = nullptr, *d_Gam = nullptr;  // n_out*n_in
     double2 *d_qsrc = nullptr;   // nx: source-row coefficient q[m] of the substrate side
     double2 *d_refl = nullptr;   // nx*n_in: reflection block (apf_reflection)
@@ -165,7 +165,7 @@ GridDev make_grid(const apf_ctx *c);
 // boundary.cu
 void launch_boundary(apf_ctx *c, cudaStream_t s);
 void launch_boundary_n(apf_ctx *const *cs, int nb, cudaStream_t s);  // contexts of one grid
-void launch_build_rhs(apf_ctx *c, double2 *E, cudaStream_t s);
+void launch_build_rhs(apf_ctx *c, double2 *E, int rows, cudaStream_t s);
 void launch_adjoint_rhs(apf_ctx *c, const double2 *Gamma, double2 *E, cudaStream_t s);
 void launch_source_row(apf_ctx *c, double2 *q, cudaStream_t s);
 void launch_reflection(apf_ctx *c, const double2 *fft0, const double2 *q, const int *m_ref, int n_ref, double2 *R,

@@ -333,8 +333,9 @@ void launch_boundary_n(apf_ctx *const *cs, int nb, cudaStream_t s) {
 
 void launch_boundary(apf_ctx *c, cudaStream_t s) { launch_boundary_n(&c, 1, s); }
 
-void launch_build_rhs(apf_ctx *c, double2 *E, cudaStream_t s) {
+void launch_build_rhs(apf_ctx *c, double2 *E, int rows, cudaStream_t s) {
     GridDev g = make_grid(c);
+    g.h = rows;  // E holds `rows` rows, the first and the last slab row among them
     // the columns of the current layout: cf forward (inputs), ca adjoint (outputs)
     int nf = c->cf, na = c->ca;
     dim3 grid((c->nx + 255) / 256, nf + na);

@@ -2,14 +2,22 @@
 //
 // The slab Schur blocks X_j and their inverses G_j are held in float32
 // (separate real / imaginary planes).  Every product runs on the tensor cores
-// (tc_gemm.cu) with operands split into bf16 planes: two planes and three
+// (cgemm.cu) with operands split into bf16 planes: two planes and three
 // products ("bf16x3") for the elimination and the field sweeps, three planes
-// and six products for the gradient contraction.  Accuracy is then won back
-// by float64 iterative refinement of the slab fields:
+// and six products for the gradient contraction (tc_gemm.cu).  Accuracy is then
+// won back by float64 iterative refinement of the slab fields:
 //     r = R - K E (float64 5-point stencil + boundary circulants),
 //     E <- E + Khat^-1 r,
 // where Khat^-1 is the block-LU solve with the stored low-precision G_j.
+//
+// The slab rows are eliminated from both ends towards the middle row m = h / 2:
+// X_j = K_j - G_{j-1} below it, X_j = K_j - G_{j+1} above it, X_m = K_m - G_{m-1} -
+// G_{m+1}.  The two chains are independent, so one launch carries a row of each
+// (of every design of a batch): half as many dependent steps, which is what a
+// single design's time consists of (one CTA per 128 x 128 diagonal block, a few
+// tiles per product of the lower recursion levels).
 #include "apf_internal.h"
+#include "cgemm.h"
 #include "tc_gemm.h"
 #include "leaf.cuh"
 
@@ -19,31 +27,41 @@
 #include <stdlib.h>
 #include <vector>
 
+// Work arrays of one of the two chains of a design.
+struct SideWork {
+    float *Xre = nullptr, *Xim = nullptr;  // n x n working block
+    Mirror XP;                             // its split form
+    __nv_bfloat16 *TP = nullptr, *TT = nullptr;  // T and T^T of every recursion level, split
+    float *O32 = nullptr;                  // field products (re, im), ncol x n each
+    Mirror PA;                             // field operand, ncol x n
+};
+
 struct MixedWork {
     int nsplit_elim = 2, nsplit_grad = 3, leaf = 128, leaf_variant = 0;
-    float *Xre = nullptr, *Xim = nullptr;            // n x n working block
-    float *Tre = nullptr, *Tim = nullptr;            // recursion scratch (n*n/2 each)
-    float *Vre = nullptr, *Vim = nullptr;
-    __nv_bfloat16 *PA = nullptr, *PB = nullptr;      // operand packs
-    long long pa_elems = 0, pb_elems = 0;
-    __nv_bfloat16 *GP = nullptr;                     // packed G_j: h of them, or seg_rows when recomputing
+    long long pitch = 0;                             // row pitch of n-column split matrices: max(n, 64)
+    int nside = 2;                                   // 1 with recomputation
+    SideWork sd[2];
+    __nv_bfloat16 *GA = nullptr, *GB = nullptr;      // gradient operands
+    __nv_bfloat16 *GP = nullptr;                     // split G_j: h of them, or seg_rows when recomputing
     long long gp_stride = 0;
-    // Recomputation of the slab Schur blocks (seg_rows > 0): the rows are cut
-    // into segments of seg_rows; only the packed inverses of one segment are
-    // held (GP slot j - start of j's segment), plus the float32 G_{c-1} at every
-    // segment start c > 0 (checkpoint s-1 for segment s), from which a
-    // segment's inverses are recomputed when a sweep needs them.
+    // Recomputation of the slab Schur blocks (seg_rows > 0).  The rows are taken
+    // in the order of the chains (lower chain, upper chain, middle row), cut into
+    // segments of seg_rows positions; only the split inverses of one segment are
+    // held (GP slot = position mod seg_rows), plus the float32 inverse before
+    // every segment start (checkpoint s - 1 for segment s), from which a
+    // segment's inverses are recomputed when a sweep needs them, and that of the
+    // lower chain's last row (CKB), which the middle row needs again.
     int seg_rows = 0, nseg = 1, seg_loaded = -1;
-    float *CK = nullptr;                             // (nseg - 1) checkpoints, 2 n^2 floats each
+    float *CK = nullptr, *CKB = nullptr;             // 2 n^2 floats per checkpoint
     // Symmetric random butterfly transform of every slab block before its
     // inversion (bfly = 1): X' = U^T X U, G = U X'^-1 U^T with a depth-2
     // recursive butterfly U; BW holds its 2 n random diagonal entries.
     int bfly = 0;
     float *BW = nullptr;
-    float *O32 = nullptr;                            // GEMM output planes, 2 * max(ncol, n_out) * nx
     double2 *r = nullptr, *delta = nullptr;          // refinement buffers (h*ncol*nx)
     double2 *cb = nullptr, *ct = nullptr;            // circulant products on the boundary rows
     double *rnorm = nullptr;                         // ||R_c||^2, ||r_c||^2
+    double *rpart = nullptr;                         // partial sums of ||r_c||^2
     int km = 0;                                      // GMRES(km) refinement (0: plain refinement)
     double2 *KV = nullptr, *KZ = nullptr;            // Krylov basis (km+1 fields) and preconditioned vectors (km)
     double2 *kdot = nullptr, *ky = nullptr;          // Gram-Schmidt coefficients (km+1)*km*ncol, update km*ncol
@@ -58,11 +76,11 @@ int recompute_segment_b(const Bat &bt, int seg, cudaStream_t s);
 
 namespace {
 
-// Per-design pointers of a batch of designs (entry blockIdx.z, or blockIdx.x
-// for the one-CTA-per-block leaf kernel); a single design uses entry 0.
+// Per-problem pointers of a launch (entry blockIdx.z, or blockIdx.x for the
+// one-CTA-per-block leaf kernels); a single problem uses entry 0.
 template <typename T>
 struct Tab {
-    T v[TC_MAX_BATCH];
+    T v[CG_MAX_PROB];
 };
 
 __device__ __forceinline__ void split_bf16(float x, int nsplit, __nv_bfloat16 *o) {
@@ -76,157 +94,21 @@ __device__ __forceinline__ void split_bf16(float x, int nsplit, __nv_bfloat16 *o
     }
 }
 
-// Pack a complex float32 planar matrix into bf16 split planes.
-// Logical element v(r, k) = trans ? src[k][r] : src[r][k], r < R, k < K.
-// layoutB = 0 (A operand): row r = [Re v(r,:), Im v(r,:)].
-// layoutB = 1 (B operand of C = A B, r indexing C's columns):
-//   row r = [Re v(r,:), -Im v(r,:)], row R + r = [Im v(r,:), Re v(r,:)].
-struct PackJob {
-    const float *re, *im;
-    long long ld;
-    int R, K, trans, layoutB, nsplit;
-    __nv_bfloat16 *out;
-    long long kp, plane_pitch;
-};
-// Up to N pack jobs per launch (blockIdx.z): the two operands of one product,
-// or those of the same product for every design of a batch.
-template <int N>
-struct PackJobsN {
-    PackJob j[N];
-};
-constexpr int MAX_JOBS = 2 * TC_MAX_BATCH;
-
-// Tile: 32 rows x 64 k; thread (tx, ty) handles k = k0 + 2 tx, +1 (bf16x2 stores).
-template <int N>
-__global__ void __launch_bounds__(256) k_pack32(const __grid_constant__ PackJobsN<N> jobs) {
-    const PackJob &J = jobs.j[blockIdx.z];
-    __shared__ float tre[32][65], tim[32][65];
-    const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
-    if (r0 >= J.R || k0 >= J.K) return;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    if (!J.trans) {
-        for (int i = ty; i < 32; i += 8) {
-            int r = r0 + i;
-            for (int kk = tx; kk < 64; kk += 32) {
-                int k = k0 + kk;
-                float a = 0.f, b = 0.f;
-                if (r < J.R && k < J.K) { a = J.re[(long long)r * J.ld + k]; b = J.im[(long long)r * J.ld + k]; }
-                tre[i][kk] = a; tim[i][kk] = b;
-            }
-        }
-    } else {
-        for (int kk = ty; kk < 64; kk += 8) {
-            int k = k0 + kk, r = r0 + tx;
-            float a = 0.f, b = 0.f;
-            if (r < J.R && k < J.K) { a = J.re[(long long)k * J.ld + r]; b = J.im[(long long)k * J.ld + r]; }
-            tre[tx][kk] = a; tim[tx][kk] = b;
-        }
-    }
-    __syncthreads();
-    const int R = J.R, K = J.K, ns = J.nsplit;
-    const long long kp = J.kp;
-    const int k = k0 + 2 * tx;
-    if (k >= K) return;
-    const bool two = (k + 1 < K);
-    for (int i = ty; i < 32; i += 8) {
-        int r = r0 + i;
-        if (r >= R) break;
-        __nv_bfloat16 a0[3], a1[3], b0[3], b1[3];
-        split_bf16(tre[i][2 * tx], ns, a0);
-        split_bf16(tim[i][2 * tx], ns, b0);
-        split_bf16(two ? tre[i][2 * tx + 1] : 0.f, ns, a1);
-        split_bf16(two ? tim[i][2 * tx + 1] : 0.f, ns, b1);
-        #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            if (p >= ns) break;
-            __nv_bfloat16 *o = J.out + p * J.plane_pitch;
-            __nv_bfloat162 re2 = __halves2bfloat162(a0[p], a1[p]);
-            __nv_bfloat162 im2 = __halves2bfloat162(b0[p], b1[p]);
-            __nv_bfloat162 nim2 = __halves2bfloat162(__hneg(b0[p]), __hneg(b1[p]));
-            auto st = [&](long long row, long long col, __nv_bfloat162 v) {
-                if (two && ((row * kp + col) & 1) == 0) {
-                    *reinterpret_cast<__nv_bfloat162 *>(o + row * kp + col) = v;
-                } else {
-                    o[row * kp + col] = v.x;
-                    if (two) o[row * kp + col + 1] = v.y;
-                }
-            };
-            if (!J.layoutB) {
-                st(r, k, re2);
-                st(r, K + k, im2);
-            } else {
-                st(r, k, re2);
-                st(r, K + k, nim2);
-                st(R + r, k, im2);
-                st(R + r, K + k, re2);
-            }
-        }
-    }
-}
-
-// Vectorised form of k_pack32 for whole 32 x 64 tiles (R % 32 == 0, K % 64 == 0,
-// ld % 4 == 0, 16-byte aligned planes): 128-bit loads into shared memory, then
-// each thread splits 8 consecutive k of one row and writes 16-byte rows of
-// every plane.
-__device__ __forceinline__ uint4 pack8(const __nv_bfloat16 (*v)[3], int p, bool neg) {
-    uint32_t w[4];
+// Split form of R x C float32 planes (trans: of their transpose, R x C): the
+// operands of the test hooks and of the leaf variants that only write float32.
+__global__ void k_mirror(const float *re, const float *im, long long ld, int R, int C, int trans, Mirror m, int planes) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (c >= C) return;
+    const long long g = trans ? (long long)c * ld + r : (long long)r * ld + c;
+    __nv_bfloat16 a[3], b[3];
+    split_bf16(re[g], planes, a);
+    split_bf16(im[g], planes, b);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        __nv_bfloat16 lo = v[2 * i][p], hi = v[2 * i + 1][p];
-        if (neg) { lo = __hneg(lo); hi = __hneg(hi); }
-        w[i] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-template <int N>
-__global__ void __launch_bounds__(256) k_pack32v(const __grid_constant__ PackJobsN<N> jobs) {
-    const PackJob &J = jobs.j[blockIdx.z];
-    __shared__ float tre[32][65], tim[32][65];
-    const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
-    if (r0 >= J.R || k0 >= J.K) return;
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int idx = t + 256 * h;
-        if (!J.trans) {
-            const int row = idx >> 4, c4 = idx & 15;
-            const long long g = (long long)(r0 + row) * J.ld + k0 + 4 * c4;
-            const float4 a = *reinterpret_cast<const float4 *>(J.re + g), b = *reinterpret_cast<const float4 *>(J.im + g);
-            tre[row][4 * c4] = a.x; tre[row][4 * c4 + 1] = a.y; tre[row][4 * c4 + 2] = a.z; tre[row][4 * c4 + 3] = a.w;
-            tim[row][4 * c4] = b.x; tim[row][4 * c4 + 1] = b.y; tim[row][4 * c4 + 2] = b.z; tim[row][4 * c4 + 3] = b.w;
-        } else {
-            const int krow = idx >> 3, c4 = idx & 7;
-            const long long g = (long long)(k0 + krow) * J.ld + r0 + 4 * c4;
-            const float4 a = *reinterpret_cast<const float4 *>(J.re + g), b = *reinterpret_cast<const float4 *>(J.im + g);
-            tre[4 * c4][krow] = a.x; tre[4 * c4 + 1][krow] = a.y; tre[4 * c4 + 2][krow] = a.z; tre[4 * c4 + 3][krow] = a.w;
-            tim[4 * c4][krow] = b.x; tim[4 * c4 + 1][krow] = b.y; tim[4 * c4 + 2][krow] = b.z; tim[4 * c4 + 3][krow] = b.w;
-        }
-    }
-    __syncthreads();
-    const int r = t >> 3, c = t & 7;
-    const int row = r0 + r, k = k0 + 8 * c;
-    __nv_bfloat16 sr[8][3], si[8][3];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        split_bf16(tre[r][8 * c + u], J.nsplit, sr[u]);
-        split_bf16(tim[r][8 * c + u], J.nsplit, si[u]);
-    }
-    const long long kp = J.kp, K = J.K, R = J.R;
-    #pragma unroll
     for (int p = 0; p < 3; ++p) {
-        if (p >= J.nsplit) break;
-        __nv_bfloat16 *o = J.out + p * J.plane_pitch;
-        const uint4 re = pack8(sr, p, false), im = pack8(si, p, false);
-        if (!J.layoutB) {
-            *reinterpret_cast<uint4 *>(o + row * kp + k) = re;
-            *reinterpret_cast<uint4 *>(o + row * kp + K + k) = im;
-        } else {
-            *reinterpret_cast<uint4 *>(o + row * kp + k) = re;
-            *reinterpret_cast<uint4 *>(o + row * kp + K + k) = pack8(si, p, true);
-            *reinterpret_cast<uint4 *>(o + (R + row) * kp + k) = im;
-            *reinterpret_cast<uint4 *>(o + (R + row) * kp + K + k) = re;
-        }
+        if (p >= planes) break;
+        __nv_bfloat16 *o = m.base + 2 * p * m.qpitch + r * m.pitch + c;
+        o[0] = a[p];
+        o[m.qpitch] = b[p];
     }
 }
 
@@ -288,127 +170,187 @@ __global__ void k_pack64_BT(const __grid_constant__ Tab<const double2 *> srct, l
     }
 }
 
-// X_j = K_j - G_{j-1} in float32 planes (K_j: 5-point slab block plus the
-// boundary circulants on the first / last slab row).
-// X_j = K_j - G_{j-1} in float32 planes (K_j: 4 - k^2 eps on the diagonal,
-// -1 on the periodic neighbours, the circulants Sigma_bot / Sigma_top on the
-// first / last slab row).  Thread: 4 consecutive columns xp of row x (n % 4 == 0).
-__global__ void k_assemble32(GridDev g, int row, const __grid_constant__ Tab<const double *> epst, const double2 *circ,
-                             const __grid_constant__ Tab<const float *> Gret, const __grid_constant__ Tab<const float *> Gimt, const __grid_constant__ Tab<float *> Xret, const __grid_constant__ Tab<float *> Ximt) {
-    const int b = blockIdx.z;
-    const double *eps = epst.v[b];
-    const float *Gre = Gret.v[b], *Gim = Gimt.v[b];
-    float *Xre = Xret.v[b], *Xim = Ximt.v[b];
-    const int n = g.nx;
-    const int x = blockIdx.y;
-    const int xp0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (xp0 >= n) return;
-    const long long idx = (long long)x * n + xp0;
-    float vr[4] = {0.f, 0.f, 0.f, 0.f}, vi[4] = {0.f, 0.f, 0.f, 0.f};
-    if (Gre) {
-        const float4 a = *reinterpret_cast<const float4 *>(Gre + idx), b = *reinterpret_cast<const float4 *>(Gim + idx);
-        vr[0] = -a.x; vr[1] = -a.y; vr[2] = -a.z; vr[3] = -a.w;
-        vi[0] = -b.x; vi[1] = -b.y; vi[2] = -b.z; vi[3] = -b.w;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int xp = xp0 + u;
-        float kr = 0.f, ki = 0.f;
-        // float64 only on the one diagonal element (the FP64 pipe is narrow)
-        if (xp == x) kr = (float)(4.0 - g.k * g.k * eps[(long long)row * n + x]);
-        const int dx = x - xp;
-        if (dx == 1 || dx == -1 || dx == n - 1 || dx == 1 - n) kr -= 1.f;
-        if (n == 2 && dx != 0) kr -= 1.f;  // both periodic neighbours coincide
-        const int d = dx < 0 ? dx + n : dx;
-        if (row == 0) { kr += (float)circ[d].x; ki += (float)circ[d].y; }
-        if (row == g.h - 1) { kr += (float)circ[n + d].x; ki += (float)circ[n + d].y; }
-        vr[u] += kr;
-        vi[u] += ki;
-    }
-    *reinterpret_cast<float4 *>(Xre + idx) = make_float4(vr[0], vr[1], vr[2], vr[3]);
-    *reinterpret_cast<float4 *>(Xim + idx) = make_float4(vi[0], vi[1], vi[2], vi[3]);
-}
+// ---------------------------------------------------------------------------
+// One step of the slab elimination between two inversions, for 4 x 4 groups of
+// elements (rows {i, i+n/4, i+n/2, i+3n/4} x the same columns), two column
+// groups per thread:
+//   * the inverses just computed (transformed, "y space") become G = U Y U^T and
+//     are written in split form (for the sweeps) and, at a checkpoint, in float32;
+//   * the next block X = K_row - G (- G of the other chain) is assembled and
+//     transformed, X' = U^T X U, and written as the recursion reads it: float32 on
+//     and below the diagonal blocks, split form below them.
+// U = P Q with Q the n-point butterfly (1/sqrt2)[R0 R1; R0 -R1] and P = diag of two
+// n/2-point butterflies, R* random diagonals near 1; such a two-sided transform
+// spreads every row over rows n/4 apart, so that the leading blocks of the Schur
+// recursion (which pivots only inside its 32 x 32 leaves) are not the nearly
+// singular sub-blocks of a strongly structured slab (high-contrast ridges) --
+// the randomisation that lets symmetric indefinite elimination run without
+// pivoting.  w[0 .. n): level-Q diagonals (R0 at i, R1 at n/2 + i); w[n .. 2n):
+// level-P, half h (0 / 1) at n + h n/2 (R0 at i, R1 at n/4 + i).
+// Bound by HBM: 24 n^2 bytes against the 72 n^2 of the five passes it replaces
+// (inverse transform, packing, assembly, forward transform).
+struct RowSrc {
+    const float *re, *im;     // n x n block (null: no such source)
+    int yspace, use;          // still transformed; subtracted from the next block
+    Mirror gp;                // split G goes here (null base: not written)
+    float *ck_re, *ck_im;     // float32 G goes here (null: not written)
+};
+struct RowJob {
+    RowSrc s[2];
+    const double *eps;        // slab permittivity
+    int row, out;             // row of K (-1: none); whether the next block is written
+    float sgn;                // X = K + sgn G
+    float *Xre, *Xim;
+    Mirror XP;                // (null base: float32 only)
+};
+template <int N>
+struct RowJobs {
+    RowJob j[N];
+};
 
-// Symmetric random butterfly transform (depth 2) of an n x n complex-symmetric
-// block in planar float32, in place.  U = P Q with Q the n-point butterfly
-// (1/sqrt2)[R0 R1; R0 -R1] and P = diag of two n/2-point butterflies, R* random
-// diagonals near 1; such a two-sided transform spreads every row over rows
-// n/4 apart, so that the leading blocks of the Schur recursion (which pivots
-// only inside its 32 x 32 leaves) are not the nearly singular sub-blocks of a
-// strongly structured slab (high-contrast ridges) -- the randomisation that
-// lets symmetric indefinite elimination run without pivoting.
-//   forward: X' = U^T X U   (rows and columns: P^T then Q^T);
-//   inverse: G  = U Y U^T   (rows and columns: Q then P).
-// w[0 .. n): level-Q diagonals (R0 at i, R1 at n/2 + i); w[n .. 2n): level-P,
-// half h (0 / 1) at n + h n/2 (R0 at i, R1 at n/4 + i).  One thread per 4 x 4
-// group of rows {i, i+n/4, i+n/2, i+3n/4} x columns {j, ...}, i, j < n/4.
 __device__ __forceinline__ void bf_fwd(float2 &t, float2 &b, float wa, float wb) {
     const float c = 0.70710678118654752f;
     const float2 s = make_float2(t.x + b.x, t.y + b.y), d = make_float2(t.x - b.x, t.y - b.y);
     t = make_float2(c * wa * s.x, c * wa * s.y);
     b = make_float2(c * wb * d.x, c * wb * d.y);
 }
+// The last product is not contracted into a following subtraction, so that G is
+// the same number whether it is used at once or read back from a checkpoint.
 __device__ __forceinline__ void bf_inv(float2 &t, float2 &b, float wa, float wb) {
     const float c = 0.70710678118654752f;
     const float2 u = make_float2(wa * t.x, wa * t.y), v = make_float2(wb * b.x, wb * b.y);
-    t = make_float2(c * (u.x + v.x), c * (u.y + v.y));
-    b = make_float2(c * (u.x - v.x), c * (u.y - v.y));
+    t = make_float2(__fmul_rn(c, u.x + v.x), __fmul_rn(c, u.y + v.y));
+    b = make_float2(__fmul_rn(c, u.x - v.x), __fmul_rn(c, u.y - v.y));
 }
-template <bool INV>
-__global__ void k_butterfly(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, int n, const float *w) {
-    float *re = ret.v[blockIdx.z], *im = imt.v[blockIdx.z];
-    const int q = n >> 2;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
-    if (j >= q || i >= q) return;
-    float2 m[4][4];
+
+__device__ __forceinline__ void store_split2(const Mirror &m, int planes, long long r, long long c, float2 a, float2 b) {
+    __nv_bfloat16 ar[3], ai[3], br[3], bi[3];
+    split_bf16(a.x, planes, ar);
+    split_bf16(a.y, planes, ai);
+    split_bf16(b.x, planes, br);
+    split_bf16(b.y, planes, bi);
+    __nv_bfloat16 *o = m.base + r * m.pitch + c;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        if (p >= planes) break;
+        *reinterpret_cast<__nv_bfloat162 *>(o + 2 * p * m.qpitch) = __halves2bfloat162(ar[p], br[p]);
+        *reinterpret_cast<__nv_bfloat162 *>(o + (2 * p + 1) * m.qpitch) = __halves2bfloat162(ai[p], bi[p]);
+    }
+}
+
+template <bool BF, int N>
+__global__ void __launch_bounds__(128) k_row_step(GridDev g, const __grid_constant__ RowJobs<N> jobs, int n, const double2 *circ,
+                                                  const float *w, int planes, int leaf) {
+    const RowJob &J = jobs.j[blockIdx.z];
+    const int q = n >> 2, half = n >> 3;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= q * half) return;
+    const int i = idx / half, j = 2 * (idx - i * half);
+    const float *wq = w, *wp0 = w + n, *wp1 = w + n + n / 2;
+    float2 x[4][8];  // [row group][2 column group + column]
+    // K: 4 - k^2 eps on the diagonal, -1 on the periodic neighbours, the circulants
+    // Sigma_bot / Sigma_top on the first / last slab row; float64 only on the diagonal
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const long long g = (long long)(i + r * q) * ld + (j + c * q);
-            m[r][c] = make_float2(re[g], im[g]);
+        for (int c = 0; c < 8; ++c) {
+            float kr = 0.f, ki = 0.f;
+            if (J.row >= 0) {
+                const int row = i + r * q, col = j + (c & 1) + (c >> 1) * q, dx = row - col;
+                if (dx == 0) kr = (float)(4.0 - g.k * g.k * J.eps[(long long)J.row * n + row]);
+                if (dx == 1 || dx == -1 || dx == n - 1 || dx == 1 - n) kr -= 1.f;
+                const int d = dx < 0 ? dx + n : dx;
+                if (J.row == 0) { kr += (float)circ[d].x; ki += (float)circ[d].y; }
+                if (J.row == g.h - 1) { kr += (float)circ[n + d].x; ki += (float)circ[n + d].y; }
+            }
+            x[r][c] = make_float2(kr, ki);
         }
-    // P level pairs (0,1) [half 0] and (2,3) [half 1] at local index i / j;
-    // Q level pairs (0,2) and (1,3) at index i, i + q (resp. j, j + q)
-    auto rows = [&](int a, int b, float wa, float wb) {
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+        const RowSrc &S = J.s[s];
+        if (!S.re) continue;
+        float2 v[4][8];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            if (INV) bf_inv(m[a][c], m[b][c], wa, wb);
-            else bf_fwd(m[a][c], m[b][c], wa, wb);
-        }
-    };
-    auto cols = [&](int a, int b, float wa, float wb) {
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (INV) bf_inv(m[r][a], m[r][b], wa, wb);
-            else bf_fwd(m[r][a], m[r][b], wa, wb);
+            for (int c = 0; c < 4; ++c) {
+                const long long o = (long long)(i + r * q) * n + j + c * q;
+                const float2 a = *reinterpret_cast<const float2 *>(S.re + o), b = *reinterpret_cast<const float2 *>(S.im + o);
+                v[r][2 * c] = make_float2(a.x, b.x);
+                v[r][2 * c + 1] = make_float2(a.y, b.y);
+            }
+        if (BF && S.yspace) {  // G = U Y U^T: rows and columns, Q then P
+            auto rows = [&](int a, int b, float wa, float wb) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) bf_inv(v[a][c], v[b][c], wa, wb);
+            };
+            auto cols = [&](int a, int b, const float *wa, const float *wb) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) bf_inv(v[r][2 * a + u], v[r][2 * b + u], wa[j + u], wb[j + u]);
+            };
+            rows(0, 2, wq[i], wq[2 * q + i]); rows(1, 3, wq[q + i], wq[3 * q + i]);
+            rows(0, 1, wp0[i], wp0[q + i]); rows(2, 3, wp1[i], wp1[q + i]);
+            cols(0, 2, wq, wq + 2 * q); cols(1, 3, wq + q, wq + 3 * q);
+            cols(0, 1, wp0, wp0 + q); cols(2, 3, wp1, wp1 + q);
         }
-    };
-    const float *wq = w, *wp0 = w + n, *wp1 = w + n + n / 2;
-    if (!INV) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int row = i + r * q, col = j + c * q;
+                const float2 a = v[r][2 * c], b = v[r][2 * c + 1];
+                if (S.gp.base) store_split2(S.gp, planes, row, col, a, b);
+                if (S.ck_re) {
+                    const long long o = (long long)row * n + col;
+                    *reinterpret_cast<float2 *>(S.ck_re + o) = make_float2(a.x, b.x);
+                    *reinterpret_cast<float2 *>(S.ck_im + o) = make_float2(a.y, b.y);
+                }
+                if (S.use) {
+                    float2 &xa = x[r][2 * c], &xb = x[r][2 * c + 1];
+                    xa = make_float2(__fadd_rn(xa.x, J.sgn * a.x), __fadd_rn(xa.y, J.sgn * a.y));
+                    xb = make_float2(__fadd_rn(xb.x, J.sgn * b.x), __fadd_rn(xb.y, J.sgn * b.y));
+                }
+            }
+    }
+    if (!J.out) return;
+    if (BF) {  // X' = U^T X U: rows and columns, P^T then Q^T
+        auto rows = [&](int a, int b, float wa, float wb) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) bf_fwd(x[a][c], x[b][c], wa, wb);
+        };
+        auto cols = [&](int a, int b, const float *wa, const float *wb) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) bf_fwd(x[r][2 * a + u], x[r][2 * b + u], wa[j + u], wb[j + u]);
+        };
         rows(0, 1, wp0[i], wp0[q + i]); rows(2, 3, wp1[i], wp1[q + i]);
         rows(0, 2, wq[i], wq[2 * q + i]); rows(1, 3, wq[q + i], wq[3 * q + i]);
-        cols(0, 1, wp0[j], wp0[q + j]); cols(2, 3, wp1[j], wp1[q + j]);
-        cols(0, 2, wq[j], wq[2 * q + j]); cols(1, 3, wq[q + j], wq[3 * q + j]);
-    } else {
-        rows(0, 2, wq[i], wq[2 * q + i]); rows(1, 3, wq[q + i], wq[3 * q + i]);
-        rows(0, 1, wp0[i], wp0[q + i]); rows(2, 3, wp1[i], wp1[q + i]);
-        cols(0, 2, wq[j], wq[2 * q + j]); cols(1, 3, wq[q + j], wq[3 * q + j]);
-        cols(0, 1, wp0[j], wp0[q + j]); cols(2, 3, wp1[j], wp1[q + j]);
+        cols(0, 1, wp0, wp0 + q); cols(2, 3, wp1, wp1 + q);
+        cols(0, 2, wq, wq + 2 * q); cols(1, 3, wq + q, wq + 3 * q);
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const long long g = (long long)(i + r * q) * ld + (j + c * q);
-            re[g] = m[r][c].x;
-            im[g] = m[r][c].y;
+            const int row = i + r * q, col = j + c * q;
+            const int br = row / leaf, bc = col / leaf;
+            if (bc > br) continue;
+            const float2 a = x[r][2 * c], b = x[r][2 * c + 1];
+            const long long o = (long long)row * n + col;
+            *reinterpret_cast<float2 *>(J.Xre + o) = make_float2(a.x, b.x);
+            *reinterpret_cast<float2 *>(J.Xim + o) = make_float2(a.y, b.y);
+            if (J.XP.base && bc < br) store_split2(J.XP, planes, row, col, a, b);
         }
 }
 
 // Float32 Gauss-Jordan inverse of an n x n (n <= 128) diagonal block with
 // partial pivoting, in shared memory (planar in global memory).
-__global__ void __launch_bounds__(512) k_leaf_inv32(float *re, float *im, long long ld, int n, int *flags) {
+__global__ void __launch_bounds__(512) k_leaf_inv32(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, int n, const __grid_constant__ Tab<int *> flt) {
+    float *re = ret.v[blockIdx.x], *im = imt.v[blockIdx.x];
+    int *flags = flt.v[blockIdx.x];
     extern __shared__ float2 a32[];
     __shared__ float2 colk[128];
     __shared__ int piv[128];
@@ -493,77 +435,108 @@ __global__ void __launch_bounds__(512) k_leaf_inv32(float *re, float *im, long l
 }
 
 template <int NB>
-__global__ void __launch_bounds__(NB * 4) k_leaf32(float *re, float *im, long long ld, int *flags) {
-    LeafIO<float, true> io{re, im, nullptr, ld};
-    leaf_gj<float, NB, true>(io, flags);
+__global__ void __launch_bounds__(NB * 4) k_leaf32(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<int *> flags) {
+    const int b = blockIdx.x;
+    LeafIO<float, true> io{re.v[b], im.v[b], nullptr, ld};
+    leaf_gj<float, NB, true>(io, flags.v[b]);
 }
 
 template <int NB>
-__global__ void __launch_bounds__(NB * 4) k_leaf32r(float *re, float *im, long long ld, int *flags) {
-    leaf_gj_regs<NB>(re, im, ld, flags);
+__global__ void __launch_bounds__(NB * 4) k_leaf32r(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<int *> flags) {
+    const int b = blockIdx.x;
+    leaf_gj_regs<NB>(re.v[b], im.v[b], ld, flags.v[b]);
 }
 
-__global__ void __launch_bounds__(512) k_leaf128rec(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<int *> flags) {
+// 128 x 128 diagonal blocks: the inverse in place and in split form (XP.base null: float32 only).
+__global__ void __launch_bounds__(512) k_leaf128rec(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
     const int b = blockIdx.x;
     leaf128_recursive(re.v[b], im.v[b], ld, flags.v[b]);
+    const Mirror m = XP.v[b];
+    if (!m.base) return;
+    __syncthreads();  // the block's float32 stores are read back by other threads
+    for (int e = threadIdx.x; e < 128 * 64; e += 512) {
+        const int r = e >> 6, c = 2 * (e & 63);
+        const float2 a = *reinterpret_cast<const float2 *>(re.v[b] + (long long)r * ld + c);
+        const float2 d = *reinterpret_cast<const float2 *>(im.v[b] + (long long)r * ld + c);
+        store_split2(m, planes, r, c, make_float2(a.x, d.x), make_float2(a.y, d.y));
+    }
 }
 
 template <int NB>
-__global__ void __launch_bounds__(NB * 4) k_leaf32r2(float *re, float *im, long long ld, int *flags) {
-    leaf_gj_regs2<NB>(re, im, ld, flags);
+__global__ void __launch_bounds__(NB * 4) k_leaf32r2(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<int *> flags) {
+    const int b = blockIdx.x;
+    leaf_gj_regs2<NB>(re.v[b], im.v[b], ld, flags.v[b]);
 }
 
-// C block <- -V, B block <- -V^T (planar float32).
-__global__ void k_negoff32(const __grid_constant__ Tab<float *> Bret, const __grid_constant__ Tab<float *> Bimt, const __grid_constant__ Tab<float *> Cret, const __grid_constant__ Tab<float *> Cimt, long long ld,
-                           const __grid_constant__ Tab<const float *> Vret, const __grid_constant__ Tab<const float *> Vimt, int h) {
-    __shared__ float tr[32][33], ti[32][33];
-    const int b = blockIdx.z;
-    float *Bre = Bret.v[b], *Bim = Bimt.v[b], *Cre = Cret.v[b], *Cim = Cimt.v[b];
-    const float *Vre = Vret.v[b], *Vim = Vimt.v[b];
-    int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    int tx = threadIdx.x, ty = threadIdx.y;
-    for (int i = ty; i < 32; i += 8) {
-        int gi = i0 + i, gj = j0 + tx;
-        if (gi < h && gj < h) {
-            float vr = Vre[(long long)gi * h + gj], vi = Vim[(long long)gi * h + gj];
-            Cre[(long long)gi * ld + gj] = -vr;
-            Cim[(long long)gi * ld + gj] = -vi;
-            tr[i][tx] = vr; ti[i][tx] = vi;
-        }
-    }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        int gj = j0 + i, gi = i0 + tx;  // B[gj][gi] = -V[gi][gj]
-        if (gi < h && gj < h) {
-            Bre[(long long)gj * ld + gi] = -tr[tx][i];
-            Bim[(long long)gj * ld + gi] = -ti[tx][i];
-        }
-    }
-}
+// Element-wise step of a field sweep between two products: o = the product's
+// rows (float32 planes O for columns [o0, o1), plus O2 for [p0, p1)), v = o + add
+// (float64 rows, columns [a0, a1)); out = v, out = o or out += o; and v in split
+// form as the next product's operand (row c - c0 for column c).  Two x per thread.
+struct FieldJob {
+    const float *O, *O2;      // re plane, im plane at + olen (null: none)
+    long long olen;
+    int o0, o1, p0, p1;
+    const double2 *add;
+    int a0, a1;
+    double2 *out;
+    int mode;                 // 1: out = v, 2: out = o, 3: out += o
+    Mirror m;
+    int c0, c1;               // columns of this job
+};
+template <int N>
+struct FieldJobs {
+    FieldJob j[N];
+};
 
-// E[c][x] = (R ? R[c][x] : 0) + O[c][x] for c < mcols;  E = R for c >= mcols.
-__global__ void k_combine(const __grid_constant__ Tab<double2 *> Et, const __grid_constant__ Tab<const double2 *> Rt, const __grid_constant__ Tab<const float *> Oret,
-                          const __grid_constant__ Tab<const float *> Oimt, int ncol, int mcols, int nx) {
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int c = blockIdx.y;
-    if (x >= nx) return;
-    const int b = blockIdx.z;
-    double2 *E = Et.v[b];
-    const double2 *R = Rt.v[b];
-    const float *Ore = Oret.v[b], *Oim = Oimt.v[b];
-    long long i = (long long)c * nx + x;
-    double2 v = R ? R[i] : cmk(0, 0);
-    if (c < mcols) { v.x += (double)Ore[i]; v.y += (double)Oim[i]; }
-    E[i] = v;
-    (void)ncol;
+template <int N>
+__global__ void __launch_bounds__(128) k_field_step(const __grid_constant__ FieldJobs<N> jobs, int nx, int planes) {
+    const FieldJob &J = jobs.j[blockIdx.z];
+    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x), c = J.c0 + blockIdx.y;
+    if (x >= nx || c >= J.c1) return;
+    double2 o[2] = {cmk(0.0, 0.0), cmk(0.0, 0.0)};
+    if (J.O && c >= J.o0 && c < J.o1) {
+        const float *p = J.O + (long long)(c - J.o0) * nx + x;
+        const float2 a = *reinterpret_cast<const float2 *>(p), b = *reinterpret_cast<const float2 *>(p + J.olen);
+        o[0] = cmk(a.x, b.x);
+        o[1] = cmk(a.y, b.y);
+    }
+    if (J.O2 && c >= J.p0 && c < J.p1) {
+        const float *p = J.O2 + (long long)(c - J.p0) * nx + x;
+        const float2 a = *reinterpret_cast<const float2 *>(p), b = *reinterpret_cast<const float2 *>(p + J.olen);
+        o[0] = cadd(o[0], cmk(a.x, b.x));
+        o[1] = cadd(o[1], cmk(a.y, b.y));
+    }
+    const long long g = (long long)c * nx + x;
+    double2 v[2] = {o[0], o[1]};
+    if (J.add && c >= J.a0 && c < J.a1) {
+        v[0] = cadd(J.add[g], v[0]);
+        v[1] = cadd(J.add[g + 1], v[1]);
+    }
+    if (J.mode == 1) {
+        J.out[g] = v[0];
+        J.out[g + 1] = v[1];
+    } else if (J.mode == 2) {
+        J.out[g] = o[0];
+        J.out[g + 1] = o[1];
+    } else if (J.mode == 3) {
+        J.out[g] = cadd(J.out[g], o[0]);
+        J.out[g + 1] = cadd(J.out[g + 1], o[1]);
+    }
+    if (J.m.base)
+        store_split2(J.m, planes, c - J.c0, x, make_float2((float)v[0].x, (float)v[0].y),
+                     make_float2((float)v[1].x, (float)v[1].y));
 }
 
 // out = Sigma in, Sigma = U diag(sigma) U^H (a circulant), per column:
 // inverse DFT of sigma times the DFT of the column.
-__global__ void k_circ_apply(const double2 *in, double2 *out, int n, int logn, const double2 *sigma,
-                             const double2 *tw) {
+// blockIdx.y: 0 the first slab row (Sigma_bot, out cb), 1 the last (Sigma_top, ct);
+// blockIdx.z: design.
+__global__ void k_circ_apply(const __grid_constant__ Tab<const double2 *> Et, long long last, const __grid_constant__ Tab<double2 *> cbt, const __grid_constant__ Tab<double2 *> ctt,
+                             int n, int logn, const double2 *sigma, const double2 *tw) {
     extern __shared__ double2 a[];
-    const double2 *src = in + (long long)blockIdx.x * n;
+    const double2 *src = Et.v[blockIdx.z] + (blockIdx.y ? last : 0) + (long long)blockIdx.x * n;
+    double2 *out = blockIdx.y ? ctt.v[blockIdx.z] : cbt.v[blockIdx.z];
+    sigma += blockIdx.y * n;
     for (int i = threadIdx.x; i < n; i += blockDim.x) a[__brev((unsigned)i) >> (32 - logn)] = src[i];
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
@@ -603,33 +576,69 @@ __global__ void k_circ_apply(const double2 *in, double2 *out, int n, int logn, c
 // r_j = R_j - K E restricted to the slab, float64.  K E at a pixel is
 // d E - (sum of the four neighbours) + boundary terms, d = 4 - k^2 eps; the
 // neighbour sum and the boundary terms are gathered first so that the
-// diagonal term is one fused multiply-add per component.
-__global__ void k_residual(GridDev g, const double *eps, const double2 *E, const double2 *R, const double2 *cb,
-                           const double2 *ct, double2 *r, int ncol) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int c = blockIdx.y, j = blockIdx.z;
-    const int n = g.nx;
-    if (x >= n) return;
+// diagonal term is one fused multiply-add per component.  One thread walks the
+// slab rows of one (column, x), so each field value is loaded three times (as
+// centre, left, right) instead of five, and the squared norm of the column is
+// summed on the way (part: one value per block, see k_normsum).  R is zero
+// except on the first and last slab rows (Rt: those two rows; null: r = K E).
+// Bound by the float64 pipe (11 operations per point, 2 per clock and SM).
+__global__ void __launch_bounds__(128) k_residual(GridDev g, const __grid_constant__ Tab<const double *> epst, const __grid_constant__ Tab<const double2 *> Et, const __grid_constant__ Tab<const double2 *> Rt, const __grid_constant__ Tab<double2 *> cbt,
+                                                  const __grid_constant__ Tab<double2 *> ctt, const __grid_constant__ Tab<double2 *> rt, const __grid_constant__ Tab<double *> partt, int ncol) {
+    const int b = blockIdx.z, c = blockIdx.y, n = g.nx, h = g.h;
+    const int x = blockIdx.x * 128 + threadIdx.x;
     const long long L = (long long)ncol * n;
-    const double2 *e = E + j * L + (long long)c * n;
-    const double d = fma(-(g.k * g.k), eps[(long long)j * n + x], 4.0);
-    const int xr = (x + 1 == n) ? 0 : x + 1, xl = (x == 0) ? n - 1 : x - 1;
-    double2 nbr = cadd(e[xr], e[xl]);  // neighbours minus boundary terms
-    if (j > 0) nbr = cadd(nbr, e[x - L]);
-    if (j < g.h - 1) nbr = cadd(nbr, e[x + L]);
-    if (j == 0) nbr = csub(nbr, cb[(long long)c * n + x]);
-    if (j == g.h - 1) nbr = csub(nbr, ct[(long long)c * n + x]);
-    const double2 ex = e[x];
-    const double2 v = make_double2(fma(d, ex.x, -nbr.x), fma(d, ex.y, -nbr.y));
-    const long long idx = j * L + (long long)c * n + x;
-    r[idx] = R ? csub(R[idx], v) : v;  // without R: K E
+    double acc = 0.0;
+    if (x < n) {
+        const double *eps = epst.v[b] + x;
+        const double2 *R = Rt.v[b];
+        const double2 *e = Et.v[b] + (long long)c * n;
+        double2 *r = rt.v[b] + (long long)c * n + x;
+        const double k2 = -(g.k * g.k);
+        const int xr = (x + 1 == n) ? 0 : x + 1, xl = (x == 0) ? n - 1 : x - 1;
+        double2 below = cmk(0.0, 0.0), here = e[x];
+        for (int j = 0; j < h; ++j, e += L, r += L) {
+            const double2 above = j + 1 < h ? e[L + x] : cmk(0.0, 0.0);
+            double2 nbr = cadd(e[xr], e[xl]);  // neighbours minus boundary terms (plus the right-hand side)
+            if (j > 0) nbr = cadd(nbr, below);
+            if (j + 1 < h) nbr = cadd(nbr, above);
+            if (j == 0) nbr = csub(nbr, cbt.v[b][(long long)c * n + x]);
+            if (j == h - 1) nbr = csub(nbr, ctt.v[b][(long long)c * n + x]);
+            if (R) {
+                if (j == 0) nbr = cadd(nbr, R[(long long)c * n + x]);
+                if (j == h - 1 && h > 1) nbr = cadd(nbr, R[L + (long long)c * n + x]);
+            }
+            const double d = fma(k2, eps[(long long)j * n], 4.0);
+            double2 v = make_double2(fma(-d, here.x, nbr.x), fma(-d, here.y, nbr.y));
+            if (!R) v = make_double2(-v.x, -v.y);  // K E
+            *r = v;
+            acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+            below = here;
+            here = above;
+        }
+    }
+    double *part = partt.v[b];
+    if (!part) return;
+    __shared__ double red[4];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) part[(long long)c * gridDim.x + blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// out[c] = the sum of column c's np partial sums, in a fixed order (one warp per column).
+__global__ void __launch_bounds__(32) k_normsum(const __grid_constant__ Tab<double *> partt, int np, const __grid_constant__ Tab<double *> outt) {
+    const double *p = partt.v[blockIdx.z] + (long long)blockIdx.x * np;
+    double a = 0.0;
+    for (int i = threadIdx.x; i < np; i += 32) a += p[i];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if (threadIdx.x == 0) outt.v[blockIdx.z][blockIdx.x] = a;
 }
 
 // out[c] = sum_{j,x} |X_j[c][x]|^2 (one block of 256 threads per column, a
-// fixed summation order; two independent loads in flight per thread).  With
-// `copy`, X is also copied there.
-__global__ void __launch_bounds__(256) k_colnorm(const double2 *X, int h, int ncol, int nx, double *out,
-                                                 double2 *copy) {
+// fixed summation order; two independent loads in flight per thread).
+__global__ void __launch_bounds__(256) k_colnorm(const double2 *X, int h, int ncol, int nx, double *out) {
     __shared__ double red[256];
     const int c = blockIdx.x;
     double a0 = 0.0, a1 = 0.0;
@@ -639,16 +648,11 @@ __global__ void __launch_bounds__(256) k_colnorm(const double2 *X, int h, int nc
         int x = threadIdx.x;
         for (; x + 256 < nx; x += 512) {
             const double2 u = p[x], v = p[x + 256];
-            if (copy) {
-                copy[o + x] = u;
-                copy[o + x + 256] = v;
-            }
             a0 += cabs2(u);
             a1 += cabs2(v);
         }
         if (x < nx) {
             const double2 u = p[x];
-            if (copy) copy[o + x] = u;
             a0 += cabs2(u);
         }
     }
@@ -694,11 +698,6 @@ __global__ void k_colscale(double2 *Y, const double2 *X, const double *nrm2, int
     const long long i = ((long long)j * ncol + c) * nx + x;
     const double n2 = nrm2[c];
     Y[i] = n2 > 0.0 ? cscale(X[i], 1.0 / sqrt(n2)) : cmk(0.0, 0.0);
-}
-
-__global__ void k_axpy(double2 *E, const double2 *d, long long n) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < n) E[i] = cadd(E[i], d[i]);
 }
 
 // g_j(x) = 2 k^2 Re sum_b Phi_j[b][x] Q[b][x].  Block: 32 consecutive x (lanes)
@@ -757,63 +756,24 @@ struct PV {  // planar complex view
     PV off(long long r, long long c) const { return PV{re + r * ld + c, im + r * ld + c, ld}; }
 };
 
-PackJob make_job(__nv_bfloat16 *dst, const PV &src, int R, int K, bool trans, bool layoutB, int nsplit,
-                 PackView *view) {
-    long long kp = round_up(2LL * K, 64);
-    long long rows = layoutB ? 2LL * R : R;
-    *view = PackView{dst, rows, kp, nsplit, rows * kp};
-    return PackJob{src.re, src.im, src.ld, R, K, trans ? 1 : 0, layoutB ? 1 : 0, nsplit, dst, kp, rows * kp};
-}
-
-template <int N>
-void launch_jobs_n(apf_ctx *c, const PackJob *js, int nj, cudaStream_t s) {
-    PackJobsN<N> jobs{};
-    int maxR = 0, maxK = 0;
-    for (int i = 0; i < nj; ++i) {
-        jobs.j[i] = js[i];
-        if (js[i].kp != 2LL * js[i].K)
-            cudaMemsetAsync(js[i].out, 0, sizeof(__nv_bfloat16) * (js[i].plane_pitch * js[i].nsplit), s);
-        maxR = std::max(maxR, js[i].R);
-        maxK = std::max(maxK, js[i].K);
-    }
-    dim3 grid((maxK + 63) / 64, (maxR + 31) / 32, nj);
-    bool vec = true;
-    for (int i = 0; i < nj; ++i) {
-        const PackJob &J = js[i];
-        vec = vec && J.R % 32 == 0 && J.K % 64 == 0 && J.ld % 4 == 0 && J.R == maxR && J.K == maxK &&
-              ((((uintptr_t)J.re) | ((uintptr_t)J.im) | ((uintptr_t)J.out)) & 15) == 0 && J.kp % 8 == 0 &&
-              J.plane_pitch % 8 == 0;
-    }
-    if (vec) APF_LAUNCH(c, k_pack32v<N>, grid, 256, 0, s, jobs);
-    else APF_LAUNCH(c, k_pack32<N>, grid, dim3(32, 8), 0, s, jobs);
-}
-
-void launch_jobs(apf_ctx *c, const PackJob *js, int nj, cudaStream_t s) {
-    if (nj <= 2) launch_jobs_n<2>(c, js, nj, s);
-    else launch_jobs_n<MAX_JOBS>(c, js, nj, s);
-}
-
-PackView pack32(apf_ctx *c, __nv_bfloat16 *dst, const PV &src, int R, int K, bool trans, bool layoutB, int nsplit,
-                cudaStream_t s) {
-    PackView v;
-    PackJob j = make_job(dst, src, R, K, trans, layoutB, nsplit, &v);
-    launch_jobs(c, &j, 1, s);
-    return v;
-}
-
-// The designs of one call: every step below launches once for all of them
-// (they share grid, slab height, channel set and settings; each has its own
-// buffers).  A single design is a batch of one.
+// The problems of one launch: designs, and for the elimination and the sweeps
+// also the two chains of each (sd[b]); they share grid, slab height, channel set
+// and settings, each has its own buffers.
 struct Bat {
-    int n = 1;
-    apf_ctx *c[TC_MAX_BATCH] = {};
+    int n = 0;
+    apf_ctx *c[CG_MAX_PROB] = {};
+    int sd[CG_MAX_PROB] = {};
     apf_ctx *lead() const { return c[0]; }
+    SideWork &w(int b) const { return c[b]->mw->sd[sd[b]]; }
+    void add(apf_ctx *ctx, int side) {
+        c[n] = ctx;
+        sd[n++] = side;
+    }
 };
 
 Bat one(apf_ctx *c) {
     Bat b;
-    b.n = 1;
-    b.c[0] = c;
+    b.add(c, 0);
     return b;
 }
 
@@ -822,26 +782,6 @@ Tab<T> tab(const Bat &bt, F f) {
     Tab<T> t{};
     for (int b = 0; b < bt.n; ++b) t.v[b] = f(b);
     return t;
-}
-
-// Pack the A operand sa[b] and the B operand sb[b] of one product for every
-// design (in w->PA / w->PB of each design) in one launch.
-void pack2_b(const Bat &bt, PackView *va, const PV *sa, int Ra, int Ka, bool ta, PackView *vb, const PV *sb, int Rb,
-             int Kb, bool tb, int nsplit, cudaStream_t s) {
-    PackJob js[2 * TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b) {
-        MixedWork *w = bt.c[b]->mw;
-        js[2 * b] = make_job(w->PA, sa[b], Ra, Ka, ta, false, nsplit, &va[b]);
-        js[2 * b + 1] = make_job(w->PB, sb[b], Rb, Kb, tb, true, nsplit, &vb[b]);
-    }
-    launch_jobs(bt.lead(), js, 2 * bt.n, s);
-}
-
-void pack32_b(const Bat &bt, PackView *v, __nv_bfloat16 *const *dst, const PV *src, int R, int K, bool trans,
-              bool layoutB, int nsplit, cudaStream_t s) {
-    PackJob js[TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b) js[b] = make_job(dst[b], src[b], R, K, trans, layoutB, nsplit, &v[b]);
-    launch_jobs(bt.lead(), js, bt.n, s);
 }
 
 void pack64A_b(const Bat &bt, PackView *v, __nv_bfloat16 *const *dst, const double2 *const *s1,
@@ -871,202 +811,372 @@ void pack64BT_b(const Bat &bt, PackView *v, __nv_bfloat16 *const *dst, const dou
                tab<__nv_bfloat16 *>(bt, [&](int b) { return dst[b]; }), kp, rows * kp);
 }
 
-// out[b] = alpha A[b] B[b]^T + beta in[b] for every design, one launch.
-int gemm_b(const Bat &bt, const PackView *A, const PackView *B, int nsplit, int M, int N, int n_cplx, float alpha,
-           float beta, const PV *out, const PV *in, cudaStream_t s) {
-    TcProblem pb[TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b)
-        pb[b] = TcProblem{A[b], B[b], out[b].re, out[b].im, in ? in[b].re : nullptr, in ? in[b].im : nullptr,
-                          bt.c[b]->d_flags};
-    return tc_gemm_n(bt.lead(), bt.n, pb, nsplit, M, N, n_cplx, alpha, beta, out[0].ld, in ? in[0].ld : 0, s);
-}
-
 int leaf_size(const MixedWork *w) { return w->leaf; }
 
-// Diagonal block of the recursion, one design (kernel variant per the context's knobs).
-void leaf_one(apf_ctx *lead, const PV &X, int n, int *flags, cudaStream_t s) {
-    MixedWork *w = lead->mw;
-    Tab<float *> re{}, im{};
-    Tab<int *> fl{};
-    re.v[0] = X.re; im.v[0] = X.im; fl.v[0] = flags;
-    // 128 blocks: in-CTA Schur recursion over 32 x 32 Gauss-Jordan leaves
-    // (default); variants 1-3 are the single-level Gauss-Jordan kernels.
-    if (n == 128 && w->leaf_variant == 1)
-        APF_LAUNCH(lead, k_leaf32r2<128>, 1, 512, 0, s, X.re, X.im, X.ld, flags);
-    else if (n == 128 && w->leaf_variant == 2)
-        APF_LAUNCH(lead, k_leaf32<128>, 1, 512, leaf_smem_bytes<128>(8), s, X.re, X.im, X.ld, flags);
-    else if (n == 128 && w->leaf_variant == 3)
-        APF_LAUNCH(lead, k_leaf32r<128>, 1, 512, 0, s, X.re, X.im, X.ld, flags);
-    else if (n == 128)
-        APF_LAUNCH(lead, k_leaf128rec, 1, 512, rec_smem_bytes(), s, re, im, X.ld, fl);
-    else if (n == 64 && w->leaf_variant == 1)
-        APF_LAUNCH(lead, k_leaf32r2<64>, 1, 256, 0, s, X.re, X.im, X.ld, flags);
-    else if (n == 64)
-        APF_LAUNCH(lead, k_leaf32r<64>, 1, 256, 0, s, X.re, X.im, X.ld, flags);
-    else if (n == 32)
-        APF_LAUNCH(lead, k_leaf32<32>, 1, 128, leaf_smem_bytes<32>(8), s, X.re, X.im, X.ld, flags);
-    else if (n == 16)
-        APF_LAUNCH(lead, k_leaf32<16>, 1, 64, leaf_smem_bytes<16>(8), s, X.re, X.im, X.ld, flags);
-    else
-        APF_LAUNCH(lead, k_leaf_inv32, 1, 256, n * n * (int)sizeof(float2), s, X.re, X.im, X.ld, n, flags);
+void mirror_b(const Bat &bt, const PV *X, const Mirror *m, int R, int C, bool trans, int planes, cudaStream_t s) {
+    for (int b = 0; b < bt.n; ++b)
+        APF_LAUNCH(bt.lead(), k_mirror, dim3((C + 127) / 128, R), 128, 0, s, (const float *)X[b].re,
+                   (const float *)X[b].im, X[b].ld, R, C, trans ? 1 : 0, m[b], planes);
 }
 
-// X[b] <- X[b]^-1 in place for complex-symmetric X[b], every design of the
-// batch: the 2x2 block Schur recursion of the float64 path with all four
-// products on the tensor cores.
-int inv32_b(const Bat &bt, const PV *X, int n, float *const *Tre, float *const *Tim, float *const *Vre,
-            float *const *Vim, cudaStream_t s) {
+// Diagonal blocks of the recursion, one CTA per problem (kernel variant per the
+// context's knobs); m: where the split form of the inverse goes (null base: nowhere).
+void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) {
+    apf_ctx *c = bt.lead();
+    const MixedWork *w = c->mw;
+    const int nb = bt.n, v = w->leaf_variant;
+    const long long ld = X[0].ld;
+    const auto re = tab<float *>(bt, [&](int b) { return X[b].re; }), im = tab<float *>(bt, [&](int b) { return X[b].im; });
+    const auto fl = tab<int *>(bt, [&](int b) { return bt.c[b]->d_flags; });
+    // 128 blocks: in-CTA Schur recursion over 32 x 32 Gauss-Jordan leaves
+    // (default); variants 1-3 are the single-level Gauss-Jordan kernels.
+    if (n == 128 && v == 0) {
+        APF_LAUNCH(c, k_leaf128rec, nb, 512, rec_smem_bytes(), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+                   w->nsplit_elim, fl);
+        return;
+    }
+    if (n == 128 && v == 1) APF_LAUNCH(c, k_leaf32r2<128>, nb, 512, 0, s, re, im, ld, fl);
+    else if (n == 128 && v == 2) APF_LAUNCH(c, k_leaf32<128>, nb, 512, leaf_smem_bytes<128>(8), s, re, im, ld, fl);
+    else if (n == 128) APF_LAUNCH(c, k_leaf32r<128>, nb, 512, 0, s, re, im, ld, fl);
+    else if (n == 64 && v == 1) APF_LAUNCH(c, k_leaf32r2<64>, nb, 256, 0, s, re, im, ld, fl);
+    else if (n == 64) APF_LAUNCH(c, k_leaf32r<64>, nb, 256, 0, s, re, im, ld, fl);
+    else if (n == 32) APF_LAUNCH(c, k_leaf32<32>, nb, 128, leaf_smem_bytes<32>(8), s, re, im, ld, fl);
+    else if (n == 16) APF_LAUNCH(c, k_leaf32<16>, nb, 64, leaf_smem_bytes<16>(8), s, re, im, ld, fl);
+    else APF_LAUNCH(c, k_leaf_inv32, nb, 256, n * n * (int)sizeof(float2), s, re, im, ld, n, fl);
+    if (m[0].base) mirror_b(bt, X, m, n, n, false, w->nsplit_elim, s);
+}
+
+// X[b] <- X[b]^-1 in place for complex-symmetric X[b] (n a power of two), by the
+// 2x2 block Schur recursion of the float64 path,
+//   [A B; C D]^-1 = [Ai + T^T V, -V^T; -V, Si],  T = C Ai, S = D - T C^T, V = Si T,
+// with all four products on the tensor cores, two of them symmetric.  X holds the
+// block in float32 (on and below its diagonal blocks) and XP the split form of
+// what lies below them; both come out as the whole inverse.  Every product reads
+// split operands where the previous steps' epilogues left them (T only exists
+// split, as T and T^T; V is written as -V to C and, transposed, to B, and read
+// back from B as the operand of T^T V), so nothing runs between the products.
+// toff: offset of this level's T in the T buffers.
+int inv32_b(const Bat &bt, const PV *X, const Mirror *XP, int n, bool want_mirror, long long toff, cudaStream_t s) {
     apf_ctx *c = bt.lead();
     MixedWork *w = c->mw;
-    const int nb = bt.n;
+    const int nb = bt.n, planes = w->nsplit_elim;
     if (n <= leaf_size(w)) {
-        if (n == 128 && w->leaf_variant == 0) {
-            // one CTA per design's block
-            APF_LAUNCH(c, k_leaf128rec, nb, 512, rec_smem_bytes(), s, tab<float *>(bt, [&](int b) { return X[b].re; }),
-                       tab<float *>(bt, [&](int b) { return X[b].im; }), X[0].ld,
-                       tab<int *>(bt, [&](int b) { return bt.c[b]->d_flags; }));
-        } else {
-            for (int b = 0; b < nb; ++b) leaf_one(c, X[b], n, bt.c[b]->d_flags, s);
-        }
+        Mirror none[CG_MAX_PROB];
+        leaf_b(bt, X, n, want_mirror ? XP : none, s);
         return APF_OK;
     }
     const int h = n / 2;
-    const int ns = w->nsplit_elim;
-    const long long hh = (long long)h * h;
-    PV A[TC_MAX_BATCH], B[TC_MAX_BATCH], C[TC_MAX_BATCH], D[TC_MAX_BATCH], T[TC_MAX_BATCH], V[TC_MAX_BATCH];
-    float *tr2[TC_MAX_BATCH], *ti2[TC_MAX_BATCH], *vr2[TC_MAX_BATCH], *vi2[TC_MAX_BATCH];
+    const long long hh = (long long)h * h, sub = toff + 2 * planes * hh;
+    PV A[CG_MAX_PROB], B[CG_MAX_PROB], C[CG_MAX_PROB], D[CG_MAX_PROB];
+    Mirror mA[CG_MAX_PROB], mB[CG_MAX_PROB], mC[CG_MAX_PROB], mD[CG_MAX_PROB], mT[CG_MAX_PROB], mTT[CG_MAX_PROB];
     for (int b = 0; b < nb; ++b) {
         A[b] = X[b]; B[b] = X[b].off(0, h); C[b] = X[b].off(h, 0); D[b] = X[b].off(h, h);
-        T[b] = PV{Tre[b], Tim[b], h}; V[b] = PV{Vre[b], Vim[b], h};
-        tr2[b] = Tre[b] + hh; ti2[b] = Tim[b] + hh; vr2[b] = Vre[b] + hh; vi2[b] = Vim[b] + hh;
+        mA[b] = XP[b]; mB[b] = XP[b].off(0, h); mC[b] = XP[b].off(h, 0); mD[b] = XP[b].off(h, h);
+        mT[b] = Mirror{bt.w(b).TP + toff, h, hh};
+        mTT[b] = Mirror{bt.w(b).TT + toff, h, hh};
     }
+    auto out = [](const PV &v, const Mirror &m) { return CgOut{v.re, v.im, v.ld, m}; };
+    CgProblem pb[CG_MAX_PROB];
+    auto product = [&](const Mirror *P, const Mirror *Q, float alpha, const PV *in, const PV *o, const Mirror *om,
+                       const PV *ot, const Mirror *otm, bool sym) {
+        for (int b = 0; b < nb; ++b) {
+            pb[b] = CgProblem{};
+            pb[b].A = P[b];
+            pb[b].B = Q[b];
+            pb[b].M = h;
+            pb[b].out = out(o ? o[b] : PV{}, om[b]);
+            pb[b].outT = out(ot ? ot[b] : PV{}, otm[b]);
+            if (in) {
+                pb[b].in_re = in[b].re;
+                pb[b].in_im = in[b].im;
+                pb[b].ldi = in[b].ld;
+            }
+            pb[b].flags = bt.c[b]->d_flags;
+        }
+        return cgemm_n(c, nb, pb, planes, h, h, h, alpha, in ? 1.f : 0.f, sym, false, s);
+    };
     int rc;
-    PackView pa[TC_MAX_BATCH], pb[TC_MAX_BATCH];
-    if ((rc = inv32_b(bt, A, h, tr2, ti2, vr2, vi2, s))) return rc;
-    // T = C Ai
-    pack2_b(bt, pa, C, h, h, false, pb, A, h, h, false, ns, s);
-    if ((rc = gemm_b(bt, pa, pb, ns, h, 2 * h, h, 1.f, 0.f, T, nullptr, s))) return rc;
-    // D = D - T B   (B-operand columns = rows of C)
-    pack2_b(bt, pa, T, h, h, false, pb, C, h, h, false, ns, s);
-    if ((rc = gemm_b(bt, pa, pb, ns, h, 2 * h, h, -1.f, 1.f, D, D, s))) return rc;
-    if ((rc = inv32_b(bt, D, h, tr2, ti2, vr2, vi2, s))) return rc;
-    // V = Si T
-    pack2_b(bt, pa, D, h, h, false, pb, T, h, h, true, ns, s);
-    if ((rc = gemm_b(bt, pa, pb, ns, h, 2 * h, h, 1.f, 0.f, V, nullptr, s))) return rc;
-    // A = Ai + V^T T   (the B operand is still the packed T^T)
-    __nv_bfloat16 *padst[TC_MAX_BATCH];
-    for (int b = 0; b < nb; ++b) padst[b] = bt.c[b]->mw->PA;
-    pack32_b(bt, pa, padst, V, h, h, true, false, ns, s);
-    if ((rc = gemm_b(bt, pa, pb, ns, h, 2 * h, h, 1.f, 1.f, A, A, s))) return rc;
-    dim3 grid((h + 31) / 32, (h + 31) / 32, nb);
-    APF_LAUNCH(c, k_negoff32, grid, dim3(32, 8), 0, s, tab<float *>(bt, [&](int b) { return B[b].re; }),
-               tab<float *>(bt, [&](int b) { return B[b].im; }), tab<float *>(bt, [&](int b) { return C[b].re; }),
-               tab<float *>(bt, [&](int b) { return C[b].im; }), X[0].ld,
-               tab<const float *>(bt, [&](int b) { return (const float *)V[b].re; }),
-               tab<const float *>(bt, [&](int b) { return (const float *)V[b].im; }), h);
-    return APF_OK;
+    if ((rc = inv32_b(bt, A, mA, h, true, sub, s))) return rc;
+    // T = C Ai (Ai symmetric: its rows are its columns)
+    if ((rc = product(mC, mA, 1.f, nullptr, nullptr, mT, nullptr, mTT, false))) return rc;
+    // D = D - T C^T
+    if ((rc = product(mT, mC, -1.f, D, D, mD, D, mD, true))) return rc;
+    if ((rc = inv32_b(bt, D, mD, h, true, sub, s))) return rc;
+    // C = -Si T, B = its transpose
+    if ((rc = product(mD, mTT, -1.f, nullptr, C, mC, B, mB, false))) return rc;
+    // A = Ai + V^T T = Ai - B T
+    return product(mB, mTT, -1.f, A, A, mA, A, mA, true);
 }
 
-int inv32(apf_ctx *c, const PV &X, int n, float *Tre, float *Tim, float *Vre, float *Vim, cudaStream_t s) {
-    return inv32_b(one(c), &X, n, &Tre, &Tim, &Vre, &Vim, s);
+// The G_j of a context in split form: slot j, or with recomputation the slot of j's position.
+int row_pos(const apf_ctx *c, int row) {
+    const int m = c->h / 2;
+    return row < m ? row : row == m ? c->h - 1 : m + (c->h - 1 - row);
 }
-
-// Packed operand view of G_j (slot j, or j's slot in its segment).
-PackView gp_view(const apf_ctx *c, int j) {
+int pos_row(const apf_ctx *c, int p) {
+    const int m = c->h / 2;
+    return p < m ? p : p == c->h - 1 ? m : c->h - 1 - (p - m);
+}
+Mirror gp_view(const apf_ctx *c, int row) {
     const MixedWork *w = c->mw;
-    const long long rows = 2LL * c->nx, kp = 2LL * c->nx;
-    const int slot = w->seg_rows > 0 ? j % w->seg_rows : j;
-    return PackView{w->GP + slot * w->gp_stride, rows, kp, w->nsplit_elim, rows * kp};
+    const int slot = w->seg_rows > 0 ? row_pos(c, row) % w->seg_rows : row;
+    return Mirror{w->GP + slot * w->gp_stride, w->pitch, w->pitch * c->nx};
 }
 
-// E[b] ~= Khat[b]^-1 Rin[b] with the stored (or recomputed) G_j of each design
-// (block forward sweep + back substitution).  mcols: columns that the forward
-// sweep must carry.
-int approx_solve_b(const Bat &bt, const double2 *const *Rin, double2 *const *Eout, int mcols, cudaStream_t s) {
+// Launch one k_row_step per problem of `bt` (n: block size; jobs without an
+// output and sources do nothing).
+void row_step_b(const Bat &bt, const RowJob *jobs, int nj, int n, bool bf, cudaStream_t s) {
+    apf_ctx *c = bt.lead();
+    const MixedWork *w = c->mw;
+    const int leaf = std::min(leaf_size(w), n);
+    const GridDev g = make_grid(c);
+    const dim3 grid((unsigned)(((long long)(n / 4) * (n / 8) + 127) / 128), 1, nj);
+    auto run = [&](auto &pack) {
+        for (int i = 0; i < nj; ++i) pack.j[i] = jobs[i];
+        constexpr int N = sizeof(pack.j) / sizeof(RowJob);
+        if (bf) APF_LAUNCH(c, (k_row_step<true, N>), grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
+        else APF_LAUNCH(c, (k_row_step<false, N>), grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
+    };
+    if (nj <= 2) {
+        RowJobs<2> p{};
+        run(p);
+    } else {
+        RowJobs<CG_MAX_PROB> p{};
+        run(p);
+    }
+}
+
+bool uses_butterfly(const MixedWork *w, int n) { return w->bfly && n > leaf_size(w) && n >= 16; }
+
+// The working block of problem b, as a source (its transformed inverse) and as
+// the block to write.
+RowSrc work_src(const SideWork &w, bool use) {
+    RowSrc s{};
+    s.re = w.Xre; s.im = w.Xim;
+    s.yspace = 1;
+    s.use = use ? 1 : 0;
+    return s;
+}
+RowJob row_job(const apf_ctx *c, const SideWork &w, int row) {
+    RowJob j{};
+    j.eps = c->d_eps;
+    j.row = row;
+    j.out = row >= 0 ? 1 : 0;
+    j.sgn = -1.f;
+    j.Xre = w.Xre; j.Xim = w.Xim;
+    j.XP = w.XP;
+    return j;
+}
+
+int invert_work_b(const Bat &bt, cudaStream_t s) {
+    const int n = bt.lead()->nx;
+    PV X[CG_MAX_PROB];
+    Mirror XP[CG_MAX_PROB];
+    for (int b = 0; b < bt.n; ++b) {
+        X[b] = PV{bt.w(b).Xre, bt.w(b).Xim, n};
+        XP[b] = bt.w(b).XP;
+    }
+    return inv32_b(bt, X, XP, n, false, 0, s);
+}
+
+// E ~= Khat^-1 R with the stored (or recomputed) G_j of each design: the
+// right-hand sides are carried along both chains to the middle row, solved
+// there, and substituted back outwards.  R(b, j): row j of design b's right-hand
+// side (null: zero); Y: rows kept on the way in; E: the solution, written, or
+// added to with `accumulate` (then Y is another array).  full: all columns are
+// carried by both chains, else the inputs [0, cf) by the lower and the outputs
+// [cf, ncol) by the upper one (where R is not zero).
+template <typename F>
+int approx_solve_b(const Bat &bt, F R, double2 *const *Y, double2 *const *E, bool accumulate, bool full, cudaStream_t s) {
     apf_ctx *c = bt.lead();
     MixedWork *w = c->mw;
-    const int nb = bt.n;
-    const int ncol = c->cf + c->ca;
-    const int nx = c->nx, ns = w->nsplit_elim;
+    const int nb = bt.n, ncol = c->cf + c->ca, nx = c->nx, h = c->h, m = h / 2, top = h - 1 - m;
+    const int planes = w->nsplit_elim, K = w->seg_rows;
     const long long L = (long long)ncol * nx;
-    const int K = w->seg_rows;
-    // with recomputation: the segment whose inverses row j needs must be loaded
-    auto need = [&](int j) -> int {
+    const int lo[2] = {0, full ? 0 : c->cf}, hi[2] = {full ? ncol : c->cf, ncol};  // columns of each chain
+    // with recomputation: the segment whose inverses `row` needs must be loaded
+    auto need = [&](int row) -> int {
         if (K <= 0) return APF_OK;
-        const int sg = j / K;
+        const int sg = row_pos(c, row) / K;
         if (sg == w->seg_loaded) return APF_OK;
         return recompute_segment_b(bt, sg, s);
     };
-    PV O[TC_MAX_BATCH];
-    __nv_bfloat16 *padst[TC_MAX_BATCH];
-    for (int b = 0; b < nb; ++b) {
-        MixedWork *wb = bt.c[b]->mw;
-        O[b] = PV{wb->O32, wb->O32 + L, nx};
-        padst[b] = wb->PA;
-        cudaMemcpyAsync(Eout[b], Rin[b], sizeof(double2) * L, cudaMemcpyDeviceToDevice, s);
-    }
-    auto otab_re = tab<const float *>(bt, [&](int b) { return (const float *)O[b].re; });
-    auto otab_im = tab<const float *>(bt, [&](int b) { return (const float *)O[b].im; });
-    dim3 cgrid((nx + 255) / 256, ncol, nb);
-    PackView pa[TC_MAX_BATCH], gv[TC_MAX_BATCH];
-    const double2 *src[TC_MAX_BATCH], *src2[TC_MAX_BATCH];
-    int rc;
-    for (int j = 1; j < c->h; ++j) {
-        if (mcols > 0) {
-            if ((rc = need(j - 1))) return rc;
+    auto side = [&](int b, int sd) -> SideWork & { return bt.c[b]->mw->sd[sd]; };
+    const int form_rows = full ? ncol : std::max(c->cf, c->ca);  // the same for both chains and in every step
+    // O32 of each chain <- (operand of the chain) G_row^T for the chains that take part
+    auto multiply = [&](const int *row, const int *cols) -> int {
+        CgProblem pb[CG_MAX_PROB];
+        int n = 0, M = 0;
+        for (int sd = 0; sd < 2; ++sd) {
+            if (row[sd] < 0 || cols[sd] <= 0) continue;
+            if (int rc = need(row[sd])) return rc;
+            M = std::max(M, cols[sd]);
             for (int b = 0; b < nb; ++b) {
-                src[b] = Eout[b] + (j - 1) * L;
-                gv[b] = gp_view(bt.c[b], j - 1);
+                SideWork &sw = side(b, sd);
+                CgProblem &p = pb[n++];
+                p.A = sw.PA;
+                p.B = gp_view(bt.c[b], row[sd]);
+                p.M = cols[sd];
+                p.out = CgOut{sw.O32, sw.O32 + L, nx, Mirror{}};
+                p.flags = bt.c[b]->d_flags;
             }
-            pack64A_b(bt, pa, padst, src, nullptr, nx, mcols, nx, ns, s);
-            if ((rc = gemm_b(bt, pa, gv, ns, mcols, 2 * nx, nx, 1.f, 0.f, O, nullptr, s))) return rc;
         }
-        APF_LAUNCH(c, k_combine, cgrid, 256, 0, s, tab<double2 *>(bt, [&](int b) { return Eout[b] + j * L; }),
-                   tab<const double2 *>(bt, [&](int b) { return Rin[b] + j * L; }), otab_re, otab_im, ncol, mcols,
-                   nx);
-    }
-    for (int j = c->h - 1; j >= 0; --j) {
-        if ((rc = need(j))) return rc;
-        for (int b = 0; b < nb; ++b) {
-            src[b] = Eout[b] + j * L;
-            src2[b] = (j == c->h - 1) ? nullptr : Eout[b] + (j + 1) * L;
-            gv[b] = gp_view(bt.c[b], j);
+        return n ? cgemm_n(c, n, pb, planes, M, nx, nx, 1.f, 0.f, false, true, s, form_rows) : APF_OK;
+    };
+    FieldJob fj[CG_MAX_PROB];
+    int nj = 0;
+    auto push = [&](const FieldJob &j) {
+        if (j.c1 > j.c0) fj[nj++] = j;
+    };
+    auto flush = [&]() {
+        if (!nj) return;
+        int rows = 0;
+        for (int i = 0; i < nj; ++i) rows = std::max(rows, fj[i].c1 - fj[i].c0);
+        const int threads = nx >= 256 ? 128 : 32;
+        const dim3 grid((nx / 2 + threads - 1) / threads, rows, nj);
+        auto run = [&](auto &pack) {
+            for (int i = 0; i < nj; ++i) pack.j[i] = fj[i];
+            constexpr int N = sizeof(pack.j) / sizeof(FieldJob);
+            APF_LAUNCH(c, k_field_step<N>, grid, threads, 0, s, pack, nx, planes);
+        };
+        if (nj <= 2) {
+            FieldJobs<2> p{};
+            run(p);
+        } else {
+            FieldJobs<CG_MAX_PROB> p{};
+            run(p);
         }
-        pack64A_b(bt, pa, padst, src, (j == c->h - 1) ? nullptr : src2, nx, ncol, nx, ns, s);
-        if ((rc = gemm_b(bt, pa, gv, ns, ncol, 2 * nx, nx, 1.f, 0.f, O, nullptr, s))) return rc;
-        APF_LAUNCH(c, k_combine, cgrid, 256, 0, s, tab<double2 *>(bt, [&](int b) { return Eout[b] + j * L; }),
-                   tab<const double2 *>(bt, [&](int b) { return (const double2 *)nullptr; }), otab_re, otab_im,
-                   ncol, ncol, nx);
+        nj = 0;
+    };
+    // one design's jobs at a time in Y / R rows; chain sd's row t steps from its end
+    auto chain_row = [&](int sd, int t) { return sd ? h - 1 - t : t; };
+    const int len[2] = {m, top};
+    // carried rows: row t's operand (Y_t = R_t + O) and, past the end row, Y_t itself
+    auto carry = [&](int b, int sd, int t) {
+        SideWork &sw = side(b, sd);
+        const int row = chain_row(sd, t);
+        FieldJob j{};
+        j.O = t > 0 ? sw.O32 : nullptr;
+        j.olen = L;
+        j.o0 = lo[sd]; j.o1 = hi[sd];
+        j.add = R(b, row);
+        j.a0 = 0; j.a1 = ncol;
+        if (t > 0) { j.out = Y[b] + row * L; j.mode = 1; }
+        j.m = sw.PA;
+        j.c0 = lo[sd]; j.c1 = hi[sd];
+        push(j);
+    };
+    // inwards; with recomputation one chain after the other, so that each segment is loaded once
+    auto inwards = [&](bool s0, bool s1) -> int {
+        const bool on[2] = {s0 && m > 0 && hi[0] > lo[0], s1 && top > 0 && hi[1] > lo[1]};
+        for (int sd = 0; sd < 2; ++sd)
+            if (on[sd])
+                for (int b = 0; b < nb; ++b) carry(b, sd, 0);
+        flush();
+        for (int t = 1; t <= std::max(on[0] ? m : 0, on[1] ? top : 0); ++t) {
+            int row[2], cols[2];
+            for (int sd = 0; sd < 2; ++sd) {
+                row[sd] = on[sd] && t <= len[sd] ? chain_row(sd, t - 1) : -1;
+                cols[sd] = hi[sd] - lo[sd];
+            }
+            if (int e = multiply(row, cols)) return e;
+            for (int sd = 0; sd < 2; ++sd)
+                if (on[sd] && t < len[sd])
+                    for (int b = 0; b < nb; ++b) carry(b, sd, t);
+            flush();
+        }
+        return APF_OK;
+    };
+    int rc = inwards(true, K <= 0);
+    if (rc == APF_OK && K > 0) rc = inwards(false, true);
+    if (rc) return rc;
+    // the middle row: both chains' contributions, then its own inverse
+    for (int b = 0; b < nb; ++b) {
+        FieldJob j{};
+        j.O = m > 0 && hi[0] > lo[0] ? side(b, 0).O32 : nullptr;
+        j.O2 = top > 0 && hi[1] > lo[1] ? side(b, 1).O32 : nullptr;
+        j.olen = L;
+        j.o0 = lo[0]; j.o1 = hi[0]; j.p0 = lo[1]; j.p1 = hi[1];
+        j.add = R(b, m);
+        j.a0 = 0; j.a1 = ncol;
+        j.m = side(b, 0).PA;
+        j.c0 = 0; j.c1 = ncol;
+        push(j);
     }
-    return APF_OK;
+    flush();
+    {
+        const int row[2] = {m, -1}, cols[2] = {ncol, 0};
+        if ((rc = multiply(row, cols))) return rc;
+    }
+    // outwards: E_row = o (in O32 of `from`), and chain sd's next operand, Y_next + o
+    auto outward = [&](int b, int sd, int row, const SideWork &from, bool store) {
+        const int next = sd ? row + 1 : row - 1;
+        FieldJob j{};
+        j.O = from.O32;
+        j.olen = L;
+        j.o0 = 0; j.o1 = ncol;
+        if (store) { j.out = E[b] + row * L; j.mode = accumulate ? 3 : 2; }
+        if (next >= 0 && next < h) {
+            // (on the chain's end row nothing was added to R)
+            j.add = next == chain_row(sd, 0) ? R(b, next) : Y[b] + next * L;
+            j.a0 = lo[sd]; j.a1 = hi[sd];
+            j.m = side(b, sd).PA;
+        }
+        j.c0 = 0; j.c1 = ncol;
+        push(j);
+    };
+    for (int b = 0; b < nb; ++b) {
+        outward(b, 0, m, side(b, 0), true);
+        if (top > 0) outward(b, 1, m, side(b, 0), false);
+    }
+    flush();
+    auto outwards = [&](bool s0, bool s1) -> int {
+        for (int t = 1; t <= std::max(s0 ? m : 0, s1 ? top : 0); ++t) {
+            const int row[2] = {s0 && t <= m ? m - t : -1, s1 && t <= top ? m + t : -1}, cols[2] = {ncol, ncol};
+            if (int e = multiply(row, cols)) return e;
+            for (int sd = 0; sd < 2; ++sd)
+                if (row[sd] >= 0)
+                    for (int b = 0; b < nb; ++b) outward(b, sd, row[sd], side(b, sd), true);
+            flush();
+        }
+        return APF_OK;
+    };
+    if (K <= 0) return outwards(true, true);
+    if ((rc = outwards(false, true))) return rc;  // the upper chain first: segment 0 is loaded at the end
+    return outwards(true, false);
 }
 
-int approx_solve(apf_ctx *c, const double2 *Rin, double2 *Eout, int mcols, cudaStream_t s) {
-    return approx_solve_b(one(c), &Rin, &Eout, mcols, s);
-}
-
-int residual(apf_ctx *c, const double2 *E, double2 *r, cudaStream_t s) {
-    MixedWork *w = c->mw;
-    int ncol = c->cf + c->ca;
-    int nx = c->nx;
-    long long L = (long long)ncol * nx;
+// r = R - K E and the squared column norms of r (rhs), or r = K E (not rhs), for
+// every design: E(b), r(b) fields.
+template <typename FE, typename FR>
+void residual_b(const Bat &bt, FE E, FR r, bool rhs, cudaStream_t s) {
+    apf_ctx *c = bt.lead();
+    const int ncol = c->cf + c->ca, nx = c->nx, nb = bt.n;
+    const long long L = (long long)ncol * nx;
     int logn = 0;
     while ((1 << logn) < nx) ++logn;
-    int threads = nx / 2 < 256 ? nx / 2 : 256;
-    int smem = nx * (int)sizeof(double2);
-    APF_LAUNCH(c, k_circ_apply, ncol, threads, smem, s, E, w->cb, nx, logn, c->d_modes, c->d_tw);
-    APF_LAUNCH(c, k_circ_apply, ncol, threads, smem, s, E + (c->h - 1) * L, w->ct, nx, logn, c->d_modes + nx,
-               c->d_tw);
-    GridDev g = make_grid(c);
-    dim3 grid((nx + 255) / 256, ncol, c->h);
-    APF_LAUNCH(c, k_residual, grid, 256, 0, s, g, c->d_eps, E, c->d_R, w->cb, w->ct, r, ncol);
-    return APF_OK;
+    const int threads = nx / 2 < 256 ? nx / 2 : 256;
+    const auto Et = tab<const double2 *>(bt, [&](int b) { return (const double2 *)E(b); });
+    const auto cb = tab<double2 *>(bt, [&](int b) { return bt.c[b]->mw->cb; });
+    const auto ct = tab<double2 *>(bt, [&](int b) { return bt.c[b]->mw->ct; });
+    const auto part = tab<double *>(bt, [&](int b) { return rhs ? bt.c[b]->mw->rpart : nullptr; });
+    APF_LAUNCH(c, k_circ_apply, dim3(ncol, 2, nb), threads, nx * (int)sizeof(double2), s, Et, (c->h - 1) * L, cb, ct, nx,
+               logn, (const double2 *)c->d_modes, (const double2 *)c->d_tw);
+    const dim3 grid((nx + 127) / 128, ncol, nb);
+    APF_LAUNCH(c, k_residual, grid, 128, 0, s, make_grid(c),
+               tab<const double *>(bt, [&](int b) { return (const double *)bt.c[b]->d_eps; }), Et,
+               tab<const double2 *>(bt, [&](int b) { return rhs ? (const double2 *)bt.c[b]->d_R : nullptr; }), cb, ct,
+               tab<double2 *>(bt, [&](int b) { return (double2 *)r(b); }), part, ncol);
+    if (rhs)
+        APF_LAUNCH(c, k_normsum, dim3(ncol, 1, nb), 32, 0, s, part, (int)grid.x,
+                   tab<double *>(bt, [&](int b) { return bt.c[b]->mw->rnorm + ncol; }));
 }
 
 }  // namespace
 
 void mixed_init_attrs() {
     tc_init_attrs();
+    cgemm_init_attrs();
     cudaFuncSetAttribute(k_leaf_inv32, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * (int)sizeof(float2));
     cudaFuncSetAttribute(k_leaf32<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<128>(8));
     cudaFuncSetAttribute(k_leaf32<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<64>(8));
@@ -1094,21 +1204,31 @@ int mixed_alloc(apf_ctx *c) {
         int v = atoi(e);
         if (v >= 0 && v <= 3) w->leaf_variant = v;
     }
-    long long n = c->nx, h = c->h;
-    int nin = c->nin, nout = c->nout;
-    long long ncol = nin + nout;
+    const long long n = c->nx, h = c->h, q = 2 * w->nsplit_elim;  // q: component planes of a split matrix
+    const int nin = c->nin, nout = c->nout;
+    const long long ncol = std::max(nin + nout, nin);
+    w->pitch = std::max<long long>(n, 64);
+    w->seg_rows = (c->schur_seg > 0 && c->schur_seg < h) ? c->schur_seg : 0;
+    w->nseg = w->seg_rows > 0 ? (int)((h + w->seg_rows - 1) / w->seg_rows) : 1;
+    w->nside = w->seg_rows > 0 || h < 3 ? 1 : 2;  // chains eliminated at the same time
     int rc;
 #define WA(p, cnt) if ((rc = walloc(c, w, &(p), (cnt))) != APF_OK) return rc;
-    WA(w->Xre, n * n); WA(w->Xim, n * n);
-    WA(w->Tre, n * n / 2); WA(w->Tim, n * n / 2); WA(w->Vre, n * n / 2); WA(w->Vim, n * n / 2);
-    int ns_max = std::max(w->nsplit_elim, w->nsplit_grad);
-    // A operands: recursion (h x 2h), fields (ncol x 2n), Gamma (n_out x kp)
-    long long kp_g = round_up(2LL * nin, 64);
-    w->pa_elems = std::max({(n / 2) * n * w->nsplit_elim, ncol * 2 * n * w->nsplit_elim, (long long)nout * kp_g * ns_max});
-    // B operands: recursion (2h x 2h), gradient (2n x kp_g)
-    w->pb_elems = std::max(n * n * w->nsplit_elim, 2 * n * kp_g * ns_max);
-    WA(w->PA, w->pa_elems);
-    WA(w->PB, w->pb_elems);
+    for (int sd = 0; sd < 2; ++sd) {
+        SideWork &sw = w->sd[sd];
+        if (sd < w->nside) {
+            WA(sw.Xre, n * n); WA(sw.Xim, n * n);
+            WA(sw.XP.base, q * n * w->pitch);
+            sw.XP.pitch = w->pitch; sw.XP.qpitch = n * w->pitch;
+            // T of the levels n/2, n/4, ..: q (n^2/4 + n^2/16 + ..) < q n^2 / 3
+            WA(sw.TP, q * (n * n * 11 / 32 + 64)); WA(sw.TT, q * (n * n * 11 / 32 + 64));
+        }
+        WA(sw.O32, 2 * ncol * n);
+        WA(sw.PA.base, q * ncol * w->pitch);
+        sw.PA.pitch = w->pitch; sw.PA.qpitch = ncol * w->pitch;
+    }
+    const long long kp_g = round_up(2LL * nin, 64);
+    WA(w->GA, (long long)nout * kp_g * w->nsplit_grad);
+    WA(w->GB, 2 * n * kp_g * w->nsplit_grad);
     if (const char *e = getenv("APF_BUTTERFLY")) w->bfly = (e[0] == '1');  // diagnostic knob; default from ctx
     else w->bfly = c->butterfly;
     WA(w->BW, 2 * n);
@@ -1129,15 +1249,23 @@ int mixed_alloc(apf_ctx *c) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap_stream);
         if (e != cudaSuccess) return check_cuda(c, e, "butterfly weights");
     }
-    w->gp_stride = 2 * n * 2 * n * w->nsplit_elim;
-    w->seg_rows = (c->schur_seg > 0 && c->schur_seg < h) ? c->schur_seg : 0;
-    w->nseg = w->seg_rows > 0 ? (int)((h + w->seg_rows - 1) / w->seg_rows) : 1;
-    WA(w->GP, (w->seg_rows > 0 ? w->seg_rows : h) * w->gp_stride);
-    if (w->seg_rows > 0) { WA(w->CK, (long long)(w->nseg - 1) * 2 * n * n); }
-    WA(w->O32, 2 * std::max<long long>(ncol, nout) * n);
+    w->gp_stride = q * n * w->pitch;
+    const long long slots = w->seg_rows > 0 ? w->seg_rows : h;
+    WA(w->GP, slots * w->gp_stride);
+    if (w->seg_rows > 0) {
+        WA(w->CK, (long long)(w->nseg - 1) * 2 * n * n);
+        WA(w->CKB, 2 * n * n);
+    }
+    if (w->pitch > n) {  // the padding columns of the products' operands are read: zero
+        cudaError_t e = cudaMemsetAsync(w->GP, 0, sizeof(__nv_bfloat16) * slots * w->gp_stride, c->cap_stream);
+        for (int sd = 0; sd < 2 && e == cudaSuccess; ++sd)
+            e = cudaMemsetAsync(w->sd[sd].PA.base, 0, sizeof(__nv_bfloat16) * q * ncol * w->pitch, c->cap_stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap_stream);
+        if (e != cudaSuccess) return check_cuda(c, e, "clear operand padding");
+    }
     WA(w->r, h * ncol * n); WA(w->delta, h * ncol * n);
     WA(w->cb, ncol * n); WA(w->ct, ncol * n);
-    WA(w->rnorm, 2 * ncol);
+    WA(w->rnorm, 2 * ncol); WA(w->rpart, ncol * ((n + 127) / 128));
     w->km = c->krylov_m;
     if (w->km > 0) {
         WA(w->KV, (long long)(w->km + 1) * h * ncol * n);
@@ -1150,56 +1278,51 @@ int mixed_alloc(apf_ctx *c) {
     return APF_OK;
 }
 
-// G_j = X_j^-1 in place (the block in w->Xre / w->Xim of every design),
-// through the symmetric random butterfly transform when it is on and the
-// recursion has levels.
-int invert_block_b(const Bat &bt, cudaStream_t s) {
+// Positions [p0, p1) of the chain order, one row at a time on the first side's
+// work arrays (recomputation of the slab inverses): the elimination (p0 = 0, p1 =
+// h) or one segment from the checkpoint before it.
+static int eliminate_positions(const Bat &bt, int p0, int p1, cudaStream_t s) {
     apf_ctx *c = bt.lead();
-    MixedWork *w = c->mw;
-    const int n = c->nx, nb = bt.n;
-    PV X[TC_MAX_BATCH];
-    float *tre[TC_MAX_BATCH], *tim[TC_MAX_BATCH], *vre[TC_MAX_BATCH], *vim[TC_MAX_BATCH];
-    for (int b = 0; b < nb; ++b) {
-        MixedWork *wb = bt.c[b]->mw;
-        X[b] = PV{wb->Xre, wb->Xim, n};
-        tre[b] = wb->Tre; tim[b] = wb->Tim; vre[b] = wb->Vre; vim[b] = wb->Vim;
+    const MixedWork *w = c->mw;
+    const int n = c->nx, h = c->h, m = h / 2, K = w->seg_rows, nb = bt.n;
+    const long long nn = (long long)n * n;
+    const bool bf = uses_butterfly(w, n);
+    RowJob jobs[CG_MAX_PROB];
+    auto plane = [&](float *p) {  // a checkpoint as a source
+        RowSrc src{};
+        src.re = p; src.im = p + nn;
+        src.use = 1;
+        return src;
+    };
+    for (int p = p0; p <= p1; ++p) {
+        const bool more = p < p1;
+        const bool middle = p == h - 1, first_up = p == m && !middle;
+        const bool two = middle && m < h - 1;  // the middle row takes both chains
+        for (int b = 0; b < nb; ++b) {
+            MixedWork *wb = bt.c[b]->mw;
+            RowJob &j = jobs[b];
+            j = row_job(bt.c[b], wb->sd[0], more ? pos_row(c, p) : -1);
+            RowSrc prev{};
+            if (p > p0) {  // the inverse just computed: into its slot, and kept where a later step starts from it
+                prev = work_src(wb->sd[0], more && !first_up);
+                prev.gp = gp_view(bt.c[b], pos_row(c, p - 1));
+                float *ck = p == m && m < h - 1 ? wb->CKB : p < h && p % K == 0 ? wb->CK + (long long)(p / K - 1) * 2 * nn : nullptr;
+                if (ck) { prev.ck_re = ck; prev.ck_im = ck + nn; }
+            } else if (p > 0 && !first_up) {
+                prev = plane(wb->CK + (long long)(p / K - 1) * 2 * nn);
+            }
+            if (two && more) {
+                if (m > 0) j.s[0] = plane(wb->CKB);
+                j.s[1] = prev;
+            } else {
+                j.s[0] = prev;
+            }
+        }
+        row_step_b(bt, jobs, nb, n, bf, s);
+        if (more)
+            if (int rc = invert_work_b(bt, s)) return rc;
     }
-    const bool bf = w->bfly && n > leaf_size(w) && n >= 16;
-    const dim3 bgrid((n / 4 + 127) / 128, n / 4, nb);
-    auto xre = tab<float *>(bt, [&](int b) { return X[b].re; });
-    auto xim = tab<float *>(bt, [&](int b) { return X[b].im; });
-    if (bf) APF_LAUNCH(c, k_butterfly<false>, bgrid, 128, 0, s, xre, xim, (long long)n, n, (const float *)w->BW);
-    int rc = inv32_b(bt, X, n, tre, tim, vre, vim, s);
-    if (rc) return rc;
-    if (bf) APF_LAUNCH(c, k_butterfly<true>, bgrid, 128, 0, s, xre, xim, (long long)n, n, (const float *)w->BW);
     return APF_OK;
-}
-
-// X_row = K_row - G (G: the float32 planes gre/gim of each design, or none) into w->Xre / w->Xim.
-static void assemble_b(const Bat &bt, int row, const float *const *gre, const float *const *gim, cudaStream_t s) {
-    apf_ctx *c = bt.lead();
-    const int n = c->nx;
-    dim3 agrid((n / 4 + 255) / 256, n, bt.n);
-    APF_LAUNCH(c, k_assemble32, agrid, 256, 0, s, make_grid(c), row,
-               tab<const double *>(bt, [&](int b) { return (const double *)bt.c[b]->d_eps; }),
-               (const double2 *)c->d_circ, tab<const float *>(bt, [&](int b) { return gre ? gre[b] : nullptr; }),
-               tab<const float *>(bt, [&](int b) { return gim ? gim[b] : nullptr; }),
-               tab<float *>(bt, [&](int b) { return bt.c[b]->mw->Xre; }),
-               tab<float *>(bt, [&](int b) { return bt.c[b]->mw->Xim; }));
-}
-
-// Pack every design's G_j (its working block) into its GP slot of row j.
-static void pack_gp_b(const Bat &bt, int j, cudaStream_t s) {
-    const int n = bt.lead()->nx;
-    PackView v[TC_MAX_BATCH];
-    PV X[TC_MAX_BATCH];
-    __nv_bfloat16 *dst[TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b) {
-        MixedWork *wb = bt.c[b]->mw;
-        X[b] = PV{wb->Xre, wb->Xim, n};
-        dst[b] = (__nv_bfloat16 *)gp_view(bt.c[b], j).base;
-    }
-    pack32_b(bt, v, dst, X, n, n, false, true, bt.lead()->mw->nsplit_elim, s);
 }
 
 int mixed_eliminate_b(const Bat &bt, cudaStream_t s) {
@@ -1207,105 +1330,106 @@ int mixed_eliminate_b(const Bat &bt, cudaStream_t s) {
     for (int b = 0; b < bt.n; ++b)
         if (!bt.c[b]->mw) return set_err(bt.c[b], APF_ESTATE, "mixed workspace missing");
     MixedWork *w = c->mw;
-    const int n = c->nx;
-    const long long nn = (long long)n * n;
-    const int K = w->seg_rows;
-    const float *xre[TC_MAX_BATCH], *xim[TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b) { xre[b] = bt.c[b]->mw->Xre; xim[b] = bt.c[b]->mw->Xim; }
-    assemble_b(bt, 0, nullptr, nullptr, s);
-    for (int j = 0; j < c->h; ++j) {
-        int rc = invert_block_b(bt, s);
-        if (rc) return rc;
-        pack_gp_b(bt, j, s);
-        if (K > 0 && j + 1 < c->h && (j + 1) % K == 0) {
-            // checkpoint G_j (float32) for the segment that starts at row j + 1
-            for (int b = 0; b < bt.n; ++b) {
-                MixedWork *wb = bt.c[b]->mw;
-                float *ck = wb->CK + (long long)((j + 1) / K - 1) * 2 * nn;
-                cudaMemcpyAsync(ck, wb->Xre, sizeof(float) * nn, cudaMemcpyDeviceToDevice, s);
-                cudaMemcpyAsync(ck + nn, wb->Xim, sizeof(float) * nn, cudaMemcpyDeviceToDevice, s);
+    const int n = c->nx, h = c->h, m = h / 2, top = h - 1 - m, nb = bt.n;
+    if (w->seg_rows > 0) {
+        int rc = eliminate_positions(bt, 0, h, s);
+        for (int b = 0; b < nb; ++b) bt.c[b]->mw->seg_loaded = (h - 1) / w->seg_rows;
+        return rc;
+    }
+    const bool bf = uses_butterfly(w, n);
+    RowJob jobs[CG_MAX_PROB];
+    // both chains: the rows t and h - 1 - t of every design in the same launches
+    for (int t = 0; t < m; ++t) {
+        Bat both;
+        for (int sd = 0; sd < (t < top ? 2 : 1); ++sd)
+            for (int b = 0; b < nb; ++b) both.add(bt.c[b], sd);
+        for (int b = 0; b < both.n; ++b) {
+            const int sd = both.sd[b], row = sd ? h - 1 - t : t;
+            jobs[b] = row_job(both.c[b], both.w(b), row);
+            if (t > 0) {
+                jobs[b].s[0] = work_src(both.w(b), true);
+                jobs[b].s[0].gp = gp_view(both.c[b], sd ? row + 1 : row - 1);
             }
         }
-        if (j + 1 < c->h) assemble_b(bt, j + 1, xre, xim, s);
+        row_step_b(both, jobs, both.n, n, bf, s);
+        if (int rc = invert_work_b(both, s)) return rc;
     }
-    for (int b = 0; b < bt.n; ++b) bt.c[b]->mw->seg_loaded = K > 0 ? (c->h - 1) / K : -1;
+    // the middle row
+    for (int b = 0; b < nb; ++b) {
+        MixedWork *wb = bt.c[b]->mw;
+        jobs[b] = row_job(bt.c[b], wb->sd[0], m);
+        if (m > 0) {
+            jobs[b].s[0] = work_src(wb->sd[0], true);
+            jobs[b].s[0].gp = gp_view(bt.c[b], m - 1);
+        }
+        if (top > 0) {
+            jobs[b].s[1] = work_src(wb->sd[1], true);
+            jobs[b].s[1].gp = gp_view(bt.c[b], m + 1);
+        }
+    }
+    row_step_b(bt, jobs, nb, n, bf, s);
+    if (int rc = invert_work_b(bt, s)) return rc;
+    for (int b = 0; b < nb; ++b) {
+        jobs[b] = row_job(bt.c[b], bt.c[b]->mw->sd[0], -1);
+        jobs[b].s[0] = work_src(bt.c[b]->mw->sd[0], false);
+        jobs[b].s[0].gp = gp_view(bt.c[b], m);
+    }
+    row_step_b(bt, jobs, nb, n, bf, s);
     return APF_OK;
 }
 
 int mixed_eliminate(apf_ctx *c, cudaStream_t s) { return mixed_eliminate_b(one(c), s); }
 
-// Recompute the packed inverses of segment `seg` (rows c .. c + seg_rows - 1)
-// into the GP slots of every design: X_c = K_c - G_{c-1} from the float32
-// checkpoint, then the same inversions and assemblies as the elimination
-// (bit-identical results).
+// Recompute the split inverses of segment `seg` into the GP slots of every
+// design, from the float32 checkpoint before it and by the same kernels as the
+// elimination (bit-identical results).
 int recompute_segment_b(const Bat &bt, int seg, cudaStream_t s) {
     apf_ctx *c = bt.lead();
-    MixedWork *w = c->mw;
-    const int n = c->nx, K = w->seg_rows;
-    const long long nn = (long long)n * n;
-    const int r0 = seg * K, r1 = std::min(c->h, r0 + K);
-    const float *gre[TC_MAX_BATCH], *gim[TC_MAX_BATCH], *xre[TC_MAX_BATCH], *xim[TC_MAX_BATCH];
-    for (int b = 0; b < bt.n; ++b) {
-        MixedWork *wb = bt.c[b]->mw;
-        gre[b] = seg > 0 ? wb->CK + (long long)(seg - 1) * 2 * nn : nullptr;
-        gim[b] = seg > 0 ? gre[b] + nn : nullptr;
-        xre[b] = wb->Xre;
-        xim[b] = wb->Xim;
-    }
-    assemble_b(bt, r0, seg > 0 ? gre : nullptr, seg > 0 ? gim : nullptr, s);
-    for (int j = r0; j < r1; ++j) {
-        int rc = invert_block_b(bt, s);
-        if (rc) return rc;
-        pack_gp_b(bt, j, s);
-        if (j + 1 < r1) assemble_b(bt, j + 1, xre, xim, s);
-    }
+    const int K = c->mw->seg_rows;
+    int rc = eliminate_positions(bt, seg * K, std::min(c->h, (seg + 1) * K), s);
     for (int b = 0; b < bt.n; ++b) bt.c[b]->mw->seg_loaded = seg;
-    return APF_OK;
+    return rc;
 }
 
-// Right-hand side R (written into d_E by the caller), its column norms, and
-// the first low-precision solve E = Khat^-1 R.
+// The column norms of the right-hand side (its two rows in d_R, see
+// launch_build_rhs) and the first low-precision solve E = Khat^-1 R.
 int mixed_fields_begin_b(const Bat &bt, cudaStream_t s) {
-    const double2 *R[TC_MAX_BATCH];
-    double2 *E[TC_MAX_BATCH];
+    double2 *E[CG_MAX_PROB];
+    apf_ctx *c0 = bt.lead();
+    const int ncol = c0->cf + c0->ca, h = c0->h;
+    const long long L = (long long)ncol * c0->nx;
     for (int b = 0; b < bt.n; ++b) {
         apf_ctx *c = bt.c[b];
-        const int ncol = c->cf + c->ca;
-        // R = the right-hand side (kept for the residuals) and its column norms, in one pass
-        APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, (const double2 *)c->d_Ew, c->h, ncol, c->nx, c->mw->rnorm, c->d_R);
-        R[b] = c->d_R;
+        APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, (const double2 *)c->d_R, std::min(h, 2), ncol, c->nx, c->mw->rnorm);
         E[b] = c->d_Ew;
     }
-    return approx_solve_b(bt, R, E, bt.lead()->cf, s);
+    auto R = [&](int b, int row) -> const double2 * {
+        return row == 0 ? bt.c[b]->d_R : row == h - 1 ? bt.c[b]->d_R + L : nullptr;
+    };
+    return approx_solve_b(bt, R, E, E, false, false, s);
 }
 
 int mixed_fields_begin(apf_ctx *c, cudaStream_t s) { return mixed_fields_begin_b(one(c), s); }
 
+static void resid_b(const Bat &bt, cudaStream_t s) {
+    residual_b(bt, [&](int b) { return bt.c[b]->d_Ew; }, [&](int b) { return bt.c[b]->mw->r; }, true, s);
+}
+
 static int resid_body(apf_ctx *c, cudaStream_t s) {
-    MixedWork *w = c->mw;
-    int ncol = c->cf + c->ca;
-    residual(c, c->d_Ew, w->r, s);
-    APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, w->r, c->h, ncol, c->nx, w->rnorm + ncol, (double2 *)nullptr);
+    resid_b(one(c), s);
     return APF_OK;
 }
 
 // E += Khat^-1 r for every design of the batch.
 static int correct_b(const Bat &bt, cudaStream_t s) {
-    const double2 *r[TC_MAX_BATCH];
-    double2 *d[TC_MAX_BATCH];
+    double2 *Y[CG_MAX_PROB], *E[CG_MAX_PROB];
     for (int b = 0; b < bt.n; ++b) {
-        r[b] = bt.c[b]->mw->r;
-        d[b] = bt.c[b]->mw->delta;
+        Y[b] = bt.c[b]->mw->delta;
+        E[b] = bt.c[b]->d_Ew;
     }
-    apf_ctx *c0 = bt.lead();
-    int rc = approx_solve_b(bt, r, d, c0->cf + c0->ca, s);
-    if (rc) return rc;
-    for (int b = 0; b < bt.n; ++b) {
-        apf_ctx *c = bt.c[b];
-        const long long total = (long long)(c->cf + c->ca) * c->nx * c->h;
-        APF_LAUNCH(c, k_axpy, (unsigned)((total + 255) / 256), 256, 0, s, c->d_Ew, c->mw->delta, total);
-    }
-    return APF_OK;
+    const long long L = (long long)(bt.lead()->cf + bt.lead()->ca) * bt.lead()->nx;
+    auto R = [&](int b, int row) -> const double2 * { return bt.c[b]->mw->r + row * L; };
+    return approx_solve_b(bt, R, Y, E, true, true, s);
 }
 
 static int correct_body(apf_ctx *c, cudaStream_t s) { return correct_b(one(c), s); }
@@ -1317,21 +1441,8 @@ static const bool g_ir_verbose = [] {
 }();
 
 // K E (the slab operator in float64) into out.
-static int apply_K(apf_ctx *c, const double2 *E, double2 *out, cudaStream_t s) {
-    MixedWork *w = c->mw;
-    const int ncol = c->cf + c->ca, nx = c->nx;
-    const long long L = (long long)ncol * nx;
-    int logn = 0;
-    while ((1 << logn) < nx) ++logn;
-    const int threads = nx / 2 < 256 ? nx / 2 : 256;
-    const int smem = nx * (int)sizeof(double2);
-    APF_LAUNCH(c, k_circ_apply, ncol, threads, smem, s, E, w->cb, nx, logn, c->d_modes, c->d_tw);
-    APF_LAUNCH(c, k_circ_apply, ncol, threads, smem, s, E + (c->h - 1) * L, w->ct, nx, logn, c->d_modes + nx,
-               c->d_tw);
-    GridDev g = make_grid(c);
-    dim3 grid((nx + 255) / 256, ncol, c->h);
-    APF_LAUNCH(c, k_residual, grid, 256, 0, s, g, c->d_eps, E, (const double2 *)nullptr, w->cb, w->ct, out, ncol);
-    return APF_OK;
+static void apply_K(apf_ctx *c, const double2 *E, double2 *out, cudaStream_t s) {
+    residual_b(one(c), [&](int) { return E; }, [&](int) { return out; }, false, s);
 }
 
 // min || beta e1 - H y || for one column by complex Givens rotations; H is
@@ -1391,8 +1502,7 @@ static int mixed_refine_gmres(apf_ctx *c, cudaStream_t s) {
     double ratio = 0.0, prev = INFINITY;
     cudaMemcpyAsync(nr.data(), w->rnorm, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s);
     for (;;) {
-        residual(c, c->d_Ew, w->r, s);
-        APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, w->r, c->h, ncol, nx, w->rnorm + ncol, (double2 *)nullptr);
+        resid_b(one(c), s);
         cudaMemcpyAsync(ne.data(), w->rnorm + ncol, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s);
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return check_cuda(c, e, "refinement");
@@ -1411,15 +1521,16 @@ static int mixed_refine_gmres(apf_ctx *c, cudaStream_t s) {
         APF_LAUNCH(c, k_colscale, fgrid, 256, 0, s, w->KV, w->r, w->rnorm + ncol, ncol, nx);
         for (int j = 0; j < m; ++j) {
             double2 *Vj = w->KV + j * L, *Wn = w->KV + (j + 1) * L, *Zj = w->KZ + j * L;
-            if ((rc = approx_solve(c, Vj, Zj, ncol, s))) return rc;
+            const long long row = (long long)ncol * nx;
+            auto R = [&](int, int j2) -> const double2 * { return Vj + j2 * row; };
+            if ((rc = approx_solve_b(one(c), R, &Zj, &Zj, false, true, s))) return rc;
             apply_K(c, Zj, Wn, s);
             for (int i = 0; i <= j; ++i) {
                 double2 *hij = w->kdot + ((long long)j * (m + 1) + i) * ncol;
                 APF_LAUNCH(c, k_coldot, ncol, 256, 0, s, w->KV + i * L, Wn, c->h, ncol, nx, hij);
                 APF_LAUNCH(c, k_colaxpy, fgrid, 256, 0, s, Wn, w->KV + i * L, hij, -1.0, ncol, nx);
             }
-            APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, Wn, c->h, ncol, nx, w->knrm + (long long)j * ncol,
-                       (double2 *)nullptr);
+            APF_LAUNCH(c, k_colnorm, ncol, 256, 0, s, Wn, c->h, ncol, nx, w->knrm + (long long)j * ncol);
             APF_LAUNCH(c, k_colscale, fgrid, 256, 0, s, Wn, Wn, w->knrm + (long long)j * ncol, ncol, nx);
         }
         cudaMemcpyAsync(hd.data(), w->kdot, sizeof(double2) * hd.size(), cudaMemcpyDeviceToHost, s);
@@ -1485,8 +1596,6 @@ int mixed_refine(apf_ctx *c, cudaStream_t s) {
     return ratio <= c->ir_tol ? APF_OK : APF_ENOCONV;
 }
 
-// Gradient contraction with tensor-core products: Q_j = Gamma F_j, then
-// g_j(x) = 2 k^2 Re sum_b Phi_j[b][x] Q_j[b][x] in float64.
 // Gradient contraction with tensor-core products for every design of the
 // batch: Q_j = Gamma F_j, then g_j(x) = 2 k^2 Re sum_b Phi_j[b][x] Q_j[b][x] in
 // float64.  Gamma[b]: the design's n_out x n_in Gamma on the device.
@@ -1496,22 +1605,24 @@ int mixed_gradient_b(const Bat &bt, const double2 *const *Gamma, cudaStream_t s)
     const int nin = c->nin, nout = c->nout, ncol = nin + nout;
     const int nx = c->nx, ns = w->nsplit_grad, nb = bt.n;
     const long long L = (long long)ncol * nx;
-    PackView pa[TC_MAX_BATCH], pb[TC_MAX_BATCH];
-    __nv_bfloat16 *padst[TC_MAX_BATCH], *pbdst[TC_MAX_BATCH];
-    PV Q[TC_MAX_BATCH];
-    const double2 *src[TC_MAX_BATCH];
+    PackView pa[APF_MAX_BATCH], pb[APF_MAX_BATCH];
+    __nv_bfloat16 *padst[APF_MAX_BATCH], *pbdst[APF_MAX_BATCH];
+    PV Q[APF_MAX_BATCH];
+    const double2 *src[APF_MAX_BATCH];
     for (int b = 0; b < nb; ++b) {
         MixedWork *wb = bt.c[b]->mw;
-        padst[b] = wb->PA;
-        pbdst[b] = wb->PB;
-        Q[b] = PV{wb->O32, wb->O32 + (long long)nout * nx, nx};
+        padst[b] = wb->GA;
+        pbdst[b] = wb->GB;
+        Q[b] = PV{wb->sd[0].O32, wb->sd[0].O32 + (long long)nout * nx, nx};
     }
     pack64A_b(bt, pa, padst, Gamma, nullptr, nin, nout, nin, ns, s);
     for (int j = 0; j < c->h; ++j) {
         for (int b = 0; b < nb; ++b) src[b] = bt.c[b]->d_E + j * L;
         pack64BT_b(bt, pb, pbdst, src, nx, nx, nin, ns, s);
-        int rc = gemm_b(bt, pa, pb, ns, nout, 2 * nx, nx, 1.f, 0.f, Q, nullptr, s);
-        if (rc) return rc;
+        TcProblem pr[APF_MAX_BATCH];
+        for (int b = 0; b < nb; ++b)
+            pr[b] = TcProblem{pa[b], pb[b], Q[b].re, Q[b].im, nullptr, nullptr, bt.c[b]->d_flags};
+        if (int rc = tc_gemm_n(c, nb, pr, ns, nout, 2 * nx, nx, 1.f, 0.f, nx, 0, s)) return rc;
         APF_LAUNCH(c, k_grad_rowdot32, dim3((nx + 31) / 32, 1, nb), 256, 0, s,
                    tab<const double2 *>(bt, [&](int b) { return (const double2 *)bt.c[b]->d_E; }),
                    tab<const float *>(bt, [&](int b) { return (const float *)Q[b].re; }),
@@ -1535,17 +1646,19 @@ int mixed_refine_b(const Bat &bt, cudaStream_t s, int *rcs) {
     std::vector<int> iters(nb, 0), rising(nb, 0), active(nb, 1);
     std::vector<double> ratio(nb, 0.0), prev(nb, INFINITY);
     for (;;) {
+        Bat act;
+        for (int b = 0; b < nb; ++b)
+            if (active[b]) act.add(bt.c[b], 0);
+        resid_b(act, s);
         for (int b = 0; b < nb; ++b) {
             if (!active[b]) continue;
             apf_ctx *c = bt.c[b];
-            resid_body(c, s);
             cudaMemcpyAsync(nr[b].data(), c->mw->rnorm, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s);
             cudaMemcpyAsync(ne[b].data(), c->mw->rnorm + ncol, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s);
         }
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return check_cuda(c0, e, "refinement");
         Bat next;
-        next.n = 0;
         for (int b = 0; b < nb; ++b) {
             if (!active[b]) continue;
             apf_ctx *c = bt.c[b];
@@ -1559,7 +1672,7 @@ int mixed_refine_b(const Bat &bt, cudaStream_t s, int *rcs) {
             }
             prev[b] = r;
             if (stop) active[b] = 0;
-            else next.c[next.n++] = c;
+            else next.add(c, 0);
         }
         if (next.n == 0) break;
         int rc = correct_b(next, s);
@@ -1579,8 +1692,7 @@ int mixed_refine_b(const Bat &bt, cudaStream_t s, int *rcs) {
 // Entry points for a batch of contexts (apf_solve_S_grad_batch).
 static Bat make_bat(apf_ctx *const *cs, int nb) {
     Bat bt;
-    bt.n = nb;
-    for (int b = 0; b < nb; ++b) bt.c[b] = cs[b];
+    for (int b = 0; b < nb; ++b) bt.add(cs[b], 0);
     return bt;
 }
 int mixed_eliminate_n(apf_ctx *const *cs, int nb, cudaStream_t s) { return mixed_eliminate_b(make_bat(cs, nb), s); }
@@ -1591,7 +1703,7 @@ int mixed_refine_n(apf_ctx *const *cs, int nb, cudaStream_t s, int *rcs) {
     return mixed_refine_b(make_bat(cs, nb), s, rcs);
 }
 int mixed_gradient_n(apf_ctx *const *cs, int nb, cudaStream_t s) {
-    const double2 *g[TC_MAX_BATCH];
+    const double2 *g[APF_MAX_BATCH];
     for (int b = 0; b < nb; ++b) g[b] = cs[b]->d_Gam;
     return mixed_gradient_b(make_bat(cs, nb), g, s);
 }
@@ -1605,8 +1717,8 @@ bool mixed_batch_compatible(const apf_ctx *a, const apf_ctx *b) {
 }
 
 // ---------------------------------------------------------------------------
-// Test hooks (not part of the public ABI in include/): exercise the packing +
-// tensor-core GEMM and the mixed recursive inversion in isolation.  They
+// Test hooks (not part of the public ABI in include/): exercise the splitting +
+// tensor-core product and the mixed recursive inversion in isolation.  They
 // allocate their own temporaries.
 // ---------------------------------------------------------------------------
 extern "C" int apf_debug_cgemm(apf_ctx *c, int m, int n, int k, const float *Are, const float *Aim,
@@ -1615,27 +1727,37 @@ extern "C" int apf_debug_cgemm(apf_ctx *c, int m, int n, int k, const float *Are
     SolveGate gate(c->device);
     if (m < 1 || n < 1 || k < 1 || nsplit < 1 || nsplit > 3) return APF_EINVAL;
     cudaSetDevice(c->device);
-    long long kp = round_up(2LL * k, 64);
-    __nv_bfloat16 *pa = nullptr, *pb = nullptr;
-    if (cudaMalloc(&pa, sizeof(__nv_bfloat16) * m * kp * nsplit) != cudaSuccess) return APF_ENOMEM;
-    if (cudaMalloc(&pb, sizeof(__nv_bfloat16) * 2LL * n * kp * nsplit) != cudaSuccess) { cudaFree(pa); return APF_ENOMEM; }
-    int *flags = c->d_flags;
-    int *tmpflags = nullptr;
-    if (!flags) { cudaMalloc(&tmpflags, 16); cudaMemset(tmpflags, 0, 16); c->d_flags = tmpflags; }
+    const long long kp = round_up(k, 64);
+    Mirror A{nullptr, kp, m * kp}, B{nullptr, kp, n * kp};
+    const size_t abytes = sizeof(__nv_bfloat16) * 2 * nsplit * m * kp, bbytes = sizeof(__nv_bfloat16) * 2 * nsplit * n * kp;
+    if (cudaMalloc(&A.base, abytes) != cudaSuccess) return APF_ENOMEM;
+    if (cudaMalloc(&B.base, bbytes) != cudaSuccess) { cudaFree(A.base); return APF_ENOMEM; }
+    int *flags = nullptr;
+    if (cudaMalloc(&flags, 16) != cudaSuccess) { cudaFree(A.base); cudaFree(B.base); return APF_ENOMEM; }
     cudaStream_t s = 0;
-    PackView A = pack32(c, pa, PV{(float *)Are, (float *)Aim, k}, m, k, false, false, nsplit, s);
-    PackView B = pack32(c, pb, PV{(float *)Bre, (float *)Bim, n}, n, k, true, true, nsplit, s);
-    int rc = tc_gemm(c, A, B, nsplit, m, 2 * n, n, 1.f, 0.f, Cre, Cim, n, nullptr, nullptr, 0, s);
+    cudaMemsetAsync(A.base, 0, abytes, s);
+    cudaMemsetAsync(B.base, 0, bbytes, s);
+    cudaMemsetAsync(flags, 0, 16, s);
+    const PV av{(float *)Are, (float *)Aim, k}, bv{(float *)Bre, (float *)Bim, n};
+    mirror_b(one(c), &av, &A, m, k, false, nsplit, s);
+    mirror_b(one(c), &bv, &B, n, k, true, nsplit, s);
+    CgProblem p;
+    p.A = A;
+    p.B = B;
+    p.M = m;
+    p.out = CgOut{Cre, Cim, n, Mirror{}};
+    p.flags = flags;
+    int rc = cgemm_n(c, 1, &p, nsplit, m, n, k, 1.f, 0.f, false, true, s);
     cudaError_t e = cudaDeviceSynchronize();
     if (c->prof_on) prof_collect(c);  // GEMM event timings of this call
     int fl = 0;
-    cudaMemcpy(&fl, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost);
-    if (tmpflags) { cudaFree(tmpflags); c->d_flags = nullptr; }
-    cudaFree(pa);
-    cudaFree(pb);
+    cudaMemcpy(&fl, flags, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(flags);
+    cudaFree(A.base);
+    cudaFree(B.base);
     if (rc) return rc;
     if (e != cudaSuccess) return check_cuda(c, e, "debug cgemm");
-    if (fl & FLAG_TIMEOUT) return set_err(c, APF_ETIMEOUT, "tc_gemm wait gave up");
+    if (fl & FLAG_TIMEOUT) return set_err(c, APF_ETIMEOUT, "cgemm wait gave up");
     return APF_OK;
 }
 
@@ -1644,31 +1766,46 @@ extern "C" int apf_debug_cgemm(apf_ctx *c, int m, int n, int k, const float *Are
 extern "C" int apf_debug_inv32(apf_ctx *c, int n, float *re, float *im, int leaf) {
     if (!c) return APF_EINVAL;
     SolveGate gate(c->device);
-    if (!c || !c->mw || n < 1 || n > c->nx || (n & (n - 1))) return APF_EINVAL;
+    if (!c->mw || n < 1 || n > c->nx || (n & (n - 1))) return APF_EINVAL;
     cudaSetDevice(c->device);
-    int old = c->mw->leaf, oldv = c->mw->leaf_variant;
+    MixedWork *w = c->mw;
+    const int old = w->leaf, oldv = w->leaf_variant;
     // leaf = block size + 1000 * kernel variant (test and tuning hook);
     // + 100000: through the symmetric random butterfly transform
     const bool bf = leaf >= 100000 && n >= 16;
     leaf %= 100000;
-    if (leaf > 0) { c->mw->leaf = leaf % 1000; c->mw->leaf_variant = leaf / 1000; }
-    cudaMemset(c->d_flags, 0, 16);
-    const dim3 bgrid((n / 4 + 127) / 128, n / 4);
-    Tab<float *> tre{}, tim{};
-    tre.v[0] = re;
-    tim.v[0] = im;
-    if (bf) APF_LAUNCH(c, k_butterfly<false>, bgrid, 128, 0, (cudaStream_t)0, tre, tim, (long long)n, n, (const float *)c->mw->BW);
-    int rc = inv32(c, PV{re, im, n}, n, c->mw->Tre, c->mw->Tim, c->mw->Vre, c->mw->Vim, 0);
-    if (bf && rc == APF_OK)
-        APF_LAUNCH(c, k_butterfly<true>, bgrid, 128, 0, (cudaStream_t)0, tre, tim, (long long)n, n, (const float *)c->mw->BW);
+    if (leaf > 0) { w->leaf = leaf % 1000; w->leaf_variant = leaf / 1000; }
+    cudaStream_t s = 0;
+    cudaMemsetAsync(c->d_flags, 0, 16, s);
+    const Bat bt = one(c);
+    const PV X{w->sd[0].Xre, w->sd[0].Xim, n}, user{re, im, n};
+    const Mirror XP{w->sd[0].XP.base, std::max<long long>(n, 64), n * std::max<long long>(n, 64)};
+    int rc = APF_OK;
+    if (n < 8) {
+        Mirror none;
+        leaf_b(bt, &user, n, &none, s);
+    } else {
+        RowJob j = row_job(c, w->sd[0], -1);  // load: X = U^T user U
+        j.s[0].re = re; j.s[0].im = im;
+        j.s[0].use = 1;
+        j.out = 1;
+        j.sgn = 1.f;
+        j.XP = XP;
+        row_step_b(bt, &j, 1, n, bf, s);
+        rc = inv32_b(bt, &X, &XP, n, false, 0, s);
+        j = row_job(c, w->sd[0], -1);  // store: user = U X U^T
+        j.s[0] = work_src(w->sd[0], false);
+        j.s[0].ck_re = re; j.s[0].ck_im = im;
+        if (rc == APF_OK) row_step_b(bt, &j, 1, n, bf, s);
+    }
     cudaError_t e = cudaDeviceSynchronize();
-    c->mw->leaf = old;
-    c->mw->leaf_variant = oldv;
+    w->leaf = old;
+    w->leaf_variant = oldv;
     if (rc) return rc;
     if (e != cudaSuccess) return check_cuda(c, e, "debug inv32");
     int fl = 0;
     cudaMemcpy(&fl, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost);
-    if (fl & FLAG_TIMEOUT) return set_err(c, APF_ETIMEOUT, "tc_gemm wait gave up");
+    if (fl & FLAG_TIMEOUT) return set_err(c, APF_ETIMEOUT, "cgemm wait gave up");
     if (fl & FLAG_SINGULAR) return set_err(c, APF_ESINGULAR, "singular leaf");
     return APF_OK;
 }

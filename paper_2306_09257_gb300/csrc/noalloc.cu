@@ -160,7 +160,7 @@ extern "C" int apf_solve_S_noalloc(int nx, int ny, int npml_bot, int npml_top, d
     launch_boundary(&c, s);
     eliminate64(&c, s);
     launch_zero(&c, c.d_E, sizeof(double2) * h * ncol * n, s);  // the fields must start at zero
-    launch_build_rhs(&c, c.d_E, s);
+    launch_build_rhs(&c, c.d_E, c.h, s);
     fields64(&c, s);
     launch_readout(&c, s);
     // a failed launch (configuration or resources) is reported here, before the

@@ -35,7 +35,6 @@ struct TcArgs {
     TcParams p[P];
     int nprob;
 };
-constexpr int TC_MAX_BATCH = 16;
 
 // One product of a batch: operands, output (and beta input) planes, error flags.
 struct TcProblem {
@@ -46,14 +45,15 @@ struct TcProblem {
 };
 
 uint32_t tc_seg_pairs(int nsplit, int *nseg);
+bool tc_make_map(CUtensorMap *m, const void *base, long long cols, long long rows, long long planes,
+                 long long row_pitch, long long plane_pitch, int box_rows, int box_planes);
 void tc_init_attrs();
 
 // out = alpha * (A B^T) + beta * in, where output column col < n_cplx goes to
 // the real plane (column col) and col >= n_cplx to the imaginary plane
-// (column col - n_cplx).  A: M rows; B: N rows; both with the same kp.
-int tc_gemm(apf_ctx *c, const PackView &A, const PackView &B, int nsplit, int M, int N, int n_cplx, float alpha,
-            float beta, float *out_re, float *out_im, long long ldo, const float *in_re, const float *in_im,
-            long long ldi, cudaStream_t s);
-// nprob (<= TC_MAX_BATCH) products of the same shape in one launch.
+// (column col - n_cplx).  A: M rows; B: N rows; both with the same kp.  Used by
+// the gradient contraction (three planes); the slab elimination and the field
+// sweeps use cgemm.h.
+// nprob (<= APF_MAX_BATCH) products of the same shape in one launch.
 int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int N, int n_cplx, float alpha,
               float beta, long long ldo, long long ldi, cudaStream_t s);
