@@ -1,8 +1,7 @@
 // Diagonal-block inversion shared by the float64 and the mixed path.
 // (1) leaf_gj / leaf_gj_regs: Gauss-Jordan elimination with partial (row)
-// pivoting of one NB x NB block.  (2) leaf128_recursive: the mixed path's
-// 128 x 128 blocks, by the 2x2 Schur recursion in shared memory down to
-// 32 x 32 Gauss-Jordan leaves held in registers.
+// pivoting of one NB x NB block.  (2) lc: the mixed path's 128 x 128 blocks, by a
+// cluster of four CTAs.
 // In (1), for the shared-memory form:  Thread t owns row t/4 and the columns sub + 4q
 // (sub = t%4), so the 4 threads of a row sit in adjacent lanes and the
 // pivot-row reads are conflict-free; rows are padded by 4 elements.
@@ -361,343 +360,278 @@ __device__ void leaf_gj_regs2(float *re, float *im, long long ld, int *flags) {
 }
 
 // ---------------------------------------------------------------------------
+// Inverse of a 128 x 128 float32 block by a cluster of four CTAs (one per block,
+// 512 threads each): block Gauss-Jordan elimination in place over four 32-column
+// panels, CTA q holding the panel of columns 32 q .. 32 q + 31 in shared memory.
+// Step p: every CTA copies panel p (distributed shared memory), inverts its 32 x 32
+// pivot block (each for itself, which saves a broadcast), and updates its own
+// panel: R = P^-1 A_p, A_i -= F_i R, A_p = R (on panel p itself: P^-1 and -F_i P^-1).
+// These blocks sit one after the other on the critical path of every
+// inversion, so what counts is latency: 4 x (a chain of 32 pivots, 128 x 32 x 32
+// multiply-adds per SM, a panel copy and a cluster barrier).  The four SMs
+// divide the multiply-adds that a single CTA would spend most of its time on.
+// Measured: 93 -> 60 us per block against one CTA (2 x 2 Schur recursion with
+// 32 x 32 leaves of one barrier, two shared-memory round trips and a division
+// per pivot).
 // ---------------------------------------------------------------------------
-// In-CTA recursive inverse of a 128 x 128 complex-symmetric fp32 block.
-// The block stays in shared memory; the 2x2 Schur recursion of the global
-// inversion (T = C Ai, D -= T B, D <- D^-1, V = D T, A += T^T V, C = -V,
-// B = -V^T) runs down to 32 x 32 diagonal blocks, which are inverted by
-// pivoted Gauss-Jordan on 8 warps with the rows in registers.  The products
-// are CTA-wide fp32 GEMMs from shared memory.  512 threads, one CTA per block.
-// ---------------------------------------------------------------------------
-namespace rec {
-constexpr int NT = 512;
-constexpr int P128 = 130, P64 = 66, P32 = 34;  // padded pitches (float2)
+namespace lc {
+constexpr int NT = 512, PT = 34;  // threads, row pitch (float2; rows 16-byte aligned, columns conflict-free)
 
+struct Smem {
+    float2 own[128 * PT], F[128 * PT], cur[2][32 * PT], inv[32 * PT], R[32 * PT];
+    float2 v[128], y[128], ypart[128];
+    float part[NT / 32], e2;
+    float2 s_inv[2];
+    int s_p[2], piv[32], bad;
+};
 
-// C = (ACC ? C : 0) + sgn * op(A) B, all H x H (H = 32 or 64), in shared memory
-// (every block offset and pitch even, so column pairs are 16-byte aligned).
-// Thread (rt, ct) computes rows rt + i * RT (i < RB) and the column pairs
-// 2 (ct + q * CT) (q < NP), with the operands of step k + 1 loaded while
-// step k is multiplied.
-template <int H, bool TRANS_A, bool ACC>
-__device__ void gemm(const float2 *A, int lda, const float2 *B, int ldb, float2 *C, int ldc, float sgn) {
-    constexpr int CT = 16;                 // column-pair threads
-    constexpr int RT = NT / CT;            // row threads (32)
-    constexpr int RB = H / RT;             // rows per thread (2 for H = 64, 1 for H = 32)
-    constexpr int NP = H / (2 * CT);       // column pairs per thread (2 or 1)
-    const int t = threadIdx.x;
-    const int rt = t / CT, ct = t % CT;
-    float2 acc[RB][2 * NP];
-#pragma unroll
-    for (int i = 0; i < RB; ++i)
-#pragma unroll
-        for (int u = 0; u < 2 * NP; ++u) acc[i][u] = make_float2(0.f, 0.f);
-    auto lda_ = [&](int k, int i) { const int r = rt + i * RT; return TRANS_A ? A[k * lda + r] : A[r * lda + k]; };
-    auto ldb_ = [&](int k, int q) { return *reinterpret_cast<const float4 *>(B + k * ldb + 2 * (ct + q * CT)); };
-    float2 a[RB];
-    float4 b[NP];
-#pragma unroll
-    for (int i = 0; i < RB; ++i) a[i] = lda_(0, i);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) b[q] = ldb_(0, q);
-#pragma unroll 2
-    for (int k = 0; k < H; ++k) {
-        float2 an[RB];
-        float4 bn[NP];
-        const int kn = k + 1 < H ? k + 1 : k;
-#pragma unroll
-        for (int i = 0; i < RB; ++i) an[i] = lda_(kn, i);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) bn[q] = ldb_(kn, q);
-#pragma unroll
-        for (int i = 0; i < RB; ++i)
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                const float2 b0 = make_float2(b[q].x, b[q].y), b1 = make_float2(b[q].z, b[q].w);
-                float2 &c0 = acc[i][2 * q], &c1 = acc[i][2 * q + 1];
-                c0.x = fmaf(a[i].x, b0.x, fmaf(-a[i].y, b0.y, c0.x));
-                c0.y = fmaf(a[i].x, b0.y, fmaf(a[i].y, b0.x, c0.y));
-                c1.x = fmaf(a[i].x, b1.x, fmaf(-a[i].y, b1.y, c1.x));
-                c1.y = fmaf(a[i].x, b1.y, fmaf(a[i].y, b1.x, c1.y));
-            }
-#pragma unroll
-        for (int i = 0; i < RB; ++i) a[i] = an[i];
-#pragma unroll
-        for (int q = 0; q < NP; ++q) b[q] = bn[q];
-    }
-#pragma unroll
-    for (int i = 0; i < RB; ++i)
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            float4 *c = reinterpret_cast<float4 *>(C + (rt + i * RT) * ldc + 2 * (ct + q * CT));
-            float4 v = make_float4(sgn * acc[i][2 * q].x, sgn * acc[i][2 * q].y, sgn * acc[i][2 * q + 1].x,
-                                   sgn * acc[i][2 * q + 1].y);
-            if (ACC) {
-                const float4 o = *c;
-                v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
-            }
-            *c = v;
-        }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Shared-memory object `p` of cluster CTA `rank` (generic address).
+template <typename T>
+__device__ __forceinline__ const T *peer(const T *p, int rank) {
+    uint64_t a;
+    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"((uint64_t)p), "r"(rank));
+    return reinterpret_cast<const T *>(a);
 }
 
-// Pivoted Gauss-Jordan inverse of a 32 x 32 block (pitch ld) by NW warps
-// (8 by default): lane i holds row i, warp w the columns CW w .. CW w + CW - 1
-// (CW = 32 / NW), in registers.  Pivot rows are not swapped: step k takes the
-// unused row p_k with the largest |a[p][k]| and eliminates column k from every
-// other row, so that at the end storage row r holds row ipiv[r] of the inverse
-// with its columns in pivot order: inv[ipiv[r]][p_c] = a[r][c].
-// After each step every warp also stores its columns to a copy in shared
-// memory (two copies, alternating by step), and the warp owning the next
-// pivot column picks the pivot with one warp max-reduction over the key
-// (|a[i][k]|^2 with its five low mantissa bits replaced by 31 - i, so ties go
-// to the lowest row); after the step's one barrier of the NW warps each warp
-// reads the pivot row and column from the copy.  `scr` holds 2 x 32 x LEAF_SP
-// float2, 16-byte aligned.
-constexpr int LEAF_SP = 34;
-
-template <int NW>
-static __device__ void leaf32t(float2 *a, int ld, float2 *scr, int *flags) {
-    constexpr int CW = 32 / NW;  // columns per warp
-    __shared__ int pp[2], piv[32];
-    if (threadIdx.x >= 32 * NW) return;
-    auto bar = [] { asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory"); };
+// Pivoted Gauss-Jordan inverse of the 32 x 32 block `a` (pitch PT) into sm.inv, by
+// warps 0-3: lane i of every warp holds row i, warp w the columns 8w .. 8w+7.  Rows
+// are not swapped: step k takes the unused row with the largest |a[p][k]| (a warp
+// maximum over |.|^2 with its low five bits replaced by 31 - row).  The warp that
+// owns the next pivot column updates that column first and finds the pivot, with
+// every lane's reciprocal computed beside the maximum, while the others finish
+// their updates: one barrier of the four warps per step.  A zero pivot leaves
+// infinities or NaN, which the caller's check of the result finds.
+static __device__ void leaf32(Smem &sm, const float2 *a) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float2 x[CW];
+    float2 x[8];
 #pragma unroll
-    for (int j = 0; j < CW; ++j) x[j] = a[lane * ld + CW * w + j];
-    // store this warp's columns to copy `b`; the owner of column k picks its pivot
-    auto stage = [&](int b, int k, bool used) {
-        float4 *dst = reinterpret_cast<float4 *>(scr + (b * 32 + lane) * LEAF_SP + CW * w);
-#pragma unroll
-        for (int j = 0; j < CW / 2; ++j) dst[j] = make_float4(x[2 * j].x, x[2 * j].y, x[2 * j + 1].x, x[2 * j + 1].y);
-        if (w == k / CW) {
-            const int kl = k % CW;
-            float2 fk;
-            if constexpr (CW == 8) {
-                const float2 s0 = (kl & 1) ? x[1] : x[0], s1 = (kl & 1) ? x[3] : x[2];
-                const float2 s2 = (kl & 1) ? x[5] : x[4], s3 = (kl & 1) ? x[7] : x[6];
-                const float2 t0 = (kl & 2) ? s1 : s0, t1 = (kl & 2) ? s3 : s2;
-                fk = (kl & 4) ? t1 : t0;
-            } else {
-                const float2 s0 = (kl & 1) ? x[1] : x[0], s1 = (kl & 1) ? x[3] : x[2];
-                fk = (kl & 2) ? s1 : s0;
-            }
-            const unsigned bits = __float_as_uint(fk.x * fk.x + fk.y * fk.y);
-            const unsigned key = used ? 0u : ((bits & ~31u) | (unsigned)(31 - lane));
-            const unsigned best = __reduce_max_sync(0xffffffffu, key);
-            if (lane == 0) {
-                const int p = 31 - (int)(best & 31u);
-                pp[b] = p;
-                piv[k] = p;
-            }
-        }
-    };
+    for (int j = 0; j < 8; ++j) x[j] = a[lane * PT + 8 * w + j];
     bool used = false;
     int mystep = 0;
-    stage(0, 0, false);
-    bar();
-    for (int k = 0; k < 32; ++k) {
-        const int buf = k & 1;
-        const int p = pp[buf];
-        const float2 *cur = scr + buf * 32 * LEAF_SP;
-        const float2 fk = cur[lane * LEAF_SP + k], d = cur[p * LEAF_SP + k];
-        float2 rr[CW];
-#pragma unroll
-        for (int j = 0; j < CW / 2; ++j) {
-            const float4 q = reinterpret_cast<const float4 *>(cur + p * LEAF_SP + CW * w)[j];
-            rr[2 * j] = make_float2(q.x, q.y);
-            rr[2 * j + 1] = make_float2(q.z, q.w);
-        }
-        const float den = d.x * d.x + d.y * d.y;
-        if (threadIdx.x == 0 && (!(den > 0.f) || !isfinite(den))) atomicOr(flags, FLAG_SINGULAR);
+    auto bar = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+    auto pivot = [&](float2 v, int k, int b) {
+        const float den = fmaf(v.x, v.x, v.y * v.y);
+        const unsigned key = used ? 0u : ((__float_as_uint(den) & ~31u) | (unsigned)(31 - lane));
+        const unsigned best = __reduce_max_sync(0xffffffffu, key);
         const float rd = __fdividef(1.f, den);
-        const float2 inv = make_float2(d.x * rd, -d.y * rd);
-        const bool isp = lane == p;
-        if (isp) { used = true; mystep = k; }
-        // pivot row: x <- x * inv; other rows: x <- x - f * (pivot row * inv)
-        const float2 fe = isp ? make_float2(-1.f, 0.f) : fk;
-        const float keep = isp ? 0.f : 1.f;
-        const float2 ck = make_float2(-(fe.x * inv.x - fe.y * inv.y), -(fe.x * inv.y + fe.y * inv.x));
-        const bool own = w == k / CW;
-        const int kl = k % CW;
-#pragma unroll
-        for (int j = 0; j < CW; ++j) {
-            const float2 r = rr[j];
-            const float2 n = make_float2(r.x * inv.x - r.y * inv.y, r.x * inv.y + r.y * inv.x);
-            float2 v;
-            v.x = fmaf(keep, x[j].x, -(fe.x * n.x - fe.y * n.y));
-            v.y = fmaf(keep, x[j].y, -(fe.x * n.y + fe.y * n.x));
-            x[j] = (own && j == kl) ? ck : v;
+        if (lane == 31 - (int)(best & 31u)) {
+            sm.s_p[b] = lane;
+            sm.piv[k] = lane;
+            sm.s_inv[b] = make_float2(v.x * rd, -v.y * rd);
         }
-        if (k + 1 < 32) stage(buf ^ 1, k + 1, used);
-        bar();
-    }
+    };
+    auto stage = [&](int b) {
+        float4 *d = reinterpret_cast<float4 *>(sm.cur[b] + lane * PT + 8 * w);
 #pragma unroll
-    for (int j = 0; j < CW; ++j) a[mystep * ld + piv[CW * w + j]] = x[j];
+        for (int j = 0; j < 4; ++j) d[j] = make_float4(x[2 * j].x, x[2 * j].y, x[2 * j + 1].x, x[2 * j + 1].y);
+    };
+    if (w == 0) pivot(x[0], 0, 0);
+    stage(0);
     bar();
-}
-
-static __device__ void leaf32(float2 *a, int ld, float2 *scr, int *flags) { leaf32t<8>(a, ld, scr, flags); }
-
-// Symmetric 2x2 recursion on the n x n block at `a` (n = 32 or 64) with
-// temporaries T, V (pitch P32) and the leaf scratch W.
-template <int N>
-__device__ void inv_sym(float2 *a, int ld, float2 *T, float2 *V, float2 *W, int *flags) {
-    if constexpr (N == 32) {
-        leaf32(a, ld, W, flags);
-        __syncthreads();
-    } else {
-        constexpr int H = N / 2;
-        float2 *A = a, *B = a + H, *C = a + H * ld, *D = a + H * ld + H;
-        inv_sym<H>(A, ld, nullptr, nullptr, W, flags);
-        gemm<H, false, false>(C, ld, A, ld, T, P32, 1.f);         // T = C Ai
-        __syncthreads();
-        gemm<H, false, true>(T, P32, B, ld, D, ld, -1.f);          // D -= T B
-        __syncthreads();
-        inv_sym<H>(D, ld, nullptr, nullptr, W, flags);
-        gemm<H, false, false>(D, ld, T, P32, V, P32, 1.f);         // V = Si T
-        __syncthreads();
-        gemm<H, true, true>(T, P32, V, P32, A, ld, 1.f);           // A += T^T V
-        for (int e = threadIdx.x; e < H * H; e += NT) {            // C = -V, B = -V^T
-            const int r = e / H, cc = e % H;
-            const float2 v = V[r * P32 + cc];
-            C[r * ld + cc] = make_float2(-v.x, -v.y);
-            B[cc * ld + r] = make_float2(-v.x, -v.y);
+    for (int kw = 0; kw < 4; ++kw) {
+#pragma unroll
+        for (int kl = 0; kl < 8; ++kl) {
+            const int k = 8 * kw + kl, b = kl & 1;
+            const int p = sm.s_p[b];
+            const float2 inv = sm.s_inv[b], f = sm.cur[b][lane * PT + k];
+            float2 r[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 q = reinterpret_cast<const float4 *>(sm.cur[b] + p * PT + 8 * w)[j];
+                r[2 * j] = make_float2(q.x, q.y);
+                r[2 * j + 1] = make_float2(q.z, q.w);
+            }
+            // other rows: x - (f inv) row_p; the pivot row: 0 - (-inv) row_p
+            const bool isp = lane == p;
+            const float2 g = isp ? make_float2(-inv.x, -inv.y)
+                                 : make_float2(fmaf(f.x, inv.x, -f.y * inv.y), fmaf(f.x, inv.y, f.y * inv.x));
+            if (isp) {
+                used = true;
+                mystep = k;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = make_float2(0.f, 0.f);
+            }
+            auto update = [&](int j) {
+                x[j].x = fmaf(-g.x, r[j].x, fmaf(g.y, r[j].y, x[j].x));
+                x[j].y = fmaf(-g.x, r[j].y, fmaf(-g.y, r[j].x, x[j].y));
+            };
+            const int jn = kl < 7 ? kl + 1 : 0;  // the next pivot column, in warp kw (or kw + 1)
+            update(jn);
+            if (w == (kl < 7 ? kw : kw + 1)) pivot(x[jn], k + 1, b ^ 1);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j != jn) update(j);
+            if (w == kw) x[kl] = make_float2(-g.x, -g.y);
+            if (k + 1 < 32) {
+                stage(b ^ 1);
+                bar();
+            }
         }
-        __syncthreads();
     }
-}
-}  // namespace rec
-
-constexpr int rec_smem_bytes() {
-    return (128 * rec::P128 + 2 * 64 * rec::P64 + 2 * 32 * rec::P32) * 8;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sm.inv[mystep * PT + sm.piv[8 * w + j]] = x[j];
 }
 
-static __device__ void leaf128_recursive(float *re, float *im, long long ld, int *flags) {
-    extern __shared__ __align__(16) unsigned char rec_smem[];
-    // zero pivots of the recursive attempt are recorded here, not in `flags`:
-    // the self-check below catches their effect and the fallback reports
-    __shared__ int s_sing;
-    if (threadIdx.x == 0) s_sing = 0;
-    float2 *M = reinterpret_cast<float2 *>(rec_smem);
-    float2 *T64 = M + 128 * rec::P128, *V64 = T64 + 64 * rec::P64;
-    float2 *T32 = V64 + 64 * rec::P64, *V32 = T32 + 32 * rec::P32;
-    for (int e = threadIdx.x; e < 128 * 128; e += rec::NT) {
-        const int r = e >> 7, c = e & 127;
-        const long long g = (long long)r * ld + c;
-        M[r * rec::P128 + c] = make_float2(re[g], im[g]);
+// The inverse of the block at (re, im) into the CTAs' panels sm.own; returns
+// (in every thread of the cluster) whether it passed the check below.
+static __device__ bool invert128(Smem &sm, const float *re, const float *im, long long ld, int rank) {
+    const int t = threadIdx.x;
+    for (int e = t; e < 128 * 32; e += NT) {
+        const int r = e >> 5, c = e & 31;
+        const long long g = (long long)r * ld + 32 * rank + c;
+        sm.own[r * PT + c] = make_float2(re[g], im[g]);
     }
-    __syncthreads();
-    // 128: split into 64 blocks (temps T64/V64), the 64 blocks use T32/V32
-    {
-        constexpr int H = 64;
-        float2 *A = M, *B = M + H, *C = M + H * rec::P128, *D = M + H * rec::P128 + H;
-        const int ld0 = rec::P128;
-        rec::inv_sym<64>(A, ld0, T32, V32, V64, &s_sing);
-        rec::gemm<H, false, false>(C, ld0, A, ld0, T64, rec::P64, 1.f);
+    const int cp = 2 * (t & 15), row = t >> 4;  // this thread's column pair and row of each block
+    for (int p = 0; p < 4; ++p) {
+        cluster_arrive();
+        cluster_wait();  // every panel is up to date
+        const float2 *src = peer(sm.own, p);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(sm.F + (row + 32 * i) * PT + cp) =
+                *reinterpret_cast<const float4 *>(src + (row + 32 * i) * PT + cp);
+        cluster_arrive();  // panel p has been read
         __syncthreads();
-        rec::gemm<H, false, true>(T64, rec::P64, B, ld0, D, ld0, -1.f);
+        if (t < 128) leaf32(sm, sm.F + 32 * p * PT);
         __syncthreads();
-        rec::inv_sym<64>(D, ld0, T32, V32, V64, &s_sing);
-        rec::gemm<H, false, false>(D, ld0, T64, rec::P64, V64, rec::P64, 1.f);
-        __syncthreads();
-        rec::gemm<H, true, true>(T64, rec::P64, V64, rec::P64, A, ld0, 1.f);
-        for (int e = threadIdx.x; e < H * H; e += rec::NT) {
-            const int r = e / H, cc = e % H;
-            const float2 v = V64[r * rec::P64 + cc];
-            C[r * ld0 + cc] = make_float2(-v.x, -v.y);
-            B[cc * ld0 + r] = make_float2(-v.x, -v.y);
+        // R = P^-1 A_p (the panel's own columns: R = P^-1)
+        float2 a0 = sm.inv[row * PT + cp], a1 = sm.inv[row * PT + cp + 1];
+        if (rank != p) {
+            a0 = a1 = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int k = 0; k < 32; k += 2) {
+                const float4 q = *reinterpret_cast<const float4 *>(sm.inv + row * PT + k);
+                const float4 u = *reinterpret_cast<const float4 *>(sm.own + (32 * p + k) * PT + cp);
+                const float4 w = *reinterpret_cast<const float4 *>(sm.own + (32 * p + k + 1) * PT + cp);
+                a0.x = fmaf(q.x, u.x, fmaf(-q.y, u.y, a0.x));
+                a0.y = fmaf(q.x, u.y, fmaf(q.y, u.x, a0.y));
+                a1.x = fmaf(q.x, u.z, fmaf(-q.y, u.w, a1.x));
+                a1.y = fmaf(q.x, u.w, fmaf(q.y, u.z, a1.y));
+                a0.x = fmaf(q.z, w.x, fmaf(-q.w, w.y, a0.x));
+                a0.y = fmaf(q.z, w.y, fmaf(q.w, w.x, a0.y));
+                a1.x = fmaf(q.z, w.z, fmaf(-q.w, w.w, a1.x));
+                a1.y = fmaf(q.z, w.w, fmaf(q.w, w.z, a1.y));
+            }
         }
+        *reinterpret_cast<float4 *>(sm.R + row * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
         __syncthreads();
+        cluster_wait();  // no CTA reads panel p any more
+        // A_i -= F_i R for the other three row blocks
+        float2 acc[3][2];
+        int ri[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            ri[i] = 32 * (i < p ? i : i + 1) + row;
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (rank != p) o = *reinterpret_cast<const float4 *>(sm.own + ri[i] * PT + cp);
+            acc[i][0] = make_float2(o.x, o.y);
+            acc[i][1] = make_float2(o.z, o.w);
+        }
+#pragma unroll 4
+        for (int k = 0; k < 32; k += 2) {
+            const float4 u = *reinterpret_cast<const float4 *>(sm.R + k * PT + cp);
+            const float4 w = *reinterpret_cast<const float4 *>(sm.R + (k + 1) * PT + cp);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 q = *reinterpret_cast<const float4 *>(sm.F + ri[i] * PT + k);
+                float2 &c0 = acc[i][0], &c1 = acc[i][1];
+                c0.x = fmaf(-q.x, u.x, fmaf(q.y, u.y, c0.x));
+                c0.y = fmaf(-q.x, u.y, fmaf(-q.y, u.x, c0.y));
+                c1.x = fmaf(-q.x, u.z, fmaf(q.y, u.w, c1.x));
+                c1.y = fmaf(-q.x, u.w, fmaf(-q.y, u.z, c1.y));
+                c0.x = fmaf(-q.z, w.x, fmaf(q.w, w.y, c0.x));
+                c0.y = fmaf(-q.z, w.y, fmaf(-q.w, w.x, c0.y));
+                c1.x = fmaf(-q.z, w.z, fmaf(q.w, w.w, c1.x));
+                c1.y = fmaf(-q.z, w.w, fmaf(-q.w, w.z, c1.y));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            *reinterpret_cast<float4 *>(sm.own + ri[i] * PT + cp) =
+                make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        *reinterpret_cast<float4 *>(sm.own + (32 * p + row) * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
     }
     // Self-check before the block is overwritten.  Pivoting stays inside the
-    // 32 x 32 leaves, so a nearly singular leading sub-block of a block that
-    // is itself well conditioned spoils the recursion; apply the computed
-    // inverse to a fixed unit-modulus probe v and compare X (X^-1 v) with v.
-    // Above 2e-5 relative residual (a sound block gives a few 1e-7) the block
-    // is inverted again by Gauss-Jordan with pivoting over all 128 rows.
-    __shared__ float2 s_y[128], s_v[128];
-    __shared__ float s_part[rec::NT / 32];
-    __shared__ int s_bad;
+    // 32 x 32 blocks, so a nearly singular leading sub-block of a block that is
+    // itself well conditioned spoils the elimination; apply the computed inverse to
+    // a fixed unit-modulus probe v and compare X (X^-1 v) with v.  Above 2e-5
+    // relative residual (a sound block gives a few 1e-7) the block is inverted
+    // again by Gauss-Jordan with pivoting over all 128 rows.
+    if (t < 128) {
+        float sn, cs;
+        sincosf(2.3999632f * (float)t, &sn, &cs);
+        sm.v[t] = make_float2(cs, sn);
+    }
+    __syncthreads();
     {
-        const int t = threadIdx.x, r = t >> 2, sub = t & 3;
-        if (t < 128) {
-            float sn, cs;
-            sincosf(2.3999632f * (float)t, &sn, &cs);
-            s_v[t] = make_float2(cs, sn);
-        }
-        __syncthreads();
+        const int r = t >> 2, c0 = 8 * (t & 3);
         float2 y = make_float2(0.f, 0.f);
-        for (int q = 0; q < 32; ++q) {
-            const int c = sub + 4 * q;
-            const float2 m = M[r * rec::P128 + c], v = s_v[c];
+#pragma unroll
+        for (int c = c0; c < c0 + 8; ++c) {
+            const float2 m = sm.own[r * PT + c], v = sm.v[32 * rank + c];
             y.x += m.x * v.x - m.y * v.y;
             y.y += m.x * v.y + m.y * v.x;
         }
-        y.x += __shfl_xor_sync(0xffffffffu, y.x, 1);
-        y.y += __shfl_xor_sync(0xffffffffu, y.y, 1);
-        y.x += __shfl_xor_sync(0xffffffffu, y.x, 2);
-        y.y += __shfl_xor_sync(0xffffffffu, y.y, 2);
-        if (sub == 0) s_y[r] = y;
-        __syncthreads();
-        // row r of the original block, columns [32 sub, 32 sub + 32), 16-byte loads
+#pragma unroll
+        for (int off = 1; off < 4; off <<= 1) {
+            y.x += __shfl_xor_sync(0xffffffffu, y.x, off);
+            y.y += __shfl_xor_sync(0xffffffffu, y.y, off);
+        }
+        if ((t & 3) == 0) sm.ypart[r] = y;
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (t < 128) {
+        float2 y = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 u = peer(sm.ypart, q)[t];
+            y.x += u.x;
+            y.y += u.y;
+        }
+        sm.y[t] = y;
+    }
+    __syncthreads();
+    {
+        // rows 32 rank .. + 31 of the original block, 16 threads per row
+        const int r = 32 * rank + row, c0 = 8 * (t & 15);
         float2 z = make_float2(0.f, 0.f);
-        const float *rr = re + (long long)r * ld + 32 * sub, *ri = im + (long long)r * ld + 32 * sub;
-        if (((((uintptr_t)rr) | ((uintptr_t)ri)) & 15) == 0) {
-            float4 a[8], b[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                a[q] = reinterpret_cast<const float4 *>(rr)[q];
-                b[q] = reinterpret_cast<const float4 *>(ri)[q];
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float xr[4] = {a[q].x, a[q].y, a[q].z, a[q].w}, xi[4] = {b[q].x, b[q].y, b[q].z, b[q].w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float2 yc = s_y[32 * sub + 4 * q + u];
-                    z.x += xr[u] * yc.x - xi[u] * yc.y;
-                    z.y += xr[u] * yc.y + xi[u] * yc.x;
-                }
-            }
-        } else {
-            for (int q = 0; q < 32; ++q) {
-                const float xr = rr[q], xi = ri[q];
-                const float2 yc = s_y[32 * sub + q];
-                z.x += xr * yc.x - xi * yc.y;
-                z.y += xr * yc.y + xi * yc.x;
-            }
-        }
-        z.x += __shfl_xor_sync(0xffffffffu, z.x, 1);
-        z.y += __shfl_xor_sync(0xffffffffu, z.y, 1);
-        z.x += __shfl_xor_sync(0xffffffffu, z.x, 2);
-        z.y += __shfl_xor_sync(0xffffffffu, z.y, 2);
-        float e2 = 0.f;
-        if (sub == 0) {
-            const float2 v = s_v[r];
-            e2 = (z.x - v.x) * (z.x - v.x) + (z.y - v.y) * (z.y - v.y);
+        for (int c = c0; c < c0 + 8; ++c) {
+            const float xr = re[(long long)r * ld + c], xi = im[(long long)r * ld + c];
+            const float2 y = sm.y[c];
+            z.x += xr * y.x - xi * y.y;
+            z.y += xr * y.y + xi * y.x;
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
-        if ((t & 31) == 0) s_part[t >> 5] = e2;
+        for (int off = 1; off < 16; off <<= 1) {
+            z.x += __shfl_xor_sync(0xffffffffu, z.x, off);
+            z.y += __shfl_xor_sync(0xffffffffu, z.y, off);
+        }
+        const float2 v = sm.v[r];
+        float e2 = (z.x - v.x) * (z.x - v.x) + (z.y - v.y) * (z.y - v.y);
+        e2 += __shfl_xor_sync(0xffffffffu, e2, 16);  // the warp's other row
+        if ((t & 31) == 0) sm.part[t >> 5] = e2;
         __syncthreads();
         if (t == 0) {
             float tot = 0.f;
-            for (int i = 0; i < rec::NT / 32; ++i) tot += s_part[i];
-            s_bad = !(tot <= 4e-10f * 128.f);  // (2e-5)^2 |v|^2; also catches NaN
+            for (int i = 0; i < NT / 32; ++i) tot += sm.part[i];
+            sm.e2 = tot;
         }
-        __syncthreads();
     }
-    if (s_bad) {
-        if (threadIdx.x == 0) atomicAdd(flags + 1, 1);  // fallback count (flags[1])
-        leaf_gj_regs<128>(re, im, ld, flags);
-        return;
+    cluster_arrive();
+    cluster_wait();
+    if (t == 0) {
+        float tot = 0.f;
+        for (int q = 0; q < 4; ++q) tot += *peer(&sm.e2, q);
+        sm.bad = !(tot <= 4e-10f * 128.f);  // (2e-5)^2 |v|^2; also catches NaN
     }
-    for (int e = threadIdx.x; e < 128 * 128; e += rec::NT) {
-        const int r = e >> 7, c = e & 127;
-        const long long g = (long long)r * ld + c;
-        const float2 v = M[r * rec::P128 + c];
-        re[g] = v.x;
-        im[g] = v.y;
-    }
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();  // no CTA leaves while another reads its shared memory
+    return !sm.bad;
 }
+}  // namespace lc

@@ -447,17 +447,34 @@ __global__ void __launch_bounds__(NB * 4) k_leaf32r(const __grid_constant__ Tab<
     leaf_gj_regs<NB>(re.v[b], im.v[b], ld, flags.v[b]);
 }
 
-// 128 x 128 diagonal blocks: the inverse in place and in split form (XP.base null: float32 only).
-__global__ void __launch_bounds__(512) k_leaf128rec(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
-    const int b = blockIdx.x;
-    leaf128_recursive(re.v[b], im.v[b], ld, flags.v[b]);
+// 128 x 128 diagonal blocks (one cluster of four CTAs each): the inverse in place
+// and in split form (XP.base null: float32 only).
+__global__ void __launch_bounds__(lc::NT) __cluster_dims__(4, 1, 1) k_leaf128(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
+    extern __shared__ __align__(16) unsigned char lc_smem[];
+    lc::Smem &sm = *reinterpret_cast<lc::Smem *>(lc_smem);
+    const int b = blockIdx.x >> 2, rank = blockIdx.x & 3;
+    float *re = ret.v[b], *im = imt.v[b];
     const Mirror m = XP.v[b];
+    if (lc::invert128(sm, re, im, ld, rank)) {
+        for (int e = threadIdx.x; e < 128 * 16; e += lc::NT) {
+            const int r = e >> 4, c = 2 * (e & 15), col = 32 * rank + c;
+            const float2 u = sm.own[r * lc::PT + c], v = sm.own[r * lc::PT + c + 1];
+            const long long g = (long long)r * ld + col;
+            *reinterpret_cast<float2 *>(re + g) = make_float2(u.x, v.x);
+            *reinterpret_cast<float2 *>(im + g) = make_float2(u.y, v.y);
+            if (m.base) store_split2(m, planes, r, col, u, v);
+        }
+        return;
+    }
+    if (rank != 0) return;
+    if (threadIdx.x == 0) atomicAdd(flags.v[b] + 1, 1);  // fallback count (flags[1])
+    leaf_gj_regs<128>(re, im, ld, flags.v[b]);
     if (!m.base) return;
     __syncthreads();  // the block's float32 stores are read back by other threads
-    for (int e = threadIdx.x; e < 128 * 64; e += 512) {
+    for (int e = threadIdx.x; e < 128 * 64; e += lc::NT) {
         const int r = e >> 6, c = 2 * (e & 63);
-        const float2 a = *reinterpret_cast<const float2 *>(re.v[b] + (long long)r * ld + c);
-        const float2 d = *reinterpret_cast<const float2 *>(im.v[b] + (long long)r * ld + c);
+        const float2 a = *reinterpret_cast<const float2 *>(re + (long long)r * ld + c);
+        const float2 d = *reinterpret_cast<const float2 *>(im + (long long)r * ld + c);
         store_split2(m, planes, r, c, make_float2(a.x, d.x), make_float2(a.y, d.y));
     }
 }
@@ -819,7 +836,7 @@ void mirror_b(const Bat &bt, const PV *X, const Mirror *m, int R, int C, bool tr
                    (const float *)X[b].im, X[b].ld, R, C, trans ? 1 : 0, m[b], planes);
 }
 
-// Diagonal blocks of the recursion, one CTA per problem (kernel variant per the
+// Diagonal blocks of the recursion, one CTA or cluster per problem (kernel variant per the
 // context's knobs); m: where the split form of the inverse goes (null base: nowhere).
 void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) {
     apf_ctx *c = bt.lead();
@@ -828,10 +845,9 @@ void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) 
     const long long ld = X[0].ld;
     const auto re = tab<float *>(bt, [&](int b) { return X[b].re; }), im = tab<float *>(bt, [&](int b) { return X[b].im; });
     const auto fl = tab<int *>(bt, [&](int b) { return bt.c[b]->d_flags; });
-    // 128 blocks: in-CTA Schur recursion over 32 x 32 Gauss-Jordan leaves
-    // (default); variants 1-3 are the single-level Gauss-Jordan kernels.
+    // 128 blocks: block elimination by a cluster of four CTAs (default); variants 1-3 are the single-level Gauss-Jordan kernels.
     if (n == 128 && v == 0) {
-        APF_LAUNCH(c, k_leaf128rec, nb, 512, rec_smem_bytes(), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+        APF_LAUNCH(c, k_leaf128, 4 * nb, lc::NT, (int)sizeof(lc::Smem), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
                    w->nsplit_elim, fl);
         return;
     }
@@ -1180,7 +1196,7 @@ void mixed_init_attrs() {
     cudaFuncSetAttribute(k_leaf_inv32, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * (int)sizeof(float2));
     cudaFuncSetAttribute(k_leaf32<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<128>(8));
     cudaFuncSetAttribute(k_leaf32<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<64>(8));
-    cudaFuncSetAttribute(k_leaf128rec, cudaFuncAttributeMaxDynamicSharedMemorySize, rec_smem_bytes());
+    cudaFuncSetAttribute(k_leaf128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem));
     cudaFuncSetAttribute(k_circ_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * (int)sizeof(double2));
 }
 
