@@ -19,6 +19,7 @@
 
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 struct apf_sno {
@@ -32,7 +33,7 @@ struct apf_sno {
     float2 *tw = nullptr;          // M x n: (cos, sin)(2 pi m x / n)
     float *h = nullptr, *z = nullptr;       // (L+1) x B x C x n, L x B x C x n
     float2 *X = nullptr, *Y = nullptr;      // L x B x C x M
-    float *dh = nullptr, *dhp = nullptr, *dz = nullptr;  // B x C x n each
+    float *dh = nullptr, *dz = nullptr;     // B x C x n each
     float2 *dY = nullptr, *dX = nullptr;    // B x C x M
     float *pooled = nullptr, *out = nullptr, *dout = nullptr, *dpooled = nullptr, *loss = nullptr;
     long long step = 0;
@@ -60,94 +61,351 @@ __global__ void k_tw(float2 *tw, int n, int M) {
     tw[(long long)m * n + x] = make_float2(c, s);
 }
 
-// h0[b][o][x] = b0[o] + sum_i W0[o][i] eps[b][i][x]
-__global__ void k_lift(const float *eps, const __nv_bfloat16 *pb, long long oW0, long long ob0, float *h0, int B,
-                       int CI, int C, int n) {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long total = (long long)B * C * n;
-    if (idx >= total) return;
-    int x = idx % n;
-    int o = (idx / n) % C;
-    int b = idx / ((long long)n * C);
-    float acc = bf(pb, ob0 + o);
-    for (int i = 0; i < CI; ++i) acc += bf(pb, oW0 + (long long)o * CI + i) * eps[((long long)b * CI + i) * n + x];
-    h0[idx] = acc;
+// h0[b][o][x] = b0[o] + sum_i W0[o][i] eps[b][i][x].  Block: 64 positions of one
+// sample, staged in shared memory; each of the 4 thread rows takes every fourth
+// group of 8 outputs.
+__global__ void __launch_bounds__(256) k_lift(const float *eps, const __nv_bfloat16 *pb, long long oW0, long long ob0,
+                                              float *h0, int CI, int C, int n) {
+    __shared__ float es[64][64], ws[64][72];  // [i][x], [i][o]
+    const int b = blockIdx.y, x0 = blockIdx.x * 64, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int Cp = (C + 7) & ~7;
+    for (int i = ty; i < CI; i += 4) es[i][tx] = eps[((long long)b * CI + i) * n + x0 + tx];
+    for (int e = threadIdx.x; e < CI * Cp; e += 256) {
+        const int i = e / Cp, o = e - i * Cp;
+        ws[i][o] = o < C ? bf(pb, oW0 + (long long)o * CI + i) : 0.f;
+    }
+    __syncthreads();
+    for (int o0 = 8 * ty; o0 < Cp; o0 += 32) {
+        float acc[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] = o0 + u < C ? bf(pb, ob0 + o0 + u) : 0.f;
+        for (int i = 0; i < CI; ++i) {
+            const float e = es[i][tx];
+            const float4 w0 = *reinterpret_cast<const float4 *>(&ws[i][o0]), w1 = *reinterpret_cast<const float4 *>(&ws[i][o0 + 4]);
+            acc[0] = fmaf(w0.x, e, acc[0]); acc[1] = fmaf(w0.y, e, acc[1]);
+            acc[2] = fmaf(w0.z, e, acc[2]); acc[3] = fmaf(w0.w, e, acc[3]);
+            acc[4] = fmaf(w1.x, e, acc[4]); acc[5] = fmaf(w1.y, e, acc[5]);
+            acc[6] = fmaf(w1.z, e, acc[6]); acc[7] = fmaf(w1.w, e, acc[7]);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (o0 + u < C) h0[((long long)b * C + o0 + u) * n + x0 + tx] = acc[u];
+    }
 }
+
+// The transforms use the symmetries of cos and sin: with theta = 2 pi m x / n, the
+// four positions x, n/2 - x, n/2 + x, n - x (0 <= x < n/4) share cos theta and
+// sin theta up to signs that depend on the parity of m only.  So the analysis
+// first folds a row into four sums per x (cos / sin part, even / odd m), and the
+// synthesis makes the four positions' values from four sums (even / odd m, cos /
+// sin part): a quarter of the multiply-adds of the plain transforms.  x = 0 has
+// only the positions 0 and n/2; x = n/4 (positions n/4, 3n/4), where cos and sin
+// are 0 or +-1, is added separately.
 
 // out[row][m] = scale_m * sum_x in[row][x] (cos, -sin)(theta_mx), rows = B*C.
 // scale_m = 1 (analysis) or the synthesis weights (1/n, 2/n) for the backward.
-__global__ void k_dft(const float *in, float2 *out, const float2 *tw, int n, int M, int synth_weights) {
-    extern __shared__ float row[];
-    const long long r = blockIdx.x;
-    for (int x = threadIdx.x; x < n; x += blockDim.x) row[x] = in[r * n + x];
-    __syncthreads();
-    // 4 threads per mode
-    const int m = threadIdx.x >> 2, part = threadIdx.x & 3;
-    float ar = 0.f, ai = 0.f;
-    if (m < M) {
-        const float2 *t = tw + (long long)m * n;
-        for (int x = part; x < n; x += 4) {
-            float v = row[x];
-            float2 w = t[x];
-            ar += v * w.x;
-            ai -= v * w.y;
+// Block: 16 rows x 64 modes, x in chunks of 32; thread: 4 rows x 4 modes of every
+// fourth x, the four partial sums added in a fixed order.  Bound by the float32
+// pipe (32 multiply-adds per 6 shared-memory loads): 64 samples of 48 channels,
+// 1024 positions, 64 modes 212 -> 21 us (one thread per mode and quarter of
+// x, two loads per multiply-add pair, before).
+__global__ void __launch_bounds__(256) k_dft(const float *__restrict__ in, float2 *out, const float2 *__restrict__ tw,
+                                             int rows, int n, int M, int synth_weights) {
+    constexpr int XC = 32, RP = 17;
+    __shared__ __align__(16) float4 sm[3 * XC * RP];
+    float4 *fold = sm, *ta = sm + XC * RP, *tb = ta + XC * RP;  // [x][row]; [x][mode group]: modes 4g, 4g+1 and 4g+2, 4g+3
+    const int tid = threadIdx.x, mg = tid & 15, ks = (tid >> 4) & 3, rg = tid >> 6;
+    const int r0 = blockIdx.x * 16, m0 = blockIdx.y * 64, q = n >> 2;
+    float re[4][4] = {}, im[4][4] = {};
+    for (int x0 = 0; x0 < q; x0 += XC) {
+        __syncthreads();
+        for (int e = tid; e < 16 * XC; e += 256) {
+            const int xx = e & (XC - 1), r = e / XC, x = x0 + xx;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (x < q && r0 + r < rows) {
+                const float *p = in + (long long)(r0 + r) * n;
+                const float a = p[x], bb = p[n / 2 - x];
+                const float c = x ? p[n / 2 + x] : 0.f, d = x ? p[n - x] : 0.f;
+                const float ad = a + d, bc = bb + c, am = a - d, bm = bb - c;
+                v = make_float4(ad + bc, ad - bc, am - bm, am + bm);  // cos even, cos odd, sin even, sin odd
+            }
+            fold[xx * RP + r] = v;
+        }
+        for (int e = tid; e < 64 * XC; e += 256) {
+            const int xx = e & (XC - 1), m = e / XC, x = x0 + xx;
+            float2 w = make_float2(0.f, 0.f);
+            if (x < q && m0 + m < M) w = tw[(long long)(m0 + m) * n + x];
+            float2 *d = reinterpret_cast<float2 *>((m & 2 ? tb : ta) + xx * RP + (m >> 2));
+            d[m & 1] = w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int xx = 0; xx < XC; xx += 4) {
+            const float4 wa = ta[(xx + ks) * RP + mg], wb = tb[(xx + ks) * RP + mg];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 f = fold[(xx + ks) * RP + 4 * rg + r];
+                re[r][0] = fmaf(f.x, wa.x, re[r][0]); im[r][0] = fmaf(-f.z, wa.y, im[r][0]);
+                re[r][1] = fmaf(f.y, wa.z, re[r][1]); im[r][1] = fmaf(-f.w, wa.w, im[r][1]);
+                re[r][2] = fmaf(f.x, wb.x, re[r][2]); im[r][2] = fmaf(-f.z, wb.y, im[r][2]);
+                re[r][3] = fmaf(f.y, wb.z, re[r][3]); im[r][3] = fmaf(-f.w, wb.w, im[r][3]);
+            }
         }
     }
-    ar += __shfl_xor_sync(0xffffffffu, ar, 1);
-    ai += __shfl_xor_sync(0xffffffffu, ai, 1);
-    ar += __shfl_xor_sync(0xffffffffu, ar, 2);
-    ai += __shfl_xor_sync(0xffffffffu, ai, 2);
-    if (m < M && part == 0) {
-        float s = 1.f;
-        if (synth_weights) s = (m == 0 ? 1.f : 2.f) / (float)n;
-        out[r * M + m] = make_float2(ar * s, ai * s);
-    }
-}
-
-// Y[b][o][m] = sum_i W[i][o][m] X[b][i][m]
-__global__ void k_mix(const float2 *X, const __nv_bfloat16 *pb, long long oWr, long long oWi, float2 *Y, int B, int C,
-                      int M) {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= (long long)B * C * M) return;
-    int m = idx % M;
-    int o = (idx / M) % C;
-    int b = idx / ((long long)M * C);
-    float yr = 0.f, yi = 0.f;
-    for (int i = 0; i < C; ++i) {
-        float2 x = X[((long long)b * C + i) * M + m];
-        long long wi = ((long long)i * C + o) * M + m;
-        float wr = bf(pb, oWr + wi), wim = bf(pb, oWi + wi);
-        yr += wr * x.x - wim * x.y;
-        yi += wr * x.y + wim * x.x;
-    }
-    Y[idx] = make_float2(yr, yi);
-}
-
-// z[b][o][x] = sum_m w_m Re(Y e^{i theta}) + sum_i P[o][i] h[b][i][x] + c[o];  hn = act(z)
-__global__ void k_synth(const float2 *Y, const float *h, const __nv_bfloat16 *pb, long long oP, long long oc,
-                        const float2 *tw, float *z, float *hn, int C, int n, int M, int act) {
-    extern __shared__ float sm[];
-    float2 *ys = reinterpret_cast<float2 *>(sm);  // M
-    float *ps = sm + 2 * M;                         // C
-    const int bo = blockIdx.y;                      // b * C + o
-    const int b = bo / C, o = bo % C;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) ys[m] = Y[(long long)bo * M + m];
-    for (int i = threadIdx.x; i < C; i += blockDim.x) ps[i] = bf(pb, oP + (long long)o * C + i);
+    // add the four x slices: lane bit 4 by shuffle, the warp pair through shared memory
     __syncthreads();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    float acc = 0.f;
-    for (int m = 0; m < M; ++m) {
-        float2 w = tw[(long long)m * n + x];
-        float2 y = ys[m];
-        float s = (m == 0 ? 1.f : 2.f) / (float)n;
-        acc += s * (y.x * w.x - y.y * w.y);
+    float *red = reinterpret_cast<float *>(sm);
+    const int slot = rg * 16 + mg;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            re[r][j] += __shfl_xor_sync(0xffffffffu, re[r][j], 16);
+            im[r][j] += __shfl_xor_sync(0xffffffffu, im[r][j], 16);
+            if (ks == 2) {
+                red[(8 * r + 2 * j) * 64 + slot] = re[r][j];
+                red[(8 * r + 2 * j + 1) * 64 + slot] = im[r][j];
+            }
+        }
+    __syncthreads();
+    if (ks != 0) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int row = r0 + 4 * rg + r;
+        if (row >= rows) break;
+        const float a = in[(long long)row * n + q], d = in[(long long)row * n + 3 * q];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int m = m0 + 4 * mg + j;
+            if (m >= M) break;
+            float vr = re[r][j] + red[(8 * r + 2 * j) * 64 + slot], vi = im[r][j] + red[(8 * r + 2 * j + 1) * 64 + slot];
+            const float sg = (m >> 1) & 1 ? -1.f : 1.f;
+            if (m & 1) vi -= sg * (a - d);
+            else vr += sg * (a + d);
+            const float s = !synth_weights ? 1.f : (m == 0 ? 1.f : 2.f) / (float)n;
+            out[(long long)row * M + m] = make_float2(vr * s, vi * s);
+        }
     }
-    for (int i = 0; i < C; ++i) acc += ps[i] * h[((long long)b * C + i) * n + x];
-    acc += bf(pb, oc + o);
-    long long idx = (long long)bo * n + x;
-    z[idx] = acc;
-    hn[idx] = act ? gelu(acc) : acc;
+}
+
+// Y[b][o][m] = sum_i W[i][o][m] X[b][i][m], or its adjoint (BWD) dX[b][i][m] =
+// sum_o conj(W[i][o][m]) dY[b][o][m].  Thread: one mode, OT outputs, four samples,
+// so that a weight serves four samples and a spectrum value OT outputs (from L2:
+// 3 loads per 16 multiply-adds with OT = 4); latency-bound, so OT = 1 where four
+// outputs per thread would leave too few threads.
+template <bool BWD, int OT>
+__global__ void __launch_bounds__(256) k_mix(const float2 *__restrict__ X, const __nv_bfloat16 *__restrict__ pb, long long oWr,
+                                             long long oWi, float2 *Y, int B, int C, int M) {
+    const int idx = blockIdx.x * 256 + threadIdx.x, groups = (C + OT - 1) / OT;
+    if (idx >= groups * M) return;
+    const int m = idx % M, o0 = OT * (idx / M), b0 = 4 * blockIdx.y;
+    const int nb = min(4, B - b0);
+    const long long sb = (long long)C * M;
+    const float2 *x = X + (long long)b0 * sb + m;
+    const __nv_bfloat16 *wrp[OT], *wip[OT];
+#pragma unroll
+    for (int j = 0; j < OT; ++j) {
+        const int o = min(o0 + j, C - 1);
+        const long long w = (BWD ? (long long)o * C : (long long)o) * M + m;
+        wrp[j] = pb + oWr + w;
+        wip[j] = pb + oWi + w;
+    }
+    const long long ws = BWD ? M : (long long)C * M;
+    float2 y[OT][4] = {};
+#pragma unroll 4
+    for (int i = 0; i < C; ++i) {
+        float2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = x[(u < nb ? u : 0) * sb + (long long)i * M];
+#pragma unroll
+        for (int j = 0; j < OT; ++j) {
+            const float wr = __bfloat162float(wrp[j][i * ws]), wi = __bfloat162float(wip[j][i * ws]);
+            const float wim = BWD ? -wi : wi;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                y[j][u].x = fmaf(wr, v[u].x, fmaf(-wim, v[u].y, y[j][u].x));
+                y[j][u].y = fmaf(wr, v[u].y, fmaf(wim, v[u].x, y[j][u].y));
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < OT; ++j)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u < nb && o0 + j < C) Y[(long long)(b0 + u) * sb + (long long)(o0 + j) * M + m] = y[j][u];
+}
+
+// v[b][o][x] = sum_m w_m Re(Y_om e^{i theta}) + sum_i P[o][i] h[b][i][x] (+ c[o]).
+// Forward: w = (1/n, 2/n, ..), z = v + c, hn = act(z).  Backward (BWD): w = 1, P
+// transposed, Y the mixing's gradient, h = dz of this layer; hn = v times the
+// derivative of the previous layer's activation at z (z null: none).
+// Block: one sample, 32 XT values of x below n/4 (so 128 XT positions), all
+// channels, 8 per warp; thread: 8 channels x XT x x 4 positions.  Bound by the
+// float32 pipe: 32 XT multiply-adds per 8 + XT (transform) or 2 + XT (map)
+// shared-memory loads.  64 samples of 48 channels, 1024 positions, 64 modes: 104 ->
+// 27 us.
+constexpr int SY_MC = 16, SY_IC = 16;  // mode pairs and channels staged at a time
+template <bool BWD, int XT, int NT>
+__global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *__restrict__ Y, const float *__restrict__ h, const __nv_bfloat16 *__restrict__ pb,
+                                               long long oP, long long oc, const float2 *__restrict__ tw, float *z, float *hn, int C, int n,
+                                               int M, int act) {
+    constexpr int XW = 32 * XT;
+    extern __shared__ __align__(16) unsigned char sy_smem[];
+    const int Cp = (C + 7) & ~7;
+    float4 *ys = reinterpret_cast<float4 *>(sy_smem);  // [mode pair][o]: w Y of modes 2q, 2q + 1
+    float4 *ts = ys + SY_MC * Cp;                       // [mode pair][x]
+    float4 *hs = ts + SY_MC * XW;                       // [i][x]: the four positions
+    float *ps = reinterpret_cast<float *>(hs + SY_IC * XW);  // [i][o]
+    const int b = blockIdx.y, x0 = blockIdx.x * XW, q = n >> 2;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, o0 = 8 * (tid >> 5);
+    for (int e = tid; e < C * Cp; e += nt) {
+        const int i = e / Cp, o = e - i * Cp;
+        ps[e] = o < C ? bf(pb, oP + (BWD ? (long long)i * C + o : (long long)o * C + i)) : 0.f;
+    }
+    auto weight = [&](int m) { return m >= M ? 0.f : BWD ? 1.f : (m == 0 ? 1.f : 2.f) / (float)n; };
+    float acc[XT][8][4];  // even cos, odd cos, even sin, odd sin
+#pragma unroll
+    for (int u = 0; u < XT; ++u)
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[u][j][k] = 0.f;
+    const int pairs = (M + 1) / 2;
+    for (int p0 = 0; p0 < pairs; p0 += SY_MC) {
+        const int np = min(SY_MC, pairs - p0);
+        __syncthreads();
+        for (int e = tid; e < np * Cp; e += nt) {
+            const int o = e / np, pr = e - o * np, m = 2 * (p0 + pr);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (o < C) {
+                const float2 *y = Y + ((long long)b * C + o) * M + m;
+                const float w0 = weight(m), w1 = weight(m + 1);
+                const float2 a = y[0], d = m + 1 < M ? y[1] : make_float2(0.f, 0.f);
+                v = make_float4(w0 * a.x, w0 * a.y, w1 * d.x, w1 * d.y);
+            }
+            ys[pr * Cp + o] = v;
+        }
+        for (int e = tid; e < np * XW; e += nt) {
+            const int pr = e / XW, xx = e - pr * XW, x = x0 + xx, m = 2 * (p0 + pr);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (x < q) {
+                const float2 a = tw[(long long)m * n + x], d = m + 1 < M ? tw[(long long)(m + 1) * n + x] : make_float2(0.f, 0.f);
+                v = make_float4(a.x, a.y, d.x, d.y);
+            }
+            ts[e] = v;
+        }
+        __syncthreads();
+        if (o0 < C) {
+            for (int pr = 0; pr < np; ++pr) {
+                float4 t[XT];
+#pragma unroll
+                for (int u = 0; u < XT; ++u) t[u] = ts[pr * XW + 32 * u + lane];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4 y = ys[pr * Cp + o0 + j];
+#pragma unroll
+                    for (int u = 0; u < XT; ++u) {
+                        acc[u][j][0] = fmaf(y.x, t[u].x, acc[u][j][0]);
+                        acc[u][j][1] = fmaf(y.z, t[u].z, acc[u][j][1]);
+                        acc[u][j][2] = fmaf(y.y, t[u].y, acc[u][j][2]);
+                        acc[u][j][3] = fmaf(y.w, t[u].w, acc[u][j][3]);
+                    }
+                }
+            }
+        }
+    }
+    // positions x, n/2 - x, n/2 + x, n - x
+#pragma unroll
+    for (int u = 0; u < XT; ++u)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float *a = acc[u][j];
+            const float cp = a[0] + a[1], cm = a[0] - a[1], sp = a[2] + a[3], sd = a[2] - a[3];
+            a[0] = cp - sp;
+            a[1] = cm + sd;
+            a[2] = cm - sd;
+            a[3] = cp + sp;
+        }
+    for (int i0 = 0; i0 < C; i0 += SY_IC) {
+        const int ni = min(SY_IC, C - i0);
+        __syncthreads();
+        for (int e = tid; e < ni * XW; e += nt) {
+            const int i = e / XW, xx = e - i * XW, x = x0 + xx;
+            const float *p = h + ((long long)b * C + i0 + i) * n;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (x < q) v = make_float4(p[x], p[n / 2 - x], x ? p[n / 2 + x] : 0.f, x ? p[n - x] : 0.f);
+            hs[e] = v;
+        }
+        __syncthreads();
+        if (o0 >= C) continue;
+        for (int i = 0; i < ni; ++i) {
+            const float *pr = ps + (i0 + i) * Cp + o0;
+            const float4 p0 = *reinterpret_cast<const float4 *>(pr), p1 = *reinterpret_cast<const float4 *>(pr + 4);
+            const float pw[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+            for (int u = 0; u < XT; ++u) {
+                const float4 v = hs[i * XW + 32 * u + lane];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    acc[u][j][0] = fmaf(pw[j], v.x, acc[u][j][0]);
+                    acc[u][j][1] = fmaf(pw[j], v.y, acc[u][j][1]);
+                    acc[u][j][2] = fmaf(pw[j], v.z, acc[u][j][2]);
+                    acc[u][j][3] = fmaf(pw[j], v.w, acc[u][j][3]);
+                }
+            }
+        }
+    }
+    if (o0 >= C) return;
+    auto store = [&](int o, int x, float v) {
+        const long long idx = ((long long)b * C + o) * n + x;
+        if (BWD) {
+            hn[idx] = z ? v * gelu_d(z[idx]) : v;
+        } else {
+            v += bf(pb, oc + o);
+            z[idx] = v;
+            hn[idx] = act ? gelu(v) : v;
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < XT; ++u) {
+        const int x = x0 + 32 * u + lane;
+        if (x >= q) continue;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (o0 + j >= C) break;
+            store(o0 + j, x, acc[u][j][0]);
+            store(o0 + j, n / 2 - x, acc[u][j][1]);
+            if (x) {
+                store(o0 + j, n / 2 + x, acc[u][j][2]);
+                store(o0 + j, n - x, acc[u][j][3]);
+            }
+        }
+    }
+    if (blockIdx.x != 0) return;
+    // positions n/4 and 3n/4: lanes share the modes and the channels
+    for (int j = 0; j < 8 && o0 + j < C; ++j) {
+        const int o = o0 + j;
+        float even = 0.f, odd = 0.f, p1 = 0.f, p3 = 0.f;
+        for (int m = lane; m < M; m += 32) {
+            const float2 y = Y[((long long)b * C + o) * M + m];
+            const float w = (m >> 1) & 1 ? -weight(m) : weight(m);
+            if (m & 1) odd = fmaf(w, y.y, odd);
+            else even = fmaf(w, y.x, even);
+        }
+        for (int i = lane; i < C; i += 32) {
+            const float *hp = h + ((long long)b * C + i) * n;
+            p1 = fmaf(ps[i * Cp + o], hp[q], p1);
+            p3 = fmaf(ps[i * Cp + o], hp[3 * q], p3);
+        }
+        float v1 = even - odd + p1, v3 = even + odd + p3;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            v1 += __shfl_xor_sync(0xffffffffu, v1, off);
+            v3 += __shfl_xor_sync(0xffffffffu, v3, off);
+        }
+        if (lane == 0) store(o, q, v1);
+        if (lane == 1) store(o, 3 * q, v3);
+    }
 }
 
 // pooled[b][c] = mean_x h[b][c][x]
@@ -212,113 +470,149 @@ __global__ void k_head_bwd(const float *out, const float *tgt, const float *pool
     }
 }
 
-// dz = dh * act'(z)  (dh of the last layer is the broadcast of dpooled / n)
-__global__ void k_act_bwd(const float *dh, const float *dpooled, const float *z, float *dz, long long total, int n,
-                          int act) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    float d = dpooled ? dpooled[i / n] / (float)n : dh[i];
-    dz[i] = act ? d * gelu_d(z[i]) : d;
+// dz of the last layer (no activation): dpooled / n at every position.
+__global__ void k_pool_bwd(const float *dpooled, float4 *dz, long long total4, int n) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= total4) return;
+    const float d = dpooled[4 * i / n] / (float)n;
+    dz[i] = make_float4(d, d, d, d);
 }
 
-// G[o][i] += sum_{b,x} D[b][o][x] H[b][i][x] and gc[o] += sum D  (one block per batch
-// sample, x staged in chunks of 64, fp32 atomics into the gradient)
-__global__ void k_outer(const float *D, const float *H, float *G, float *gc, int CO, int CI, int n) {
-    extern __shared__ float sm[];
-    float *ds = sm;             // CO x 64
-    float *hs = sm + CO * 64;   // CI x 64
-    const int b = blockIdx.x;
-    const int pairs = CO * CI;
-    float acc[12];
-    float cacc = 0.f;
+// G[o][i] += sum_{b,x} D[b][o][x] H[b][i][x] and gc[o] += sum D.  Block: one
+// sample, the positions in chunks of 32 staged as [x][channel]; a thread holds an
+// 8 x 4 tile of one of the slices of every chunk, summed per chunk first; the
+// slices are added in shared memory and the block's sums to G by one float32
+// atomic each; the next chunk is loaded while this one is multiplied.  The groups of four channels
+// are permuted by x / 4, so that both the transposing stores (8 x 4 channels
+// per warp) and the 16-byte loads are free of bank conflicts.  32 multiply-adds
+// per 3 loads: 128 samples, 48 x 48, 1024 positions 408 -> 40 us.
+__global__ void __launch_bounds__(512) k_outer(const float *__restrict__ D, const float *__restrict__ H, float *G, float *gc,
+                                               int CO, int CI, int n) {
+    constexpr int XC = 32;
+    __shared__ __align__(16) float ds[XC * 64], hs[XC * 64];
+    const int b = blockIdx.x, tid = threadIdx.x;
+    const int to = (CO + 7) / 8, ti = (CI + 3) / 4, nt = to * ti, ns = min(512 / nt, XC);  // tiles, slices (CO, CI <= 64)
+    const int slice = tid / nt, tile = tid - slice * nt, og = 2 * (tile / ti), ig = tile % ti;  // groups of 4 channels
+    const bool on = slice < ns;
+    float tot[8][4] = {}, ctot[8] = {};
+    // positions 4 xq .. 4 xq + 3 of channel c of a chunk (8 x 64 threads)
+    const int xq = tid & 7, c = tid >> 3, at = (((c >> 2) ^ xq) << 2) + (c & 3) + 4 * xq * 64;
+    const float *pd = D + ((long long)b * CO + c) * n + 4 * xq, *ph = H + ((long long)b * CI + c) * n + 4 * xq;
+    float rd[4], rh[4];
+    auto fetch = [&](int x0) {
 #pragma unroll
-    for (int q = 0; q < 12; ++q) acc[q] = 0.f;
-    for (int x0 = 0; x0 < n; x0 += 64) {
-        for (int e = threadIdx.x; e < CO * 64; e += blockDim.x)
-            ds[e] = D[((long long)b * CO + e / 64) * n + x0 + (e % 64)];
-        for (int e = threadIdx.x; e < CI * 64; e += blockDim.x)
-            hs[e] = H[((long long)b * CI + e / 64) * n + x0 + (e % 64)];
+        for (int u = 0; u < 4; ++u) {
+            rd[u] = c < CO ? pd[x0 + u] : 0.f;
+            rh[u] = c < CI ? ph[x0 + u] : 0.f;
+        }
+    };
+    fetch(0);
+    for (int x0 = 0; x0 < n; x0 += XC) {
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 12; ++q) {
-            int pr = threadIdx.x + q * blockDim.x;
-            if (pr < pairs) {
-                int o = pr / CI, i = pr % CI;
-                float s = 0.f;
-                for (int x = 0; x < 64; ++x) s += ds[o * 64 + x] * hs[i * 64 + x];
-                acc[q] += s;
+        for (int u = 0; u < 4; ++u) {
+            ds[at + 64 * u] = rd[u];
+            hs[at + 64 * u] = rh[u];
+        }
+        __syncthreads();
+        if (x0 + XC < n) fetch(x0 + XC);
+        if (!on) continue;
+        float acc[8][4] = {}, cacc[8] = {};
+        for (int x = slice; x < XC; x += ns) {
+            const int sw = (x >> 2) & 7;
+            const float4 a = *reinterpret_cast<const float4 *>(ds + 64 * x + ((og ^ sw) << 2));
+            const float4 c = *reinterpret_cast<const float4 *>(ds + 64 * x + (((og + 1) ^ sw) << 2));
+            const float4 h = *reinterpret_cast<const float4 *>(hs + 64 * x + ((ig ^ sw) << 2));
+            const float dv[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                if (ig == 0) cacc[r] += dv[r];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[r][k] = fmaf(dv[r], hv[k], acc[r][k]);
             }
         }
-        if (gc && (int)threadIdx.x < CO)
-            for (int x = 0; x < 64; ++x) cacc += ds[threadIdx.x * 64 + x];
-        __syncthreads();
-    }
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        int pr = threadIdx.x + q * blockDim.x;
-        if (pr < pairs) atomicAdd(&G[pr], acc[q]);
+        for (int r = 0; r < 8; ++r) {
+            ctot[r] += cacc[r];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tot[r][k] += acc[r][k];
+        }
     }
-    if (gc && (int)threadIdx.x < CO) atomicAdd(&gc[threadIdx.x], cacc);
+    // one row of every tile at a time: 5 values per thread, the slices added in order
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        __syncthreads();
+        if (on) {
+            *reinterpret_cast<float4 *>(ds + 4 * tid) = make_float4(tot[r][0], tot[r][1], tot[r][2], tot[r][3]);
+            hs[tid] = ctot[r];
+        }
+        __syncthreads();
+        const int o = 4 * og + r;
+        if (tid >= nt || o >= CO) continue;
+        float v[4] = {}, cv = 0.f;
+        for (int q = 0; q < ns; ++q) {
+            const float4 t = *reinterpret_cast<const float4 *>(ds + 4 * (q * nt + tid));
+            v[0] += t.x; v[1] += t.y; v[2] += t.z; v[3] += t.w;
+            cv += hs[q * nt + tid];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (4 * ig + k < CI) atomicAdd(&G[o * CI + 4 * ig + k], v[k]);
+        if (ig == 0) atomicAdd(&gc[o], cv);
+    }
 }
 
-// Mixing backward: dX[b][i][m] = sum_o conj-pair(W) dY;  dW[i][o][m] = sum_b ...
-__global__ void k_mix_bwd_x(const float2 *dY, const __nv_bfloat16 *pb, long long oWr, long long oWi, float2 *dX, int B,
-                            int C, int M) {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= (long long)B * C * M) return;
-    int m = idx % M;
-    int i = (idx / M) % C;
-    int b = idx / ((long long)M * C);
-    float xr = 0.f, xi = 0.f;
-    for (int o = 0; o < C; ++o) {
-        float2 d = dY[((long long)b * C + o) * M + m];
-        long long wi = ((long long)i * C + o) * M + m;
-        float wr = bf(pb, oWr + wi), wim = bf(pb, oWi + wi);
-        xr += wr * d.x + wim * d.y;
-        xi += -wim * d.x + wr * d.y;
+// Mixing backward, weights: dW[i][o][m] = sum_b conj(X[b][i][m]) dY[b][o][m].
+// Thread: one mode and a 4 x 4 tile of (i, o), every eighth sample; the eight
+// partial sums are added through shared memory in a fixed order.  Latency-bound
+// (8 loads from L2 per 64 multiply-adds).
+constexpr int MW_S = 8;
+__global__ void __launch_bounds__(32 * MW_S) k_mix_bwd_w(const float2 *__restrict__ X, const float2 *__restrict__ dY, float *g,
+                                                   long long gWr, long long gWi, int B, int C, int M) {
+    __shared__ float2 red[MW_S - 1][16][32];
+    const int ml = threadIdx.x & 31, sl = threadIdx.x >> 5, m = blockIdx.x * 32 + ml;
+    const int i0 = 4 * blockIdx.y, o0 = 4 * blockIdx.z;
+    float2 acc[4][4] = {};
+    if (m < M) {
+#pragma unroll 2
+        for (int b = sl; b < B; b += MW_S) {
+            const float2 *x = X + (long long)b * C * M + m, *d = dY + (long long)b * C * M + m;
+            float2 xv[4], dv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                xv[u] = x[(long long)min(i0 + u, C - 1) * M];
+                dv[u] = d[(long long)min(o0 + u, C - 1) * M];
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    acc[r][c].x = fmaf(xv[r].x, dv[c].x, fmaf(xv[r].y, dv[c].y, acc[r][c].x));
+                    acc[r][c].y = fmaf(-xv[r].y, dv[c].x, fmaf(xv[r].x, dv[c].y, acc[r][c].y));
+                }
+        }
     }
-    dX[idx] = make_float2(xr, xi);
-}
-
-__global__ void k_mix_bwd_w(const float2 *X, const float2 *dY, float *g, long long gWr, long long gWi, int B, int C,
-                            int M) {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= (long long)C * C * M) return;
-    int m = idx % M;
-    int o = (idx / M) % C;
-    int i = idx / ((long long)M * C);
-    float ar = 0.f, ai = 0.f;
-    for (int b = 0; b < B; ++b) {
-        float2 x = X[((long long)b * C + i) * M + m];
-        float2 d = dY[((long long)b * C + o) * M + m];
-        ar += x.x * d.x + x.y * d.y;
-        ai += -x.y * d.x + x.x * d.y;
+    if (sl > 0) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) red[sl - 1][e][ml] = acc[e >> 2][e & 3];
     }
-    g[gWr + idx] = ar;
-    g[gWi + idx] = ai;
-}
-
-// dh_prev[b][i][x] = sum_o P[o][i] dz[b][o][x] + sum_m (dXr cos - dXi sin)
-__global__ void k_dh_prev(const float *dz, const float2 *dX, const __nv_bfloat16 *pb, long long oP, const float2 *tw,
-                          float *dhp, int C, int n, int M) {
-    extern __shared__ float sm[];
-    float2 *xs = reinterpret_cast<float2 *>(sm);
-    float *ps = sm + 2 * M;
-    const int bi = blockIdx.y;
-    const int b = bi / C, i = bi % C;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) xs[m] = dX[(long long)bi * M + m];
-    for (int o = threadIdx.x; o < C; o += blockDim.x) ps[o] = bf(pb, oP + (long long)o * C + i);
     __syncthreads();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    float acc = 0.f;
-    for (int o = 0; o < C; ++o) acc += ps[o] * dz[((long long)b * C + o) * n + x];
-    for (int m = 0; m < M; ++m) {
-        float2 w = tw[(long long)m * n + x];
-        float2 d = xs[m];
-        acc += d.x * w.x - d.y * w.y;
+    if (sl > 0 || m >= M) return;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int i = i0 + (e >> 2), o = o0 + (e & 3);
+        float2 v = acc[e >> 2][e & 3];
+#pragma unroll
+        for (int q = 0; q < MW_S - 1; ++q) {
+            v.x += red[q][e][ml].x;
+            v.y += red[q][e][ml].y;
+        }
+        if (i < C && o < C) {
+            const long long w = ((long long)i * C + o) * M + m;
+            g[gWr + w] = v.x;
+            g[gWi + w] = v.y;
+        }
     }
-    dhp[(long long)bi * n + x] = acc;
 }
 
 __global__ void k_adam(float *p, const float *g, float *m1, float *m2, __nv_bfloat16 *pb, long long np, float lr,
@@ -347,24 +641,72 @@ int serr(apf_sno *s, int code, const char *msg) {
     return set_err(nullptr, code, "%s", msg);
 }
 
+void launch_dft(apf_sno *s, const float *in, float2 *out, int B, int weights, cudaStream_t st) {
+    const int rows = B * s->c;
+    k_dft<<<dim3((rows + 15) / 16, (s->m + 63) / 64), 256, 0, st>>>(in, out, s->tw, rows, s->n, s->m, weights);
+}
+
+size_t synth_smem(int C, int XT) {
+    const size_t Cp = (C + 7) & ~7, XW = 32 * XT;
+    return 16 * (SY_MC * Cp + SY_MC * XW + SY_IC * XW) + 4 * C * Cp;
+}
+
+// x per block: 64 where that still gives about two blocks per SM, else 32; up to
+// 48 channels the block has 192 threads, so that three fit the register file.
+template <bool BWD, int XT, int NT>
+void launch_synth_t(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
+                    int act, cudaStream_t st) {
+    const int q = s->n / 4, threads = 32 * ((s->c + 7) / 8);
+    k_synth<BWD, XT, NT><<<dim3((q + 32 * XT - 1) / (32 * XT), B), threads, synth_smem(s->c, XT), st>>>(
+        Y, h, s->pb, oP, oc, s->tw, z, hn, s->c, s->n, s->m, act);
+}
+
+template <bool BWD>
+void launch_synth(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
+                  int act, cudaStream_t st) {
+    const bool two = (long long)B * ((s->n / 4 + 63) / 64) >= 256, small = s->c <= 48;
+    auto f = two ? (small ? launch_synth_t<BWD, 2, 192> : launch_synth_t<BWD, 2, 256>)
+                 : (small ? launch_synth_t<BWD, 1, 192> : launch_synth_t<BWD, 1, 256>);
+    f(s, Y, h, oP, oc, z, hn, B, act, st);
+}
+
+// Shared memory instead of L1 for the kernels that stage their operands (the
+// default split left room for two blocks per SM).
+template <bool BWD, int XT, int NT>
+void synth_attrs() {
+    cudaFuncSetAttribute(k_synth<BWD, XT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)synth_smem(64, XT));
+    cudaFuncSetAttribute(k_synth<BWD, XT, NT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+}
+void init_attrs() {
+    synth_attrs<false, 1, 192>(); synth_attrs<false, 2, 192>(); synth_attrs<false, 1, 256>(); synth_attrs<false, 2, 256>();
+    synth_attrs<true, 1, 192>(); synth_attrs<true, 2, 192>(); synth_attrs<true, 1, 256>(); synth_attrs<true, 2, 256>();
+    cudaFuncSetAttribute(k_dft, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncSetAttribute(k_outer, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+}
+
+template <bool BWD>
+void launch_mix(apf_sno *s, const float2 *X, float2 *Y, int l, int B, cudaStream_t st) {
+    const int C = s->c, M = s->m;
+    const long long wr = s->oWr + (long long)l * C * C * M, wi = s->oWi + (long long)l * C * C * M;
+    const int bg = (B + 3) / 4;
+    if ((long long)((C + 3) / 4) * M * bg >= 16384)
+        k_mix<BWD, 4><<<dim3(nb((long long)((C + 3) / 4) * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
+    else
+        k_mix<BWD, 1><<<dim3(nb((long long)C * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
+}
+
 void forward(apf_sno *s, const float *x, int B, cudaStream_t st) {
     const int C = s->c, n = s->n, M = s->m, L = s->layers;
-    const long long act = (long long)B * C * n, spec = (long long)B * C * M;
-    k_lift<<<nb(act), 256, 0, st>>>(x, s->pb, s->oW0, s->ob0, s->h, B, s->ci, C, n);
+    k_lift<<<dim3(n / 64, B), 256, 0, st>>>(x, s->pb, s->oW0, s->ob0, s->h, s->ci, C, n);
     for (int l = 0; l < L; ++l) {
         const float *hp = s->h + (long long)l * s->bmax * C * n;
         float *hn = s->h + (long long)(l + 1) * s->bmax * C * n;
         float *z = s->z + (long long)l * s->bmax * C * n;
         float2 *X = s->X + (long long)l * s->bmax * C * M, *Y = s->Y + (long long)l * s->bmax * C * M;
-        k_dft<<<B * C, 4 * M, n * sizeof(float), st>>>(hp, X, s->tw, n, M, 0);
-        k_mix<<<nb(spec), 256, 0, st>>>(X, s->pb, s->oWr + (long long)l * C * C * M, s->oWi + (long long)l * C * C * M,
-                                       Y, B, C, M);
-        dim3 g((n + 255) / 256, B * C);
-        k_synth<<<g, 256, (2 * M + C) * sizeof(float), st>>>(Y, hp, s->pb, s->oP + (long long)l * C * C,
-                                                           s->oc + (long long)l * C, s->tw, z, hn, C, n, M,
-                                                           l < L - 1 ? 1 : 0);
+        launch_dft(s, hp, X, B, 0, st);
+        launch_mix<false>(s, X, Y, l, B, st);
+        launch_synth<false>(s, Y, hp, s->oP + (long long)l * C * C, s->oc + (long long)l * C, z, hn, B, l < L - 1 ? 1 : 0, st);
     }
-    (void)act;
     k_pool<<<B * C, 256, 0, st>>>(s->h + (long long)L * s->bmax * C * n, s->pooled, n);
     k_head<<<nb(B * s->no), 256, 0, st>>>(s->pooled, s->pb, s->oWh, s->obh, s->out, B, C, s->no);
 }
@@ -372,32 +714,26 @@ void forward(apf_sno *s, const float *x, int B, cudaStream_t st) {
 // Gradients of the loss w.r.t. every parameter into s->g (after forward).
 void backward(apf_sno *s, const float *x, const float *tgt, int B, cudaStream_t st) {
     const int C = s->c, n = s->n, M = s->m, L = s->layers, NO = s->no;
-    const long long act = (long long)B * C * n, spec = (long long)B * C * M;
+    const long long act = (long long)B * C * n;
     cudaMemsetAsync(s->g, 0, sizeof(float) * s->nparams, st);
     k_head_bwd<<<1, 256, 0, st>>>(s->out, tgt, s->pooled, s->pb, s->oWh, s->g, s->oWh, s->obh, s->dout, s->dpooled,
                                   s->loss, B, C, NO);
+    k_pool_bwd<<<nb(act / 4), 256, 0, st>>>(s->dpooled, reinterpret_cast<float4 *>(s->dz), act / 4, n);
     for (int l = L - 1; l >= 0; --l) {
         const float *hp = s->h + (long long)l * s->bmax * C * n;
-        const float *z = s->z + (long long)l * s->bmax * C * n;
         const float2 *X = s->X + (long long)l * s->bmax * C * M;
-        k_act_bwd<<<nb(act), 256, 0, st>>>(s->dh, l == L - 1 ? s->dpooled : nullptr, z, s->dz, act, n,
-                                           l < L - 1 ? 1 : 0);
-        k_outer<<<B, 256, (C + C) * 64 * sizeof(float), st>>>(s->dz, hp, s->g + s->oP + (long long)l * C * C,
-                                                             s->g + s->oc + (long long)l * C, C, C, n);
-        k_dft<<<B * C, 4 * M, n * sizeof(float), st>>>(s->dz, s->dY, s->tw, n, M, 1);
-        k_mix_bwd_w<<<nb((long long)C * C * M), 256, 0, st>>>(X, s->dY, s->g, s->oWr + (long long)l * C * C * M,
-                                                              s->oWi + (long long)l * C * C * M, B, C, M);
-        k_mix_bwd_x<<<nb(spec), 256, 0, st>>>(s->dY, s->pb, s->oWr + (long long)l * C * C * M,
-                                              s->oWi + (long long)l * C * C * M, s->dX, B, C, M);
-        dim3 g((n + 255) / 256, B * C);
-        k_dh_prev<<<g, 256, (2 * M + C) * sizeof(float), st>>>(s->dz, s->dX, s->pb, s->oP + (long long)l * C * C,
-                                                             s->tw, s->dhp, C, n, M);
-        float *t = s->dh;
-        s->dh = s->dhp;
-        s->dhp = t;
+        k_outer<<<B, 512, 0, st>>>(s->dz, hp, s->g + s->oP + (long long)l * C * C, s->g + s->oc + (long long)l * C, C, C, n);
+        launch_dft(s, s->dz, s->dY, B, 1, st);
+        k_mix_bwd_w<<<dim3((M + 31) / 32, (C + 3) / 4, (C + 3) / 4), 32 * MW_S, 0, st>>>(
+            X, s->dY, s->g, s->oWr + (long long)l * C * C * M, s->oWi + (long long)l * C * C * M, B, C, M);
+        launch_mix<true>(s, s->dY, s->dX, l, B, st);
+        // dz of the layer below (of the lifted input: no activation)
+        float *zp = l > 0 ? s->z + (long long)(l - 1) * s->bmax * C * n : nullptr;
+        launch_synth<true>(s, s->dX, s->dz, s->oP + (long long)l * C * C, 0, zp, s->dh, B, 0, st);
+        std::swap(s->dh, s->dz);
     }
     // lift: dW0[o][i] = sum dh0[b][o][x] eps[b][i][x], db0 = sum dh0
-    k_outer<<<B, 256, (C + s->ci) * 64 * sizeof(float), st>>>(s->dh, x, s->g + s->oW0, s->g + s->ob0, C, s->ci, n);
+    k_outer<<<B, 512, 0, st>>>(s->dz, x, s->g + s->oW0, s->g + s->ob0, C, s->ci, n);
 }
 
 }  // namespace
@@ -413,6 +749,7 @@ int apf_sno_create(apf_sno **out, int device, int n, int in_ch, int width, int m
         width * width > 12 * 256 || width * in_ch > 12 * 256)
         return set_err(nullptr, APF_EINVAL, "apf_sno_create: sizes out of range");
     if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return set_err(nullptr, APF_ECUDA, "bad device"); }
+    init_attrs();
     apf_sno *s = new apf_sno();
     s->device = device; s->n = n; s->ci = in_ch; s->c = width; s->m = modes; s->layers = layers; s->no = n_out;
     s->bmax = max_batch;
@@ -438,7 +775,7 @@ int apf_sno_create(apf_sno **out, int device, int n, int in_ch, int width, int m
               al((void **)&s->pb, sizeof(__nv_bfloat16) * o) && al((void **)&s->tw, sizeof(float2) * M * n) &&
               al((void **)&s->h, sizeof(float) * (L + 1) * Bn) && al((void **)&s->z, sizeof(float) * L * Bn) &&
               al((void **)&s->X, sizeof(float2) * L * BM) && al((void **)&s->Y, sizeof(float2) * L * BM) &&
-              al((void **)&s->dh, sizeof(float) * Bn) && al((void **)&s->dhp, sizeof(float) * Bn) &&
+              al((void **)&s->dh, sizeof(float) * Bn) &&
               al((void **)&s->dz, sizeof(float) * Bn) && al((void **)&s->dY, sizeof(float2) * BM) &&
               al((void **)&s->dX, sizeof(float2) * BM) &&
               al((void **)&s->pooled, sizeof(float) * max_batch * C) &&
