@@ -190,9 +190,10 @@ __global__ void __launch_bounds__(256) k_dft(const float *__restrict__ in, float
 
 // Y[b][o][m] = sum_i W[i][o][m] X[b][i][m], or its adjoint (BWD) dX[b][i][m] =
 // sum_o conj(W[i][o][m]) dY[b][o][m].  Thread: one mode, OT outputs, four samples,
-// so that a weight serves four samples and a spectrum value OT outputs (from L2:
-// 3 loads per 16 multiply-adds with OT = 4); latency-bound, so OT = 1 where four
-// outputs per thread would leave too few threads.
+// so that a weight serves four samples and a spectrum value OT outputs; bound by
+// the latency of L2, so OT = 1 where two outputs per thread would leave too few
+// threads (64 samples of 48 channels: 20 us per call with one output and sample
+// per thread, 14 with OT = 2).
 template <bool BWD, int OT>
 __global__ void __launch_bounds__(256) k_mix(const float2 *__restrict__ X, const __nv_bfloat16 *__restrict__ pb, long long oWr,
                                              long long oWi, float2 *Y, int B, int C, int M) {
@@ -245,8 +246,8 @@ __global__ void __launch_bounds__(256) k_mix(const float2 *__restrict__ X, const
 // shared-memory loads.  64 samples of 48 channels, 1024 positions, 64 modes: 104 ->
 // 27 us.
 constexpr int SY_MC = 16, SY_IC = 16;  // mode pairs and channels staged at a time
-template <bool BWD, int XT, int NT>
-__global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *__restrict__ Y, const float *__restrict__ h, const __nv_bfloat16 *__restrict__ pb,
+template <bool BWD, int XT>
+__global__ void __launch_bounds__(256, 2) k_synth(const float2 *__restrict__ Y, const float *__restrict__ h, const __nv_bfloat16 *__restrict__ pb,
                                                long long oP, long long oc, const float2 *__restrict__ tw, float *z, float *hn, int C, int n,
                                                int M, int act) {
     constexpr int XW = 32 * XT;
@@ -274,10 +275,11 @@ __global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *_
     for (int p0 = 0; p0 < pairs; p0 += SY_MC) {
         const int np = min(SY_MC, pairs - p0);
         __syncthreads();
-        for (int e = tid; e < np * Cp; e += nt) {
-            const int o = e / np, pr = e - o * np, m = 2 * (p0 + pr);
+#pragma unroll 4
+        for (int e = tid; e < SY_MC * Cp; e += nt) {
+            const int o = e / SY_MC, pr = e % SY_MC, m = 2 * (p0 + pr);
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (o < C) {
+            if (o < C && pr < np) {
                 const float2 *y = Y + ((long long)b * C + o) * M + m;
                 const float w0 = weight(m), w1 = weight(m + 1);
                 const float2 a = y[0], d = m + 1 < M ? y[1] : make_float2(0.f, 0.f);
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *_
             }
             ys[pr * Cp + o] = v;
         }
+#pragma unroll 4
         for (int e = tid; e < np * XW; e += nt) {
             const int pr = e / XW, xx = e - pr * XW, x = x0 + xx, m = 2 * (p0 + pr);
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *_
     for (int i0 = 0; i0 < C; i0 += SY_IC) {
         const int ni = min(SY_IC, C - i0);
         __syncthreads();
+#pragma unroll 4
         for (int e = tid; e < ni * XW; e += nt) {
             const int i = e / XW, xx = e - i * XW, x = x0 + xx;
             const float *p = h + ((long long)b * C + i0 + i) * n;
@@ -356,55 +360,74 @@ __global__ void __launch_bounds__(NT, NT == 192 ? 3 : 2) k_synth(const float2 *_
         }
     }
     if (o0 >= C) return;
-    auto store = [&](int o, int x, float v) {
-        const long long idx = ((long long)b * C + o) * n + x;
+    const long long base = ((long long)b * C + o0) * n;
+    const float *zr = BWD && z ? z + base : nullptr;
+    float *zw = BWD ? nullptr : z + base, *hw = hn + base;
+    auto store = [&](int at, float v, float bias, float zv) {
         if (BWD) {
-            hn[idx] = z ? v * gelu_d(z[idx]) : v;
+            hw[at] = zr ? v * gelu_d(zv) : v;
         } else {
-            v += bf(pb, oc + o);
-            z[idx] = v;
-            hn[idx] = act ? gelu(v) : v;
+            v += bias;
+            zw[at] = v;
+            hw[at] = act ? gelu(v) : v;
         }
     };
 #pragma unroll
-    for (int u = 0; u < XT; ++u) {
-        const int x = x0 + 32 * u + lane;
-        if (x >= q) continue;
+    for (int j = 0; j < 8; ++j) {
+        if (o0 + j >= C) break;
+        const float bias = BWD ? 0.f : bf(pb, oc + o0 + j);
+        int at[XT][4];
+        float zv[XT][4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (o0 + j >= C) break;
-            store(o0 + j, x, acc[u][j][0]);
-            store(o0 + j, n / 2 - x, acc[u][j][1]);
-            if (x) {
-                store(o0 + j, n / 2 + x, acc[u][j][2]);
-                store(o0 + j, n - x, acc[u][j][3]);
+        for (int u = 0; u < XT; ++u) {
+            const int x = x0 + 32 * u + lane;
+            const int pos[4] = {x, n / 2 - x, n / 2 + x, n - x};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                at[u][k] = x < q && (x > 0 || k < 2) ? j * n + pos[k] : -1;
+                zv[u][k] = BWD && zr && at[u][k] >= 0 ? zr[at[u][k]] : 0.f;  // all loads before the first store
             }
         }
+#pragma unroll
+        for (int u = 0; u < XT; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (at[u][k] >= 0) store(at[u][k], acc[u][j][k], bias, zv[u][k]);
     }
     if (blockIdx.x != 0) return;
-    // positions n/4 and 3n/4: lanes share the modes and the channels
-    for (int j = 0; j < 8 && o0 + j < C; ++j) {
-        const int o = o0 + j;
-        float even = 0.f, odd = 0.f, p1 = 0.f, p3 = 0.f;
-        for (int m = lane; m < M; m += 32) {
-            const float2 y = Y[((long long)b * C + o) * M + m];
-            const float w = (m >> 1) & 1 ? -weight(m) : weight(m);
-            if (m & 1) odd = fmaf(w, y.y, odd);
-            else even = fmaf(w, y.x, even);
+    // positions n/4 and 3n/4 of the warp's 8 channels: lanes share modes and channels
+    float even[8] = {}, odd[8] = {};
+    for (int m = lane; m < M; m += 32) {
+        const float w = (m >> 1) & 1 ? -weight(m) : weight(m);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float2 y = Y[((long long)b * C + min(o0 + j, C - 1)) * M + m];
+            if (m & 1) odd[j] = fmaf(w, y.y, odd[j]);
+            else even[j] = fmaf(w, y.x, even[j]);
         }
-        for (int i = lane; i < C; i += 32) {
-            const float *hp = h + ((long long)b * C + i) * n;
-            p1 = fmaf(ps[i * Cp + o], hp[q], p1);
-            p3 = fmaf(ps[i * Cp + o], hp[3 * q], p3);
+    }
+    float p1[8] = {}, p3[8] = {};
+    for (int i = lane; i < C; i += 32) {
+        const float *hp = h + ((long long)b * C + i) * n;
+        const float h1 = hp[q], h3 = hp[3 * q];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            p1[j] = fmaf(ps[i * Cp + o0 + j], h1, p1[j]);
+            p3[j] = fmaf(ps[i * Cp + o0 + j], h3, p3[j]);
         }
-        float v1 = even - odd + p1, v3 = even + odd + p3;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        float v1 = even[j] - odd[j] + p1[j], v3 = even[j] + odd[j] + p3[j];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             v1 += __shfl_xor_sync(0xffffffffu, v1, off);
             v3 += __shfl_xor_sync(0xffffffffu, v3, off);
         }
-        if (lane == 0) store(o, q, v1);
-        if (lane == 1) store(o, 3 * q, v3);
+        if (o0 + j < C && lane < 2) {
+            const int at = j * n + (lane ? 3 * q : q);
+            store(at, lane ? v3 : v1, BWD ? 0.f : bf(pb, oc + o0 + j), zr ? zr[at] : 0.f);
+        }
     }
 }
 
@@ -651,37 +674,28 @@ size_t synth_smem(int C, int XT) {
     return 16 * (SY_MC * Cp + SY_MC * XW + SY_IC * XW) + 4 * C * Cp;
 }
 
-// x per block: 64 where that still gives about two blocks per SM, else 32; up to
-// 48 channels the block has 192 threads, so that three fit the register file.
-template <bool BWD, int XT, int NT>
+// x per block: 64 where that still gives about two blocks per SM, else 32.
+template <bool BWD, int XT>
 void launch_synth_t(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
                     int act, cudaStream_t st) {
     const int q = s->n / 4, threads = 32 * ((s->c + 7) / 8);
-    k_synth<BWD, XT, NT><<<dim3((q + 32 * XT - 1) / (32 * XT), B), threads, synth_smem(s->c, XT), st>>>(
+    k_synth<BWD, XT><<<dim3((q + 32 * XT - 1) / (32 * XT), B), threads, synth_smem(s->c, XT), st>>>(
         Y, h, s->pb, oP, oc, s->tw, z, hn, s->c, s->n, s->m, act);
 }
 
 template <bool BWD>
 void launch_synth(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
                   int act, cudaStream_t st) {
-    const bool two = (long long)B * ((s->n / 4 + 63) / 64) >= 256, small = s->c <= 48;
-    auto f = two ? (small ? launch_synth_t<BWD, 2, 192> : launch_synth_t<BWD, 2, 256>)
-                 : (small ? launch_synth_t<BWD, 1, 192> : launch_synth_t<BWD, 1, 256>);
-    f(s, Y, h, oP, oc, z, hn, B, act, st);
+    if ((long long)B * ((s->n / 4 + 63) / 64) >= 256) launch_synth_t<BWD, 2>(s, Y, h, oP, oc, z, hn, B, act, st);
+    else launch_synth_t<BWD, 1>(s, Y, h, oP, oc, z, hn, B, act, st);
 }
 
-// Shared memory instead of L1 for the kernels that stage their operands (the
-// default split left room for two blocks per SM).
-template <bool BWD, int XT, int NT>
-void synth_attrs() {
-    cudaFuncSetAttribute(k_synth<BWD, XT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)synth_smem(64, XT));
-    cudaFuncSetAttribute(k_synth<BWD, XT, NT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+template <bool BWD, int XT>
+void synth_attr() {
+    cudaFuncSetAttribute(k_synth<BWD, XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)synth_smem(64, XT));
 }
 void init_attrs() {
-    synth_attrs<false, 1, 192>(); synth_attrs<false, 2, 192>(); synth_attrs<false, 1, 256>(); synth_attrs<false, 2, 256>();
-    synth_attrs<true, 1, 192>(); synth_attrs<true, 2, 192>(); synth_attrs<true, 1, 256>(); synth_attrs<true, 2, 256>();
-    cudaFuncSetAttribute(k_dft, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    cudaFuncSetAttribute(k_outer, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    synth_attr<false, 1>(); synth_attr<false, 2>(); synth_attr<true, 1>(); synth_attr<true, 2>();
 }
 
 template <bool BWD>
@@ -689,8 +703,8 @@ void launch_mix(apf_sno *s, const float2 *X, float2 *Y, int l, int B, cudaStream
     const int C = s->c, M = s->m;
     const long long wr = s->oWr + (long long)l * C * C * M, wi = s->oWi + (long long)l * C * C * M;
     const int bg = (B + 3) / 4;
-    if ((long long)((C + 3) / 4) * M * bg >= 16384)
-        k_mix<BWD, 4><<<dim3(nb((long long)((C + 3) / 4) * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
+    if ((long long)((C + 1) / 2) * M * bg >= 16384)
+        k_mix<BWD, 2><<<dim3(nb((long long)((C + 1) / 2) * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
     else
         k_mix<BWD, 1><<<dim3(nb((long long)C * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
 }
