@@ -187,8 +187,11 @@ __global__ void k_pack64_BT(const __grid_constant__ Tab<const double2 *> srct, l
 // the randomisation that lets symmetric indefinite elimination run without
 // pivoting.  w[0 .. n): level-Q diagonals (R0 at i, R1 at n/2 + i); w[n .. 2n):
 // level-P, half h (0 / 1) at n + h n/2 (R0 at i, R1 at n/4 + i).
-// Bound by HBM: 24 n^2 bytes against the 72 n^2 of the five passes it replaces
-// (inverse transform, packing, assembly, forward transform).
+// 24 n^2 bytes against the 72 n^2 of the five passes it replaces (inverse
+// transform, packing, assembly, forward transform).  Two 4096 blocks: 179 us, 4.5
+// TB/s (0.66 of the copy rate; about 100 instructions per element); 399 us with
+// the source and the next block in separate registers and K evaluated for
+// every element.
 struct RowSrc {
     const float *re, *im;     // n x n block (null: no such source)
     int yspace, use;          // still transformed; subtracted from the next block
@@ -238,9 +241,11 @@ __device__ __forceinline__ void store_split2(const Mirror &m, int planes, long l
     }
 }
 
-template <bool BF, int N>
-__global__ void __launch_bounds__(128) k_row_step(GridDev g, const __grid_constant__ RowJobs<N> jobs, int n, const double2 *circ,
-                                                  const float *w, int planes, int leaf) {
+// TWO: both sources (the middle row); otherwise only s[0] is looked at, and the
+// block is assembled in the registers that held the source.
+template <bool BF, bool TWO, int N>
+__global__ void __launch_bounds__(128, TWO ? 2 : 4) k_row_step(GridDev g, const __grid_constant__ RowJobs<N> jobs, int n, const double2 *__restrict__ circ,
+                                                               const float *__restrict__ w, int planes, int leaf) {
     const RowJob &J = jobs.j[blockIdx.z];
     const int q = n >> 2, half = n >> 3;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -248,28 +253,8 @@ __global__ void __launch_bounds__(128) k_row_step(GridDev g, const __grid_consta
     const int i = idx / half, j = 2 * (idx - i * half);
     const float *wq = w, *wp0 = w + n, *wp1 = w + n + n / 2;
     float2 x[4][8];  // [row group][2 column group + column]
-    // K: 4 - k^2 eps on the diagonal, -1 on the periodic neighbours, the circulants
-    // Sigma_bot / Sigma_top on the first / last slab row; float64 only on the diagonal
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            float kr = 0.f, ki = 0.f;
-            if (J.row >= 0) {
-                const int row = i + r * q, col = j + (c & 1) + (c >> 1) * q, dx = row - col;
-                if (dx == 0) kr = (float)(4.0 - g.k * g.k * J.eps[(long long)J.row * n + row]);
-                if (dx == 1 || dx == -1 || dx == n - 1 || dx == 1 - n) kr -= 1.f;
-                const int d = dx < 0 ? dx + n : dx;
-                if (J.row == 0) { kr += (float)circ[d].x; ki += (float)circ[d].y; }
-                if (J.row == g.h - 1) { kr += (float)circ[n + d].x; ki += (float)circ[n + d].y; }
-            }
-            x[r][c] = make_float2(kr, ki);
-        }
-#pragma unroll 1
-    for (int s = 0; s < 2; ++s) {
-        const RowSrc &S = J.s[s];
-        if (!S.re) continue;
-        float2 v[4][8];
+    // a source into v: load, transform, write out
+    auto source = [&](const RowSrc &S, float2 (&v)[4][8]) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -285,10 +270,12 @@ __global__ void __launch_bounds__(128) k_row_step(GridDev g, const __grid_consta
                 for (int c = 0; c < 8; ++c) bf_inv(v[a][c], v[b][c], wa, wb);
             };
             auto cols = [&](int a, int b, const float *wa, const float *wb) {
+                const float2 fa = *reinterpret_cast<const float2 *>(wa + j), fb = *reinterpret_cast<const float2 *>(wb + j);
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) bf_inv(v[r][2 * a + u], v[r][2 * b + u], wa[j + u], wb[j + u]);
+                for (int r = 0; r < 4; ++r) {
+                    bf_inv(v[r][2 * a], v[r][2 * b], fa.x, fb.x);
+                    bf_inv(v[r][2 * a + 1], v[r][2 * b + 1], fa.y, fb.y);
+                }
             };
             rows(0, 2, wq[i], wq[2 * q + i]); rows(1, 3, wq[q + i], wq[3 * q + i]);
             rows(0, 1, wp0[i], wp0[q + i]); rows(2, 3, wp1[i], wp1[q + i]);
@@ -307,36 +294,76 @@ __global__ void __launch_bounds__(128) k_row_step(GridDev g, const __grid_consta
                     *reinterpret_cast<float2 *>(S.ck_re + o) = make_float2(a.x, b.x);
                     *reinterpret_cast<float2 *>(S.ck_im + o) = make_float2(a.y, b.y);
                 }
-                if (S.use) {
-                    float2 &xa = x[r][2 * c], &xb = x[r][2 * c + 1];
-                    xa = make_float2(__fadd_rn(xa.x, J.sgn * a.x), __fadd_rn(xa.y, J.sgn * a.y));
-                    xb = make_float2(__fadd_rn(xb.x, J.sgn * b.x), __fadd_rn(xb.y, J.sgn * b.y));
-                }
             }
+    };
+    if (J.s[0].re) source(J.s[0], x);
+    if (!TWO && !J.out) return;
+    // X = K + sgn G.  K: 4 - k^2 eps on the diagonal, -1 on the periodic neighbours,
+    // the circulants Sigma_bot / Sigma_top on the first / last slab row; float64 only
+    // on the diagonal
+    const float s0 = J.s[0].re && J.s[0].use ? J.sgn : 0.f;
+    const bool c0 = J.row == 0, c1 = J.row == g.h - 1;
+    // off the end rows K touches a thread's elements only where i and j are (almost) equal modulo q
+    const int off = i > j ? i - j : j - i;
+    if (J.row >= 0 && (c0 || c1 || off <= 2 || off >= q - 2)) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float kr = 0.f, ki = 0.f;
+                const int row = i + r * q, col = j + (c & 1) + (c >> 1) * q, dx = row - col;
+                if (dx == 0) kr = (float)(4.0 - g.k * g.k * J.eps[(long long)J.row * n + row]);
+                if (dx == 1 || dx == -1 || dx == n - 1 || dx == 1 - n) kr -= 1.f;
+                const int d = dx < 0 ? dx + n : dx;
+                if (c0) { kr += (float)circ[d].x; ki += (float)circ[d].y; }
+                if (c1) { kr += (float)circ[n + d].x; ki += (float)circ[n + d].y; }
+                // (sgn = +-1: the product is exact)
+                x[r][c] = s0 != 0.f ? make_float2(__fadd_rn(kr, s0 * x[r][c].x), __fadd_rn(ki, s0 * x[r][c].y)) : make_float2(kr, ki);
+            }
+    } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) x[r][c] = s0 != 0.f ? make_float2(s0 * x[r][c].x, s0 * x[r][c].y) : make_float2(0.f, 0.f);
     }
-    if (!J.out) return;
+    if constexpr (TWO) {
+        if (J.s[1].re) {
+            float2 v[4][8];
+            source(J.s[1], v);
+            if (J.s[1].use)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        x[r][c] = make_float2(__fadd_rn(x[r][c].x, J.sgn * v[r][c].x), __fadd_rn(x[r][c].y, J.sgn * v[r][c].y));
+        }
+        if (!J.out) return;
+    }
     if (BF) {  // X' = U^T X U: rows and columns, P^T then Q^T
         auto rows = [&](int a, int b, float wa, float wb) {
 #pragma unroll
             for (int c = 0; c < 8; ++c) bf_fwd(x[a][c], x[b][c], wa, wb);
         };
         auto cols = [&](int a, int b, const float *wa, const float *wb) {
+            const float2 fa = *reinterpret_cast<const float2 *>(wa + j), fb = *reinterpret_cast<const float2 *>(wb + j);
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int u = 0; u < 2; ++u) bf_fwd(x[r][2 * a + u], x[r][2 * b + u], wa[j + u], wb[j + u]);
+            for (int r = 0; r < 4; ++r) {
+                bf_fwd(x[r][2 * a], x[r][2 * b], fa.x, fb.x);
+                bf_fwd(x[r][2 * a + 1], x[r][2 * b + 1], fa.y, fb.y);
+            }
         };
         rows(0, 1, wp0[i], wp0[q + i]); rows(2, 3, wp1[i], wp1[q + i]);
         rows(0, 2, wq[i], wq[2 * q + i]); rows(1, 3, wq[q + i], wq[3 * q + i]);
         cols(0, 1, wp0, wp0 + q); cols(2, 3, wp1, wp1 + q);
         cols(0, 2, wq, wq + 2 * q); cols(1, 3, wq + q, wq + 3 * q);
     }
+    const int ls = 31 - __clz(leaf);  // leaf sizes are powers of two
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const int row = i + r * q, col = j + c * q;
-            const int br = row / leaf, bc = col / leaf;
+            const int br = row >> ls, bc = col >> ls;
             if (bc > br) continue;
             const float2 a = x[r][2 * c], b = x[r][2 * c + 1];
             const long long o = (long long)row * n + col;
@@ -594,53 +621,102 @@ __global__ void k_circ_apply(const __grid_constant__ Tab<const double2 *> Et, lo
 // d E - (sum of the four neighbours) + boundary terms, d = 4 - k^2 eps; the
 // neighbour sum and the boundary terms are gathered first so that the
 // diagonal term is one fused multiply-add per component.  One thread walks the
-// slab rows of one (column, x), so each field value is loaded three times (as
-// centre, left, right) instead of five, and the squared norm of the column is
-// summed on the way (part: one value per block, see k_normsum).  R is zero
-// except on the first and last slab rows (Rt: those two rows; null: r = K E).
-// Bound by the float64 pipe (11 operations per point, 2 per clock and SM).
+// slab rows of RC columns at one x, so each field value is loaded three times (as
+// centre, left, right) instead of five, with the next row's loads in flight, and
+// the squared norms of the columns are summed on the way (part: one value per
+// block and column, see k_normsum).  R is zero except on the first and last slab
+// rows (Rt: those two rows; null: r = K E).  Bound by the float64 pipe: 10.5
+// operations per point at 2 per clock and SM (4096 x 260, 686 columns: 0.82 ms of
+// them, 1.15 ms measured; 1.62 ms with the end rows' conditions in the loop).
+constexpr int RC = 2;
 __global__ void __launch_bounds__(128) k_residual(GridDev g, const __grid_constant__ Tab<const double *> epst, const __grid_constant__ Tab<const double2 *> Et, const __grid_constant__ Tab<const double2 *> Rt, const __grid_constant__ Tab<double2 *> cbt,
                                                   const __grid_constant__ Tab<double2 *> ctt, const __grid_constant__ Tab<double2 *> rt, const __grid_constant__ Tab<double *> partt, int ncol) {
-    const int b = blockIdx.z, c = blockIdx.y, n = g.nx, h = g.h;
+    const int b = blockIdx.z, n = g.nx, h = g.h, c0 = RC * blockIdx.y;
     const int x = blockIdx.x * 128 + threadIdx.x;
     const long long L = (long long)ncol * n;
-    double acc = 0.0;
+    double acc[RC] = {};
     if (x < n) {
         const double *eps = epst.v[b] + x;
         const double2 *R = Rt.v[b];
-        const double2 *e = Et.v[b] + (long long)c * n;
-        double2 *r = rt.v[b] + (long long)c * n + x;
         const double k2 = -(g.k * g.k);
         const int xr = (x + 1 == n) ? 0 : x + 1, xl = (x == 0) ? n - 1 : x - 1;
-        double2 below = cmk(0.0, 0.0), here = e[x];
-        for (int j = 0; j < h; ++j, e += L, r += L) {
-            const double2 above = j + 1 < h ? e[L + x] : cmk(0.0, 0.0);
-            double2 nbr = cadd(e[xr], e[xl]);  // neighbours minus boundary terms (plus the right-hand side)
-            if (j > 0) nbr = cadd(nbr, below);
-            if (j + 1 < h) nbr = cadd(nbr, above);
-            if (j == 0) nbr = csub(nbr, cbt.v[b][(long long)c * n + x]);
-            if (j == h - 1) nbr = csub(nbr, ctt.v[b][(long long)c * n + x]);
-            if (R) {
-                if (j == 0) nbr = cadd(nbr, R[(long long)c * n + x]);
-                if (j == h - 1 && h > 1) nbr = cadd(nbr, R[L + (long long)c * n + x]);
-            }
-            const double d = fma(k2, eps[(long long)j * n], 4.0);
-            double2 v = make_double2(fma(-d, here.x, nbr.x), fma(-d, here.y, nbr.y));
-            if (!R) v = make_double2(-v.x, -v.y);  // K E
-            *r = v;
-            acc = fma(v.x, v.x, fma(v.y, v.y, acc));
-            below = here;
-            here = above;
+        long long col[RC];
+        const double2 *e[RC];
+#pragma unroll
+        for (int u = 0; u < RC; ++u) {
+            col[u] = (long long)min(c0 + u, ncol - 1) * n;  // (an odd last column is computed twice, written once)
+            e[u] = Et.v[b] + col[u];
         }
+        double2 below[RC], here[RC], above[RC], lr[RC], rr[RC];
+        double ep = eps[0];
+#pragma unroll
+        for (int u = 0; u < RC; ++u) {
+            below[u] = cmk(0.0, 0.0);
+            here[u] = e[u][x];
+            lr[u] = e[u][xl];
+            rr[u] = e[u][xr];
+            above[u] = h > 1 ? e[u][L + x] : cmk(0.0, 0.0);
+        }
+        // extra: what an end row adds to the neighbour sum.  The rows between them
+        // run without a condition (one would be turned into float64 operations
+        // that are always executed: 21 per point instead of 10.5).
+        auto row = [&](int j, const double2 (&extra)[RC], bool end) {
+            // the next row's neighbours and the row above it
+            double2 nl[RC], nr[RC], na[RC];
+            double en = 0.0;
+#pragma unroll
+            for (int u = 0; u < RC; ++u) {
+                e[u] += L;
+                nl[u] = nr[u] = na[u] = cmk(0.0, 0.0);
+                if (j + 1 < h) {
+                    nl[u] = e[u][xl];
+                    nr[u] = e[u][xr];
+                    if (j + 2 < h) na[u] = e[u][L + x];
+                }
+            }
+            if (j + 1 < h) en = eps[(long long)(j + 1) * n];
+            const double d = fma(k2, ep, 4.0);
+#pragma unroll
+            for (int u = 0; u < RC; ++u) {
+                double2 nbr = cadd(cadd(rr[u], lr[u]), cadd(below[u], above[u]));  // neighbours, zero outside the slab
+                if (end) nbr = cadd(nbr, extra[u]);
+                const double2 v = make_double2(fma(-d, here[u].x, nbr.x), fma(-d, here[u].y, nbr.y));
+                if (c0 + u < ncol) rt.v[b][j * L + col[u] + x] = R ? v : make_double2(-v.x, -v.y);  // without R: K E
+                acc[u] = fma(v.x, v.x, fma(v.y, v.y, acc[u]));
+                below[u] = here[u];
+                here[u] = above[u];
+                above[u] = na[u];
+                lr[u] = nl[u];
+                rr[u] = nr[u];
+            }
+            ep = en;
+        };
+        double2 first[RC], last[RC];
+#pragma unroll
+        for (int u = 0; u < RC; ++u) {
+            const double2 sb = cbt.v[b][col[u] + x], st = ctt.v[b][col[u] + x];
+            first[u] = R ? csub(R[col[u] + x], sb) : make_double2(-sb.x, -sb.y);
+            last[u] = R && h > 1 ? csub(R[L + col[u] + x], st) : make_double2(-st.x, -st.y);
+            if (h == 1) first[u] = cadd(first[u], last[u]);
+        }
+        row(0, first, true);
+#pragma unroll 1
+        for (int j = 1; j < h - 1; ++j) row(j, first, false);
+        if (h > 1) row(h - 1, last, true);
     }
     double *part = partt.v[b];
     if (!part) return;
-    __shared__ double red[4];
+    __shared__ double red[RC][4];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    for (int u = 0; u < RC; ++u) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], off);
+        if ((threadIdx.x & 31) == 0) red[u][threadIdx.x >> 5] = acc[u];
+    }
     __syncthreads();
-    if (threadIdx.x == 0) part[(long long)c * gridDim.x + blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+    const int u = threadIdx.x;
+    if (u < RC && c0 + u < ncol)
+        part[(long long)(c0 + u) * gridDim.x + blockIdx.x] = (red[u][0] + red[u][1]) + (red[u][2] + red[u][3]);
 }
 
 // out[c] = the sum of column c's np partial sums, in a fixed order (one warp per column).
@@ -947,11 +1023,16 @@ void row_step_b(const Bat &bt, const RowJob *jobs, int nj, int n, bool bf, cudaS
     const int leaf = std::min(leaf_size(w), n);
     const GridDev g = make_grid(c);
     const dim3 grid((unsigned)(((long long)(n / 4) * (n / 8) + 127) / 128), 1, nj);
+    bool two = false;
+    for (int i = 0; i < nj; ++i) two = two || jobs[i].s[1].re;
     auto run = [&](auto &pack) {
         for (int i = 0; i < nj; ++i) pack.j[i] = jobs[i];
         constexpr int N = sizeof(pack.j) / sizeof(RowJob);
-        if (bf) APF_LAUNCH(c, (k_row_step<true, N>), grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
-        else APF_LAUNCH(c, (k_row_step<false, N>), grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
+        auto launch = [&](auto kernel) {
+            APF_LAUNCH(c, kernel, grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
+        };
+        if (bf) two ? launch(k_row_step<true, true, N>) : launch(k_row_step<true, false, N>);
+        else two ? launch(k_row_step<false, true, N>) : launch(k_row_step<false, false, N>);
     };
     if (nj <= 2) {
         RowJobs<2> p{};
@@ -1178,7 +1259,7 @@ void residual_b(const Bat &bt, FE E, FR r, bool rhs, cudaStream_t s) {
     const auto part = tab<double *>(bt, [&](int b) { return rhs ? bt.c[b]->mw->rpart : nullptr; });
     APF_LAUNCH(c, k_circ_apply, dim3(ncol, 2, nb), threads, nx * (int)sizeof(double2), s, Et, (c->h - 1) * L, cb, ct, nx,
                logn, (const double2 *)c->d_modes, (const double2 *)c->d_tw);
-    const dim3 grid((nx + 127) / 128, ncol, nb);
+    const dim3 grid((nx + 127) / 128, (ncol + RC - 1) / RC, nb);
     APF_LAUNCH(c, k_residual, grid, 128, 0, s, make_grid(c),
                tab<const double *>(bt, [&](int b) { return (const double *)bt.c[b]->d_eps; }), Et,
                tab<const double2 *>(bt, [&](int b) { return rhs ? (const double2 *)bt.c[b]->d_R : nullptr; }), cb, ct,
