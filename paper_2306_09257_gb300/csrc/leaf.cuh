@@ -363,26 +363,27 @@ __device__ void leaf_gj_regs2(float *re, float *im, long long ld, int *flags) {
 // Inverse of a 128 x 128 float32 block by a cluster of four CTAs (one per block,
 // 512 threads each): block Gauss-Jordan elimination in place over four 32-column
 // panels, CTA q holding the panel of columns 32 q .. 32 q + 31 in shared memory.
-// Step p: every CTA copies panel p (distributed shared memory), inverts its 32 x 32
-// pivot block (each for itself, which saves a broadcast), and updates its own
-// panel: R = P^-1 A_p, A_i -= F_i R, A_p = R (on panel p itself: P^-1 and -F_i P^-1).
-// These blocks sit one after the other on the critical path of every
-// inversion, so what counts is latency: 4 x (a chain of 32 pivots, 128 x 32 x 32
-// multiply-adds per SM, a panel copy and a cluster barrier).  The four SMs
-// divide the multiply-adds that a single CTA would spend most of its time on.
-// Measured: 93 -> 60 us per block against one CTA (2 x 2 Schur recursion with
-// 32 x 32 leaves of one barrier, two shared-memory round trips and a division
-// per pivot).
+// Step p, with panel p as it stands (F) and the inverse P^-1 of its 32 x 32 pivot
+// block in every CTA: R = P^-1 A_p, A_i -= F_i R, A_p = R (on panel p itself:
+// P^-1 and -F_i P^-1).
+// These blocks sit one after the other on the critical path of every inversion,
+// so what counts is latency, and the chain of 4 x 32 pivots bounds it.  Four
+// warps of the next panel's CTA invert its pivot block and store the inverse to the
+// four CTAs (distributed shared memory) while the other three copy the panel.
+// Updating the next pivot block alone first, and the rest beside its inversion,
+// is no faster: the inversion then takes twice as long (it shares the SM's issue slots).
+// Measured: 36 us per block; 60 us with every CTA inverting the pivot block (400 clocks
+// a pivot) after copying the panel, 93 us in one CTA.
 // ---------------------------------------------------------------------------
 namespace lc {
 constexpr int NT = 512, PT = 34;  // threads, row pitch (float2; rows 16-byte aligned, columns conflict-free)
 
 struct Smem {
-    float2 own[128 * PT], F[128 * PT], cur[2][32 * PT], inv[32 * PT], R[32 * PT];
-    float2 v[128], y[128], ypart[128];
-    float part[NT / 32], e2;
-    float2 s_inv[2];
-    int s_p[2], piv[32], bad;
+    float2 own[128 * PT], F[128 * PT], inv[32 * PT], R[32 * PT];
+    float2 g[32 * 32], scale[32];
+    float2 v[128], wpart[16][32], w[32], zpart[4][4][128];
+    float part[4];
+    int piv[32];
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -390,118 +391,169 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 
 // Shared-memory object `p` of cluster CTA `rank` (generic address).
 template <typename T>
-__device__ __forceinline__ const T *peer(const T *p, int rank) {
+__device__ __forceinline__ T *peer(T *p, int rank) {
     uint64_t a;
     asm volatile("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"((uint64_t)p), "r"(rank));
-    return reinterpret_cast<const T *>(a);
+    return reinterpret_cast<T *>(a);
+}
+// Store to the same place in all four CTAs.
+template <typename T>
+__device__ __forceinline__ void store_all(T *p, T v) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) *peer(p, q) = v;
 }
 
-// Pivoted Gauss-Jordan inverse of the 32 x 32 block `a` (pitch PT) into sm.inv, by
+// Pivoted Gauss-Jordan inverse of the 32 x 32 block `a` (pitch PT) into `out`, by
 // warps 0-3: lane i of every warp holds row i, warp w the columns 8w .. 8w+7.  Rows
 // are not swapped: step k takes the unused row with the largest |a[p][k]| (a warp
-// maximum over |.|^2 with its low five bits replaced by 31 - row).  The warp that
-// owns the next pivot column updates that column first and finds the pivot, with
-// every lane's reciprocal computed beside the maximum, while the others finish
-// their updates: one barrier of the four warps per step.  A zero pivot leaves
+// maximum over |.|^2 with its low five bits replaced by the row), and rows are
+// divided by their pivots only at the end, so that a step leaves its own row
+// alone.  All that a step's pivot needs lies in the warp that holds its column: for
+// eight steps that warp runs ahead on its own (pivot row by shuffles, all issued
+// before their first use; reciprocals beside the maximum) and leaves the column's
+// factors in shared memory; the other warps follow two steps at a time behind
+// named barriers, at which it does not wait (1-4 and 5-8 by turns: it waits for the
+// next warp's while the others may still be at its own).  A zero pivot leaves
 // infinities or NaN, which the caller's check of the result finds.
-static __device__ void leaf32(Smem &sm, const float2 *a) {
+// Measured: 195 clocks per pivot; 400 with a barrier of all four warps and the
+// pivot row through shared memory.
+static __device__ void leaf32(Smem &sm, const float2 *a, float2 *out) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float2 x[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = a[lane * PT + 8 * w + j];
-    bool used = false;
+    for (int j = 0; j < 8; j += 2) {
+        const float4 q = *reinterpret_cast<const float4 *>(a + lane * PT + 8 * w + j);
+        x[j] = make_float2(q.x, q.y);
+        x[j + 1] = make_float2(q.z, q.w);
+    }
+    unsigned keep = ~31u, low = lane;  // both 0 once the row has been a pivot
     int mystep = 0;
-    auto bar = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
-    auto pivot = [&](float2 v, int k, int b) {
-        const float den = fmaf(v.x, v.x, v.y * v.y);
-        const unsigned key = used ? 0u : ((__float_as_uint(den) & ~31u) | (unsigned)(31 - lane));
-        const unsigned best = __reduce_max_sync(0xffffffffu, key);
-        const float rd = __fdividef(1.f, den);
-        if (lane == 31 - (int)(best & 31u)) {
-            sm.s_p[b] = lane;
-            sm.piv[k] = lane;
-            sm.s_inv[b] = make_float2(v.x * rd, -v.y * rd);
-        }
+    auto shuffle = [](float2 v, int p) {
+        return make_float2(__shfl_sync(0xffffffffu, v.x, p), __shfl_sync(0xffffffffu, v.y, p));
     };
-    auto stage = [&](int b) {
-        float4 *d = reinterpret_cast<float4 *>(sm.cur[b] + lane * PT + 8 * w);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) d[j] = make_float4(x[2 * j].x, x[2 * j].y, x[2 * j + 1].x, x[2 * j + 1].y);
+    auto apply = [](float2 &c, float2 g, float2 r) {
+        c.x = fmaf(-g.x, r.x, fmaf(g.y, r.y, c.x));
+        c.y = fmaf(-g.x, r.y, fmaf(-g.y, r.x, c.y));
     };
-    if (w == 0) pivot(x[0], 0, 0);
-    stage(0);
-    bar();
     for (int kw = 0; kw < 4; ++kw) {
-#pragma unroll
-        for (int kl = 0; kl < 8; ++kl) {
-            const int k = 8 * kw + kl, b = kl & 1;
-            const int p = sm.s_p[b];
-            const float2 inv = sm.s_inv[b], f = sm.cur[b][lane * PT + k];
-            float2 r[8];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 q = reinterpret_cast<const float4 *>(sm.cur[b] + p * PT + 8 * w)[j];
-                r[2 * j] = make_float2(q.x, q.y);
-                r[2 * j + 1] = make_float2(q.z, q.w);
-            }
-            // other rows: x - (f inv) row_p; the pivot row: 0 - (-inv) row_p
-            const bool isp = lane == p;
-            const float2 g = isp ? make_float2(-inv.x, -inv.y)
-                                 : make_float2(fmaf(f.x, inv.x, -f.y * inv.y), fmaf(f.x, inv.y, f.y * inv.x));
-            if (isp) {
-                used = true;
-                mystep = k;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] = make_float2(0.f, 0.f);
-            }
-            auto update = [&](int j) {
-                x[j].x = fmaf(-g.x, r[j].x, fmaf(g.y, r[j].y, x[j].x));
-                x[j].y = fmaf(-g.x, r[j].y, fmaf(-g.y, r[j].x, x[j].y));
+        const int bar = 1 + 4 * (kw & 1);
+        if (w == kw) {
+            unsigned key, best;
+            float2 rec;  // this lane's 1 / x
+            auto search = [&](float2 v) {
+                const float den = fmaf(v.x, v.x, v.y * v.y);
+                key = (__float_as_uint(den) & keep) | low;
+                best = __reduce_max_sync(0xffffffffu, key);
+                float rd;
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(den));
+                rec = make_float2(v.x * rd, -v.y * rd);
             };
-            const int jn = kl < 7 ? kl + 1 : 0;  // the next pivot column, in warp kw (or kw + 1)
-            update(jn);
-            if (w == (kl < 7 ? kw : kw + 1)) pivot(x[jn], k + 1, b ^ 1);
+            search(x[0]);
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j != jn) update(j);
-            if (w == kw) x[kl] = make_float2(-g.x, -g.y);
-            if (k + 1 < 32) {
-                stage(b ^ 1);
-                bar();
+            for (int kl = 0; kl < 8; ++kl) {
+                const int k = 8 * kw + kl, p = (int)(best & 31u);
+                const float2 inv = shuffle(rec, p), f = x[kl];
+                float2 r[8];
+#pragma unroll
+                for (int i = 1; i < 8; ++i) r[(kl + i) & 7] = shuffle(x[(kl + i) & 7], p);
+                const bool isp = lane == p;
+                const float2 g = isp ? make_float2(0.f, 0.f)
+                                     : make_float2(fmaf(f.x, inv.x, -f.y * inv.y), fmaf(f.x, inv.y, f.y * inv.x));
+                if (isp) {
+                    keep = low = 0u;
+                    mystep = k;
+                }
+                apply(x[(kl + 1) & 7], g, r[(kl + 1) & 7]);
+                if (kl < 7) search(x[(kl + 1) & 7]);
+                sm.piv[k] = p;
+                sm.scale[k] = inv;
+                sm.g[32 * k + lane] = g;
+                if (kl & 1) {
+                    __syncwarp();
+                    asm volatile("bar.arrive %0, 128;" ::"r"(bar + (kl >> 1)) : "memory");
+                }
+#pragma unroll
+                for (int i = 2; i < 8; ++i) apply(x[(kl + i) & 7], g, r[(kl + i) & 7]);
+                x[kl] = isp ? make_float2(1.f, 0.f) : make_float2(-g.x, -g.y);
+            }
+            __syncwarp();
+        } else {
+#pragma unroll
+            for (int kl = 0; kl < 8; kl += 2) {
+                asm volatile("bar.sync %0, 128;" ::"r"(bar + (kl >> 1)) : "memory");
+                const int k = 8 * kw + kl;
+                const int p0 = sm.piv[k], p1 = sm.piv[k + 1];
+                const float2 g0 = sm.g[32 * k + lane], g1 = sm.g[32 * (k + 1) + lane];
+                if (lane == p0 || lane == p1) {
+                    keep = low = 0u;
+                    mystep = lane == p0 ? k : k + 1;
+                }
+                float2 r[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) r[j] = shuffle(x[j], p0);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) apply(x[j], g0, r[j]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) r[j] = shuffle(x[j], p1);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) apply(x[j], g1, r[j]);
             }
         }
     }
+    const float2 q = sm.scale[mystep];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sm.inv[mystep * PT + sm.piv[8 * w + j]] = x[j];
+    for (int j = 0; j < 8; ++j)
+        out[mystep * PT + sm.piv[8 * w + j]] = make_float2(x[j].x * q.x - x[j].y * q.y, x[j].x * q.y + x[j].y * q.x);
 }
 
-// The inverse of the block at (re, im) into the CTAs' panels sm.own; returns
-// (in every thread of the cluster) whether it passed the check below.
-static __device__ bool invert128(Smem &sm, const float *re, const float *im, long long ld, int rank) {
+// The inverse of the block at (re, im), in place; each CTA passes its panel
+// (sm.own) to `also` as well.  Returns (the same in every thread of the cluster)
+// whether the result passed the check below; if not, the block is as it was.
+template <typename Also>
+static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, int rank, Also also) {
     const int t = threadIdx.x;
-    for (int e = t; e < 128 * 32; e += NT) {
-        const int r = e >> 5, c = e & 31;
-        const long long g = (long long)r * ld + 32 * rank + c;
-        sm.own[r * PT + c] = make_float2(re[g], im[g]);
+    cluster_arrive();
+    {
+        float2 x[8], f[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long g = (long long)((t >> 5) + 16 * i) * ld + (t & 31);
+            f[i] = make_float2(re[g], im[g]);
+            x[i] = make_float2(re[g + 32 * rank], im[g + 32 * rank]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = ((t >> 5) + 16 * i) * PT + (t & 31);
+            sm.F[e] = f[i];
+            sm.own[e] = x[i];
+        }
     }
+    __syncthreads();
+    if (t < 128) {
+        leaf32(sm, sm.F, sm.inv);
+    } else if (t < 256) {
+        float sn, cs;
+        sincosf(2.3999632f * (float)(t - 128), &sn, &cs);
+        sm.v[t - 128] = make_float2(cs, sn);
+    }
+    // this thread's share of the original block, for the check: a column, eight rows
+    float *const ore = re + (32 * rank + 8 * (t >> 7)) * ld + (t & 127), *const oim = im + (ore - re);
+    float xr[8], xi[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        xr[i] = ore[i * ld];
+        xi[i] = oim[i * ld];
+    }
+    __syncthreads();
+    cluster_wait();  // every CTA has started: its shared memory can be written
     const int cp = 2 * (t & 15), row = t >> 4;  // this thread's column pair and row of each block
     for (int p = 0; p < 4; ++p) {
-        cluster_arrive();
-        cluster_wait();  // every panel is up to date
-        const float2 *src = peer(sm.own, p);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4 *>(sm.F + (row + 32 * i) * PT + cp) =
-                *reinterpret_cast<const float4 *>(src + (row + 32 * i) * PT + cp);
-        cluster_arrive();  // panel p has been read
-        __syncthreads();
-        if (t < 128) leaf32(sm, sm.F + 32 * p * PT);
-        __syncthreads();
+        const float2 *F = rank == p ? sm.own : sm.F;  // rows are read and written by the same half warp
         // R = P^-1 A_p (the panel's own columns: R = P^-1)
         float2 a0 = sm.inv[row * PT + cp], a1 = sm.inv[row * PT + cp + 1];
         if (rank != p) {
             a0 = a1 = make_float2(0.f, 0.f);
-#pragma unroll 4
+#pragma unroll 8
             for (int k = 0; k < 32; k += 2) {
                 const float4 q = *reinterpret_cast<const float4 *>(sm.inv + row * PT + k);
                 const float4 u = *reinterpret_cast<const float4 *>(sm.own + (32 * p + k) * PT + cp);
@@ -518,7 +570,6 @@ static __device__ bool invert128(Smem &sm, const float *re, const float *im, lon
         }
         *reinterpret_cast<float4 *>(sm.R + row * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
         __syncthreads();
-        cluster_wait();  // no CTA reads panel p any more
         // A_i -= F_i R for the other three row blocks
         float2 acc[3][2];
         int ri[3];
@@ -536,7 +587,7 @@ static __device__ bool invert128(Smem &sm, const float *re, const float *im, lon
             const float4 w = *reinterpret_cast<const float4 *>(sm.R + (k + 1) * PT + cp);
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const float4 q = *reinterpret_cast<const float4 *>(sm.F + ri[i] * PT + k);
+                const float4 q = *reinterpret_cast<const float4 *>(F + ri[i] * PT + k);
                 float2 &c0 = acc[i][0], &c1 = acc[i][1];
                 c0.x = fmaf(-q.x, u.x, fmaf(q.y, u.y, c0.x));
                 c0.y = fmaf(-q.x, u.y, fmaf(-q.y, u.x, c0.y));
@@ -548,90 +599,118 @@ static __device__ bool invert128(Smem &sm, const float *re, const float *im, lon
                 c1.y = fmaf(-q.z, w.w, fmaf(-q.w, w.z, c1.y));
             }
         }
+        __syncwarp();
 #pragma unroll
         for (int i = 0; i < 3; ++i)
             *reinterpret_cast<float4 *>(sm.own + ri[i] * PT + cp) =
                 make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
         *reinterpret_cast<float4 *>(sm.own + (32 * p + row) * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
-    }
-    // Self-check before the block is overwritten.  Pivoting stays inside the
-    // 32 x 32 blocks, so a nearly singular leading sub-block of a block that is
-    // itself well conditioned spoils the elimination; apply the computed inverse to
-    // a fixed unit-modulus probe v and compare X (X^-1 v) with v.  Above 2e-5
-    // relative residual (a sound block gives a few 1e-7) the block is inverted
-    // again by Gauss-Jordan with pivoting over all 128 rows.
-    if (t < 128) {
-        float sn, cs;
-        sincosf(2.3999632f * (float)t, &sn, &cs);
-        sm.v[t] = make_float2(cs, sn);
+        if (p == 3) break;
+        cluster_arrive();
+        if (rank == p + 1) {
+            __syncthreads();
+            if (t < 128) {
+                leaf32(sm, sm.own + 32 * (p + 1) * PT, sm.inv);
+                asm volatile("bar.sync 9, 128;" ::: "memory");
+                cluster_wait();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float2 *e = sm.inv + (8 * i + (t >> 4)) * PT + cp;
+                    const float4 v = *reinterpret_cast<const float4 *>(e);
+#pragma unroll
+                    for (int q = 1; q < 4; ++q) *reinterpret_cast<float4 *>(peer(e, (rank + q) & 3)) = v;
+                }
+            } else {
+                cluster_wait();
+            }
+        } else {
+            cluster_wait();  // panel p + 1 is up to date
+            const float2 *src = peer(sm.own, p + 1);
+            float4 f[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int r = 32 * (i < p + 1 ? i : i + 1) + row;
+                f[i] = *reinterpret_cast<const float4 *>(src + r * PT + cp);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int r = 32 * (i < p + 1 ? i : i + 1) + row;
+                *reinterpret_cast<float4 *>(sm.F + r * PT + cp) = f[i];
+            }
+        }
+        cluster_arrive();  // every CTA has panel p + 1 and its pivot block's inverse
+        cluster_wait();
     }
     __syncthreads();
+    for (int e = t; e < 128 * 16; e += NT) {
+        const int r = e >> 4, c = 2 * (e & 15);
+        const float2 u = sm.own[r * PT + c], v = sm.own[r * PT + c + 1];
+        const long long g = r * ld + 32 * rank + c;
+        *reinterpret_cast<float2 *>(re + g) = make_float2(u.x, v.x);
+        *reinterpret_cast<float2 *>(im + g) = make_float2(u.y, v.y);
+        also(r, 32 * rank + c, u, v);
+    }
+    // Self-check.  Pivoting stays inside the 32 x 32 blocks, so a nearly singular
+    // leading sub-block of a block that is itself well conditioned spoils the
+    // elimination; apply the computed inverse to a fixed unit-modulus probe v and
+    // compare (v^T X^-1) X with v^T.  Above 2e-5 relative residual (a sound block
+    // gives a few 1e-7) the block is inverted again by Gauss-Jordan with pivoting
+    // over all 128 rows.
     {
-        const int r = t >> 2, c0 = 8 * (t & 3);
+        const int g = t >> 5, c = t & 31;
         float2 y = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int c = c0; c < c0 + 8; ++c) {
-            const float2 m = sm.own[r * PT + c], v = sm.v[32 * rank + c];
+        for (int r = 8 * g; r < 8 * g + 8; ++r) {
+            const float2 m = sm.own[r * PT + c], v = sm.v[r];
             y.x += m.x * v.x - m.y * v.y;
             y.y += m.x * v.y + m.y * v.x;
         }
-#pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
-            y.x += __shfl_xor_sync(0xffffffffu, y.x, off);
-            y.y += __shfl_xor_sync(0xffffffffu, y.y, off);
-        }
-        if ((t & 3) == 0) sm.ypart[r] = y;
+        sm.wpart[g][c] = y;
     }
-    cluster_arrive();
-    cluster_wait();
-    if (t < 128) {
+    __syncthreads();
+    if (t < 32) {
         float2 y = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 u = peer(sm.ypart, q)[t];
-            y.x += u.x;
-            y.y += u.y;
+        for (int g = 0; g < 16; ++g) {
+            y.x += sm.wpart[g][t].x;
+            y.y += sm.wpart[g][t].y;
         }
-        sm.y[t] = y;
+        sm.w[t] = y;
     }
     __syncthreads();
     {
-        // rows 32 rank .. + 31 of the original block, 16 threads per row
-        const int r = 32 * rank + row, c0 = 8 * (t & 15);
         float2 z = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int c = c0; c < c0 + 8; ++c) {
-            const float xr = re[(long long)r * ld + c], xi = im[(long long)r * ld + c];
-            const float2 y = sm.y[c];
-            z.x += xr * y.x - xi * y.y;
-            z.y += xr * y.y + xi * y.x;
+        for (int i = 0; i < 8; ++i) {
+            const float2 y = sm.w[8 * (t >> 7) + i];
+            z.x += xr[i] * y.x - xi[i] * y.y;
+            z.y += xr[i] * y.y + xi[i] * y.x;
         }
-#pragma unroll
-        for (int off = 1; off < 16; off <<= 1) {
-            z.x += __shfl_xor_sync(0xffffffffu, z.x, off);
-            z.y += __shfl_xor_sync(0xffffffffu, z.y, off);
-        }
-        const float2 v = sm.v[r];
-        float e2 = (z.x - v.x) * (z.x - v.x) + (z.y - v.y) * (z.y - v.y);
-        e2 += __shfl_xor_sync(0xffffffffu, e2, 16);  // the warp's other row
-        if ((t & 31) == 0) sm.part[t >> 5] = e2;
-        __syncthreads();
-        if (t == 0) {
-            float tot = 0.f;
-            for (int i = 0; i < NT / 32; ++i) tot += sm.part[i];
-            sm.e2 = tot;
-        }
+        store_all(&sm.zpart[rank][t >> 7][t & 127], z);
     }
     cluster_arrive();
-    cluster_wait();
-    if (t == 0) {
-        float tot = 0.f;
-        for (int q = 0; q < 4; ++q) tot += *peer(&sm.e2, q);
-        sm.bad = !(tot <= 4e-10f * 128.f);  // (2e-5)^2 |v|^2; also catches NaN
+    cluster_wait();  // the last access to another CTA's shared memory is done
+    if (t < 128) {
+        float2 z = make_float2(-sm.v[t].x, -sm.v[t].y);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            z.x += sm.zpart[q >> 2][q & 3][t].x;
+            z.y += sm.zpart[q >> 2][q & 3][t].y;
+        }
+        float e2 = z.x * z.x + z.y * z.y;
+#pragma unroll
+        for (int off = 16; off; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+        if ((t & 31) == 0) sm.part[t >> 5] = e2;
     }
     __syncthreads();
+    if ((sm.part[0] + sm.part[1]) + (sm.part[2] + sm.part[3]) <= 4e-10f * 128.f) return true;  // (2e-5)^2 |v|^2; NaN fails
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        ore[i * ld] = xr[i];
+        oim[i * ld] = xi[i];
+    }
     cluster_arrive();
-    cluster_wait();  // no CTA leaves while another reads its shared memory
-    return !sm.bad;
+    cluster_wait();  // the block is whole again
+    return false;
 }
 }  // namespace lc

@@ -482,17 +482,10 @@ __global__ void __launch_bounds__(lc::NT) __cluster_dims__(4, 1, 1) k_leaf128(co
     const int b = blockIdx.x >> 2, rank = blockIdx.x & 3;
     float *re = ret.v[b], *im = imt.v[b];
     const Mirror m = XP.v[b];
-    if (lc::invert128(sm, re, im, ld, rank)) {
-        for (int e = threadIdx.x; e < 128 * 16; e += lc::NT) {
-            const int r = e >> 4, c = 2 * (e & 15), col = 32 * rank + c;
-            const float2 u = sm.own[r * lc::PT + c], v = sm.own[r * lc::PT + c + 1];
-            const long long g = (long long)r * ld + col;
-            *reinterpret_cast<float2 *>(re + g) = make_float2(u.x, v.x);
-            *reinterpret_cast<float2 *>(im + g) = make_float2(u.y, v.y);
-            if (m.base) store_split2(m, planes, r, col, u, v);
-        }
-        return;
-    }
+    const bool sound = lc::invert128(sm, re, im, ld, rank, [&](int r, int c, float2 u, float2 v) {
+        if (m.base) store_split2(m, planes, r, c, u, v);
+    });
+    if (sound) return;
     if (rank != 0) return;
     if (threadIdx.x == 0) atomicAdd(flags.v[b] + 1, 1);  // fallback count (flags[1])
     leaf_gj_regs<128>(re, im, ld, flags.v[b]);
