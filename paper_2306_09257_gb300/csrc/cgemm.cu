@@ -75,7 +75,8 @@ struct CgLayout {
     static constexpr int B_ROWS = BNC / CG;
     static constexpr int B_TILE = B_ROWS * BK * 2;
     static constexpr int STAGE = NQ * (A_TILE + B_TILE);
-    static constexpr int BAR = STAGES * STAGE;
+    static constexpr int OUT = STAGES * STAGE;                // one 32 x 32 float block per epilogue warp
+    static constexpr int BAR = OUT + EPI_WARPS * 32 * 32 * 4;
     static constexpr int TOTAL = BAR + (2 * STAGES + 4) * 8 + 16 + 1024;
     static constexpr int GROUP = (CG == 1 ? 4 : 2) * BNC;  // tensor-memory columns
     static constexpr int ACC = (CROSS ? 2 : 1) * GROUP;
@@ -96,79 +97,78 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Split planes of x, plane p in bits [16 p, 16 p + 16) of lo (p = 0, 1) and of hi (p = 2).
-__device__ __forceinline__ void split_words(float x, int planes, uint32_t &lo, uint32_t &hi) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(x);
-    lo = __bfloat16_as_ushort(h0);
-    hi = 0;
-    if (planes > 1) {
-        const float x1 = x - __bfloat162float(h0);
-        const __nv_bfloat16 h1 = __float2bfloat16_rn(x1);
-        lo |= (uint32_t)__bfloat16_as_ushort(h1) << 16;
-        if (planes > 2) hi = __bfloat16_as_ushort(__float2bfloat16_rn(x1 - __bfloat162float(h1)));
+// Split planes of (a, b), packed: a in the low half of w[p].
+__device__ __forceinline__ void split2(float a, float b, int planes, uint32_t (&w)[3]) {
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        if (p >= planes) break;
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        memcpy(&w[p], &h, 4);
+        a -= __uint_as_float(w[p] << 16);
+        b -= __uint_as_float(w[p] & 0xffff0000u);
     }
 }
 
 __device__ __forceinline__ void store_split(const Mirror &m, int q, int planes, long long r, long long c, float x) {
-    uint32_t lo, hi;
-    split_words(x, planes, lo, hi);
-    __nv_bfloat16 *d = m.base + q * m.qpitch + r * m.pitch + c;
-    d[0] = __ushort_as_bfloat16((unsigned short)lo);
-    if (planes > 1) d[2 * m.qpitch] = __ushort_as_bfloat16((unsigned short)(lo >> 16));
-    if (planes > 2) d[4 * m.qpitch] = __ushort_as_bfloat16((unsigned short)hi);
+    uint32_t w[3];
+    split2(x, 0.f, planes, w);
+    for (int p = 0; p < planes; ++p)
+        m.base[(2 * p + q) * m.qpitch + r * m.pitch + c] = __ushort_as_bfloat16((unsigned short)w[p]);
 }
 
-// One component (q: 0 re, 1 im) of 16 columns of one row per lane, whole and
-// aligned: the row as 16-byte stores, the transpose with neighbouring lanes
-// exchanging halves so that a store covers two rows (32 lanes: 2 x 64 bytes).
-__device__ __forceinline__ void store_vec(const CgOut &o, const CgOut &t, int q, int planes, int row, int c0, int lane,
-                                          const float (&v)[16]) {
-    float *o32 = q ? o.im : o.re, *t32 = q ? t.im : t.re;
-    if (o32) {
-        float4 *d = reinterpret_cast<float4 *>(o32 + (long long)row * o.ld + c0);
+// Component q (0 re, 1 im) of a 32 x 32 block whose row `row` this lane holds, to
+// the transposed output: neighbouring lanes exchange halves, so that a store covers
+// two columns of 32 rows.
+__device__ __forceinline__ void store_transposed(const CgOut &t, int q, int planes, int row, int c0, int lane,
+                                                 float (&v)[32]) {
+    const bool odd = lane & 1;
+    const long long col = c0 + (odd ? 16 : 0);
+    const int r0 = row & ~1;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    for (int i = 0; i < 16; ++i) {  // v[i], v[i + 16] <- even and odd row of column col + i
+        const float got = __shfl_xor_sync(0xffffffffu, odd ? v[i] : v[i + 16], 1);
+        if (odd) v[i] = got;
+        else v[i + 16] = got;
     }
-    if (t32) {
+    if (float *d = q ? t.im : t.re) {
+        d += col * t.ld + r0;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) t32[(long long)(c0 + i) * t.ld + row] = v[i];
-    }
-    if (!o.m.base && !t.m.base) return;
-    uint32_t lo[16], hi[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) split_words(v[i], planes, lo[i], hi[i]);
-    if (o.m.base) {
-        __nv_bfloat16 *d = o.m.base + q * o.m.qpitch + (long long)row * o.m.pitch + c0;
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            if (p >= planes) break;
-            uint32_t w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                w[i] = p == 0 ? __byte_perm(lo[2 * i], lo[2 * i + 1], 0x5410)
-                              : p == 1 ? __byte_perm(lo[2 * i], lo[2 * i + 1], 0x7632)
-                                       : __byte_perm(hi[2 * i], hi[2 * i + 1], 0x5410);
-            uint4 *dp = reinterpret_cast<uint4 *>(d + 2 * p * o.m.qpitch);
-            dp[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            dp[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        }
+        for (int i = 0; i < 16; ++i, d += t.ld) *reinterpret_cast<float2 *>(d) = make_float2(v[i], v[i + 16]);
     }
     if (t.m.base) {
-        const bool odd = lane & 1;
-        __nv_bfloat16 *d = t.m.base + q * t.m.qpitch + (row & ~1);
+        __nv_bfloat16 *d = t.m.base + q * t.m.qpitch + col * t.m.pitch + r0;
+        const long long plane = 2 * t.m.qpitch;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t ol = __shfl_xor_sync(0xffffffffu, odd ? lo[i] : lo[i + 8], 1);
-            const uint32_t ml = odd ? lo[i + 8] : lo[i];
-            __nv_bfloat16 *dc = d + (long long)(c0 + i + (odd ? 8 : 0)) * t.m.pitch;
-            const uint32_t a = odd ? ol : ml, b = odd ? ml : ol;  // even row, odd row
-            *reinterpret_cast<uint32_t *>(dc) = __byte_perm(a, b, 0x5410);
-            if (planes > 1) *reinterpret_cast<uint32_t *>(dc + 2 * t.m.qpitch) = __byte_perm(a, b, 0x7632);
-            if (planes > 2) {
-                const uint32_t oh = __shfl_xor_sync(0xffffffffu, odd ? hi[i] : hi[i + 8], 1);
-                const uint32_t mh = odd ? hi[i + 8] : hi[i];
-                *reinterpret_cast<uint32_t *>(dc + 4 * t.m.qpitch) = __byte_perm(odd ? oh : mh, odd ? mh : oh, 0x5410);
-            }
+        for (int i = 0; i < 16; ++i, d += t.m.pitch) {
+            uint32_t w[3];
+            split2(v[i], v[i + 16], planes, w);
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                if (p < planes) *reinterpret_cast<uint32_t *>(d + p * plane) = w[p];
+        }
+    }
+}
+
+// The rows of such a block from shared memory to the output, eight lanes per row
+// (x[i]: this lane's four columns of row r0 + 4 i; rows at and past M are left out).
+__device__ __forceinline__ void store_rows(const CgOut &o, int q, int planes, int r0, int M, int col, const float4 (&x)[8]) {
+    if (float *d = q ? o.im : o.re) {
+        d += (long long)r0 * o.ld + col;
+#pragma unroll
+        for (int i = 0; i < 8; ++i, d += 4 * o.ld)
+            if (r0 + 4 * i < M) *reinterpret_cast<float4 *>(d) = x[i];
+    }
+    if (o.m.base) {
+        __nv_bfloat16 *d = o.m.base + q * o.m.qpitch + (long long)r0 * o.m.pitch + col;
+        const long long plane = 2 * o.m.qpitch;
+#pragma unroll
+        for (int i = 0; i < 8; ++i, d += 4 * o.m.pitch) {
+            uint32_t w0[3], w1[3];
+            split2(x[i].x, x[i].y, planes, w0);
+            split2(x[i].z, x[i].w, planes, w1);
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                if (p < planes && r0 + 4 * i < M) *reinterpret_cast<uint2 *>(d + p * plane) = make_uint2(w0[p], w1[p]);
         }
     }
 }
@@ -344,10 +344,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             }
         }
     } else {
-        constexpr int CH = BNC / 16;               // chunks of 16 columns
-        const int q4 = warp & 3, half = (warp - 2) >> 2;  // tensor-memory lane quarter, chunk parity
+        // A warp takes one component of its 32 rows, 32 columns at a time.  It holds
+        // a row per lane, as the tensor memory hands them out; what goes to or comes
+        // from memory along the rows passes through a block of shared memory (16-byte
+        // cells, cell c of row r at c ^ (r % 8)), so that eight lanes share a row.
+        // One lane per row instead: 10k clocks for a 128 x 32 tile, 20k where it
+        // crosses the diagonal (element by element); like this 5.5k either way, which
+        // is what 128 KB take at the 32 bytes per clock that the stores of an SM reach.
+        const int q4 = warp & 3, q = (warp - 2) >> 2;  // tensor-memory lane quarter, component
         const bool use_beta = args.beta != 0.f, vec = args.vec != 0;
-        const int planes = args.planes;
+        const int planes = NQ == 4 ? 2 : args.planes;
+        float *block = reinterpret_cast<float *>(smem + L::OUT) + (warp - 2) * 1024;
+        auto cell = [&](int r, int c) { return reinterpret_cast<float4 *>(block + 32 * r + 4 * (c ^ (r & 7))); };
+        const int sr = lane >> 3, sc = lane & 7;  // this lane's row (of four) and cell in the shared layout
         int tl = 0;
         for (int t = cid; t < ntiles; t += ncl, ++tl) {
             const int b = tl % SETS, u = tl / SETS, pr = t / ntl;
@@ -355,32 +364,33 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             int m0, n0;
             tile_at(t - pr * ntl, m0, n0);
             const int row0 = m0 + (int)rank * BM + 32 * q4, row = row0 + lane;
-            float br[16], bi[16];
-            // the beta input of a chunk is fetched before the accumulator is waited
-            // for: all its loads are in flight together
+            const float *in = q ? p.in_im : p.in_re;
+            float *const o32 = q ? p.o.im : p.o.re;
+            // the beta input of a block is fetched before the accumulator is waited for
+            float4 pre[8];
             auto fetch = [&](int c0) {
-                const float *ir = p.in_re + (long long)row * p.ldi + c0, *ii = p.in_im + (long long)row * p.ldi + c0;
-                if (row < p.M && vec) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float4 x = reinterpret_cast<const float4 *>(ir)[i], y = reinterpret_cast<const float4 *>(ii)[i];
-                        br[4 * i] = x.x; br[4 * i + 1] = x.y; br[4 * i + 2] = x.z; br[4 * i + 3] = x.w;
-                        bi[4 * i] = y.x; bi[4 * i + 1] = y.y; bi[4 * i + 2] = y.z; bi[4 * i + 3] = y.w;
+                for (int i = 0; i < 8; ++i) {
+                    const int r = row0 + 4 * i + sr, c = c0 + 4 * sc;
+                    const float *src = in + (long long)r * p.ldi + c;
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r < p.M && c < args.N) {
+                        if (vec) {
+                            x = *reinterpret_cast<const float4 *>(src);
+                        } else {
+                            x.x = src[0];
+                            if (c + 1 < args.N) x.y = src[1];
+                            if (c + 2 < args.N) x.z = src[2];
+                            if (c + 3 < args.N) x.w = src[3];
+                        }
                     }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const bool in = row < p.M && c0 + i < args.N;
-                        br[i] = in ? ir[i] : 0.f;
-                        bi[i] = in ? ii[i] : 0.f;
-                    }
+                    pre[i] = x;
                 }
             };
             bool waited = false;
 #pragma unroll 1
-            for (int ch = half; ch < CH; ch += 2) {
-                const int c0 = n0 + 16 * ch;
-                const bool skip = c0 >= args.N || (args.sym && c0 > row0 + 31);  // warp-uniform
+            for (int c0 = n0; c0 < n0 + BNC; c0 += 32) {
+                const bool skip = c0 >= args.N || row0 >= p.M || (args.sym && c0 > row0);  // warp-uniform
                 if (!skip && use_beta) fetch(c0);
                 if (!waited) {
                     if (!mbar_wait(&tfull[b], u & 1, abort_flag)) { ok = false; break; }
@@ -389,63 +399,79 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     waited = true;
                 }
                 if (skip) continue;
-                const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(b * L::ACC + 16 * ch);
-                float vr[16], vi[16];
+                const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(b * L::ACC + (c0 - n0));
+                float v[32];
 #pragma unroll
                 for (int g = 0; g <= CROSS; ++g) {
-                    uint32_t u[CG == 1 ? 4 : 2][16];
 #pragma unroll
-                    for (int q = 0; q < (CG == 1 ? 4 : 2); ++q) tmem_ld16(ta + g * L::GROUP + q * BNC, u[q]);
-                    tmem_wait_ld();
+                    for (int hc = 0; hc < 32; hc += 16) {
+                        uint32_t x[16], y[16];
+                        tmem_ld16(ta + g * L::GROUP + q * BNC + hc, x);                         // rr, ri (pair: re, im)
+                        if (CG == 1) tmem_ld16(ta + g * L::GROUP + (q ? 2 : 3) * BNC + hc, y);  // ii, ir
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float x = __uint_as_float(u[0][i]), y = __uint_as_float(u[1][i]);
-                        if (CG == 1) {
-                            x -= __uint_as_float(u[CG == 1 ? 3 : 0][i]);
-                            y += __uint_as_float(u[CG == 1 ? 2 : 1][i]);
+                        for (int i = 0; i < 16; ++i) {
+                            float z = __uint_as_float(x[i]);
+                            if (CG == 1) z += q ? __uint_as_float(y[i]) : -__uint_as_float(y[i]);
+                            v[hc + i] = g ? v[hc + i] + z : z;
                         }
-                        vr[i] = g ? vr[i] + x : x;
-                        vi[i] = g ? vi[i] + y : y;
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    vr[i] *= args.alpha;
-                    vi[i] *= args.alpha;
-                    if (use_beta) {
-                        vr[i] += args.beta * br[i];
-                        vi[i] += args.beta * bi[i];
-                    }
-                }
-                if (vec && row0 + 31 < p.M && (!args.sym || c0 + 15 <= row0)) {
-                    store_vec(p.o, p.t, 0, planes, row, c0, lane, vr);
-                    store_vec(p.o, p.t, 1, planes, row, c0, lane, vi);
-                } else if (row < p.M) {
-                    for (int i = 0; i < 16; ++i) {
-                        const int col = c0 + i;
-                        if (col >= args.N || (args.sym && col > row)) break;
-                        float er = vr[0], ei = vi[0];
+                for (int i = 0; i < 32; ++i) v[i] *= args.alpha;
+                if (use_beta) {
 #pragma unroll
-                        for (int j = 1; j < 16; ++j)
-                            if (j == i) { er = vr[j]; ei = vi[j]; }
-                        if (p.o.re) {
-                            p.o.re[(long long)row * p.o.ld + col] = er;
-                            p.o.im[(long long)row * p.o.ld + col] = ei;
-                        }
-                        if (p.o.m.base) {
-                            store_split(p.o.m, 0, planes, row, col, er);
-                            store_split(p.o.m, 1, planes, row, col, ei);
-                        }
-                        if (p.t.re) {
-                            p.t.re[(long long)col * p.t.ld + row] = er;
-                            p.t.im[(long long)col * p.t.ld + row] = ei;
-                        }
-                        if (p.t.m.base) {
-                            store_split(p.t.m, 0, planes, col, row, er);
-                            store_split(p.t.m, 1, planes, col, row, ei);
+                    for (int i = 0; i < 8; ++i) *cell(4 * i + sr, sc) = pre[i];
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float4 x = *cell(lane, i);
+                        v[4 * i] += args.beta * x.x;
+                        v[4 * i + 1] += args.beta * x.y;
+                        v[4 * i + 2] += args.beta * x.z;
+                        v[4 * i + 3] += args.beta * x.w;
+                    }
+                    __syncwarp();
+                }
+                const bool diagonal = args.sym && c0 == row0;
+                const bool cols = vec && c0 + 31 < args.N, whole = cols && row0 + 31 < p.M;
+                if (o32 || p.o.m.base || !whole) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) *cell(lane, i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    __syncwarp();
+                    if (diagonal) {  // the block mirrored at its diagonal: no transposed store
+#pragma unroll
+                        for (int i = 1; i < 32; ++i)
+                            if (i > lane) v[i] = block[32 * i + 4 * ((lane >> 2) ^ (i & 7)) + (lane & 3)];
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            *cell(lane, i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        __syncwarp();
+                    }
+                    if (cols) {
+                        float4 x[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) x[i] = *cell(4 * i + sr, sc);
+                        store_rows(p.o, q, planes, row0 + sr, p.M, c0 + 4 * sc, x);
+                    }
+                    if (!whole && row < p.M) {  // ragged edges
+#pragma unroll 1
+                        for (int i = 0; i < 32 && c0 + i < args.N; ++i) {
+                            const int col = c0 + i;
+                            const float x = block[32 * lane + 4 * ((i >> 2) ^ (lane & 7)) + (i & 3)];
+                            if (!cols) {
+                                if (o32) o32[(long long)row * p.o.ld + col] = x;
+                                if (p.o.m.base) store_split(p.o.m, q, planes, row, col, x);
+                            }
+                            if (diagonal) continue;
+                            float *t32 = q ? p.t.im : p.t.re;
+                            if (t32) t32[(long long)col * p.t.ld + row] = x;
+                            if (p.t.m.base) store_split(p.t.m, q, planes, col, row, x);
                         }
                     }
                 }
+                if (!diagonal && whole && (p.t.re || p.t.m.base)) store_transposed(p.t, q, planes, row, c0, lane, v);
                 __syncwarp();
             }
             if (!ok) break;
