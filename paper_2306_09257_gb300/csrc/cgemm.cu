@@ -63,11 +63,18 @@ struct CgArgs {
 // product, and the sweeps (unlike the elimination, where it makes no difference)
 // set how far one refinement sweep gets: 4096 x 260, two sweeps, residual 8e-11
 // without and 2e-11 with it.
+// MERGED: a product with fewer than 128 columns takes the tensor core as long as one
+// with 128 (64 clocks per 16 of K), so the 128 x 32 tile multiplies x0 by both planes
+// of y at once, which leaves the cross products in accumulators of their own: 4
+// instead of 6 such products, 1100 instead of 1536 clocks per 64 of K.  The 128 x 64
+// tile gives the same bits (which of the two runs depends on how many products share
+// a launch), so one-CTA tiles of two planes always have CROSS.
 // Shared memory per stage: 128 rows of A and the CTA's rows of B (all BNC, or half
 // of them in a pair), 128 bytes each.  Tensor memory: an accumulator group is
-// [rr | ri | ir | ii] (one CTA) or [re | im] (pair), a set one group or, with
-// CROSS, two; two sets where they fit, so that the epilogue of a tile overlaps the
-// products of the next.
+// [rr | ri | ir | ii] (one CTA; MERGED: [rr | ri] and [ir | ii] of both groups side by
+// side) or [re | im] (pair), a set one group or, with CROSS, two; two sets where
+// they fit, so that the epilogue of a tile overlaps the products of the next, else
+// the one-CTA epilogue reads the whole set before its stores (HELD).
 template <int CG, int BNC, int NQ, int CROSS>
 struct CgLayout {
     static constexpr int STAGES = NQ == 4 ? 2 : 4;
@@ -81,6 +88,10 @@ struct CgLayout {
     static constexpr int GROUP = (CG == 1 ? 4 : 2) * BNC;  // tensor-memory columns
     static constexpr int ACC = (CROSS ? 2 : 1) * GROUP;
     static constexpr int SETS = 2 * ACC <= 512 ? 2 : 1;
+    static constexpr bool MERGED = CG == 1 && NQ == 4 && 4 * BNC <= 128;
+    static constexpr int HELD = SETS == 1 && BNC <= 64 ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
+    // offset of the accumulator of component q's first (x r..) or second (x i..) half in group g
+    static constexpr int acc(int g, int i, int r) { return MERGED ? (4 * i + 2 * g + r) * BNC : g * GROUP + (2 * i + r) * BNC; }
     static constexpr int TMEM = SETS * ACC;
     static_assert(B_TILE % 1024 == 0, "B tiles must fill whole 128-byte swizzle atoms");
     static_assert(TMEM == 256 || TMEM == 512, "tensor-memory allocation");
@@ -300,6 +311,21 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     if (!mbar_wait(&full[s], r & 1, abort_flag)) { ok = false; break; }
                     fence_after();
                     const uint32_t sa = smem_u32(smem + s * L::STAGE), sb = sa + NQ * L::A_TILE;
+                    if (L::MERGED) {
+                        // x0 with both planes of y at once: [rr0 | ri0 | rr1 | ri1], [ir0 | ii0 | ir1 | ii1]
+                        constexpr uint32_t idesc_all = base | ((uint32_t)((4 * BNC) >> 3) << 17);
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {  // x0 (y0, y1), x1 y0
+                            const uint32_t ar = sa + 2 * g * L::A_TILE, ai = ar + L::A_TILE;
+#pragma unroll
+                            for (int k4 = 0; k4 < BK / 16; ++k4) {
+                                const uint64_t dar = sw128_desc(ar + k4 * 32), dai = sw128_desc(ai + k4 * 32), db = sw128_desc(sb + k4 * 32);
+                                const uint32_t acc = (kk > 0 || k4 > 0 || g > 0) ? 1u : 0u, to = set + 2 * g * BNC;
+                                mma_bf16(to, dar, db, g ? idesc_both : idesc_all, acc);
+                                mma_bf16(to + 4 * BNC, dai, db, g ? idesc_both : idesc_all, acc);
+                            }
+                        }
+                    } else {
 #pragma unroll
                     for (int g = 0; g < (NQ == 4 ? 3 : 1); ++g) {  // x0 y0, x0 y1, x1 y0
                         const uint32_t ar = sa + (g == 2 ? 2 : 0) * L::A_TILE, ai = ar + L::A_TILE;
@@ -320,6 +346,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                                 mma_bf16(re + 2 * BNC, dai, dbr, idesc_both, acc);  // [ir | ii]
                             }
                         }
+                    }
                     }
                     if (CG == 2) {
                         mma_commit_pair(smem_u32(&empty[s]));
@@ -387,27 +414,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     pre[i] = x;
                 }
             };
-            bool waited = false;
-#pragma unroll 1
-            for (int c0 = n0; c0 < n0 + BNC; c0 += 32) {
-                const bool skip = c0 >= args.N || row0 >= p.M || (args.sym && c0 > row0);  // warp-uniform
-                if (!skip && use_beta) fetch(c0);
-                if (!waited) {
-                    if (!mbar_wait(&tfull[b], u & 1, abort_flag)) { ok = false; break; }
-                    __syncwarp();
-                    fence_after();
-                    waited = true;
-                }
-                if (skip) continue;
+            // one component of a block: rr - ii or ri + ir (pair: as accumulated), times alpha
+            auto read = [&](int c0, float (&v)[32]) {
                 const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(b * L::ACC + (c0 - n0));
-                float v[32];
 #pragma unroll
                 for (int g = 0; g <= CROSS; ++g) {
 #pragma unroll
                     for (int hc = 0; hc < 32; hc += 16) {
                         uint32_t x[16], y[16];
-                        tmem_ld16(ta + g * L::GROUP + q * BNC + hc, x);                         // rr, ri (pair: re, im)
-                        if (CG == 1) tmem_ld16(ta + g * L::GROUP + (q ? 2 : 3) * BNC + hc, y);  // ii, ir
+                        tmem_ld16(ta + (q ? L::acc(g, 0, 1) : L::acc(g, 0, 0)) + hc, x);
+                        if (CG == 1) tmem_ld16(ta + (q ? L::acc(g, 1, 0) : L::acc(g, 1, 1)) + hc, y);
                         tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
@@ -419,7 +435,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                 }
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] *= args.alpha;
+            };
+            auto skip = [&](int c0) { return c0 >= args.N || row0 >= p.M || (args.sym && c0 > row0); };  // warp-uniform
+            auto release = [&] {
+                fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (CG == 2) mbar_arrive_cluster(lead ? smem_u32(&tempty[b]) : peer_addr(&tempty[b], 0));
+                    else mbar_arrive(&tempty[b]);
+                }
+            };
+            if (!skip(n0) && use_beta) fetch(n0);
+            if (!mbar_wait(&tfull[b], u & 1, abort_flag)) { ok = false; break; }
+            __syncwarp();
+            fence_after();
+            float held[L::HELD][32];
+            if (L::HELD > 1) {  // a single set: free it for the next tile's products before the stores
+#pragma unroll
+                for (int i = 0; i < L::HELD; ++i)
+                    if (!skip(n0 + 32 * i)) read(n0 + 32 * i, held[i]);
+                release();
+            }
+            auto finish = [&](int c0, float (&v)[32]) {
                 if (use_beta) {
+                    if (c0 > n0) fetch(c0);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) *cell(4 * i + sr, sc) = pre[i];
                     __syncwarp();
@@ -473,13 +512,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                 }
                 if (!diagonal && whole && (p.t.re || p.t.m.base)) store_transposed(p.t, q, planes, row, c0, lane, v);
                 __syncwarp();
-            }
-            if (!ok) break;
-            fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if (CG == 2) mbar_arrive_cluster(lead ? smem_u32(&tempty[b]) : peer_addr(&tempty[b], 0));
-                else mbar_arrive(&tempty[b]);
+            };
+            if (L::HELD > 1) {
+#pragma unroll
+                for (int i = 0; i < L::HELD; ++i)
+                    if (!skip(n0 + 32 * i)) finish(n0 + 32 * i, held[i]);
+            } else {
+#pragma unroll 1
+                for (int c0 = n0; c0 < n0 + BNC; c0 += 32) {
+                    if (skip(c0)) continue;
+                    read(c0, held[0]);
+                    finish(c0, held[0]);
+                }
+                release();
             }
         }
     }
@@ -639,21 +684,15 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
         const long long mt = (M + BM - 1) / BM, nt = (N + 31) / 32;
         if ((sym ? 2 * mt * (mt + 1) : mt * nt) * nprob <= sms) kind = 0;
     }
-    switch (kind + (cross ? 3 : 0)) {
-        case 0: return launch_cg<1, 32, 4, 0, P>(c, nprob, pb, args, M, N, K, sms, s);
-        case 1: return launch_cg<1, 64, 4, 0, P>(c, nprob, pb, args, M, N, K, sms, s);
-        case 2: return launch_cg<2, 128, 4, 0, P>(c, nprob, pb, args, M, N, K, pairs, s);
-        case 3: return launch_cg<1, 32, 4, 1, P>(c, nprob, pb, args, M, N, K, sms, s);
-        case 4: return launch_cg<1, 64, 4, 1, P>(c, nprob, pb, args, M, N, K, sms, s);
-        default: return launch_cg<2, 128, 4, 1, P>(c, nprob, pb, args, M, N, K, pairs, s);
-    }
+    if (kind == 0) return launch_cg<1, 32, 4, 1, P>(c, nprob, pb, args, M, N, K, sms, s);
+    if (kind == 1) return launch_cg<1, 64, 4, 1, P>(c, nprob, pb, args, M, N, K, sms, s);
+    return cross ? launch_cg<2, 128, 4, 1, P>(c, nprob, pb, args, M, N, K, pairs, s)
+                 : launch_cg<2, 128, 4, 0, P>(c, nprob, pb, args, M, N, K, pairs, s);
 }
 
 }  // namespace
 
 void cgemm_init_attrs() {
-    set_attr<1, 32, 4, 0>();
-    set_attr<1, 64, 4, 0>();
     set_attr<2, 128, 4, 0>();
     set_attr<1, 32, 4, 1>();
     set_attr<1, 64, 4, 1>();
