@@ -74,7 +74,7 @@ struct CgArgs {
 // [rr | ri | ir | ii] (one CTA; MERGED: [rr | ri] and [ir | ii] of both groups side by
 // side) or [re | im] (pair), a set one group or, with CROSS, two; two sets where
 // they fit, so that the epilogue of a tile overlaps the products of the next, else
-// the one-CTA epilogue reads the whole set before its stores (HELD).
+// the epilogue reads the whole set before its stores (HELD).
 template <int CG, int BNC, int NQ, int CROSS>
 struct CgLayout {
     static constexpr int STAGES = NQ == 4 ? 2 : 4;
@@ -89,7 +89,7 @@ struct CgLayout {
     static constexpr int ACC = (CROSS ? 2 : 1) * GROUP;
     static constexpr int SETS = 2 * ACC <= 512 ? 2 : 1;
     static constexpr bool MERGED = CG == 1 && NQ == 4 && 4 * BNC <= 128;
-    static constexpr int HELD = SETS == 1 && BNC <= 64 ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
+    static constexpr int HELD = SETS == 1 ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
     // offset of the accumulator of component q's first (x r..) or second (x i..) half in group g
     static constexpr int acc(int g, int i, int r) { return MERGED ? (4 * i + 2 * g + r) * BNC : g * GROUP + (2 * i + r) * BNC; }
     static constexpr int TMEM = SETS * ACC;
@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             const int row0 = m0 + (int)rank * BM + 32 * q4, row = row0 + lane;
             const float *in = q ? p.in_im : p.in_re;
             float *const o32 = q ? p.o.im : p.o.re;
-            // the beta input of a block is fetched before the accumulator is waited for
+            // the first block's beta input is fetched before the accumulator is waited for
+            // (a single set: after it has been read, beside the next tile's products)
             float4 pre[8];
             auto fetch = [&](int c0) {
 #pragma unroll
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     else mbar_arrive(&tempty[b]);
                 }
             };
-            if (!skip(n0) && use_beta) fetch(n0);
+            if (L::HELD == 1 && use_beta && !skip(n0)) fetch(n0);
             if (!mbar_wait(&tfull[b], u & 1, abort_flag)) { ok = false; break; }
             __syncwarp();
             fence_after();
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             }
             auto finish = [&](int c0, float (&v)[32]) {
                 if (use_beta) {
-                    if (c0 > n0) fetch(c0);
+                    if (L::HELD > 1 || c0 > n0) fetch(c0);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) *cell(4 * i + sr, sc) = pre[i];
                     __syncwarp();
