@@ -360,30 +360,36 @@ __device__ void leaf_gj_regs2(float *re, float *im, long long ld, int *flags) {
 }
 
 // ---------------------------------------------------------------------------
-// Inverse of a 128 x 128 float32 block by a cluster of four CTAs (one per block,
-// 512 threads each): block Gauss-Jordan elimination in place over four 32-column
+// Inverse of a 128 x 128 (64 x 64) float32 block by a cluster of NP = four (two)
+// CTAs of 512 threads: block Gauss-Jordan elimination in place over NP 32-column
 // panels, CTA q holding the panel of columns 32 q .. 32 q + 31 in shared memory.
 // Step p, with panel p as it stands (F) and the inverse P^-1 of its 32 x 32 pivot
 // block in every CTA: R = P^-1 A_p, A_i -= F_i R, A_p = R (on panel p itself:
 // P^-1 and -F_i P^-1).
 // These blocks sit one after the other on the critical path of every inversion,
-// so what counts is latency, and the chain of 4 x 32 pivots bounds it.  Four
+// so what counts is latency, and the chain of 32 NP pivots bounds it.  Four
 // warps of the next panel's CTA invert its pivot block and store the inverse to the
-// four CTAs (distributed shared memory) while the other three copy the panel.
+// others (distributed shared memory) while these copy the panel.
 // Updating the next pivot block alone first, and the rest beside its inversion,
 // is no faster: the inversion then takes twice as long (it shares the SM's issue slots).
-// Measured: 36 us per block; 60 us with every CTA inverting the pivot block (400 clocks
-// a pivot) after copying the panel, 93 us in one CTA.
+// Measured: 36 us per 128 block; 60 us with every CTA inverting the pivot block (400 clocks
+// a pivot) after copying the panel, 93 us in one CTA.  64 block: 20 us; 56 us by pivots
+// over all rows in one CTA.
 // ---------------------------------------------------------------------------
 namespace lc {
 constexpr int NT = 512, PT = 34;  // threads, row pitch (float2; rows 16-byte aligned, columns conflict-free)
 
-struct Smem {
-    float2 own[128 * PT], F[128 * PT], inv[32 * PT], R[32 * PT];
+struct Leaf {  // of the 32 x 32 inversion
     float2 g[32 * 32], scale[32];
-    float2 v[128], wpart[16][32], w[32], zpart[4][4][128];
-    float part[4];
     int piv[32];
+};
+template <int NP>
+struct Smem {
+    static constexpr int N = 32 * NP, GROUPS = NT / N;  // rows and columns; threads per column
+    float2 own[N * PT], F[N * PT], inv[32 * PT], R[32 * PT];
+    float2 v[N], wpart[16][32], w[32], zpart[NP][GROUPS][N];
+    float part[NP];
+    Leaf leaf;
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -396,11 +402,11 @@ __device__ __forceinline__ T *peer(T *p, int rank) {
     asm volatile("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"((uint64_t)p), "r"(rank));
     return reinterpret_cast<T *>(a);
 }
-// Store to the same place in all four CTAs.
-template <typename T>
+// Store to the same place in all CTAs of the cluster.
+template <int NP, typename T>
 __device__ __forceinline__ void store_all(T *p, T v) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) *peer(p, q) = v;
+    for (int q = 0; q < NP; ++q) *peer(p, q) = v;
 }
 
 // Pivoted Gauss-Jordan inverse of the 32 x 32 block `a` (pitch PT) into `out`, by
@@ -417,7 +423,7 @@ __device__ __forceinline__ void store_all(T *p, T v) {
 // infinities or NaN, which the caller's check of the result finds.
 // Measured: 195 clocks per pivot; 400 with a barrier of all four warps and the
 // pivot row through shared memory.
-static __device__ void leaf32(Smem &sm, const float2 *a, float2 *out) {
+static __device__ void leaf32(Leaf &sm, const float2 *a, float2 *out) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float2 x[8];
 #pragma unroll
@@ -509,20 +515,21 @@ static __device__ void leaf32(Smem &sm, const float2 *a, float2 *out) {
 // The inverse of the block at (re, im), in place; each CTA passes its panel
 // (sm.own) to `also` as well.  Returns (the same in every thread of the cluster)
 // whether the result passed the check below; if not, the block is as it was.
-template <typename Also>
-static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, int rank, Also also) {
+template <int NP, typename Also>
+static __device__ bool invert(Smem<NP> &sm, float *re, float *im, long long ld, int rank, Also also) {
+    constexpr int N = Smem<NP>::N, GROUPS = Smem<NP>::GROUPS, NI = 32 / GROUPS;
     const int t = threadIdx.x;
     cluster_arrive();
     {
-        float2 x[8], f[8];
+        float2 x[2 * NP], f[2 * NP];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 2 * NP; ++i) {
             const long long g = (long long)((t >> 5) + 16 * i) * ld + (t & 31);
             f[i] = make_float2(re[g], im[g]);
             x[i] = make_float2(re[g + 32 * rank], im[g + 32 * rank]);
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 2 * NP; ++i) {
             const int e = ((t >> 5) + 16 * i) * PT + (t & 31);
             sm.F[e] = f[i];
             sm.own[e] = x[i];
@@ -530,24 +537,25 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
     }
     __syncthreads();
     if (t < 128) {
-        leaf32(sm, sm.F, sm.inv);
-    } else if (t < 256) {
+        leaf32(sm.leaf, sm.F, sm.inv);
+    } else if (t < 128 + N) {
         float sn, cs;
         sincosf(2.3999632f * (float)(t - 128), &sn, &cs);
         sm.v[t - 128] = make_float2(cs, sn);
     }
-    // this thread's share of the original block, for the check: a column, eight rows
-    float *const ore = re + (32 * rank + 8 * (t >> 7)) * ld + (t & 127), *const oim = im + (ore - re);
-    float xr[8], xi[8];
+    // this thread's share of the original block, for the check: a column, NI rows
+    const int grp = t / N, col = t % N;
+    float *const ore = re + (32 * rank + NI * grp) * ld + col, *const oim = im + (ore - re);
+    float xr[NI], xi[NI];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < NI; ++i) {
         xr[i] = ore[i * ld];
         xi[i] = oim[i * ld];
     }
     __syncthreads();
     cluster_wait();  // every CTA has started: its shared memory can be written
     const int cp = 2 * (t & 15), row = t >> 4;  // this thread's column pair and row of each block
-    for (int p = 0; p < 4; ++p) {
+    for (int p = 0; p < NP; ++p) {
         const float2 *F = rank == p ? sm.own : sm.F;  // rows are read and written by the same half warp
         // R = P^-1 A_p (the panel's own columns: R = P^-1)
         float2 a0 = sm.inv[row * PT + cp], a1 = sm.inv[row * PT + cp + 1];
@@ -570,11 +578,11 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
         }
         *reinterpret_cast<float4 *>(sm.R + row * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
         __syncthreads();
-        // A_i -= F_i R for the other three row blocks
-        float2 acc[3][2];
-        int ri[3];
+        // A_i -= F_i R for the other row blocks
+        float2 acc[NP - 1][2];
+        int ri[NP - 1];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < NP - 1; ++i) {
             ri[i] = 32 * (i < p ? i : i + 1) + row;
             float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
             if (rank != p) o = *reinterpret_cast<const float4 *>(sm.own + ri[i] * PT + cp);
@@ -586,7 +594,7 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
             const float4 u = *reinterpret_cast<const float4 *>(sm.R + k * PT + cp);
             const float4 w = *reinterpret_cast<const float4 *>(sm.R + (k + 1) * PT + cp);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
+            for (int i = 0; i < NP - 1; ++i) {
                 const float4 q = *reinterpret_cast<const float4 *>(F + ri[i] * PT + k);
                 float2 &c0 = acc[i][0], &c1 = acc[i][1];
                 c0.x = fmaf(-q.x, u.x, fmaf(q.y, u.y, c0.x));
@@ -601,16 +609,16 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
         }
         __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < NP - 1; ++i)
             *reinterpret_cast<float4 *>(sm.own + ri[i] * PT + cp) =
                 make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
         *reinterpret_cast<float4 *>(sm.own + (32 * p + row) * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
-        if (p == 3) break;
+        if (p == NP - 1) break;
         cluster_arrive();
         if (rank == p + 1) {
             __syncthreads();
             if (t < 128) {
-                leaf32(sm, sm.own + 32 * (p + 1) * PT, sm.inv);
+                leaf32(sm.leaf, sm.own + 32 * (p + 1) * PT, sm.inv);
                 asm volatile("bar.sync 9, 128;" ::: "memory");
                 cluster_wait();
 #pragma unroll
@@ -618,7 +626,7 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
                     float2 *e = sm.inv + (8 * i + (t >> 4)) * PT + cp;
                     const float4 v = *reinterpret_cast<const float4 *>(e);
 #pragma unroll
-                    for (int q = 1; q < 4; ++q) *reinterpret_cast<float4 *>(peer(e, (rank + q) & 3)) = v;
+                    for (int q = 1; q < NP; ++q) *reinterpret_cast<float4 *>(peer(e, (rank + q) % NP)) = v;
                 }
             } else {
                 cluster_wait();
@@ -626,14 +634,14 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
         } else {
             cluster_wait();  // panel p + 1 is up to date
             const float2 *src = peer(sm.own, p + 1);
-            float4 f[3];
+            float4 f[NP - 1];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
+            for (int i = 0; i < NP - 1; ++i) {
                 const int r = 32 * (i < p + 1 ? i : i + 1) + row;
                 f[i] = *reinterpret_cast<const float4 *>(src + r * PT + cp);
             }
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
+            for (int i = 0; i < NP - 1; ++i) {
                 const int r = 32 * (i < p + 1 ? i : i + 1) + row;
                 *reinterpret_cast<float4 *>(sm.F + r * PT + cp) = f[i];
             }
@@ -642,7 +650,7 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
         cluster_wait();
     }
     __syncthreads();
-    for (int e = t; e < 128 * 16; e += NT) {
+    for (int e = t; e < N * 16; e += NT) {
         const int r = e >> 4, c = 2 * (e & 15);
         const float2 u = sm.own[r * PT + c], v = sm.own[r * PT + c + 1];
         const long long g = r * ld + 32 * rank + c;
@@ -655,12 +663,12 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
     // elimination; apply the computed inverse to a fixed unit-modulus probe v and
     // compare (v^T X^-1) X with v^T.  Above 2e-5 relative residual (a sound block
     // gives a few 1e-7) the block is inverted again by Gauss-Jordan with pivoting
-    // over all 128 rows.
+    // over all rows.
     {
         const int g = t >> 5, c = t & 31;
         float2 y = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int r = 8 * g; r < 8 * g + 8; ++r) {
+        for (int r = 2 * NP * g; r < 2 * NP * (g + 1); ++r) {
             const float2 m = sm.own[r * PT + c], v = sm.v[r];
             y.x += m.x * v.x - m.y * v.y;
             y.y += m.x * v.y + m.y * v.x;
@@ -681,21 +689,22 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
     {
         float2 z = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 y = sm.w[8 * (t >> 7) + i];
+        for (int i = 0; i < NI; ++i) {
+            const float2 y = sm.w[NI * grp + i];
             z.x += xr[i] * y.x - xi[i] * y.y;
             z.y += xr[i] * y.y + xi[i] * y.x;
         }
-        store_all(&sm.zpart[rank][t >> 7][t & 127], z);
+        store_all<NP>(&sm.zpart[rank][grp][col], z);
     }
     cluster_arrive();
     cluster_wait();  // the last access to another CTA's shared memory is done
-    if (t < 128) {
+    if (t < N) {
         float2 z = make_float2(-sm.v[t].x, -sm.v[t].y);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            z.x += sm.zpart[q >> 2][q & 3][t].x;
-            z.y += sm.zpart[q >> 2][q & 3][t].y;
+        for (int q = 0; q < NP * GROUPS; ++q) {
+            const float2 u = sm.zpart[q / GROUPS][q % GROUPS][t];
+            z.x += u.x;
+            z.y += u.y;
         }
         float e2 = z.x * z.x + z.y * z.y;
 #pragma unroll
@@ -703,9 +712,12 @@ static __device__ bool invert128(Smem &sm, float *re, float *im, long long ld, i
         if ((t & 31) == 0) sm.part[t >> 5] = e2;
     }
     __syncthreads();
-    if ((sm.part[0] + sm.part[1]) + (sm.part[2] + sm.part[3]) <= 4e-10f * 128.f) return true;  // (2e-5)^2 |v|^2; NaN fails
+    float e2 = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < NP; ++i) e2 += sm.part[i];
+    if (e2 <= 4e-10f * N) return true;  // (2e-5)^2 |v|^2; NaN fails
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
         ore[i * ld] = xr[i];
         oim[i * ld] = xi[i];
     }

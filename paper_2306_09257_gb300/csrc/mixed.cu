@@ -477,26 +477,28 @@ __global__ void __launch_bounds__(NB * 4) k_leaf32r(const __grid_constant__ Tab<
     leaf_gj_regs<NB>(re.v[b], im.v[b], ld, flags.v[b]);
 }
 
-// 128 x 128 diagonal blocks (one cluster of four CTAs each): the inverse in place
+// 128 x 128 and 64 x 64 diagonal blocks (NP = 4, 2; one cluster of NP CTAs each): the inverse in place
 // and in split form (XP.base null: float32 only).
-__global__ void __launch_bounds__(lc::NT) __cluster_dims__(4, 1, 1) k_leaf128(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
+template <int NP>
+__global__ void __launch_bounds__(lc::NT) __cluster_dims__(NP, 1, 1) k_leaf_cluster(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
     chain_enter();
     extern __shared__ __align__(16) unsigned char lc_smem[];
-    lc::Smem &sm = *reinterpret_cast<lc::Smem *>(lc_smem);
-    const int b = blockIdx.x >> 2, rank = blockIdx.x & 3;
+    constexpr int N = 32 * NP;
+    lc::Smem<NP> &sm = *reinterpret_cast<lc::Smem<NP> *>(lc_smem);
+    const int b = blockIdx.x / NP, rank = blockIdx.x % NP;
     float *re = ret.v[b], *im = imt.v[b];
     const Mirror m = XP.v[b];
-    const bool sound = lc::invert128(sm, re, im, ld, rank, [&](int r, int c, float2 u, float2 v) {
+    const bool sound = lc::invert<NP>(sm, re, im, ld, rank, [&](int r, int c, float2 u, float2 v) {
         if (m.base) store_split2(m, planes, r, c, u, v);
     });
     if (sound) return;
-    if (rank != 0) return;
+    if (rank != 0 || threadIdx.x >= 4 * N) return;
     if (threadIdx.x == 0) atomicAdd(flags.v[b] + 1, 1);  // fallback count (flags[1])
-    leaf_gj_regs<128>(re, im, ld, flags.v[b]);
+    leaf_gj_regs<N>(re, im, ld, flags.v[b]);
     if (!m.base) return;
     __syncthreads();  // the block's float32 stores are read back by other threads
-    for (int e = threadIdx.x; e < 128 * 64; e += lc::NT) {
-        const int r = e >> 6, c = 2 * (e & 63);
+    for (int e = threadIdx.x; e < N * N / 2; e += 4 * N) {
+        const int r = e / (N / 2), c = 2 * (e % (N / 2));
         const float2 a = *reinterpret_cast<const float2 *>(re + (long long)r * ld + c);
         const float2 d = *reinterpret_cast<const float2 *>(im + (long long)r * ld + c);
         store_split2(m, planes, r, c, make_float2(a.x, d.x), make_float2(a.y, d.y));
@@ -971,10 +973,15 @@ void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) 
     const long long ld = X[0].ld;
     const auto re = tab<float *>(bt, [&](int b) { return X[b].re; }), im = tab<float *>(bt, [&](int b) { return X[b].im; });
     const auto fl = tab<int *>(bt, [&](int b) { return bt.c[b]->d_flags; });
-    // 128 blocks: block elimination by a cluster of four CTAs (default); variants 1-3 are the single-level Gauss-Jordan kernels.
+    // 128 and 64: block elimination by a cluster (default); variants 1-3 are the single-level Gauss-Jordan kernels.
     if (n == 128 && v == 0) {
-        APF_CHAIN(c, k_leaf128, 4 * nb, lc::NT, (int)sizeof(lc::Smem), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
-                   w->nsplit_elim, fl);
+        APF_CHAIN(c, k_leaf_cluster<4>, 4 * nb, lc::NT, (int)sizeof(lc::Smem<4>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+                  w->nsplit_elim, fl);
+        return;
+    }
+    if (n == 64 && v == 0) {
+        APF_CHAIN(c, k_leaf_cluster<2>, 2 * nb, lc::NT, (int)sizeof(lc::Smem<2>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+                  w->nsplit_elim, fl);
         return;
     }
     if (n == 128 && v == 1) APF_LAUNCH(c, k_leaf32r2<128>, nb, 512, 0, s, re, im, ld, fl);
@@ -1327,7 +1334,8 @@ void mixed_init_attrs() {
     cudaFuncSetAttribute(k_leaf_inv32, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * (int)sizeof(float2));
     cudaFuncSetAttribute(k_leaf32<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<128>(8));
     cudaFuncSetAttribute(k_leaf32<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<64>(8));
-    cudaFuncSetAttribute(k_leaf128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem));
+    cudaFuncSetAttribute(k_leaf_cluster<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem<4>));
+    cudaFuncSetAttribute(k_leaf_cluster<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem<2>));
     cudaFuncSetAttribute(k_circ_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * (int)sizeof(double2));
 }
 
