@@ -372,8 +372,8 @@ __device__ void leaf_gj_regs2(float *re, float *im, long long ld, int *flags) {
 // others (distributed shared memory) while these copy the panel.
 // Updating the next pivot block alone first, and the rest beside its inversion,
 // is no faster: the inversion then takes twice as long (it shares the SM's issue slots).
-// Measured: 36 us per 128 block; 60 us with every CTA inverting the pivot block (400 clocks
-// a pivot) after copying the panel, 93 us in one CTA.  64 block: 20 us; 56 us by pivots
+// Measured: 34 us per 128 block; 60 us with every CTA inverting the pivot block (400 clocks
+// a pivot) after copying the panel, 93 us in one CTA.  64 block: 18 us; 56 us by pivots
 // over all rows in one CTA.
 // ---------------------------------------------------------------------------
 namespace lc {
@@ -512,6 +512,39 @@ static __device__ void leaf32(Leaf &sm, const float2 *a, float2 *out) {
         out[mystep * PT + sm.piv[8 * w + j]] = make_float2(x[j].x * q.x - x[j].y * q.y, x[j].x * q.y + x[j].y * q.x);
 }
 
+// acc += S f u over 32 k: NR rows f (32 contiguous elements each) times the columns
+// 0, 1, 16, 17 of u (pitch PT).  Shared memory hands out 128 bytes per clock,
+// broadcasts included, so the tile counts: with two rows and four columns per
+// thread R takes 1.9k clocks, 2.7k with one row and two columns.  The update (three
+// rows, four columns) takes 4.8k, as with two columns; its multiply-adds alone are 3.1k.
+template <int S, int NR>
+__device__ __forceinline__ void multiply(float4 (&acc)[NR][2], const float2 *const (&f)[NR], const float2 *u) {
+#pragma unroll 4
+    for (int k = 0; k < 32; k += 2) {
+        float4 q[NR];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            q[i] = *reinterpret_cast<const float4 *>(f[i] + k);
+            if (S < 0) q[i] = make_float4(-q[i].x, -q[i].y, -q[i].z, -q[i].w);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float4 w = *reinterpret_cast<const float4 *>(u + (k + kk) * PT + 16 * j);
+#pragma unroll
+                for (int i = 0; i < NR; ++i) {
+                    const float qx = kk ? q[i].z : q[i].x, qy = kk ? q[i].w : q[i].y;
+                    float4 &c = acc[i][j];
+                    c.x = fmaf(qx, w.x, fmaf(-qy, w.y, c.x));
+                    c.y = fmaf(qx, w.y, fmaf(qy, w.x, c.y));
+                    c.z = fmaf(qx, w.z, fmaf(-qy, w.w, c.z));
+                    c.w = fmaf(qx, w.w, fmaf(qy, w.z, c.w));
+                }
+            }
+    }
+}
+
 // The inverse of the block at (re, im), in place; each CTA passes its panel
 // (sm.own) to `also` as well.  Returns (the same in every thread of the cluster)
 // whether the result passed the check below; if not, the block is as it was.
@@ -554,65 +587,57 @@ static __device__ bool invert(Smem<NP> &sm, float *re, float *im, long long ld, 
     }
     __syncthreads();
     cluster_wait();  // every CTA has started: its shared memory can be written
-    const int cp = 2 * (t & 15), row = t >> 4;  // this thread's column pair and row of each block
+    const int cp = 2 * (t & 15), row = t >> 4;  // this thread's share of a copy: column pair, row of each block
+    const int tc = 2 * (t & 7), tr = t >> 3;    // and of a product: columns tc, tc + 1, tc + 16, tc + 17, row
     for (int p = 0; p < NP; ++p) {
-        const float2 *F = rank == p ? sm.own : sm.F;  // rows are read and written by the same half warp
-        // R = P^-1 A_p (the panel's own columns: R = P^-1)
-        float2 a0 = sm.inv[row * PT + cp], a1 = sm.inv[row * PT + cp + 1];
-        if (rank != p) {
-            a0 = a1 = make_float2(0.f, 0.f);
-#pragma unroll 8
-            for (int k = 0; k < 32; k += 2) {
-                const float4 q = *reinterpret_cast<const float4 *>(sm.inv + row * PT + k);
-                const float4 u = *reinterpret_cast<const float4 *>(sm.own + (32 * p + k) * PT + cp);
-                const float4 w = *reinterpret_cast<const float4 *>(sm.own + (32 * p + k + 1) * PT + cp);
-                a0.x = fmaf(q.x, u.x, fmaf(-q.y, u.y, a0.x));
-                a0.y = fmaf(q.x, u.y, fmaf(q.y, u.x, a0.y));
-                a1.x = fmaf(q.x, u.z, fmaf(-q.y, u.w, a1.x));
-                a1.y = fmaf(q.x, u.w, fmaf(q.y, u.z, a1.y));
-                a0.x = fmaf(q.z, w.x, fmaf(-q.w, w.y, a0.x));
-                a0.y = fmaf(q.z, w.y, fmaf(q.w, w.x, a0.y));
-                a1.x = fmaf(q.z, w.z, fmaf(-q.w, w.w, a1.x));
-                a1.y = fmaf(q.z, w.w, fmaf(q.w, w.z, a1.y));
+        // R = P^-1 A_p (the panel's own columns: R = P^-1), two rows and four columns per thread
+        float4 r[2][2];
+        if (t < 128) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    r[i][j] = rank == p ? *reinterpret_cast<const float4 *>(sm.inv + (tr + 16 * i) * PT + tc + 16 * j)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (rank != p) {
+                const float2 *const f[2] = {sm.inv + tr * PT, sm.inv + (tr + 16) * PT};
+                multiply<1>(r, f, sm.own + 32 * p * PT + tc);
             }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) *reinterpret_cast<float4 *>(sm.R + (tr + 16 * i) * PT + tc + 16 * j) = r[i][j];
         }
-        *reinterpret_cast<float4 *>(sm.R + row * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
         __syncthreads();
-        // A_i -= F_i R for the other row blocks
-        float2 acc[NP - 1][2];
-        int ri[NP - 1];
+        // A_i -= F_i R for the other row blocks, four columns of one row of each per thread.
+        // On panel p F is the panel itself: its rows are read and written by the same lanes.
+        if (t < 256) {
+            float4 acc[NP - 1][2];
 #pragma unroll
-        for (int i = 0; i < NP - 1; ++i) {
-            ri[i] = 32 * (i < p ? i : i + 1) + row;
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (rank != p) o = *reinterpret_cast<const float4 *>(sm.own + ri[i] * PT + cp);
-            acc[i][0] = make_float2(o.x, o.y);
-            acc[i][1] = make_float2(o.z, o.w);
+            for (int i = 0; i < NP - 1; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    acc[i][j] = rank == p ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                          : *reinterpret_cast<const float4 *>(sm.own + (32 * (i < p ? i : i + 1) + tr) * PT + tc + 16 * j);
+            const float2 *F = rank == p ? sm.own : sm.F;
+            const float2 *f[NP - 1];
+#pragma unroll
+            for (int i = 0; i < NP - 1; ++i) f[i] = F + (32 * (i < p ? i : i + 1) + tr) * PT;
+            multiply<-1>(acc, f, sm.R + tc);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NP - 1; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    *reinterpret_cast<float4 *>(sm.own + (32 * (i < p ? i : i + 1) + tr) * PT + tc + 16 * j) = acc[i][j];
         }
-#pragma unroll 4
-        for (int k = 0; k < 32; k += 2) {
-            const float4 u = *reinterpret_cast<const float4 *>(sm.R + k * PT + cp);
-            const float4 w = *reinterpret_cast<const float4 *>(sm.R + (k + 1) * PT + cp);
+        if (t < 128) {
 #pragma unroll
-            for (int i = 0; i < NP - 1; ++i) {
-                const float4 q = *reinterpret_cast<const float4 *>(F + ri[i] * PT + k);
-                float2 &c0 = acc[i][0], &c1 = acc[i][1];
-                c0.x = fmaf(-q.x, u.x, fmaf(q.y, u.y, c0.x));
-                c0.y = fmaf(-q.x, u.y, fmaf(-q.y, u.x, c0.y));
-                c1.x = fmaf(-q.x, u.z, fmaf(q.y, u.w, c1.x));
-                c1.y = fmaf(-q.x, u.w, fmaf(-q.y, u.z, c1.y));
-                c0.x = fmaf(-q.z, w.x, fmaf(q.w, w.y, c0.x));
-                c0.y = fmaf(-q.z, w.y, fmaf(-q.w, w.x, c0.y));
-                c1.x = fmaf(-q.z, w.z, fmaf(q.w, w.w, c1.x));
-                c1.y = fmaf(-q.z, w.w, fmaf(-q.w, w.z, c1.y));
-            }
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    *reinterpret_cast<float4 *>(sm.own + (32 * p + tr + 16 * i) * PT + tc + 16 * j) = r[i][j];
         }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < NP - 1; ++i)
-            *reinterpret_cast<float4 *>(sm.own + ri[i] * PT + cp) =
-                make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-        *reinterpret_cast<float4 *>(sm.own + (32 * p + row) * PT + cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
         if (p == NP - 1) break;
         cluster_arrive();
         if (rank == p + 1) {
