@@ -47,7 +47,7 @@ template <int P>
 struct CgArgs {
     CUtensorMap a[P], b[P];
     CgParams p[P];
-    int nprob, N, Mt, Nt, ntl, kblocks, nseg, planes, sym, vec;
+    int nprob, N, Mt, Nt, ntl, kblocks, nseg, planes, sym, vec, t_block;
     uint32_t seg_pairs;
     float alpha, beta;
 };
@@ -128,9 +128,9 @@ __device__ __forceinline__ void store_split(const Mirror &m, int q, int planes, 
 }
 
 // Component q (0 re, 1 im) of a 32 x 32 block whose row `row` this lane holds, to
-// the transposed output: neighbouring lanes exchange halves, so that a store covers
+// the transposed output (t32: its float32 plane or null): neighbouring lanes exchange halves, so that a store covers
 // two columns of 32 rows.
-__device__ __forceinline__ void store_transposed(const CgOut &t, int q, int planes, int row, int c0, int lane,
+__device__ __forceinline__ void store_transposed(const CgOut &t, float *t32, int q, int planes, int row, int c0, int lane,
                                                  float (&v)[32]) {
     const bool odd = lane & 1;
     const long long col = c0 + (odd ? 16 : 0);
@@ -141,7 +141,7 @@ __device__ __forceinline__ void store_transposed(const CgOut &t, int q, int plan
         if (odd) v[i] = got;
         else v[i + 16] = got;
     }
-    if (float *d = q ? t.im : t.re) {
+    if (float *d = t32) {
         d += col * t.ld + r0;
 #pragma unroll
         for (int i = 0; i < 16; ++i, d += t.ld) *reinterpret_cast<float2 *>(d) = make_float2(v[i], v[i + 16]);
@@ -474,6 +474,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     __syncwarp();
                 }
                 const bool diagonal = args.sym && c0 == row0;
+                float *const t32 = !args.t_block || c0 / args.t_block == row0 / args.t_block ? (q ? p.t.im : p.t.re) : nullptr;
                 const bool cols = vec && c0 + 31 < args.N, whole = cols && row0 + 31 < p.M;
                 if (o32 || p.o.m.base || !whole) {
 #pragma unroll
@@ -505,13 +506,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                                 if (p.o.m.base) store_split(p.o.m, q, planes, row, col, x);
                             }
                             if (diagonal) continue;
-                            float *t32 = q ? p.t.im : p.t.re;
                             if (t32) t32[(long long)col * p.t.ld + row] = x;
                             if (p.t.m.base) store_split(p.t.m, q, planes, col, row, x);
                         }
                     }
                 }
-                if (!diagonal && whole && (p.t.re || p.t.m.base)) store_transposed(p.t, q, planes, row, c0, lane, v);
+                if (!diagonal && whole && (t32 || p.t.m.base)) store_transposed(p.t, t32, q, planes, row, c0, lane, v);
                 __syncwarp();
             };
             if (L::HELD > 1) {
@@ -656,6 +656,7 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
     args.alpha = alpha;
     args.beta = beta;
     args.sym = sym ? 1 : 0;
+    args.t_block = pb[0].t_block;
     bool vec = N % 16 == 0;
     for (int i = 0; i < nprob; ++i) {
         const CgProblem &q = pb[i];

@@ -32,11 +32,13 @@ struct CgProblem {
     const float *in_re = nullptr, *in_im = nullptr;
     long long ldi = 0;
     int *flags = nullptr;
+    int t_block = 0;  // != 0 (the same for all problems): outT in float32 only inside diagonal blocks of this size
 };
 
 // nprob products of the same N, K (and at most M rows) in one launch.  sym: the
-// result is symmetric (M = N, out and outT the same matrix): only elements on
-// and below the diagonal are computed, each written to both places.  cross: the
+// result is symmetric (M = N, out and outT the same matrix, or outT without what
+// nobody reads above the diagonal): only elements on and below the diagonal are
+// computed, each written to both places; 32 x 32 diagonal blocks come out whole.  cross: the
 // smaller sums of a long product in accumulators of their own (see cgemm.cu).
 // rows: the row count by which the kernel form is chosen (0: M).
 int cgemm_n(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int N, int K, float alpha, float beta,

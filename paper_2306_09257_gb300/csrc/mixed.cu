@@ -1000,12 +1000,15 @@ void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) 
 //   [A B; C D]^-1 = [Ai + T^T V, -V^T; -V, Si],  T = C Ai, S = D - T C^T, V = Si T,
 // with all four products on the tensor cores, two of them symmetric.  X holds the
 // block in float32 (on and below its diagonal blocks) and XP the split form of
-// what lies below them; both come out as the whole inverse.  Every product reads
-// split operands where the previous steps' epilogues left them (T only exists
-// split, as T and T^T; V is written as -V to C and, transposed, to B, and read
-// back from B as the operand of T^T V), so nothing runs between the products.
-// toff: offset of this level's T in the T buffers.
-int inv32_b(const Bat &bt, const PV *X, const Mirror *XP, int n, bool want_mirror, long long toff, cudaStream_t s) {
+// what lies below them; they come out as the whole inverse, XP with want_mirror
+// only.  Every product reads split operands where the previous steps' epilogues
+// left them (T only exists split, as T and T^T; V is written as -V to C and,
+// transposed, to B, and read back from B as the operand of T^T V), so nothing
+// runs between the products.
+// toff: offset of this level's T in the T buffers.  upper: the result is wanted in
+// float32 above the diagonal (outside its leaves) too, which nothing inside the recursion
+// reads: an SM stores 32 bytes per clock, and half of a product's time can be stores.
+int inv32_b(const Bat &bt, const PV *X, const Mirror *XP, int n, bool want_mirror, long long toff, cudaStream_t s, bool upper = true) {
     apf_ctx *c = bt.lead();
     MixedWork *w = c->mw;
     const int nb = bt.n, planes = w->nsplit_elim;
@@ -1026,8 +1029,9 @@ int inv32_b(const Bat &bt, const PV *X, const Mirror *XP, int n, bool want_mirro
     }
     auto out = [](const PV &v, const Mirror &m) { return CgOut{v.re, v.im, v.ld, m}; };
     CgProblem pb[CG_MAX_PROB];
+    const Mirror none[CG_MAX_PROB];
     auto product = [&](const Mirror *P, const Mirror *Q, float alpha, const PV *in, const PV *o, const Mirror *om,
-                       const PV *ot, const Mirror *otm, bool sym) {
+                       const PV *ot, const Mirror *otm, bool sym, int t_block = 0) {
         for (int b = 0; b < nb; ++b) {
             pb[b] = CgProblem{};
             pb[b].A = P[b];
@@ -1041,20 +1045,23 @@ int inv32_b(const Bat &bt, const PV *X, const Mirror *XP, int n, bool want_mirro
                 pb[b].ldi = in[b].ld;
             }
             pb[b].flags = bt.c[b]->d_flags;
+            pb[b].t_block = t_block;
         }
         return cgemm_n(c, nb, pb, planes, h, h, h, alpha, in ? 1.f : 0.f, sym, false, s);
     };
     int rc;
-    if ((rc = inv32_b(bt, A, mA, h, true, sub, s))) return rc;
+    if ((rc = inv32_b(bt, A, mA, h, true, sub, s, false))) return rc;
     // T = C Ai (Ai symmetric: its rows are its columns)
     if ((rc = product(mC, mA, 1.f, nullptr, nullptr, mT, nullptr, mTT, false))) return rc;
-    // D = D - T C^T
-    if ((rc = product(mT, mC, -1.f, D, D, mD, D, mD, true))) return rc;
-    if ((rc = inv32_b(bt, D, mD, h, true, sub, s))) return rc;
+    // D = D - T C^T, as the inversion of D reads it
+    const bool deep = h > leaf_size(w);
+    if ((rc = product(mT, mC, -1.f, D, D, deep ? mD : none, D, none, true, leaf_size(w)))) return rc;
+    if ((rc = inv32_b(bt, D, mD, h, true, sub, s, upper))) return rc;
     // C = -Si T, B = its transpose
-    if ((rc = product(mD, mTT, -1.f, nullptr, C, mC, B, mB, false))) return rc;
+    if ((rc = product(mD, mTT, -1.f, nullptr, C, want_mirror ? mC : none, upper ? B : nullptr, mB, false))) return rc;
     // A = Ai + V^T T = Ai - B T
-    return product(mB, mTT, -1.f, A, A, mA, A, mA, true);
+    const Mirror *const sA = want_mirror ? mA : none;
+    return product(mB, mTT, -1.f, A, A, sA, upper ? A : nullptr, sA, true);
 }
 
 // The G_j of a context in split form: slot j, or with recomputation the slot of j's position.
