@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                         for (int i = 0; i < 8; ++i) x[i] = *cell(4 * i + sr, sc);
                         store_rows(p.o, q, planes, row0 + sr, p.M, c0 + 4 * sc, x);
                     }
-                    if (!whole && row < p.M) {  // ragged edges
+                    if (!whole && row < p.M && (!cols || t32 || p.t.m.base)) {  // ragged edges
 #pragma unroll 1
                         for (int i = 0; i < 32 && c0 + i < args.N; ++i) {
                             const int col = c0 + i;
