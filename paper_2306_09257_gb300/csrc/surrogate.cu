@@ -106,9 +106,10 @@ __global__ void __launch_bounds__(256) k_lift(const float *eps, const __nv_bfloa
 // scale_m = 1 (analysis) or the synthesis weights (1/n, 2/n) for the backward.
 // Block: 16 rows x 64 modes, x in chunks of 32; thread: 4 rows x 4 modes of every
 // fourth x, the four partial sums added in a fixed order.  Bound by the float32
-// pipe (32 multiply-adds per 6 shared-memory loads): 64 samples of 48 channels,
-// 1024 positions, 64 modes 212 -> 21 us (one thread per mode and quarter of
-// x, two loads per multiply-add pair, before).
+// pipe (32 multiply-adds per 6 shared-memory loads), and for few rows by latency: the
+// next chunk is loaded during this one's products.  64 samples of 48 channels,
+// 1024 positions, 64 modes 212 -> 20 us, 1 sample 15 -> 10 us (one thread per mode
+// and quarter of x, two loads per multiply-add pair, before).
 __global__ void __launch_bounds__(256) k_dft(const float *__restrict__ in, float2 *out, const float2 *__restrict__ tw,
                                              int rows, int n, int M, int synth_weights) {
     constexpr int XC = 32, RP = 17;
@@ -117,27 +118,40 @@ __global__ void __launch_bounds__(256) k_dft(const float *__restrict__ in, float
     const int tid = threadIdx.x, mg = tid & 15, ks = (tid >> 4) & 3, rg = tid >> 6;
     const int r0 = blockIdx.x * 16, m0 = blockIdx.y * 64, q = n >> 2;
     float re[4][4] = {}, im[4][4] = {};
-    for (int x0 = 0; x0 < q; x0 += XC) {
-        __syncthreads();
-        for (int e = tid; e < 16 * XC; e += 256) {
-            const int xx = e & (XC - 1), r = e / XC, x = x0 + xx;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 pf[2];  // the next chunk's loads, in flight during this one's products
+    float2 pw[8];
+    auto fetch = [&](int x0) {
+        const int x = x0 + (tid & (XC - 1));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int r = tid / XC + 8 * k;
+            pf[k] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (x < q && r0 + r < rows) {
                 const float *p = in + (long long)(r0 + r) * n;
-                const float a = p[x], bb = p[n / 2 - x];
-                const float c = x ? p[n / 2 + x] : 0.f, d = x ? p[n - x] : 0.f;
-                const float ad = a + d, bc = bb + c, am = a - d, bm = bb - c;
-                v = make_float4(ad + bc, ad - bc, am - bm, am + bm);  // cos even, cos odd, sin even, sin odd
+                pf[k] = make_float4(p[x], p[n / 2 - x], x ? p[n / 2 + x] : 0.f, x ? p[n - x] : 0.f);
             }
-            fold[xx * RP + r] = v;
         }
-        for (int e = tid; e < 64 * XC; e += 256) {
-            const int xx = e & (XC - 1), m = e / XC, x = x0 + xx;
-            float2 w = make_float2(0.f, 0.f);
-            if (x < q && m0 + m < M) w = tw[(long long)(m0 + m) * n + x];
-            float2 *d = reinterpret_cast<float2 *>((m & 2 ? tb : ta) + xx * RP + (m >> 2));
-            d[m & 1] = w;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int m = m0 + tid / XC + 8 * k;
+            pw[k] = x < q && m < M ? tw[(long long)m * n + x] : make_float2(0.f, 0.f);
         }
+    };
+    fetch(0);
+    for (int x0 = 0; x0 < q; x0 += XC) {
+        __syncthreads();
+        const int xx = tid & (XC - 1);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float ad = pf[k].x + pf[k].w, bc = pf[k].y + pf[k].z, am = pf[k].x - pf[k].w, bm = pf[k].y - pf[k].z;
+            fold[xx * RP + tid / XC + 8 * k] = make_float4(ad + bc, ad - bc, am - bm, am + bm);  // cos even, cos odd, sin even, sin odd
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int m = tid / XC + 8 * k;
+            reinterpret_cast<float2 *>((m & 2 ? tb : ta) + xx * RP + (m >> 2))[m & 1] = pw[k];
+        }
+        if (x0 + XC < q) fetch(x0 + XC);
         __syncthreads();
 #pragma unroll
         for (int xx = 0; xx < XC; xx += 4) {
@@ -189,51 +203,158 @@ __global__ void __launch_bounds__(256) k_dft(const float *__restrict__ in, float
 }
 
 // Y[b][o][m] = sum_i W[i][o][m] X[b][i][m], or its adjoint (BWD) dX[b][i][m] =
-// sum_o conj(W[i][o][m]) dY[b][o][m].  Thread: one mode, OT outputs, four samples,
-// so that a weight serves four samples and a spectrum value OT outputs; bound by
-// the latency of L2, so OT = 1 where two outputs per thread would leave too few
-// threads (64 samples of 48 channels: 20 us per call with one output and sample
-// per thread, 14 with OT = 2).
-template <bool BWD, int OT>
+// sum_o conj(W[i][o][m]) dY[b][o][m].  Thread: one mode, two outputs, four samples,
+// so that a weight serves four samples and a spectrum value two outputs; bound by
+// the latency of L2, so four i are loaded before the first use (128 samples of 48
+// channels, 64 modes: 15.5 us; 27 us as the compiler ordered the loads).
+template <bool BWD>
 __global__ void __launch_bounds__(256) k_mix(const float2 *__restrict__ X, const __nv_bfloat16 *__restrict__ pb, long long oWr,
                                              long long oWi, float2 *Y, int B, int C, int M) {
+    constexpr int OT = 2;
     const int idx = blockIdx.x * 256 + threadIdx.x, groups = (C + OT - 1) / OT;
     if (idx >= groups * M) return;
     const int m = idx % M, o0 = OT * (idx / M), b0 = 4 * blockIdx.y;
     const int nb = min(4, B - b0);
     const long long sb = (long long)C * M;
     const float2 *x = X + (long long)b0 * sb + m;
-    const __nv_bfloat16 *wrp[OT], *wip[OT];
+    const unsigned short *wrp[OT], *wip[OT];
 #pragma unroll
     for (int j = 0; j < OT; ++j) {
         const int o = min(o0 + j, C - 1);
         const long long w = (BWD ? (long long)o * C : (long long)o) * M + m;
-        wrp[j] = pb + oWr + w;
-        wip[j] = pb + oWi + w;
+        wrp[j] = reinterpret_cast<const unsigned short *>(pb) + oWr + w;
+        wip[j] = reinterpret_cast<const unsigned short *>(pb) + oWi + w;
     }
     const long long ws = BWD ? M : (long long)C * M;
     float2 y[OT][4] = {};
-#pragma unroll 4
-    for (int i = 0; i < C; ++i) {
-        float2 v[4];
+    constexpr int IC = 4;  // loads before their first use
+    for (int i0 = 0; i0 < C; i0 += IC) {
+        float2 v[IC][4];
+        unsigned r[IC][OT], q[IC][OT];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = x[(u < nb ? u : 0) * sb + (long long)i * M];
+        for (int k = 0; k < IC; ++k) {
+            const long long i = min(i0 + k, C - 1);
 #pragma unroll
-        for (int j = 0; j < OT; ++j) {
-            const float wr = __bfloat162float(wrp[j][i * ws]), wi = __bfloat162float(wip[j][i * ws]);
-            const float wim = BWD ? -wi : wi;
+            for (int u = 0; u < 4; ++u) v[k][u] = x[(u < nb ? u : 0) * sb + i * M];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                y[j][u].x = fmaf(wr, v[u].x, fmaf(-wim, v[u].y, y[j][u].x));
-                y[j][u].y = fmaf(wr, v[u].y, fmaf(wim, v[u].x, y[j][u].y));
+            for (int j = 0; j < OT; ++j) {
+                r[k][j] = wrp[j][i * ws];
+                q[k][j] = wip[j][i * ws];
             }
         }
+#pragma unroll
+        for (int k = 0; k < IC; ++k)
+#pragma unroll
+            for (int j = 0; j < OT; ++j) {
+                const float wr = i0 + k < C ? __uint_as_float(r[k][j] << 16) : 0.f, wi = i0 + k < C ? __uint_as_float(q[k][j] << 16) : 0.f;
+                const float wim = BWD ? -wi : wi;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    y[j][u].x = fmaf(wr, v[k][u].x, fmaf(-wim, v[k][u].y, y[j][u].x));
+                    y[j][u].y = fmaf(wr, v[k][u].y, fmaf(wim, v[k][u].x, y[j][u].y));
+                }
+            }
     }
 #pragma unroll
     for (int j = 0; j < OT; ++j)
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (u < nb && o0 + j < C) Y[(long long)(b0 + u) * sb + (long long)(o0 + j) * M + m] = y[j][u];
+}
+
+// The same, and k_synth below, for small calls, one output per thread: as many
+// threads as there are, each with a short chain of loads (SMALL_BATCH at a time
+// before their first use; the compiler's own unrolling waited for each).
+constexpr int SMALL_BATCH = 8;
+__host__ __device__ constexpr int small_pad(int k) { return (k + SMALL_BATCH - 1) / SMALL_BATCH * SMALL_BATCH; }
+template <bool BWD>
+__global__ void __launch_bounds__(128) k_mix_small(const float2 *__restrict__ X, const __nv_bfloat16 *__restrict__ pb, long long oWr,
+                                                   long long oWi, float2 *__restrict__ Y, int B, int C, int M) {
+    const int idx = blockIdx.x * 128 + threadIdx.x;
+    if (idx >= B * C * M) return;
+    const int m = idx % M, o = (idx / M) % C, b = idx / (M * C), ws = BWD ? M : C * M;
+    const float2 *x = X + (long long)b * C * M + m;
+    const unsigned short *w = reinterpret_cast<const unsigned short *>(pb) + (BWD ? (long long)o * C : (long long)o) * M + m;
+    const unsigned short *wr = w + oWr, *wi = w + oWi;
+    float yr = 0.f, yi = 0.f;
+    for (int i0 = 0; i0 < C; i0 += SMALL_BATCH) {
+        float2 v[SMALL_BATCH];
+        unsigned r[SMALL_BATCH], q[SMALL_BATCH];
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            const int i = min(i0 + k, C - 1);
+            v[k] = x[i * M];
+            r[k] = wr[i * ws];
+            q[k] = wi[i * ws];
+        }
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            const float a = i0 + k < C ? __uint_as_float(r[k] << 16) : 0.f, d = i0 + k < C ? __uint_as_float(q[k] << 16) : 0.f;
+            yr = fmaf(a, v[k].x, fmaf(BWD ? d : -d, v[k].y, yr));
+            yi = fmaf(a, v[k].y, fmaf(BWD ? -d : d, v[k].x, yi));
+        }
+    }
+    Y[idx] = make_float2(yr, yi);
+}
+
+// Block: 128 positions (blockIdx.x) of one channel of a sample (blockIdx.y).
+template <bool BWD>
+__global__ void __launch_bounds__(128) k_synth_small(const float2 *__restrict__ Y, const float *__restrict__ h, const __nv_bfloat16 *__restrict__ pb,
+                                                     long long oP, long long oc, const float2 *__restrict__ tw, float *z, float *hn, int C,
+                                                     int n, int M, int act) {
+    extern __shared__ __align__(16) unsigned char ss_smem[];
+    const int Mp = small_pad(M), Cp = small_pad(C);  // with zeros up to whole batches
+    float2 *ys = reinterpret_cast<float2 *>(ss_smem);  // [m]: w Y
+    float *ps = reinterpret_cast<float *>(ys + Mp);     // [i]
+    const int b = blockIdx.y / C, o = blockIdx.y - b * C, x = blockIdx.x * 128 + threadIdx.x;
+    const float *hb = h + (long long)b * C * n + x;
+    float2 w[SMALL_BATCH];  // one batch ahead
+    float v[SMALL_BATCH];
+    if (x < n) {
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            w[k] = tw[min(k, M - 1) * n + x];
+            v[k] = hb[min(k, C - 1) * n];
+        }
+    }
+    for (int m = threadIdx.x; m < Mp; m += 128) {
+        const float2 y = Y[(long long)blockIdx.y * M + min(m, M - 1)];
+        const float s = m >= M ? 0.f : BWD ? 1.f : (m == 0 ? 1.f : 2.f) / (float)n;
+        ys[m] = make_float2(s * y.x, s * y.y);
+    }
+    for (int i = threadIdx.x; i < Cp; i += 128) ps[i] = i < C ? bf(pb, oP + (BWD ? (long long)i * C + o : (long long)o * C + i)) : 0.f;
+    __syncthreads();
+    if (x >= n) return;
+    const long long at = (long long)blockIdx.y * n + x;
+    const float zv = BWD && z ? z[at] : 0.f;
+    float acc = 0.f;
+    for (int m0 = 0; m0 < M; m0 += SMALL_BATCH) {
+        float2 c[SMALL_BATCH];
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            c[k] = w[k];
+            if (m0 + SMALL_BATCH < M) w[k] = tw[min(m0 + SMALL_BATCH + k, M - 1) * n + x];
+        }
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) acc = fmaf(ys[m0 + k].x, c[k].x, fmaf(-ys[m0 + k].y, c[k].y, acc));
+    }
+    for (int i0 = 0; i0 < C; i0 += SMALL_BATCH) {
+        float c[SMALL_BATCH];
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            c[k] = v[k];
+            if (i0 + SMALL_BATCH < C) v[k] = hb[min(i0 + SMALL_BATCH + k, C - 1) * n];
+        }
+#pragma unroll
+        for (int k = 0; k < SMALL_BATCH; ++k) acc = fmaf(ps[i0 + k], c[k], acc);
+    }
+    if (BWD) {
+        hn[at] = z ? acc * gelu_d(zv) : acc;
+    } else {
+        acc += bf(pb, oc + o);
+        z[at] = acc;
+        hn[at] = act ? gelu(acc) : acc;
+    }
 }
 
 // v[b][o][x] = sum_m w_m Re(Y_om e^{i theta}) + sum_i P[o][i] h[b][i][x] (+ c[o]).
@@ -674,6 +795,13 @@ size_t synth_smem(int C, int XT) {
     return 16 * (SY_MC * Cp + SY_MC * XW + SY_IC * XW) + 4 * C * Cp;
 }
 
+// Outputs up to which one thread each is faster (k_synth_small, k_mix_small).  Whole
+// screening calls, one-output kernels against the tiled ones: 1 sample of 16 channels
+// and 128 positions 132 against 182 us; 20 of 24 and 512 (246k synthesised values) 178
+// against 260 us, 8 of 48 and 1024 (393k) 315 against 296 us.  Mixing alone: 20 of
+// 48 and 64 modes (61k values) 281 against 299 us per call, 64 of them (197k) 404
+// against 402 us.
+constexpr long long SMALL_SYNTH = 262144, SMALL_MIX = 131072;
 // x per block: 64 where that still gives about two blocks per SM, else 32.
 template <bool BWD, int XT>
 void launch_synth_t(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
@@ -686,7 +814,10 @@ void launch_synth_t(apf_sno *s, const float2 *Y, const float *h, long long oP, l
 template <bool BWD>
 void launch_synth(apf_sno *s, const float2 *Y, const float *h, long long oP, long long oc, float *z, float *hn, int B,
                   int act, cudaStream_t st) {
-    if ((long long)B * ((s->n / 4 + 63) / 64) >= 256) launch_synth_t<BWD, 2>(s, Y, h, oP, oc, z, hn, B, act, st);
+    if ((long long)B * s->c * s->n <= SMALL_SYNTH)
+        k_synth_small<BWD><<<dim3((s->n + 127) / 128, B * s->c), 128, 8 * small_pad(s->m) + 4 * small_pad(s->c), st>>>(Y, h, s->pb, oP, oc, s->tw, z, hn, s->c, s->n,
+                                                                             s->m, act);
+    else if ((long long)B * ((s->n / 4 + 63) / 64) >= 256) launch_synth_t<BWD, 2>(s, Y, h, oP, oc, z, hn, B, act, st);
     else launch_synth_t<BWD, 1>(s, Y, h, oP, oc, z, hn, B, act, st);
 }
 
@@ -702,11 +833,10 @@ template <bool BWD>
 void launch_mix(apf_sno *s, const float2 *X, float2 *Y, int l, int B, cudaStream_t st) {
     const int C = s->c, M = s->m;
     const long long wr = s->oWr + (long long)l * C * C * M, wi = s->oWi + (long long)l * C * C * M;
-    const int bg = (B + 3) / 4;
-    if ((long long)((C + 1) / 2) * M * bg >= 16384)
-        k_mix<BWD, 2><<<dim3(nb((long long)((C + 1) / 2) * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
+    if ((long long)B * C * M <= SMALL_MIX)
+        k_mix_small<BWD><<<(B * C * M + 127) / 128, 128, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
     else
-        k_mix<BWD, 1><<<dim3(nb((long long)C * M), bg), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
+        k_mix<BWD><<<dim3(nb((long long)((C + 1) / 2) * M), (B + 3) / 4), 256, 0, st>>>(X, s->pb, wr, wi, Y, B, C, M);
 }
 
 void forward(apf_sno *s, const float *x, int B, cudaStream_t st) {

@@ -1,7 +1,7 @@
 """Surrogate kernels at the edges of their tiles: single channels and samples,
 odd widths, mode counts around the 32-pair and 64-mode chunks, positions that
-are no multiple of a block's, batches that take either block width of the
-synthesis; forward and every gradient against the float64 reference.
+are no multiple of a block's, batches that take the one-output kernels and either
+block width of the tiled ones; forward and every gradient against the float64 reference.
 
 Tolerance: float32 sums of up to n x width terms (relative error of the order of
 sqrt(16384) x 2^-24 = 8e-6) through three or four layers: 5e-5 forward, 2e-4 on
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 # n, in_ch, width, modes, layers, n_out, batch
 SHAPES = [(64, 1, 1, 1, 1, 1, 1), (64, 2, 9, 32, 2, 3, 5), (192, 5, 7, 31, 3, 2, 3), (320, 12, 33, 65, 2, 5, 2),
-          (256, 20, 54, 33, 2, 7, 1), (1024, 12, 48, 64, 2, 5, 66), (512, 3, 16, 130, 2, 1, 9)]
+          (256, 20, 54, 33, 2, 7, 1), (1024, 12, 48, 64, 2, 5, 66), (512, 3, 16, 130, 2, 1, 9), (960, 3, 53, 37, 2, 2, 6)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
