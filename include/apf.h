@@ -280,13 +280,14 @@ int apf_get_stats(const apf_ctx *ctx, apf_stats *stats);
 
 /* Mixed mode: storage of the slab Schur blocks.  Every field sweep needs the
    inverses G_j of all h slab rows (the blocks the partial factorization of
-   paper Sec. 2 leaves behind; 16 nx^2 bytes each in packed bf16 form, 21.5 GB
+   paper Sec. 2 leaves behind; 8 nx^2 bytes each as two bf16 planes, 10.7 GB
    for h = 20 at nx = 8192).  segment_rows = 0 (the default) stores all h.
-   segment_rows = k in [1, h) keeps the packed inverses of only one segment of
-   k rows, plus the float32 G_{c-1} (8 nx^2 bytes) at every segment start
-   c > 0, and recomputes a segment's inverses from its checkpoint whenever a
-   sweep needs them: about two eliminations more per sweep, for a workspace
-   of (k * 16 + (ceil(h/k) - 1) * 8) nx^2 bytes instead of h * 16 nx^2.  The
+   segment_rows = k in [1, h) keeps the split inverses of only one segment of
+   k rows, plus a float32 block (8 nx^2 bytes) at every segment start c > 0
+   and one for the middle row, and recomputes a segment's inverses from its
+   checkpoint whenever a sweep needs them: about two eliminations more per
+   sweep, for a workspace of (k + ceil(h/k)) * 8 nx^2 bytes instead of
+   h * 8 nx^2.  The
    recomputed inverses are bit-identical to the stored ones, so results do
    not change.  Re-creates the workspace like apf_set_krylov (the fields of
    an earlier solve are gone).  APF_EINVAL in APF_FP64 mode for k != 0. */

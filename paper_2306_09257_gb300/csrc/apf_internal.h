@@ -2,8 +2,6 @@
 #pragma once
 
 #include <cuda_runtime.h>
-
-#include <utility>
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <string>
@@ -161,42 +159,6 @@ struct apf_ctx {
         kernel<<<(grid), (block), (smem), (stream)>>>(__VA_ARGS__);           \
         (ctx)->launches++;                                                    \
     } while (0)
-
-// For kernels that begin with chain_enter() (or call chain_start and chain_wait):
-// such a launch may start while its predecessor in the stream still runs.  The
-// chains of small dependent kernels that make up a solve pay a launch latency and
-// a prologue per kernel otherwise.
-template <typename... P, typename... A>
-void chain_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
-}
-#define APF_CHAIN(ctx, kernel, grid, block, smem, stream, ...)                      \
-    do {                                                                            \
-        chain_launch(kernel, grid, block, smem, stream, __VA_ARGS__);               \
-        (ctx)->launches++;                                                          \
-    } while (0)
-
-#ifdef __CUDACC__
-// The next kernel may be placed as soon as all blocks of this one are; its
-// chain_wait returns when this one has ended and its stores can be seen.
-// Nothing that an earlier kernel writes or reads is touched before chain_wait.
-__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_enter() {
-    chain_start();
-    chain_wait();
-}
-#endif
 
 GridDev make_grid(const apf_ctx *c);
 

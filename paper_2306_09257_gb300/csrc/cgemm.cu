@@ -221,7 +221,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
         n0 = ni * BNC;
     };
 
-    chain_start();
     if (warp == 0 && lane == 0 && cid < ntiles) {
         prefetch_map(&args.a[cid / ntl]);
         prefetch_map(&args.b[cid / ntl]);
@@ -256,7 +255,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
     if (CG == 2) cluster_sync();
     else __syncthreads();
     fence_after();
-    chain_wait();
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
     int issued = 0;
@@ -583,15 +581,13 @@ int launch_cg(apf_ctx *c, int nprob, const CgProblem *pb, CgArgs<P> &args, int M
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = L::TOTAL;
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = CG == 2 ? 2 : 1;
+    cfg.numAttrs = CG == 2 ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_cgemm<CG, BNC, NQ, CROSS, P>, args);
     if (e != cudaSuccess) return check_cuda(c, e, "tensor-core GEMM launch");
     c->launches++;

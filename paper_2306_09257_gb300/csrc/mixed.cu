@@ -97,7 +97,6 @@ __device__ __forceinline__ void split_bf16(float x, int nsplit, __nv_bfloat16 *o
 // Split form of R x C float32 planes (trans: of their transpose, R x C): the
 // operands of the test hooks and of the leaf variants that only write float32.
 __global__ void k_mirror(const float *re, const float *im, long long ld, int R, int C, int trans, Mirror m, int planes) {
-    chain_enter();
     const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
     if (c >= C) return;
     const long long g = trans ? (long long)c * ld + r : (long long)r * ld + c;
@@ -247,7 +246,6 @@ __device__ __forceinline__ void store_split2(const Mirror &m, int planes, long l
 template <bool BF, bool TWO, int N>
 __global__ void __launch_bounds__(128, TWO ? 2 : 4) k_row_step(GridDev g, const __grid_constant__ RowJobs<N> jobs, int n, const double2 *__restrict__ circ,
                                                                const float *__restrict__ w, int planes, int leaf) {
-    chain_enter();
     const RowJob &J = jobs.j[blockIdx.z];
     const int q = n >> 2, half = n >> 3;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -472,7 +470,6 @@ __global__ void __launch_bounds__(NB * 4) k_leaf32(const __grid_constant__ Tab<f
 
 template <int NB>
 __global__ void __launch_bounds__(NB * 4) k_leaf32r(const __grid_constant__ Tab<float *> re, const __grid_constant__ Tab<float *> im, long long ld, const __grid_constant__ Tab<int *> flags) {
-    chain_enter();
     const int b = blockIdx.x;
     leaf_gj_regs<NB>(re.v[b], im.v[b], ld, flags.v[b]);
 }
@@ -481,7 +478,6 @@ __global__ void __launch_bounds__(NB * 4) k_leaf32r(const __grid_constant__ Tab<
 // and in split form (XP.base null: float32 only).
 template <int NP>
 __global__ void __launch_bounds__(lc::NT) __cluster_dims__(NP, 1, 1) k_leaf_cluster(const __grid_constant__ Tab<float *> ret, const __grid_constant__ Tab<float *> imt, long long ld, const __grid_constant__ Tab<Mirror> XP, int planes, const __grid_constant__ Tab<int *> flags) {
-    chain_enter();
     extern __shared__ __align__(16) unsigned char lc_smem[];
     constexpr int N = 32 * NP;
     lc::Smem<NP> &sm = *reinterpret_cast<lc::Smem<NP> *>(lc_smem);
@@ -533,7 +529,6 @@ struct FieldJobs {
 
 template <int N>
 __global__ void __launch_bounds__(128) k_field_step(const __grid_constant__ FieldJobs<N> jobs, int nx, int planes) {
-    chain_enter();
     const FieldJob &J = jobs.j[blockIdx.z];
     const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x), c = J.c0 + blockIdx.y;
     if (x >= nx || c >= J.c1) return;
@@ -582,7 +577,6 @@ __global__ void __launch_bounds__(128) k_field_step(const __grid_constant__ Fiel
 // 1.24 ms.
 __global__ void __launch_bounds__(256) k_circ_apply(const __grid_constant__ Tab<const double2 *> Et, long long last, const __grid_constant__ Tab<double2 *> cbt, const __grid_constant__ Tab<double2 *> ctt,
                              int n, int logn, const double2 *__restrict__ sigma, const double2 *__restrict__ tw) {
-    chain_enter();
     extern __shared__ double2 a[];
     const double2 *src = Et.v[blockIdx.z] + (blockIdx.y ? last : 0) + (long long)blockIdx.x * n;
     double2 *out = (blockIdx.y ? ctt.v[blockIdx.z] : cbt.v[blockIdx.z]) + (long long)blockIdx.x * n;
@@ -681,7 +675,6 @@ __global__ void __launch_bounds__(256) k_circ_apply(const __grid_constant__ Tab<
 constexpr int RC = 2;
 __global__ void __launch_bounds__(128) k_residual(GridDev g, const __grid_constant__ Tab<const double *> epst, const __grid_constant__ Tab<const double2 *> Et, const __grid_constant__ Tab<const double2 *> Rt, const __grid_constant__ Tab<double2 *> cbt,
                                                   const __grid_constant__ Tab<double2 *> ctt, const __grid_constant__ Tab<double2 *> rt, const __grid_constant__ Tab<double *> partt, int ncol) {
-    chain_enter();
     const int b = blockIdx.z, n = g.nx, h = g.h, c0 = RC * blockIdx.y;
     const int x = blockIdx.x * 128 + threadIdx.x;
     const long long L = (long long)ncol * n;
@@ -772,7 +765,6 @@ __global__ void __launch_bounds__(128) k_residual(GridDev g, const __grid_consta
 
 // out[c] = the sum of column c's np partial sums, in a fixed order (one warp per column).
 __global__ void __launch_bounds__(32) k_normsum(const __grid_constant__ Tab<double *> partt, int np, const __grid_constant__ Tab<double *> outt) {
-    chain_enter();
     const double *p = partt.v[blockIdx.z] + (long long)blockIdx.x * np;
     double a = 0.0;
     for (int i = threadIdx.x; i < np; i += 32) a += p[i];
@@ -960,7 +952,7 @@ int leaf_size(const MixedWork *w) { return w->leaf; }
 
 void mirror_b(const Bat &bt, const PV *X, const Mirror *m, int R, int C, bool trans, int planes, cudaStream_t s) {
     for (int b = 0; b < bt.n; ++b)
-        APF_CHAIN(bt.lead(), k_mirror, dim3((C + 127) / 128, R), 128, 0, s, (const float *)X[b].re,
+        APF_LAUNCH(bt.lead(), k_mirror, dim3((C + 127) / 128, R), 128, 0, s, (const float *)X[b].re,
                    (const float *)X[b].im, X[b].ld, R, C, trans ? 1 : 0, m[b], planes);
 }
 
@@ -975,20 +967,20 @@ void leaf_b(const Bat &bt, const PV *X, int n, const Mirror *m, cudaStream_t s) 
     const auto fl = tab<int *>(bt, [&](int b) { return bt.c[b]->d_flags; });
     // 128 and 64: block elimination by a cluster (default); variants 1-3 are the single-level Gauss-Jordan kernels.
     if (n == 128 && v == 0) {
-        APF_CHAIN(c, k_leaf_cluster<4>, 4 * nb, lc::NT, (int)sizeof(lc::Smem<4>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+        APF_LAUNCH(c, k_leaf_cluster<4>, 4 * nb, lc::NT, (int)sizeof(lc::Smem<4>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
                   w->nsplit_elim, fl);
         return;
     }
     if (n == 64 && v == 0) {
-        APF_CHAIN(c, k_leaf_cluster<2>, 2 * nb, lc::NT, (int)sizeof(lc::Smem<2>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
+        APF_LAUNCH(c, k_leaf_cluster<2>, 2 * nb, lc::NT, (int)sizeof(lc::Smem<2>), s, re, im, ld, tab<Mirror>(bt, [&](int b) { return m[b]; }),
                   w->nsplit_elim, fl);
         return;
     }
     if (n == 128 && v == 1) APF_LAUNCH(c, k_leaf32r2<128>, nb, 512, 0, s, re, im, ld, fl);
     else if (n == 128 && v == 2) APF_LAUNCH(c, k_leaf32<128>, nb, 512, leaf_smem_bytes<128>(8), s, re, im, ld, fl);
-    else if (n == 128) APF_CHAIN(c, k_leaf32r<128>, nb, 512, 0, s, re, im, ld, fl);
+    else if (n == 128) APF_LAUNCH(c, k_leaf32r<128>, nb, 512, 0, s, re, im, ld, fl);
     else if (n == 64 && v == 1) APF_LAUNCH(c, k_leaf32r2<64>, nb, 256, 0, s, re, im, ld, fl);
-    else if (n == 64) APF_CHAIN(c, k_leaf32r<64>, nb, 256, 0, s, re, im, ld, fl);
+    else if (n == 64) APF_LAUNCH(c, k_leaf32r<64>, nb, 256, 0, s, re, im, ld, fl);
     else if (n == 32) APF_LAUNCH(c, k_leaf32<32>, nb, 128, leaf_smem_bytes<32>(8), s, re, im, ld, fl);
     else if (n == 16) APF_LAUNCH(c, k_leaf32<16>, nb, 64, leaf_smem_bytes<16>(8), s, re, im, ld, fl);
     else APF_LAUNCH(c, k_leaf_inv32, nb, 256, n * n * (int)sizeof(float2), s, re, im, ld, n, fl);
@@ -1093,7 +1085,7 @@ void row_step_b(const Bat &bt, const RowJob *jobs, int nj, int n, bool bf, cudaS
         for (int i = 0; i < nj; ++i) pack.j[i] = jobs[i];
         constexpr int N = sizeof(pack.j) / sizeof(RowJob);
         auto launch = [&](auto kernel) {
-            APF_CHAIN(c, kernel, grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
+            APF_LAUNCH(c, kernel, grid, 128, 0, s, g, pack, n, (const double2 *)c->d_circ, (const float *)w->BW, w->nsplit_elim, leaf);
         };
         if (bf) two ? launch(k_row_step<true, true, N>) : launch(k_row_step<true, false, N>);
         else two ? launch(k_row_step<false, true, N>) : launch(k_row_step<false, false, N>);
@@ -1198,7 +1190,7 @@ int approx_solve_b(const Bat &bt, F R, double2 *const *Y, double2 *const *E, boo
         auto run = [&](auto &pack) {
             for (int i = 0; i < nj; ++i) pack.j[i] = fj[i];
             constexpr int N = sizeof(pack.j) / sizeof(FieldJob);
-            APF_CHAIN(c, k_field_step<N>, grid, threads, 0, s, pack, nx, planes);
+            APF_LAUNCH(c, k_field_step<N>, grid, threads, 0, s, pack, nx, planes);
         };
         if (nj <= 2) {
             FieldJobs<2> p{};
@@ -1321,15 +1313,15 @@ void residual_b(const Bat &bt, FE E, FR r, bool rhs, cudaStream_t s) {
     const auto cb = tab<double2 *>(bt, [&](int b) { return bt.c[b]->mw->cb; });
     const auto ct = tab<double2 *>(bt, [&](int b) { return bt.c[b]->mw->ct; });
     const auto part = tab<double *>(bt, [&](int b) { return rhs ? bt.c[b]->mw->rpart : nullptr; });
-    APF_CHAIN(c, k_circ_apply, dim3(ncol, 2, nb), threads, nx * (int)sizeof(double2), s, Et, (c->h - 1) * L, cb, ct, nx,
+    APF_LAUNCH(c, k_circ_apply, dim3(ncol, 2, nb), threads, nx * (int)sizeof(double2), s, Et, (c->h - 1) * L, cb, ct, nx,
                logn, (const double2 *)c->d_modes, (const double2 *)c->d_tw);
     const dim3 grid((nx + 127) / 128, (ncol + RC - 1) / RC, nb);
-    APF_CHAIN(c, k_residual, grid, 128, 0, s, make_grid(c),
+    APF_LAUNCH(c, k_residual, grid, 128, 0, s, make_grid(c),
                tab<const double *>(bt, [&](int b) { return (const double *)bt.c[b]->d_eps; }), Et,
                tab<const double2 *>(bt, [&](int b) { return rhs ? (const double2 *)bt.c[b]->d_R : nullptr; }), cb, ct,
                tab<double2 *>(bt, [&](int b) { return (double2 *)r(b); }), part, ncol);
     if (rhs)
-        APF_CHAIN(c, k_normsum, dim3(ncol, 1, nb), 32, 0, s, part, (int)grid.x,
+        APF_LAUNCH(c, k_normsum, dim3(ncol, 1, nb), 32, 0, s, part, (int)grid.x,
                    tab<double *>(bt, [&](int b) { return bt.c[b]->mw->rnorm + ncol; }));
 }
 
