@@ -45,8 +45,8 @@ WL = {"mid": W.MID, "large": W.LARGE, "xlarge": W.XLARGE, "tiny": W.TINY}
 # capture of the field-sweep product (dram__bytes_read.sum + dram__bytes_write.sum
 # divided by 8 m n k x 3 plane products of that launch); a launch's traffic is
 # this times its flops.  None until a capture of the current kernel exists.
-GEMM_CAPTURE = {"bytes_per_hw_flop": 336.3e6 / (8.0 * 686 * 4096 * 4096 * 3),
-                "profile": "profiles/k_tc_gemm_pair_field_sweep_686x4096x4096.md"}
+GEMM_CAPTURE = {"bytes_per_hw_flop": 189.8e6 / (8.0 * 686 * 4096 * 4096 * 3),
+                "profile": "profiles/k_cgemm_field_sweep_686x4096x4096.md"}
 
 
 def args_parse():
@@ -716,7 +716,7 @@ def main():
         per_launch = pr["gemm_hw_flops"] / max(1, pr["gemm_launches"])
         tr = GEMM_CAPTURE["bytes_per_hw_flop"] * per_launch if GEMM_CAPTURE["bytes_per_hw_flop"] else None
         return {"bound": "tensor", "achieved": hw, "peak": peak_sus, "unit": "TFLOP/s", "frac": hw / peak_sus,
-                "traffic": tr, "kernel": "k_tc_gemm_pair / k_tc_gemm (tcgen05 bf16, fp32 accumulate)",
+                "traffic": tr, "kernel": "k_cgemm / k_tc_gemm (tcgen05 bf16, fp32 accumulate)",
                 "achieved_algorithmic_complex_tflops": alg, "gemm_launches": pr["gemm_launches"],
                 "note": (f"{where}: achieved = bf16 tensor flops (8 m n k per complex product x plane products) / "
                          f"summed CUDA-event launch time of the GEMMs; peak = bf16_tflops_sustained ({src}, of "

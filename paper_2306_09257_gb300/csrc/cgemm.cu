@@ -47,7 +47,7 @@ template <int P>
 struct CgArgs {
     CUtensorMap a[P], b[P];
     CgParams p[P];
-    int nprob, N, Mt, Nt, ntl, kblocks, nseg, planes, sym, vec, t_block;
+    int nprob, N, Mt, Nt, ntl, kblocks, nseg, planes, sym, vec, t_block, passes;
     uint32_t seg_pairs;
     float alpha, beta;
 };
@@ -62,7 +62,10 @@ struct CgArgs {
 // magnitude; a third as many of them leaves a third of the error of a K = 4096
 // product, and the sweeps (unlike the elimination, where it makes no difference)
 // set how far one refinement sweep gets: 4096 x 260, two sweeps, residual 8e-11
-// without and 2e-11 with it.
+// without and 2e-11 with it.  PASSES: for the same reason the pair tile adds up at
+// most 32 k blocks in the tensor memory; the passes are added in registers (4096 x
+// 260: residual of the first solve 3.9e-4 in one pass, 2.6e-4 in two, 3.8e-8 and not
+// 1.0e-7 after a sweep).
 // MERGED: a product with fewer than 128 columns takes the tensor core as long as one
 // with 128 (64 clocks per 16 of K), so the 128 x 32 tile multiplies x0 by both planes
 // of y at once, which leaves the cross products in accumulators of their own: 4
@@ -90,6 +93,7 @@ struct CgLayout {
     static constexpr int SETS = 2 * ACC <= 512 ? 2 : 1;
     static constexpr bool MERGED = CG == 1 && NQ == 4 && 4 * BNC <= 128;
     static constexpr int HELD = SETS == 1 ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
+    static constexpr bool PASSES = CG == 2 && CROSS;  // long sums in several passes
     // offset of the accumulator of component q's first (x r..) or second (x i..) half in group g
     static constexpr int acc(int g, int i, int r) { return MERGED ? (4 * i + 2 * g + r) * BNC : g * GROUP + (2 * i + r) * BNC; }
     static constexpr int TMEM = SETS * ACC;
@@ -204,6 +208,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
     const int ntl = args.ntl, ntiles = ntl * args.nprob;  // tiles of problem pr: [pr ntl, (pr + 1) ntl)
     const int cid = (int)blockIdx.x / CG, ncl = (int)gridDim.x / CG;
     const int total = args.kblocks * (NQ == 4 ? 1 : args.nseg);
+    const int passes = L::PASSES ? args.passes : 1;
     // first row and column of tile tt (pair: of the whole 256-row tile); with
     // sym, row block mi has the column blocks up to its last row
     auto tile_at = [&](int tt, int &m0, int &n0) {
@@ -299,12 +304,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate A
             constexpr uint32_t idesc_both = base | ((uint32_t)((2 * BNC) >> 3) << 17);
             int it = 0, tl = 0;
-            for (int t = cid; t < ntiles && ok; t += ncl, ++tl) {
+            for (int w = 0; w < passes * ((ntiles - cid + ncl - 1) / ncl) && ok; ++w, ++tl) {  // tiles times passes
                 const int b = tl % SETS, u = tl / SETS;
                 if (!mbar_wait(&tempty[b], (u & 1) ^ 1, abort_flag)) { ok = false; break; }
                 fence_after();
                 const uint32_t set = tmem + (uint32_t)(b * L::ACC);
-                for (int kk = 0; kk < total; ++kk, ++it) {
+                const int ps = w % passes, k0 = total * ps / passes, k1 = total * (ps + 1) / passes;
+                for (int kk = k0; kk < k1; ++kk, ++it) {
                     const int s = it % STAGES, r = it / STAGES;
                     if (!mbar_wait(&full[s], r & 1, abort_flag)) { ok = false; break; }
                     fence_after();
@@ -318,7 +324,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
 #pragma unroll
                             for (int k4 = 0; k4 < BK / 16; ++k4) {
                                 const uint64_t dar = sw128_desc(ar + k4 * 32), dai = sw128_desc(ai + k4 * 32), db = sw128_desc(sb + k4 * 32);
-                                const uint32_t acc = (kk > 0 || k4 > 0 || g > 0) ? 1u : 0u, to = set + 2 * g * BNC;
+                                const uint32_t acc = (kk > k0 || k4 > 0 || g > 0) ? 1u : 0u, to = set + 2 * g * BNC;
                                 mma_bf16(to, dar, db, g ? idesc_both : idesc_all, acc);
                                 mma_bf16(to + 4 * BNC, dai, db, g ? idesc_both : idesc_all, acc);
                             }
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                         const uint32_t re = set + (CROSS && g > 0 ? L::GROUP : 0), im = re + BNC;
 #pragma unroll
                         for (int k4 = 0; k4 < BK / 16; ++k4) {
-                            const uint32_t acc = (kk > 0 || k4 > 0 || g > CROSS) ? 1u : 0u;
+                            const uint32_t acc = (kk > k0 || k4 > 0 || g > CROSS) ? 1u : 0u;
                             const uint64_t dar = sw128_desc(ar + k4 * 32), dai = sw128_desc(ai + k4 * 32);
                             const uint64_t dbr = sw128_desc(br + k4 * 32), dbi = sw128_desc(bi + k4 * 32);
                             if (CG == 2) {
@@ -384,7 +390,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
         const int sr = lane >> 3, sc = lane & 7;  // this lane's row (of four) and cell in the shared layout
         int tl = 0;
         for (int t = cid; t < ntiles; t += ncl, ++tl) {
-            const int b = tl % SETS, u = tl / SETS, pr = t / ntl;
+            const int b = L::PASSES ? 0 : tl % SETS, u = tl / SETS, pr = t / ntl;  // (PASSES: one set, uses counted in the loop below)
             const CgParams &p = args.p[pr];
             int m0, n0;
             tile_at(t - pr * ntl, m0, n0);
@@ -413,8 +419,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                     pre[i] = x;
                 }
             };
-            // one component of a block: rr - ii or ri + ir (pair: as accumulated), times alpha
-            auto read = [&](int c0, float (&v)[32]) {
+            // one component of a block: rr - ii or ri + ir (pair: as accumulated), added to v
+            auto read = [&](int c0, float (&v)[32], bool add) {
                 const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(b * L::ACC + (c0 - n0));
 #pragma unroll
                 for (int g = 0; g <= CROSS; ++g) {
@@ -428,12 +434,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                         for (int i = 0; i < 16; ++i) {
                             float z = __uint_as_float(x[i]);
                             if (CG == 1) z += q ? __uint_as_float(y[i]) : -__uint_as_float(y[i]);
-                            v[hc + i] = g ? v[hc + i] + z : z;
+                            v[hc + i] = add || g ? v[hc + i] + z : z;
                         }
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] *= args.alpha;
             };
             auto skip = [&](int c0) { return c0 >= args.N || row0 >= p.M || (args.sym && c0 > row0); };  // warp-uniform
             auto release = [&] {
@@ -445,17 +449,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                 }
             };
             if (L::HELD == 1 && use_beta && !skip(n0)) fetch(n0);
-            if (!mbar_wait(&tfull[b], u & 1, abort_flag)) { ok = false; break; }
-            __syncwarp();
-            fence_after();
             float held[L::HELD][32];
-            if (L::HELD > 1) {  // a single set: free it for the next tile's products before the stores
+            for (int ps = 0; ps < passes; ++ps) {
+                if (!mbar_wait(&tfull[b], (L::PASSES ? tl * passes + ps : u) & 1, abort_flag)) { ok = false; break; }
+                __syncwarp();
+                fence_after();
+                if (L::HELD > 1) {  // a single set: free it for the next products before the stores
 #pragma unroll
-                for (int i = 0; i < L::HELD; ++i)
-                    if (!skip(n0 + 32 * i)) read(n0 + 32 * i, held[i]);
-                release();
+                    for (int i = 0; i < L::HELD; ++i)
+                        if (!skip(n0 + 32 * i)) read(n0 + 32 * i, held[i], L::PASSES && ps > 0);
+                    release();
+                }
             }
+            if (!ok) break;
             auto finish = [&](int c0, float (&v)[32]) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] *= args.alpha;
                 if (use_beta) {
                     if (L::HELD > 1 || c0 > n0) fetch(c0);
 #pragma unroll
@@ -520,7 +529,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
 #pragma unroll 1
                 for (int c0 = n0; c0 < n0 + BNC; c0 += 32) {
                     if (skip(c0)) continue;
-                    read(c0, held[0]);
+                    read(c0, held[0], false);
                     finish(c0, held[0]);
                 }
                 release();
@@ -653,6 +662,7 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
     args.beta = beta;
     args.sym = sym ? 1 : 0;
     args.t_block = pb[0].t_block;
+    args.passes = (args.kblocks + 31) / 32;
     bool vec = N % 16 == 0;
     for (int i = 0; i < nprob; ++i) {
         const CgProblem &q = pb[i];
