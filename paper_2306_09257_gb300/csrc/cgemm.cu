@@ -63,9 +63,9 @@ struct CgArgs {
 // product, and the sweeps (unlike the elimination, where it makes no difference)
 // set how far one refinement sweep gets: 4096 x 260, two sweeps, residual 8e-11
 // without and 2e-11 with it.  PASSES: for the same reason the pair tile adds up at
-// most 32 k blocks in the tensor memory; the passes are added in registers (4096 x
-// 260: residual of the first solve 3.9e-4 in one pass, 2.6e-4 in two, 3.8e-8 and not
-// 1.0e-7 after a sweep).
+// most 32 k blocks in the tensor memory, and half of a product of up to 64; the
+// passes are added in registers (4096 x 260: residual of the first solve 3.9e-4 in
+// one pass, 2.6e-4 in two, 1.0e-7 and 3.8e-8 after a sweep).
 // MERGED: a product with fewer than 128 columns takes the tensor core as long as one
 // with 128 (64 clocks per 16 of K), so the 128 x 32 tile multiplies x0 by both planes
 // of y at once, which leaves the cross products in accumulators of their own: 4
@@ -662,7 +662,7 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
     args.beta = beta;
     args.sym = sym ? 1 : 0;
     args.t_block = pb[0].t_block;
-    args.passes = (args.kblocks + 31) / 32;
+    args.passes = std::max(2, (args.kblocks + 31) / 32);
     bool vec = N % 16 == 0;
     for (int i = 0; i < nprob; ++i) {
         const CgProblem &q = pb[i];
