@@ -259,11 +259,11 @@ def run_reference(a, w):
 
 def alg_flops(w, nin, nout):
     """Algorithmic real flops of one S + grad f evaluation (8 per complex
-    multiply-add): symmetric recursive inversion of the h slab blocks
-    (h (16/3) n^3), the first field sweep (8 n^2 [(h-1) n_in + h (n_in + n_out)])
+    multiply-add): symmetric recursive inversion of the h slab blocks, two of
+    the four products of a level by half (h 4 n^3), the first field sweep (8 n^2 [(h-1) n_in + h (n_in + n_out)])
     and the adjoint contraction (8 h n n_in n_out)."""
     n, h = float(w.nx), float(w.h)
-    return h * 16.0 / 3.0 * n ** 3 + 8.0 * n * n * ((h - 1) * nin + h * (nin + nout)) + 8.0 * h * n * nin * nout
+    return h * 4.0 * n ** 3 + 8.0 * n * n * ((h - 1) * nin + h * (nin + nout)) + 8.0 * h * n * nin * nout
 
 
 def fp64_peak(local):
