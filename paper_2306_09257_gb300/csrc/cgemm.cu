@@ -681,10 +681,11 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
                                         : launch_cg<1, 64, 2, 0, P>(c, nprob, pb, args, M, N, K, sms, s);
     // Pair tiles (256 x 128 over two SMs) for the long products of many rows: at
     // full load as fast per SM as the one-CTA 128 x 64 tile or faster, with half
-    // its operand traffic (4096^3: 821 against 1053 us; 2048^3: 127 against 148);
-    // below K = 2048 a product has too few of them to fill the chip (1024^3: 40
-    // against 25 us).  128 x 32 tiles take as long as 128 x 64 ones but store
-    // sooner (512^3: 15.8 against 16.1 us): where they still go in one round.
+    // its operand traffic (4096^3: 840 against 1043 us; 2048^3: 133 against 148);
+    // below K = 2048 a product has too few of them to fill the chip (1024^3 took
+    // 40 us with them, 26 with one-CTA tiles).  128 x 32 tiles, where they still go
+    // in one round, take both planes of B at once and store sooner (512^3: 13.8 us,
+    // 16.1 with 128 x 64 tiles).
     int kind = 1;
     if (pair_enabled() && K >= 2048 && rows > BM) {
         kind = 2;

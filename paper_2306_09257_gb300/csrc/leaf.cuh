@@ -1,7 +1,7 @@
 // Diagonal-block inversion shared by the float64 and the mixed path.
 // (1) leaf_gj / leaf_gj_regs: Gauss-Jordan elimination with partial (row)
-// pivoting of one NB x NB block.  (2) lc: the mixed path's 128 x 128 blocks, by a
-// cluster of four CTAs.
+// pivoting of one NB x NB block.  (2) lc: the mixed path's 128 x 128 and 64 x 64
+// blocks, by a cluster of four and two CTAs.
 // In (1), for the shared-memory form:  Thread t owns row t/4 and the columns sub + 4q
 // (sub = t%4), so the 4 threads of a row sit in adjacent lanes and the
 // pivot-row reads are conflict-free; rows are padded by 4 elements.

@@ -14,7 +14,7 @@
 // X_j = K_j - G_{j-1} below it, X_j = K_j - G_{j+1} above it, X_m = K_m - G_{m-1} -
 // G_{m+1}.  The two chains are independent, so one launch carries a row of each
 // (of every design of a batch): half as many dependent steps, which is what a
-// single design's time consists of (one CTA per 128 x 128 diagonal block, a few
+// single design's time consists of (four CTAs per 128 x 128 diagonal block, a few
 // tiles per product of the lower recursion levels).
 #include "apf_internal.h"
 #include "cgemm.h"
