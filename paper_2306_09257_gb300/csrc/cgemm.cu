@@ -575,9 +575,10 @@ int launch_cg(apf_ctx *c, int nprob, const CgProblem *pb, CgArgs<P> &args, int M
               cudaStream_t s) {
     using L = CgLayout<CG, BNC, NQ, CROSS>;
     for (int i = 0; i < nprob; ++i) {
-        const long long k64 = (K + 63) / 64 * 64;  // operands are padded with zeros to whole k blocks
-        if (!tc_make_map(&args.a[i], pb[i].A.base, k64, pb[i].M, 2 * args.planes, pb[i].A.pitch, pb[i].A.qpitch, BM, NQ) ||
-            !tc_make_map(&args.b[i], pb[i].B.base, k64, N, 2 * args.planes, pb[i].B.pitch, pb[i].B.qpitch, L::B_ROWS, NQ))
+        // K columns, not whole k blocks: what follows a sub-block in memory belongs to
+        // its neighbour, and TMA fills the rest of the last k block with zeros
+        if (!tc_make_map(&args.a[i], pb[i].A.base, K, pb[i].M, 2 * args.planes, pb[i].A.pitch, pb[i].A.qpitch, BM, NQ) ||
+            !tc_make_map(&args.b[i], pb[i].B.base, K, N, 2 * args.planes, pb[i].B.pitch, pb[i].B.qpitch, L::B_ROWS, NQ))
             return set_err(c, APF_ECUDA, "tensor map encode failed (M=%d N=%d K=%d)", pb[i].M, N, K);
     }
     args.Mt = (M + CG * BM - 1) / (CG * BM);

@@ -38,7 +38,6 @@ struct SideWork {
 
 struct MixedWork {
     int nsplit_elim = 2, nsplit_grad = 3, leaf = 128, leaf_variant = 0;
-    long long pitch = 0;                             // row pitch of n-column split matrices: max(n, 64)
     int nside = 2;                                   // 1 with recomputation
     SideWork sd[2];
     __nv_bfloat16 *GA = nullptr, *GB = nullptr;      // gradient operands
@@ -1068,7 +1067,7 @@ int pos_row(const apf_ctx *c, int p) {
 Mirror gp_view(const apf_ctx *c, int row) {
     const MixedWork *w = c->mw;
     const int slot = w->seg_rows > 0 ? row_pos(c, row) % w->seg_rows : row;
-    return Mirror{w->GP + slot * w->gp_stride, w->pitch, w->pitch * c->nx};
+    return Mirror{w->GP + slot * w->gp_stride, c->nx, (long long)c->nx * c->nx};
 }
 
 // Launch one k_row_step per problem of `bt` (n: block size; jobs without an
@@ -1361,7 +1360,6 @@ int mixed_alloc(apf_ctx *c) {
     const long long n = c->nx, h = c->h, q = 2 * w->nsplit_elim;  // q: component planes of a split matrix
     const int nin = c->nin, nout = c->nout;
     const long long ncol = std::max(nin + nout, nin);
-    w->pitch = std::max<long long>(n, 64);
     w->seg_rows = (c->schur_seg > 0 && c->schur_seg < h) ? c->schur_seg : 0;
     w->nseg = w->seg_rows > 0 ? (int)((h + w->seg_rows - 1) / w->seg_rows) : 1;
     w->nside = w->seg_rows > 0 || h < 3 ? 1 : 2;  // chains eliminated at the same time
@@ -1371,14 +1369,14 @@ int mixed_alloc(apf_ctx *c) {
         SideWork &sw = w->sd[sd];
         if (sd < w->nside) {
             WA(sw.Xre, n * n); WA(sw.Xim, n * n);
-            WA(sw.XP.base, q * n * w->pitch);
-            sw.XP.pitch = w->pitch; sw.XP.qpitch = n * w->pitch;
+            WA(sw.XP.base, q * n * n);
+            sw.XP.pitch = n; sw.XP.qpitch = n * n;
             // T of the levels n/2, n/4, ..: q (n^2/4 + n^2/16 + ..) < q n^2 / 3
             WA(sw.TP, q * (n * n * 11 / 32 + 64)); WA(sw.TT, q * (n * n * 11 / 32 + 64));
         }
         WA(sw.O32, 2 * ncol * n);
-        WA(sw.PA.base, q * ncol * w->pitch);
-        sw.PA.pitch = w->pitch; sw.PA.qpitch = ncol * w->pitch;
+        WA(sw.PA.base, q * ncol * n);
+        sw.PA.pitch = n; sw.PA.qpitch = ncol * n;
     }
     const long long kp_g = round_up(2LL * nin, 64);
     WA(w->GA, (long long)nout * kp_g * w->nsplit_grad);
@@ -1403,19 +1401,12 @@ int mixed_alloc(apf_ctx *c) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap_stream);
         if (e != cudaSuccess) return check_cuda(c, e, "butterfly weights");
     }
-    w->gp_stride = q * n * w->pitch;
+    w->gp_stride = q * n * n;
     const long long slots = w->seg_rows > 0 ? w->seg_rows : h;
     WA(w->GP, slots * w->gp_stride);
     if (w->seg_rows > 0) {
         WA(w->CK, (long long)(w->nseg - 1) * 2 * n * n);
         WA(w->CKB, 2 * n * n);
-    }
-    if (w->pitch > n) {  // the padding columns of the products' operands are read: zero
-        cudaError_t e = cudaMemsetAsync(w->GP, 0, sizeof(__nv_bfloat16) * slots * w->gp_stride, c->cap_stream);
-        for (int sd = 0; sd < 2 && e == cudaSuccess; ++sd)
-            e = cudaMemsetAsync(w->sd[sd].PA.base, 0, sizeof(__nv_bfloat16) * q * ncol * w->pitch, c->cap_stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap_stream);
-        if (e != cudaSuccess) return check_cuda(c, e, "clear operand padding");
     }
     WA(w->r, h * ncol * n); WA(w->delta, h * ncol * n);
     WA(w->cb, ncol * n); WA(w->ct, ncol * n);
@@ -1928,12 +1919,13 @@ extern "C" int apf_debug_inv32(apf_ctx *c, int n, float *re, float *im, int leaf
     // + 100000: through the symmetric random butterfly transform
     const bool bf = leaf >= 100000 && n >= 16;
     leaf %= 100000;
-    if (leaf > 0) { w->leaf = leaf % 1000; w->leaf_variant = leaf / 1000; }
+    // (blocks below 8 are taken as 8: a row of a product's operand is at least 16 bytes)
+    if (leaf > 0) { w->leaf = std::max(8, leaf % 1000); w->leaf_variant = leaf / 1000; }
     cudaStream_t s = 0;
     cudaMemsetAsync(c->d_flags, 0, 16, s);
     const Bat bt = one(c);
     const PV X{w->sd[0].Xre, w->sd[0].Xim, n}, user{re, im, n};
-    const Mirror XP{w->sd[0].XP.base, std::max<long long>(n, 64), n * std::max<long long>(n, 64)};
+    const Mirror XP{w->sd[0].XP.base, n, (long long)n * n};
     int rc = APF_OK;
     if (n < 8) {
         Mirror none;
