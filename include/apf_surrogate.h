@@ -43,7 +43,7 @@ long long apf_sno_num_params(const apf_sno *s);
 /* Copy the fp32 parameters in (also resets the Adam moments) or out. */
 int apf_sno_set_params(apf_sno *s, const float *params);
 int apf_sno_get_params(const apf_sno *s, float *params);
-/* y = net(x) for `batch` samples. */
+/* y = net(x) for `batch` samples; the bits of a sample's y do not depend on the others in the call. */
 int apf_sno_forward(apf_sno *s, const float *x, int batch, float *y, void *stream);
 /* Gradient of the mean squared error w.r.t. every parameter (same layout as
    the parameter vector; grads may be NULL) and the loss (host, may be NULL). */

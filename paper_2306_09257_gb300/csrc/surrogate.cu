@@ -297,7 +297,10 @@ __global__ void __launch_bounds__(128) k_mix_small(const float2 *__restrict__ X,
     Y[idx] = make_float2(yr, yi);
 }
 
-// Block: 128 positions (blockIdx.x) of one channel of a sample (blockIdx.y).
+// Block: 128 positions (blockIdx.x) of one channel of a sample (blockIdx.y).  Every sum
+// is taken in k_synth's order (modes folded, n/4 and 3n/4 by a warp), so that a
+// sample's result does not depend on how many others are in the call (0.3 to 0.5 us
+// of a launch's 3.5 to 7 us: 1 sample of 16 channels, 128 positions; of 48 and 1024).
 template <bool BWD>
 __global__ void __launch_bounds__(128) k_synth_small(const float2 *__restrict__ Y, const float *__restrict__ h, const __nv_bfloat16 *__restrict__ pb,
                                                      long long oP, long long oc, const float2 *__restrict__ tw, float *z, float *hn, int C,
@@ -306,20 +309,27 @@ __global__ void __launch_bounds__(128) k_synth_small(const float2 *__restrict__ 
     const int Mp = small_pad(M), Cp = small_pad(C);  // with zeros up to whole batches
     float2 *ys = reinterpret_cast<float2 *>(ss_smem);  // [m]: w Y
     float *ps = reinterpret_cast<float *>(ys + Mp);     // [i]
-    const int b = blockIdx.y / C, o = blockIdx.y - b * C, x = blockIdx.x * 128 + threadIdx.x;
-    const float *hb = h + (long long)b * C * n + x;
+    const int b = blockIdx.y / C, o = blockIdx.y - b * C, x = blockIdx.x * 128 + threadIdx.x, q = n >> 2;
+    // x is one of f, n/2 - f, n/2 + f, n - f
+    const int quarter = (x >= q) + (x >= n / 2) + (x >= 3 * q), f = quarter == 0 ? x : quarter == 1 ? n / 2 - x : quarter == 2 ? x - n / 2 : n - x;
+    const float *hb = h + (long long)b * C * n;
+    // n/4 or 3n/4 if it is one of this warp's positions; its first loads go out with the others
+    const int lane = threadIdx.x & 31, x0 = x - lane, p = (q - x0) >> 5 == 0 ? q : (3 * q - x0) >> 5 == 0 ? 3 * q : -1;
+    const float2 yp = p >= 0 && lane < M ? Y[(long long)blockIdx.y * M + lane] : make_float2(0.f, 0.f);
+    const float hp = p >= 0 && lane < C ? hb[lane * n + p] : 0.f;
+    auto weight = [&](int m) { return m >= M ? 0.f : BWD ? 1.f : (m == 0 ? 1.f : 2.f) / (float)n; };
     float2 w[SMALL_BATCH];  // one batch ahead
     float v[SMALL_BATCH];
     if (x < n) {
 #pragma unroll
         for (int k = 0; k < SMALL_BATCH; ++k) {
-            w[k] = tw[min(k, M - 1) * n + x];
-            v[k] = hb[min(k, C - 1) * n];
+            w[k] = tw[min(k, M - 1) * n + f];
+            v[k] = hb[min(k, C - 1) * n + x];
         }
     }
     for (int m = threadIdx.x; m < Mp; m += 128) {
         const float2 y = Y[(long long)blockIdx.y * M + min(m, M - 1)];
-        const float s = m >= M ? 0.f : BWD ? 1.f : (m == 0 ? 1.f : 2.f) / (float)n;
+        const float s = weight(m);
         ys[m] = make_float2(s * y.x, s * y.y);
     }
     for (int i = threadIdx.x; i < Cp; i += 128) ps[i] = i < C ? bf(pb, oP + (BWD ? (long long)i * C + o : (long long)o * C + i)) : 0.f;
@@ -327,26 +337,45 @@ __global__ void __launch_bounds__(128) k_synth_small(const float2 *__restrict__ 
     if (x >= n) return;
     const long long at = (long long)blockIdx.y * n + x;
     const float zv = BWD && z ? z[at] : 0.f;
-    float acc = 0.f;
+    float a[4] = {};  // even cos, odd cos, even sin, odd sin
     for (int m0 = 0; m0 < M; m0 += SMALL_BATCH) {
         float2 c[SMALL_BATCH];
 #pragma unroll
         for (int k = 0; k < SMALL_BATCH; ++k) {
             c[k] = w[k];
-            if (m0 + SMALL_BATCH < M) w[k] = tw[min(m0 + SMALL_BATCH + k, M - 1) * n + x];
+            if (m0 + SMALL_BATCH < M) w[k] = tw[min(m0 + SMALL_BATCH + k, M - 1) * n + f];
         }
 #pragma unroll
-        for (int k = 0; k < SMALL_BATCH; ++k) acc = fmaf(ys[m0 + k].x, c[k].x, fmaf(-ys[m0 + k].y, c[k].y, acc));
+        for (int k = 0; k < SMALL_BATCH; ++k) {
+            a[k & 1] = fmaf(ys[m0 + k].x, c[k].x, a[k & 1]);
+            a[2 + (k & 1)] = fmaf(ys[m0 + k].y, c[k].y, a[2 + (k & 1)]);
+        }
     }
+    const float cp = a[0] + a[1], cm = a[0] - a[1], sp = a[2] + a[3], sd = a[2] - a[3];
+    float acc = quarter == 0 ? cp - sp : quarter == 1 ? cm + sd : quarter == 2 ? cm - sd : cp + sp;
     for (int i0 = 0; i0 < C; i0 += SMALL_BATCH) {
         float c[SMALL_BATCH];
 #pragma unroll
         for (int k = 0; k < SMALL_BATCH; ++k) {
             c[k] = v[k];
-            if (i0 + SMALL_BATCH < C) v[k] = hb[min(i0 + SMALL_BATCH + k, C - 1) * n];
+            if (i0 + SMALL_BATCH < C) v[k] = hb[min(i0 + SMALL_BATCH + k, C - 1) * n + x];
         }
 #pragma unroll
         for (int k = 0; k < SMALL_BATCH; ++k) acc = fmaf(ps[i0 + k], c[k], acc);
+    }
+    if (p >= 0) {
+        float even = 0.f, odd = 0.f, part = 0.f;
+        for (int m = lane; m < M; m += 32) {
+            const float s = (m >> 1) & 1 ? -weight(m) : weight(m);
+            const float2 y = m == lane ? yp : Y[(long long)blockIdx.y * M + m];
+            if (m & 1) odd = fmaf(s, y.y, odd);
+            else even = fmaf(s, y.x, even);
+        }
+        for (int i = lane; i < C; i += 32) part = fmaf(ps[i], i == lane ? hp : hb[i * n + p], part);
+        float t = p == q ? even - odd + part : even + odd + part;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (x == p) acc = t;
     }
     if (BWD) {
         hn[at] = z ? acc * gelu_d(zv) : acc;
