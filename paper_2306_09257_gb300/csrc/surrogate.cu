@@ -66,7 +66,7 @@ __global__ void k_tw(float2 *tw, int n, int M) {
 // group of 8 outputs.
 __global__ void __launch_bounds__(256) k_lift(const float *eps, const __nv_bfloat16 *pb, long long oW0, long long ob0,
                                               float *h0, int CI, int C, int n) {
-    __shared__ float es[64][64], ws[64][72];  // [i][x], [i][o]
+    __shared__ __align__(16) float es[64][64], ws[64][72];  // [i][x], [i][o]
     const int b = blockIdx.y, x0 = blockIdx.x * 64, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     const int Cp = (C + 7) & ~7;
     for (int i = ty; i < CI; i += 4) es[i][tx] = eps[((long long)b * CI + i) * n + x0 + tx];
