@@ -63,9 +63,16 @@ struct CgArgs {
 // product, and the sweeps (unlike the elimination, where it makes no difference)
 // set how far one refinement sweep gets: 4096 x 260, two sweeps, residual 8e-11
 // without and 2e-11 with it.  PASSES: for the same reason the pair tile adds up at
-// most 32 k blocks in the tensor memory, and half of a product of up to 64; the
-// passes are added in registers (4096 x 260: residual of the first solve 3.9e-4 in
-// one pass, 2.6e-4 in two, 1.0e-7 and 3.8e-8 after a sweep).
+// most 16 k blocks in the tensor memory, 8 of a product of more than 64 (K > 4096),
+// and the passes are added in registers; with one plane product per stage the
+// smaller products are a pass of their own.  Residual of the first solve and after
+// a sweep, time of an evaluation, two planes: 4096 x 260 one pass 3.9e-4, 1.0e-7;
+// 32 blocks 2.5e-4, 4.0e-8, 55.7 ms; 16 blocks 2.0e-4, 1.5e-8, 55.9 ms; 8 blocks
+// 1.8e-4, 1.0e-8, 57.1 ms; 8192 x 280 32 blocks 3.7e-4, 9.0e-8, 276 ms; 16 blocks
+// 3.0e-4, 4.2e-8, 279 ms; 8 blocks 2.8e-4, 3.1e-8, 286 ms (the one-ended order of
+// elimination with 256-wide tiles left 2.4e-4, 3.3e-8 and 2.8e-4, 4.0e-8).  Three
+// planes, 4096 x 260: one pass 3.3e-4, 9.0e-8, 97.0 ms; 16 blocks 9.7e-5, 8.1e-9,
+// 98.8 ms (before: 2.3e-4, 4.2e-8).
 // MERGED: a product with fewer than 128 columns takes the tensor core as long as one
 // with 128 (64 clocks per 16 of K), so the 128 x 32 tile multiplies x0 by both planes
 // of y at once, which leaves the cross products in accumulators of their own: 4
@@ -92,8 +99,8 @@ struct CgLayout {
     static constexpr int ACC = (CROSS ? 2 : 1) * GROUP;
     static constexpr int SETS = 2 * ACC <= 512 ? 2 : 1;
     static constexpr bool MERGED = CG == 1 && NQ == 4 && 4 * BNC <= 128;
-    static constexpr int HELD = SETS == 1 ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
-    static constexpr bool PASSES = CG == 2 && CROSS;  // long sums in several passes
+    static constexpr bool PASSES = CG == 2 && (CROSS || NQ == 2);  // long sums in several passes
+    static constexpr int HELD = SETS == 1 || PASSES ? BNC / 32 : 1;  // blocks of a tile read before the first is stored
     // offset of the accumulator of component q's first (x r..) or second (x i..) half in group g
     static constexpr int acc(int g, int i, int r) { return MERGED ? (4 * i + 2 * g + r) * BNC : g * GROUP + (2 * i + r) * BNC; }
     static constexpr int TMEM = SETS * ACC;
@@ -209,6 +216,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
     const int cid = (int)blockIdx.x / CG, ncl = (int)gridDim.x / CG;
     const int total = args.kblocks * (NQ == 4 ? 1 : args.nseg);
     const int passes = L::PASSES ? args.passes : 1;
+    // first k step of pass ps: equal parts, but with one plane product per stage all the
+    // smaller products together are the first pass
+    auto pass_begin = [&](int ps) {
+        if (NQ == 4 || !L::PASSES) return total * ps / passes;
+        const int small = args.nseg > 1 ? 1 : 0;
+        return ps < small ? 0 : total - args.kblocks * (passes - ps) / (passes - small);
+    };
     // first row and column of tile tt (pair: of the whole 256-row tile); with
     // sym, row block mi has the column blocks up to its last row
     auto tile_at = [&](int tt, int &m0, int &n0) {
@@ -309,7 +323,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
                 if (!mbar_wait(&tempty[b], (u & 1) ^ 1, abort_flag)) { ok = false; break; }
                 fence_after();
                 const uint32_t set = tmem + (uint32_t)(b * L::ACC);
-                const int ps = w % passes, k0 = total * ps / passes, k1 = total * (ps + 1) / passes;
+                const int ps = w % passes, k0 = pass_begin(ps), k1 = pass_begin(ps + 1);
                 for (int kk = k0; kk < k1; ++kk, ++it) {
                     const int s = it % STAGES, r = it / STAGES;
                     if (!mbar_wait(&full[s], r & 1, abort_flag)) { ok = false; break; }
@@ -390,7 +404,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
         const int sr = lane >> 3, sc = lane & 7;  // this lane's row (of four) and cell in the shared layout
         int tl = 0;
         for (int t = cid; t < ntiles; t += ncl, ++tl) {
-            const int b = L::PASSES ? 0 : tl % SETS, u = tl / SETS, pr = t / ntl;  // (PASSES: one set, uses counted in the loop below)
+            int b = 0;  // the set in use
+            const int pr = t / ntl;
             const CgParams &p = args.p[pr];
             int m0, n0;
             tile_at(t - pr * ntl, m0, n0);
@@ -451,10 +466,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_cgemm(const __grid_constant__ Cg
             if (L::HELD == 1 && use_beta && !skip(n0)) fetch(n0);
             float held[L::HELD][32];
             for (int ps = 0; ps < passes; ++ps) {
-                if (!mbar_wait(&tfull[b], (L::PASSES ? tl * passes + ps : u) & 1, abort_flag)) { ok = false; break; }
+                const int use = tl * passes + ps;
+                b = use % SETS;
+                if (!mbar_wait(&tfull[b], (use / SETS) & 1, abort_flag)) { ok = false; break; }
                 __syncwarp();
                 fence_after();
-                if (L::HELD > 1) {  // a single set: free it for the next products before the stores
+                if (L::HELD > 1) {  // free the set for the next products before the stores
 #pragma unroll
                     for (int i = 0; i < L::HELD; ++i)
                         if (!skip(n0 + 32 * i)) read(n0 + 32 * i, held[i], L::PASSES && ps > 0);
@@ -663,7 +680,8 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
     args.beta = beta;
     args.sym = sym ? 1 : 0;
     args.t_block = pb[0].t_block;
-    args.passes = std::max(2, (args.kblocks + 31) / 32);
+    args.passes = std::max(2, args.kblocks / (args.kblocks > 64 ? 8 : 16));  // see PASSES
+    if (planes != 2 && args.nseg > 1) args.passes++;  // the smaller products
     bool vec = N % 16 == 0;
     for (int i = 0; i < nprob; ++i) {
         const CgProblem &q = pb[i];
