@@ -108,7 +108,7 @@ static void free_workspace(apf_ctx *c) {
     c->ws_bytes = 0;
     c->ws_nx = c->ws_ny = c->ws_h = c->ws_min = c->ws_mout = -1;
     c->d_min = c->d_mout = nullptr; c->d_stretch = nullptr; c->d_modes = c->d_coef = c->d_circ = c->d_tw = nullptr;
-    c->d_G = c->d_scr1 = c->d_scr2 = c->d_E = c->d_T = c->d_R = nullptr;
+    c->d_G = c->d_scr = c->d_E = c->d_T = c->d_R = nullptr;
     c->d_S = c->d_Gam = c->d_Q = c->d_fft = nullptr;
     c->d_grad = c->d_f = c->d_colnorm = nullptr;
     c->d_flags = nullptr; c->d_pairs = nullptr;
@@ -144,8 +144,7 @@ static int ensure_workspace(apf_ctx *c) {
     AL(c->d_modes, 4 * nx); AL(c->d_stretch, 2 * (c->ny + 1)); AL(c->d_coef, ncol); AL(c->d_circ, 2 * nx); AL(c->d_tw, nx / 2);
     if (c->precision == APF_FP64) {
         AL(c->d_G, h * nx * nx);
-        AL(c->d_scr1, nx * nx); AL(c->d_scr2, nx * nx);
-        AL(c->d_T, 2 * std::max<long long>(ncol, nin) * nx);
+        AL(c->d_scr, nx * nx); AL(c->d_T, ncol * nx);
     }
     // fields: the single-elimination solve's n_in + n_out columns, or the
     // conventional adjoint method's n_in forward and n_in adjoint columns

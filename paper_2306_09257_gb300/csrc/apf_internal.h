@@ -99,9 +99,9 @@ struct apf_ctx {
     double2 *d_circ = nullptr;   // 2*nx: circulant generators of Sigma_bot, Sigma_top
     double2 *d_tw = nullptr;     // nx/2 twiddles exp(-2 pi i k / nx)
     double2 *d_G = nullptr;      // h*nx*nx   (float64 mode)
-    double2 *d_scr1 = nullptr, *d_scr2 = nullptr;  // recursion scratch, nx*nx each (two blocks at a time)
+    double2 *d_scr = nullptr;    // recursion scratch, nx*nx (float64 mode)
     double2 *d_E = nullptr;      // h*ncol*nx fields, [row][column][x]
-    double2 *d_T = nullptr;      // 2*ncol*nx temp (float64 mode)
+    double2 *d_T = nullptr;      // ncol*nx temp (float64 mode)
     double2 *d_R = nullptr;      // 2*ncol*nx right-hand side, first and last slab row (mixed)
     double2 *d_S = nullptr, *d_Gam = nullptr;  // n_out*n_in
     double2 *d_qsrc = nullptr;   // nx: source-row coefficient q[m] of the substrate side
@@ -182,8 +182,8 @@ void zgemm(apf_ctx *c, bool ta, bool sym, int M, int N, int K, double2 alpha,
            const double2 *B, long long ldb, long long sB, double2 beta,
            double2 *C, long long ldc, long long sC, int batch, cudaStream_t s, int M2 = 0);
 void eliminate64(apf_ctx *c, cudaStream_t s);
-void launch_add(apf_ctx *c, double2 *T, const double2 *a, long long da, const double2 *b, long long db, long long n,
-                int nz, cudaStream_t s);
+void launch_add(apf_ctx *c, double2 *T, long long dT, const double2 *a, long long da, const double2 *b, long long db,
+                long long n, int nz, cudaStream_t s);
 void launch_zero(apf_ctx *c, void *dst, long long bytes, cudaStream_t s);
 
 void fields64(apf_ctx *c, cudaStream_t s);

@@ -137,10 +137,9 @@ extern "C" int apf_solve_S_noalloc(int nx, int ny, int npml_bot, int npml_top, d
     c.d_circ = (double2 *)carve(sizeof(double2) * 2 * n);
     c.d_tw = (double2 *)carve(sizeof(double2) * n / 2);
     c.d_G = (double2 *)carve(sizeof(double2) * h * n * n);
-    c.d_scr1 = (double2 *)carve(sizeof(double2) * n * n);
-    c.d_scr2 = (double2 *)carve(sizeof(double2) * n * n);
+    c.d_scr = (double2 *)carve(sizeof(double2) * n * n);
     c.d_E = (double2 *)carve(sizeof(double2) * h * ncol * n);
-    c.d_T = (double2 *)carve(sizeof(double2) * 2 * ncol * n);
+    c.d_T = (double2 *)carve(sizeof(double2) * ncol * n);
     c.d_fft = (double2 *)carve(sizeof(double2) * ncol * n);
     c.d_S = (double2 *)carve(sizeof(double2) * n_in * n_out);
     c.d_flags = (int *)carve(sizeof(int) * 4);

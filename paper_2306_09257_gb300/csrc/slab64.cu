@@ -16,6 +16,7 @@
 #include "leaf.cuh"
 
 #include <algorithm>
+#include <stdint.h>
 
 namespace {
 
@@ -325,12 +326,12 @@ __global__ void k_neg_offdiag(double2 *Bblk, double2 *Cblk, long long sX, long l
 }
 
 // T = a + b for the field rows of a back-substitution step (b null: T = a);
-// blockIdx.y = 1: the second row of the pair, at a + da, b + db, T + n.
-__global__ void k_add2(double2 *T, const double2 *a, long long da, const double2 *b, long long db, long long n) {
+// blockIdx.y = 1: the second row of the pair, at a + da, b + db, T + dT.
+__global__ void k_add2(double2 *T, long long dT, const double2 *a, long long da, const double2 *b, long long db, long long n) {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (blockIdx.y == 1) {
-        T += n;
+        T += dT;
         a += da;
         b += db;
     }
@@ -387,7 +388,7 @@ void zgemm(apf_ctx *c, bool ta, bool sym, int M, int N, int K, double2 alpha, co
 // which uses B = C^T and Ai = Ai^T, so four GEMMs per level, two of them with
 // a symmetric result.  Pivoting is confined to the diagonal leaf blocks.
 // nz (1 or 2) blocks sX apart are inverted by the same launches, with scratch
-// sS apart.
+// (n^2 / 3 elements at each of scr1 and scr2) sS apart.
 void invert_sym64(apf_ctx *c, double2 *X, long long sX, int nz, int n, long long ld, double2 *scr1, double2 *scr2,
                   long long sS, cudaStream_t s) {
     if (n <= LEAF64) {
@@ -411,26 +412,34 @@ void invert_sym64(apf_ctx *c, double2 *X, long long sX, int nz, int n, long long
     APF_LAUNCH(c, k_neg_offdiag, grid, 256, 0, s, B, C, sX, ld, V, sS, h);
 }
 
+// From a to b, which may lie in different allocations (all of them aligned to 256 bytes).
+static long long elements_between(const double2 *a, const double2 *b) {
+    return ((long long)(uintptr_t)b - (long long)(uintptr_t)a) / (long long)sizeof(double2);
+}
+
 // Block elimination of the slab rows from both ends towards the middle row
 // m = h / 2: rows 0, 1, .., m - 1 upwards (X_j = K_j - G_{j-1}) and rows h - 1, ..,
 // m + 1 downwards (X_j = K_j - G_{j+1}) are independent chains, so rows t and
 // h - 1 - t are inverted by the same launches; the middle row takes both
 // neighbours, X_m = K_m - G_{m-1} - G_{m+1}.  The same h inversions, but only
-// about h / 2 dependent steps of them, each with twice the parallel work.
+// about h / 2 dependent steps of them, each with twice the parallel work.  The
+// second chain's scratch lies in the middle row's block, which is not assembled
+// before both chains are done.
 void eliminate64(apf_ctx *c, cudaStream_t s) {
     const long long n = c->nx, nn = n * n;
     const int h = c->h, m = h / 2, top = h - 1 - m;  // top <= m
-    double2 *G = c->d_G;
+    double2 *G = c->d_G, *scr1 = c->d_scr, *scr2 = scr1 + nn / 2;
+    const long long dS = elements_between(scr1, G + m * nn);
     for (int t = 0; t < m; ++t) {
         const int u = h - 1 - t, nz = t < top ? 2 : 1;
         const long long d = (u - t) * nn;  // from row t's block to row u's
         launch_assemble64(c, t, nz == 2 ? u : -1, t > 0 ? G + (t - 1) * nn : nullptr, d + 2 * nn, nullptr, G + t * nn,
                           d, s);
-        invert_sym64(c, G + t * nn, d, nz, c->nx, n, c->d_scr1, c->d_scr2, nn / 2, s);
+        invert_sym64(c, G + t * nn, d, nz, c->nx, n, scr1, scr2, dS, s);
     }
     launch_assemble64(c, m, -1, m > 0 ? G + (m - 1) * nn : nullptr, 0, top > 0 ? G + (m + 1) * nn : nullptr, G + m * nn,
                       0, s);
-    invert_sym64(c, G + m * nn, 0, 1, c->nx, n, c->d_scr1, c->d_scr2, 0, s);
+    invert_sym64(c, G + m * nn, 0, 1, c->nx, n, scr1, scr2, 0, s);
 }
 
 // Slab fields from the inverses of eliminate64: the right-hand sides (inputs
@@ -440,6 +449,7 @@ void fields64(apf_ctx *c, cudaStream_t s) {
     const int nf = c->cf, na = c->ca, ncol = nf + na, h = c->h, m = h / 2, top = h - 1 - m;
     const long long nx = c->nx, L = (long long)ncol * nx, nn = nx * nx, of = (long long)nf * nx;
     double2 *E = c->d_Ew, *T = c->d_T;
+    const long long dT = elements_between(T, c->d_fft);  // the second row of a pair: in the transforms' buffer, not in use yet
     const double2 *G = c->d_G;
     const double2 one = cmk(1, 0), zero = cmk(0, 0);
     // inwards: Y_t = G_{t-1} Y_{t-1} (inputs) and Y_u = G_{u+1} Y_{u+1} (outputs), u = h - 1 - t
@@ -454,19 +464,19 @@ void fields64(apf_ctx *c, cudaStream_t s) {
                   E + t * L, nx, 0, 1, s, 0);
     }
     // the middle row, then outwards E_t = G_t (Y_t + E_{t+1}), E_u = G_u (Y_u + E_{u-1})
-    launch_add(c, T, E + m * L, 0, nullptr, 0, L, 1, s);
+    launch_add(c, T, 0, E + m * L, 0, nullptr, 0, L, 1, s);
     zgemm(c, false, false, ncol, c->nx, c->nx, one, T, nx, 0, G + m * nn, nx, 0, zero, E + m * L, nx, 0, 1, s);
     for (int t = m - 1; t >= 0; --t) {
         const int u = h - 1 - t, nz = t < top ? 2 : 1;
-        launch_add(c, T, E + t * L, (u - t) * L, E + (t + 1) * L, (u - t - 2) * L, L, nz, s);
-        zgemm(c, false, false, ncol, c->nx, c->nx, one, T, nx, L, G + t * nn, nx, (u - t) * nn, zero, E + t * L, nx,
+        launch_add(c, T, dT, E + t * L, (u - t) * L, E + (t + 1) * L, (u - t - 2) * L, L, nz, s);
+        zgemm(c, false, false, ncol, c->nx, c->nx, one, T, nx, dT, G + t * nn, nx, (u - t) * nn, zero, E + t * L, nx,
               (u - t) * L, nz, s);
     }
 }
 
-void launch_add(apf_ctx *c, double2 *T, const double2 *a, long long da, const double2 *b, long long db, long long n,
-                int nz, cudaStream_t s) {
-    APF_LAUNCH(c, k_add2, dim3((unsigned)((n + 255) / 256), nz), 256, 0, s, T, a, da, b, db, n);
+void launch_add(apf_ctx *c, double2 *T, long long dT, const double2 *a, long long da, const double2 *b, long long db,
+                long long n, int nz, cudaStream_t s) {
+    APF_LAUNCH(c, k_add2, dim3((unsigned)((n + 255) / 256), nz), 256, 0, s, T, dT, a, da, b, db, n);
 }
 
 void launch_zero(apf_ctx *c, void *dst, long long bytes, cudaStream_t s) {
