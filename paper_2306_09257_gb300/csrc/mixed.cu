@@ -1949,8 +1949,10 @@ extern "C" int apf_debug_inv32(apf_ctx *c, int n, float *re, float *im, int leaf
     w->leaf_variant = oldv;
     if (rc) return rc;
     if (e != cudaSuccess) return check_cuda(c, e, "debug inv32");
-    int fl = 0;
-    cudaMemcpy(&fl, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost);
+    int fl2[2] = {0, 0};
+    cudaMemcpy(fl2, c->d_flags, sizeof fl2, cudaMemcpyDeviceToHost);
+    const int fl = fl2[0];
+    c->stats.leaf_fallbacks = fl2[1];
     if (fl & FLAG_TIMEOUT) return set_err(c, APF_ETIMEOUT, "cgemm wait gave up");
     if (fl & FLAG_SINGULAR) return set_err(c, APF_ESINGULAR, "singular leaf");
     return APF_OK;

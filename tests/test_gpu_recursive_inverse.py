@@ -19,7 +19,7 @@ def symmetric(torch, n, seed, scale):
     return P + P.T
 
 
-def check(torch, X, leaf, levels):
+def check(torch, X, leaf, levels, planes=2):
     """X inverted with `leaf` as the hook takes it; returns the number of diagonal blocks that fell back."""
     from paper_2306_09257_gb300 import apf, build
     build.build_lib()
@@ -28,6 +28,7 @@ def check(torch, X, leaf, levels):
     L.apf_debug_inv32.argtypes = [f, ctypes.c_int, f, f, ctypes.c_int]
     n = X.shape[0]
     s = apf.Solver(0, "mixed")
+    s.set_elimination(planes, True)
     s.set_grid(n, 8 + 2 * 4 + 4, 4, 4, 8.0)
     s.set_eps(np.full((1, n), 1.5), 2.25, 1.0)
     s.set_channels([0], [0])
@@ -52,3 +53,29 @@ def test_blocks_below_64(n, leaf):
     X = symmetric(torch, n, n + leaf, 0.2)
     X[range(n), range(n)] += 2.0 + 0.5j
     check(torch, X, leaf, int(np.log2(n / max(8, leaf % 1000))))
+
+
+@pytest.mark.parametrize("planes", [2, 3])
+@pytest.mark.parametrize("leaf", [128, 100128])
+def test_pair_tiles(leaf, planes):
+    """n = 4096: the products of the top level have 2048 terms and rows and run on two-CTA tiles, with beta input,
+    the symmetric walk over the tiles, and float32, split and transposed outputs."""
+    torch = pytest.importorskip("torch")
+    n = 4096
+    X = symmetric(torch, n, leaf, 0.2)
+    X[range(n), range(n)] += 2.0 + 0.5j
+    check(torch, X, leaf, 5, planes)
+
+
+@pytest.mark.parametrize("n,leaf", [(128, 64), (256, 128), (512, 128)])
+def test_fallback_replaces_the_split_form(n, leaf):
+    """The first 32 x 32 block is zero while the leading diagonal block is well conditioned: its cluster inverse is
+    rejected after its split form has been written, and the products of the levels above read what pivoting over all
+    rows writes over it."""
+    torch = pytest.importorskip("torch")
+    X = symmetric(torch, n, n, 0.1)
+    X[range(leaf, n), range(leaf, n)] += 1.0
+    i = torch.arange(leaf)
+    X[i, (i + leaf // 2) % leaf] += 1.0
+    X[:32, :32] = 0.0
+    assert check(torch, X, leaf, int(np.log2(n / leaf))) == 1
