@@ -111,17 +111,14 @@ __global__ void k_mirror(const float *re, const float *im, long long ld, int R, 
     }
 }
 
-// A-layout pack of complex float64 rows (optionally the sum of two sources):
-// row r = [Re v(r,:), Im v(r,:)], v = s1 (+ s2).
-__global__ void k_pack64_A(const __grid_constant__ Tab<const double2 *> s1t, const __grid_constant__ Tab<const double2 *> s2t, long long ld, int R, int K,
+// A-layout pack of complex float64 rows: row r = [Re v(r,:), Im v(r,:)].
+__global__ void k_pack64_A(const __grid_constant__ Tab<const double2 *> srct, long long ld, int R, int K,
                            int nsplit, const __grid_constant__ Tab<__nv_bfloat16 *> outt, long long kp, long long plane_pitch) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     int r = blockIdx.y;
     if (k >= K || r >= R) return;
-    const double2 *__restrict__ s1 = s1t.v[blockIdx.z], *__restrict__ s2 = s2t.v[blockIdx.z];
     __nv_bfloat16 *out = outt.v[blockIdx.z];
-    double2 v = s1[(long long)r * ld + k];
-    if (s2) v = cadd(v, s2[(long long)r * ld + k]);
+    const double2 v = srct.v[blockIdx.z][(long long)r * ld + k];
     __nv_bfloat16 sa[3], sb[3];
     split_bf16((float)v.x, nsplit, sa);
     split_bf16((float)v.y, nsplit, sb);
@@ -920,16 +917,15 @@ Tab<T> tab(const Bat &bt, F f) {
     return t;
 }
 
-void pack64A_b(const Bat &bt, PackView *v, __nv_bfloat16 *const *dst, const double2 *const *s1,
-               const double2 *const *s2, long long ld, int R, int K, int nsplit, cudaStream_t s) {
+void pack64A_b(const Bat &bt, PackView *v, __nv_bfloat16 *const *dst, const double2 *const *src, long long ld, int R,
+               int K, int nsplit, cudaStream_t s) {
     const long long kp = round_up(2LL * K, 64);
     for (int b = 0; b < bt.n; ++b) {
         if (kp != 2LL * K) cudaMemsetAsync(dst[b], 0, sizeof(__nv_bfloat16) * R * kp * nsplit, s);
         v[b] = PackView{dst[b], R, kp, nsplit, (long long)R * kp};
     }
     dim3 grid((K + 255) / 256, R, bt.n);
-    APF_LAUNCH(bt.lead(), k_pack64_A, grid, 256, 0, s, tab<const double2 *>(bt, [&](int b) { return s1[b]; }),
-               tab<const double2 *>(bt, [&](int b) { return s2 ? s2[b] : nullptr; }), ld, R, K, nsplit,
+    APF_LAUNCH(bt.lead(), k_pack64_A, grid, 256, 0, s, tab<const double2 *>(bt, [&](int b) { return src[b]; }), ld, R, K, nsplit,
                tab<__nv_bfloat16 *>(bt, [&](int b) { return dst[b]; }), kp, (long long)R * kp);
 }
 
@@ -1331,7 +1327,6 @@ void mixed_init_attrs() {
     cgemm_init_attrs();
     cudaFuncSetAttribute(k_leaf_inv32, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * (int)sizeof(float2));
     cudaFuncSetAttribute(k_leaf32<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<128>(8));
-    cudaFuncSetAttribute(k_leaf32<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, leaf_smem_bytes<64>(8));
     cudaFuncSetAttribute(k_leaf_cluster<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem<4>));
     cudaFuncSetAttribute(k_leaf_cluster<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(lc::Smem<2>));
     cudaFuncSetAttribute(k_circ_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * (int)sizeof(double2));
@@ -1760,14 +1755,14 @@ int mixed_gradient_b(const Bat &bt, const double2 *const *Gamma, cudaStream_t s)
         pbdst[b] = wb->GB;
         Q[b] = PV{wb->sd[0].O32, wb->sd[0].O32 + (long long)nout * nx, nx};
     }
-    pack64A_b(bt, pa, padst, Gamma, nullptr, nin, nout, nin, ns, s);
+    pack64A_b(bt, pa, padst, Gamma, nin, nout, nin, ns, s);
     for (int j = 0; j < c->h; ++j) {
         for (int b = 0; b < nb; ++b) src[b] = bt.c[b]->d_E + j * L;
         pack64BT_b(bt, pb, pbdst, src, nx, nx, nin, ns, s);
         TcProblem pr[APF_MAX_BATCH];
         for (int b = 0; b < nb; ++b)
-            pr[b] = TcProblem{pa[b], pb[b], Q[b].re, Q[b].im, nullptr, nullptr, bt.c[b]->d_flags};
-        if (int rc = tc_gemm_n(c, nb, pr, ns, nout, 2 * nx, nx, 1.f, 0.f, nx, 0, s)) return rc;
+            pr[b] = TcProblem{pa[b], pb[b], Q[b].re, Q[b].im, bt.c[b]->d_flags};
+        if (int rc = tc_gemm_n(c, nb, pr, ns, nout, 2 * nx, nx, nx, s)) return rc;
         APF_LAUNCH(c, k_grad_rowdot32, dim3((nx + 31) / 32, 1, nb), 256, 0, s,
                    tab<const double2 *>(bt, [&](int b) { return (const double2 *)bt.c[b]->d_E; }),
                    tab<const float *>(bt, [&](int b) { return (const float *)Q[b].re; }),

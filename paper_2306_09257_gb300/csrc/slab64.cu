@@ -46,7 +46,7 @@ __global__ void k_assemble64(GridDev g, int row, int row2, const double *eps, co
     X[idx] = v;
 }
 
-// C = alpha op(A) op(B) + beta C, row-major complex float64, batched over
+// C = alpha op(A) B + beta C, row-major complex float64, batched over
 // blockIdx.z (M2 > 0: the second entry of the batch has M2 rows instead of M).
 //
 // What bounds it is the float64 pipe: 2 FMA per clock and SM on GB300, so a
@@ -71,7 +71,7 @@ struct ZArgs {
     long long lda, sA, ldb, sB, ldc, sC;
 };
 
-template <int T, bool TA, bool TB, bool SYM>
+template <int T, bool TA, bool SYM>
 __global__ void __launch_bounds__(256) k_zgemm(const ZArgs a) {
     constexpr int BK = 32, KS = 256 / (T * T), NL = (BK * T + 255) / 256;
     __shared__ double2 As[2][BK][T + 1], Bs[2][BK][T + 1];
@@ -96,11 +96,11 @@ __global__ void __launch_bounds__(256) k_zgemm(const ZArgs a) {
             const int e = tid + 256 * r;
             if (BK * T < 256 && e >= BK * T) break;
             const int ka = TA ? e / T : e % BK, ia = TA ? e % T : e / BK;  // contiguous along m / along k
-            const int kb = TB ? e % BK : e / T, jb = TB ? e / BK : e % T;  // contiguous along k / along n
+            const int kb = e / T, jb = e % T;                               // contiguous along n
             const int gi = m0 + ia, gj = n0 + jb;
             ra[r] = rb[r] = cmk(0.0, 0.0);
             if (gi < M && k0 + ka < K) ra[r] = TA ? A[(long long)(k0 + ka) * a.lda + gi] : A[(long long)gi * a.lda + k0 + ka];
-            if (gj < N && k0 + kb < K) rb[r] = TB ? B[(long long)gj * a.ldb + k0 + kb] : B[(long long)(k0 + kb) * a.ldb + gj];
+            if (gj < N && k0 + kb < K) rb[r] = B[(long long)(k0 + kb) * a.ldb + gj];
         }
     };
     fetch(0);
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k_zgemm(const ZArgs a) {
             const int e = tid + 256 * r;
             if (BK * T < 256 && e >= BK * T) break;
             As[buf][TA ? e / T : e % BK][TA ? e % T : e / BK] = ra[r];
-            Bs[buf][TB ? e % BK : e / T][TB ? e / BK : e % T] = rb[r];
+            Bs[buf][e / T][e % T] = rb[r];
         }
         __syncthreads();  // one per chunk: the other buffer was last read before the previous one
         if (k0 + BK < K) fetch(k0 + BK);
@@ -352,13 +352,12 @@ void launch_assemble64(apf_ctx *c, int row, int row2, const double2 *Gp, long lo
 namespace {
 
 template <int T>
-void launch_zgemm(apf_ctx *c, bool ta, bool tb, bool sym, int batch, const ZArgs &a, cudaStream_t s) {
+void launch_zgemm(apf_ctx *c, bool ta, bool sym, int batch, const ZArgs &a, cudaStream_t s) {
     const int mt = (std::max(a.M, a.M2) + T - 1) / T, nt = (a.N + T - 1) / T;
     dim3 grid(sym ? mt * (mt + 1) / 2 : nt, sym ? 1 : mt, batch);
-    if (sym && ta) APF_LAUNCH(c, (k_zgemm<T, true, false, true>), grid, 256, 0, s, a);
-    else if (sym) APF_LAUNCH(c, (k_zgemm<T, false, false, true>), grid, 256, 0, s, a);
-    else APF_LAUNCH(c, (k_zgemm<T, false, false, false>), grid, 256, 0, s, a);
-    (void)tb;
+    if (sym && ta) APF_LAUNCH(c, (k_zgemm<T, true, true>), grid, 256, 0, s, a);
+    else if (sym) APF_LAUNCH(c, (k_zgemm<T, false, true>), grid, 256, 0, s, a);
+    else APF_LAUNCH(c, (k_zgemm<T, false, false>), grid, 256, 0, s, a);
 }
 
 }  // namespace
@@ -376,9 +375,9 @@ void zgemm(apf_ctx *c, bool ta, bool sym, int M, int N, int K, double2 alpha, co
     };
     // at least two tiles per SM (304 on 152 SMs): with fewer, the last wave of
     // the larger tile costs more than the smaller tile's extra loads
-    if (tiles(16) >= 304) launch_zgemm<16>(c, ta, false, sym, batch, a, s);
-    else if (tiles(8) >= 304) launch_zgemm<8>(c, ta, false, sym, batch, a, s);
-    else launch_zgemm<4>(c, ta, false, sym, batch, a, s);
+    if (tiles(16) >= 304) launch_zgemm<16>(c, ta, sym, batch, a, s);
+    else if (tiles(8) >= 304) launch_zgemm<8>(c, ta, sym, batch, a, s);
+    else launch_zgemm<4>(c, ta, sym, batch, a, s);
 }
 
 // X <- X^-1 in place for complex-symmetric X (n a power of two), by the

@@ -5,15 +5,16 @@
 //
 // The GEMM is real: D[m][n] = sum_k A[m][k] B[n][k] with A and B "K-major"
 // (rows contiguous in k).  Complex products and extra precision are both
-// expressed through the operand layout, so one real kernel serves all of the
-// slab elimination:
+// expressed through the operand layout.  It serves the gradient contraction
+// Q_j = Gamma F_j in three planes (the elimination and the field sweeps have
+// their own kernel, cgemm.cu):
 //   * complex: A-row = [Re a, Im a], B-rows = [Re b, -Im b] (real part of the
 //     output) and [Im b, Re b] (imaginary part), so a complex m x k x n product
 //     is one real m x 2k x 2n product;
-//   * precision: each operand is split into 2 or 3 bf16 planes
-//     (x = x0 + x1 [+ x2]); the kernel walks "segments", one per retained
-//     plane product (x0 y0, x0 y1, x1 y0 [, x0 y2, x1 y1, x2 y0]), all
-//     accumulated in the same fp32 tensor-memory tile.
+//   * precision: each operand is split into bf16 planes (x = x0 + x1 + x2);
+//     the kernel walks "segments", one per retained plane product (x0 y0, x0 y1,
+//     x1 y0, x0 y2, x1 y1, x2 y0), all accumulated in the same fp32
+//     tensor-memory tile.
 // Operand planes live in 3-D tensor maps (k, row, plane), so rows past the
 // operand's end are zero-filled by TMA and no padding is needed in m or n.
 #include "apf_internal.h"
@@ -43,43 +44,20 @@ struct Layout {
 // Epilogue of one 32-column chunk of one accumulator row.
 __device__ __forceinline__ void store_chunk(const TcParams &p, int row, int col0, const uint32_t (&r)[32]) {
     if (row >= p.M) return;
-    const bool use_beta = (p.beta != 0.0f);
-    float *op;
-    const float *ip;
-    int cc0;
-    if (col0 < p.n_cplx) { op = p.out_re; ip = p.in_re; cc0 = col0; }
-    else { op = p.out_im; ip = p.in_im; cc0 = col0 - p.n_cplx; }
     const bool whole = (col0 + 32 <= p.N) && ((col0 < p.n_cplx) == (col0 + 31 < p.n_cplx));
-    float *dst = op + (long long)row * p.ldo + cc0;
-    const float *src = ip + (long long)row * p.ldi + cc0;
-    if (whole && ((((uintptr_t)dst) | (use_beta ? (uintptr_t)src : 0)) & 15) == 0) {
+    float *dst = (col0 < p.n_cplx ? p.out_re + col0 : p.out_im + (col0 - p.n_cplx)) + (long long)row * p.ldo;
+    if (whole && (((uintptr_t)dst) & 15) == 0) {
 #pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            float4 o;
-            o.x = p.alpha * __uint_as_float(r[4 * v + 0]);
-            o.y = p.alpha * __uint_as_float(r[4 * v + 1]);
-            o.z = p.alpha * __uint_as_float(r[4 * v + 2]);
-            o.w = p.alpha * __uint_as_float(r[4 * v + 3]);
-            if (use_beta) {
-                float4 c = *reinterpret_cast<const float4 *>(src + 4 * v);
-                o.x += p.beta * c.x; o.y += p.beta * c.y; o.z += p.beta * c.z; o.w += p.beta * c.w;
-            }
-            *reinterpret_cast<float4 *>(dst + 4 * v) = o;
-        }
+        for (int v = 0; v < 8; ++v)
+            *reinterpret_cast<float4 *>(dst + 4 * v) = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
+                                                                   __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         return;
     }
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
         const int col = col0 + i;
         if (col >= p.N) break;
-        float *o2;
-        const float *i2;
-        int cc;
-        if (col < p.n_cplx) { o2 = p.out_re; i2 = p.in_re; cc = col; }
-        else { o2 = p.out_im; i2 = p.in_im; cc = col - p.n_cplx; }
-        float v = p.alpha * __uint_as_float(r[i]);
-        if (use_beta) v += p.beta * i2[(long long)row * p.ldi + cc];
-        o2[(long long)row * p.ldo + cc] = v;
+        (col < p.n_cplx ? p.out_re + col : p.out_im + (col - p.n_cplx))[(long long)row * p.ldo] = __uint_as_float(r[i]);
     }
 }
 
@@ -312,8 +290,6 @@ int launch_variant(apf_ctx *c, bool wide, int nprob, const TcProblem *pb, const 
             return set_err(c, APF_ECUDA, "tensor map encode failed (M=%d N=%d kp=%lld)", base.M, base.N, pb[i].A.kp);
         TcParams q = base;
         q.out_re = pb[i].out_re; q.out_im = pb[i].out_im;
-        q.in_re = pb[i].in_re ? pb[i].in_re : pb[i].out_re;
-        q.in_im = pb[i].in_im ? pb[i].in_im : pb[i].out_im;
         q.flags = pb[i].flags;
         args.p[i] = q;
     }
@@ -325,8 +301,8 @@ int launch_variant(apf_ctx *c, bool wide, int nprob, const TcProblem *pb, const 
 
 }  // namespace
 
-int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int N, int n_cplx, float alpha,
-              float beta, long long ldo, long long ldi, cudaStream_t s) {
+int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int N, int n_cplx, long long ldo,
+              cudaStream_t s) {
     if (M <= 0 || N <= 0 || nprob <= 0) return APF_OK;
     if (nprob > APF_MAX_BATCH) return set_err(c, APF_EINVAL, "tc_gemm_n: %d problems > %d", nprob, APF_MAX_BATCH);
     if (!ensure_encode()) return set_err(c, APF_ECUDA, "cuTensorMapEncodeTiled unavailable");
@@ -338,9 +314,7 @@ int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int
     p.M = M; p.N = N; p.n_cplx = n_cplx;
     p.kblocks = (int)(kp / BK);
     p.seg_pairs = tc_seg_pairs(nsplit, &p.nseg);
-    p.alpha = alpha; p.beta = beta;
     p.ldo = ldo;
-    p.ldi = pb[0].in_re ? ldi : ldo;
     // Tile width: score the wave utilisation of 256- and 128-wide tiles.
     static int num_sms = 0;
     if (!num_sms) {

@@ -19,11 +19,8 @@ struct TcParams {
     int M, N, n_cplx;
     int kblocks, nseg;
     uint32_t seg_pairs;
-    float alpha, beta;
     float *out_re, *out_im;
     long long ldo;
-    const float *in_re, *in_im;
-    long long ldi;
     int *flags;
 };
 
@@ -36,11 +33,10 @@ struct TcArgs {
     int nprob;
 };
 
-// One product of a batch: operands, output (and beta input) planes, error flags.
+// One product of a batch: operands, output planes, error flags.
 struct TcProblem {
     PackView A, B;
     float *out_re, *out_im;
-    const float *in_re, *in_im;
     int *flags;
 };
 
@@ -49,11 +45,11 @@ bool tc_make_map(CUtensorMap *m, const void *base, long long cols, long long row
                  long long row_pitch, long long plane_pitch, int box_rows, int box_planes);
 void tc_init_attrs();
 
-// out = alpha * (A B^T) + beta * in, where output column col < n_cplx goes to
+// out = A B^T, where output column col < n_cplx goes to
 // the real plane (column col) and col >= n_cplx to the imaginary plane
 // (column col - n_cplx).  A: M rows; B: N rows; both with the same kp.  Used by
 // the gradient contraction (three planes); the slab elimination and the field
 // sweeps use cgemm.h.
 // nprob (<= APF_MAX_BATCH) products of the same shape in one launch.
-int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int N, int n_cplx, float alpha,
-              float beta, long long ldo, long long ldi, cudaStream_t s);
+int tc_gemm_n(apf_ctx *c, int nprob, const TcProblem *pb, int nsplit, int M, int N, int n_cplx, long long ldo,
+              cudaStream_t s);
