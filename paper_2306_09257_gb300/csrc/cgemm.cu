@@ -63,16 +63,14 @@ struct CgArgs {
 // product, and the sweeps (unlike the elimination, where it makes no difference)
 // set how far one refinement sweep gets: 4096 x 260, two sweeps, residual 8e-11
 // without and 2e-11 with it.  PASSES: for the same reason the pair tile adds up at
-// most 16 k blocks in the tensor memory, 8 of a product of more than 64 (K > 4096),
-// and the passes are added in registers; with one plane product per stage the
-// smaller products are a pass of their own.  Residual of the first solve and after
-// a sweep, time of an evaluation, two planes: 4096 x 260 one pass 3.9e-4, 1.0e-7;
-// 32 blocks 2.5e-4, 4.0e-8, 55.7 ms; 16 blocks 2.0e-4, 1.5e-8, 55.9 ms; 8 blocks
-// 1.8e-4, 1.0e-8, 57.1 ms; 8192 x 280 32 blocks 3.7e-4, 9.0e-8, 276 ms; 16 blocks
-// 3.0e-4, 4.2e-8, 279 ms; 8 blocks 2.8e-4, 3.1e-8, 286 ms (the one-ended order of
-// elimination with 256-wide tiles left 2.4e-4, 3.3e-8 and 2.8e-4, 4.0e-8).  Three
-// planes, 4096 x 260: one pass 3.3e-4, 9.0e-8, 97.0 ms; 16 blocks 9.7e-5, 8.1e-9,
-// 98.8 ms (before: 2.3e-4, 4.2e-8).
+// most 16 k blocks in the tensor memory (and half of a product of up to 32), and the
+// passes are added in registers; with one plane product per stage the smaller
+// products are a pass of their own.  Residual of the first solve and after a sweep,
+// time of an evaluation to 1e-10: 4096 x 260 in one pass 3.9e-4, 1.0e-7; passes of 32
+// blocks 2.7e-4, 4.0e-8, 55.2 ms; of 16 2.1e-4, 1.7e-8, 55.8 ms; of 8 no better by more
+// than a third, 57.1 ms.  8192 x 280: 32 blocks 3.9e-4, 1.1e-7, 274 ms; 16 blocks 3.2e-4,
+// 4.6e-8, 278 ms.  Three planes, 4096 x 260: one pass 3.6e-4, 1.0e-7, 96.6 ms; 16 blocks
+// 9.9e-5, 8.6e-9, 98.2 ms.
 // MERGED: a product with fewer than 128 columns takes the tensor core as long as one
 // with 128 (64 clocks per 16 of K), so the 128 x 32 tile multiplies x0 by both planes
 // of y at once, which leaves the cross products in accumulators of their own: 4
@@ -680,7 +678,7 @@ int dispatch(apf_ctx *c, int nprob, const CgProblem *pb, int planes, int M, int 
     args.beta = beta;
     args.sym = sym ? 1 : 0;
     args.t_block = pb[0].t_block;
-    args.passes = std::max(2, args.kblocks / (args.kblocks > 64 ? 8 : 16));  // see PASSES
+    args.passes = std::max(2, args.kblocks / 16);  // see PASSES
     if (planes != 2 && args.nseg > 1) args.passes++;  // the smaller products
     bool vec = N % 16 == 0;
     for (int i = 0; i < nprob; ++i) {
