@@ -62,7 +62,7 @@ __device__ __forceinline__ double2 crecip(double2 d) {
 // it: so one warp per SM (nx / 16 blocks), the two sides apart, one division
 // per row instead of three, and in the unstretched rows (s = 1, where the
 // couplings are 1 and the diagonal is real) none of the complex products with
-// them.  Measured at 1024 x 240: 462 -> 37 us; 64 x 100: 187 -> 18 us.
+// them.  Measured inside a solve at 1024 x 240: 462 -> 65 us; 64 x 100: 187 -> 31 us.
 __global__ void __launch_bounds__(32) k_boundary_sweep(GridDev g, const double2 *__restrict__ st, double2 *modes) {
     const int m = blockIdx.x * 32 + threadIdx.x;
     if (m >= g.nx) return;

@@ -373,7 +373,7 @@ __device__ void leaf_gj_regs2(float *re, float *im, long long ld, int *flags) {
 // Updating the next pivot block alone first, and the rest beside its inversion,
 // is no faster: the inversion then takes twice as long (it shares the SM's issue slots).
 // Measured: 34 us per 128 block; 60 us with every CTA inverting the pivot block (400 clocks
-// a pivot) after copying the panel, 93 us in one CTA.  64 block: 18 us; 56 us by pivots
+// a pivot) after copying the panel, 93 us in one CTA.  64 block: 15 us; 56 us by pivots
 // over all rows in one CTA.
 // ---------------------------------------------------------------------------
 namespace lc {
